@@ -362,10 +362,10 @@ typedef struct raypc_batch raypc_batch;
 
 /* A reusable batch of up to max_views views (1..4096). It owns a device view
  * table, per-view classification bitmasks and sub-brick lists, per-view cell
- * classes, a tile counter and a CUDA graph of the batched launch (table
- * upload, per-view brick and sub-brick classification, per-view cell classes,
- * the empty-space distance of every view that renders with skipping, one
- * persistent render kernel), captured on first use and replayed afterwards.
+ * classes and a CUDA graph of the batched launch (table upload, per-view brick
+ * and sub-brick classification, per-view cell classes, the empty-space distance
+ * of every view, and one render node per view, side by side), captured on first
+ * use and replayed afterwards with the nodes' parameters set to the views.
  * Allocates device and pinned host memory; the per-view buffers are allocated
  * for a view slot on its first use and grown for larger levels: n^3 * 2 bytes
  * of cell classes plus about n^3 / 10 bytes of masks, lists and distances per
@@ -379,9 +379,8 @@ raypc_status raypc_batch_destroy(raypc_batch *batch);
  * function, and the same storage dtype. The tile variant of the launch is view
  * 0's (after RAYPC_AUTO resolution); skipping is chosen per view, and a view
  * with skipping jumps by the empty-space distance of its own classification,
- * as a single-frame render does. Work is split into 16x8-pixel tiles
- * pulled dynamically by persistent thread blocks, so large and small images
- * balance across the GPU. The call returns after enqueueing; it may wait for
+ * as a single-frame render does. The views' renders run side by side in
+ * 16x8-pixel blocks, so large and small images balance across the GPU. The call returns after enqueueing; it may wait for
  * the batch submitted two calls earlier on this batch object to finish (the
  * view table is double-buffered). Concurrent calls on one batch object must be
  * serialised by the caller. */
@@ -401,8 +400,8 @@ raypc_status raypc_render_batch(raypc_batch *batch, const raypc_view *views, int
  * admitted work into one batched render launch per loop turn and free stream
  * (a request's coarse and full passes go into the same launch; coarse passes
  * and small images first), so requests that arrive while others run join the
- * next launch and their work overlaps on the device. The persistent kernel
- * publishes each finished view through a record in mapped host memory, so a
+ * next launch and their work overlaps on the device. Every view's render
+ * publishes its end through a record in mapped host memory, so a
  * request completes when its own passes are done, not when its whole launch
  * is. Per-request timestamps are recorded. A request's results are identical to rendering /
  * histogramming it alone. Besides the output pool, each stream's batch holds

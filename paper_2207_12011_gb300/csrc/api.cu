@@ -51,7 +51,7 @@ namespace {
 void free_level(Level& L) {
     void* ptrs[] = {L.cells, L.pairs, L.bmin, L.bmax, L.active, L.skippable, L.list, L.n_active, L.pass_count,
                     L.sbmin, L.sbmax, L.sactive, L.slist, L.scount, L.cls, L.tf_active, L.tf_sactive,
-                    L.sdist, L.sdist_tmp};
+                    L.sdist};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     L = Level{};
@@ -60,13 +60,13 @@ void free_level(Level& L) {
 void free_bricks(Level& L) {
     void* ptrs[] = {L.bmin, L.bmax, L.active, L.skippable, L.list, L.n_active, L.pass_count,
                     L.sbmin, L.sbmax, L.sactive, L.slist, L.scount, L.tf_active, L.tf_sactive,
-                    L.sdist, L.sdist_tmp};
+                    L.sdist};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     L.bmin = L.bmax = L.sbmin = L.sbmax = nullptr;
     L.active = L.skippable = L.list = L.n_active = L.sactive = L.slist = L.scount = nullptr;
     L.tf_active = L.tf_sactive = nullptr;
-    L.sdist = L.sdist_tmp = nullptr;
+    L.sdist = nullptr;
     L.sdist_of = nullptr;
     L.pass_count = nullptr;
     L.bricks = L.classified = L.cls_valid = false;
@@ -340,6 +340,9 @@ raypc_status make_render_args(Volume* V, Level* L, const raypc_camera* cam, int 
     a.lv.n = L->n;
     a.lv.nb = L->nb;
     a.lv.nsb = L->nsb;
+    a.lv.pd = subbrick_pad(L->n);
+    a.lv.pbias = narrow_bias(L->n);
+    a.lv.plast = (uint32_t)(padded_bytes(L->n) - 1);
     a.lv.sactive = L->sactive;
     a.lv.bmin = L->bmin;
     a.lv.bmax = L->bmax;
@@ -352,6 +355,17 @@ raypc_status make_render_args(Volume* V, Level* L, const raypc_camera* cam, int 
     a.w = w;
     a.h = h;
     a.dt = dt;
+    // samples that stay in a box of inactive sub-bricks extending 4 (D - 1) cells beyond the current
+    // sub-brick, D >= 2, 4, kDistCap (the lattice moves a cell index by at most dt n/2 cells per
+    // sample on any axis, 1/16 cell covers its rounding); whole numbers, 0 for coarse steps
+    const float cells_per_step = dt * (0.5f * (float)L->n);
+    const int box[3] = {1, 3, kDistCap - 1};
+    for (int i = 0; i < 3; ++i) a.jump[i] = floorf((4.0f * (float)box[i] - 0.0625f) / cells_per_step);
+    // A sample's |p| exceeds r_out by at most about |eye| 2^-20 (rounding of the sphere interval, t
+    // and p), so -1 <= u < n on every axis when r_out <= 1 and |eye| n < 2^17.
+    const float eye_max = fmaxf(fabsf(cam->eye[0]), fmaxf(fabsf(cam->eye[1]), fabsf(cam->eye[2])));
+    const size_t plane_bytes = (size_t)L->n * L->n * L->n * 2 * elem_size(V->dtype);
+    a.narrow = V->r_out <= 1.0f && eye_max * (float)L->n < 131072.0f && plane_bytes < ((size_t)1 << 32);
     a.rin2 = V->r_in * V->r_in;
     a.rout2 = V->r_out * V->r_out;
     finish_position_brush(a);
@@ -683,28 +697,29 @@ raypc_status raypc_set_tf(raypc_ctx* ctx, int vol, const float* rgbs, int color_
     return RAYPC_OK;
 }
 
-// With tf_skip, the render reads the activity bits ANDed with the TF visibility of
-// the level's bricks and sub-bricks (computed for this render on its stream).
 // Empty-space distance of the sub-bricks under the activity bits the render reads (the
-// brush's, or the TF-visible ones with tf_skip), for renders with skipping.
+// brush's, or the TF-visible ones with tf_skip): the grid the march searches. A render
+// without skipping only needs the activity, and reads the bits where the grid cannot be had.
 static raypc_status ensure_distance(raypc_ctx* ctx, Volume* V, Level& L, RenderArgs& a, bool recompute,
                                     cudaStream_t s) {
-    if (!a.skip) return RAYPC_OK;
     if (!L.sdist) {
-        const size_t bytes = L.nsbricks();
-        raypc_status st = ctx->alloc((void**)&L.sdist, bytes, &V->bytes);
-        if (st == RAYPC_OK) st = ctx->alloc((void**)&L.sdist_tmp, bytes, &V->bytes);
-        if (st) return st;
+        raypc_status st = ctx->alloc((void**)&L.sdist, padded_bytes(L.n), &V->bytes);
+        if (st) {
+            L.sdist = nullptr;
+            return a.skip ? st : RAYPC_OK;
+        }
         L.sdist_of = nullptr;
     }
     if (recompute || L.sdist_of != a.lv.sactive) {
-        CK(launch_subbrick_distance(a.lv.sactive, L.nsb, L.sdist, L.sdist_tmp, s), "empty-space distance");
+        CK(launch_subbrick_distance(a.lv.sactive, L.n, L.sdist, false, s), "empty-space distance");
         L.sdist_of = a.lv.sactive;
     }
     a.lv.sdist = L.sdist;
     return RAYPC_OK;
 }
 
+// With tf_skip, the render reads the activity bits ANDed with the TF visibility of
+// the level's bricks and sub-bricks (computed for this render on its stream).
 static raypc_status apply_tf_skip(Volume* V, Level& L, const raypc_render_opts* opts, RenderArgs& a, cudaStream_t s) {
     if (!opts || !opts->tf_skip) return RAYPC_OK;
     TfVisArgs t{};
@@ -1129,11 +1144,7 @@ raypc_status raypc_get_skip_distance(raypc_ctx* ctx, int vol, int lod, uint8_t* 
     if (V->stale) return fail(RAYPC_ERR_INVALID_ARG, "volume updated: raypc_build_bricks must run first");
     cudaStream_t s = (cudaStream_t)stream;
     if ((st = ensure_classified(V, *L, s))) return st;
-    RenderArgs a{};
-    a.skip = 1;
-    a.lv.sactive = L->sactive;
-    if ((st = ensure_distance(ctx, V, *L, a, false, s))) return st;
-    CK(cudaMemcpyAsync(out_dev, L->sdist, L->nsbricks(), cudaMemcpyDeviceToDevice, s), "copy skip distance");
+    CK(launch_subbrick_distance(L->sactive, L->n, out_dev, true, s), "empty-space distance");
     return RAYPC_OK;
 }
 

@@ -1,14 +1,16 @@
 // Batched rendering: many views (each with its own camera, image size and
-// brush box) rendered by one persistent launch, captured once in a CUDA graph
-// and replayed with new view tables.
+// brush box) in one CUDA graph, captured once and replayed with new view
+// tables and render parameters.
 //
 // Per batch the host fills a view table (double-buffered in pinned memory);
-// the graph uploads it, zeroes the tile counter and the per-view selectivity
-// counts, classifies every view's bricks under that view's brush into the
-// view's own bitmasks, and runs the persistent render kernel, whose blocks
-// pull 16x8-pixel tiles of all views from one atomic counter. Kernel
-// parameters never change between batches (everything variable lives in the
-// table), so the graph is captured once per table buffer and storage dtype.
+// the graph uploads it, zeroes the per-view counters, classifies every view's
+// sub-bricks and cells under that view's brush into the view's own buffers, and
+// renders the views in nodes side by side, so that the blocks of the next views
+// fill the GPU while the last blocks of one finish. The table's address never
+// changes; the render nodes' kernels, grids and parameters are set on the
+// instantiated graph before each replay, and the nodes beyond the batch's views
+// are switched off. A graph is captured per table buffer and storage dtype, with
+// a power of two of render nodes.
 #include <vector>
 
 #include "runtime.h"
@@ -20,7 +22,6 @@ struct raypc_batch {
     int max_views = 0;
     size_t table_bytes = 0;
     char* d_table = nullptr;          // BatchHeader, then max_views BatchView (device)
-    unsigned* d_counter = nullptr;    // tile counter
     unsigned* d_pass = nullptr;       // max_views x kMaxVars selectivity counts
     unsigned* d_tiles = nullptr;      // max_views finished-tile counters, then max_views sub-brick list lengths
     ViewDone* h_done[2] = {nullptr, nullptr};   // mapped pinned completion records per table slot
@@ -37,7 +38,11 @@ struct raypc_batch {
     std::vector<size_t> cls_cells;    // capacity (cells) per slot
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t exec[2] = {nullptr, nullptr};
-    int exec_key[2] = {-1, -1};       // dtype * 16 + variant of the captured graph
+    int exec_dtype[2] = {-1, -1};     // storage dtype of the captured graph
+    cudaGraph_t graph[2] = {nullptr, nullptr};   // the captured graph (kept: it owns the node handles)
+    std::vector<cudaGraphNode_t> nodes[2];   // its render nodes, the first `enabled` of them switched on
+    int enabled[2] = {0, 0};
+    std::vector<ViewLaunch> launch;   // their parameters, as filled for a call
     size_t charged = 0;
 };
 
@@ -57,6 +62,7 @@ void release(raypc_batch* b) {
     wait_idle(b);
     for (int i = 0; i < 2; ++i) {
         if (b->exec[i]) cudaGraphExecDestroy(b->exec[i]);
+        if (b->graph[i]) cudaGraphDestroy(b->graph[i]);
         if (b->h_table[i]) cudaFreeHost(b->h_table[i]);
         if (b->h_done[i]) cudaFreeHost(b->h_done[i]);
         if (b->done[i]) cudaEventDestroy(b->done[i]);
@@ -66,39 +72,62 @@ void release(raypc_batch* b) {
     for (uint16_t* p : b->cls)
         if (p) cudaFree(p);
     if (b->d_table) cudaFree(b->d_table);
-    if (b->d_counter) cudaFree(b->d_counter);
     if (b->d_pass) cudaFree(b->d_pass);
     if (b->d_tiles) cudaFree(b->d_tiles);
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
     if (b->ctx) b->ctx->used -= b->charged < b->ctx->used ? b->charged : b->ctx->used;
 }
 
-raypc_status capture(raypc_batch* b, int slot, int dtype, int variant, bool depth) {
+raypc_status capture(raypc_batch* b, int slot, int dtype) {
     int dev = 0, sms = 0;
     CK(cudaGetDevice(&dev), "cudaGetDevice");
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
-    const int blocks = sms * render_batch_blocks_per_sm(dtype, variant, depth);
     const unsigned cls_blocks = (unsigned)sms * 8u;
     if (b->exec[slot]) {
         cudaGraphExecDestroy(b->exec[slot]);
         b->exec[slot] = nullptr;
     }
+    if (b->graph[slot]) {
+        cudaGraphDestroy(b->graph[slot]);
+        b->graph[slot] = nullptr;
+    }
+    b->nodes[slot].clear();
     cudaStream_t s = b->cap_stream;
     CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal), "begin graph capture");
     cudaError_t e = cudaMemcpyAsync(b->d_table, b->h_table[slot], b->table_bytes, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(b->d_counter, 0, sizeof(unsigned), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_pass, 0, sizeof(unsigned) * kMaxVars * b->max_views, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_tiles, 0, sizeof(unsigned) * 2 * b->max_views, s);
     if (e == cudaSuccess)
-        e = launch_render_batch(hdr_of(b->d_table), views_of(b->d_table), b->d_counter, depth, dtype, variant,
-                                cls_blocks, blocks, s);
+        e = launch_view_classes(hdr_of(b->d_table), views_of(b->d_table), dtype, cls_blocks, s);
     cudaGraph_t graph = nullptr;
     cudaError_t e2 = cudaStreamEndCapture(s, &graph);
     if (e == cudaSuccess) e = e2;
+    // the render nodes follow the last captured launch, side by side
+    cudaGraphNode_t last = nullptr;
+    if (e == cudaSuccess) {
+        size_t n = 0;
+        e = cudaGraphGetNodes(graph, nullptr, &n);
+        std::vector<cudaGraphNode_t> all(n);
+        if (e == cudaSuccess) e = cudaGraphGetNodes(graph, all.data(), &n);
+        for (size_t i = 0; i < n && e == cudaSuccess && !last; ++i) {
+            size_t after = 0;
+            e = cudaGraphNodeGetDependentNodes(all[i], nullptr, nullptr, &after);
+            if (e == cudaSuccess && after == 0) last = all[i];
+        }
+    }
+    size_t count = 1;
+    while (count < b->launch.size()) count *= 2;
+    for (size_t i = 0; i < count && e == cudaSuccess; ++i) {
+        const cudaKernelNodeParams p = render_view_node(b->launch[i < b->launch.size() ? i : 0], dtype);
+        cudaGraphNode_t node = nullptr;
+        e = cudaGraphAddKernelNode(&node, graph, &last, 1, &p);
+        b->nodes[slot].push_back(node);
+    }
     if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec[slot], graph, 0);
-    if (graph) cudaGraphDestroy(graph);
+    b->graph[slot] = graph;
     if (e != cudaSuccess) return cuda_fail(e, "batch graph capture");
-    b->exec_key[slot] = dtype * 16 + variant + (depth ? 8 : 0);
+    b->exec_dtype[slot] = dtype;
+    b->enabled[slot] = (int)count;
     return RAYPC_OK;
 }
 
@@ -126,7 +155,6 @@ raypc_status raypc_batch_create(raypc_ctx* ctx, int max_views, raypc_batch** out
     b->cls.assign(max_views, nullptr);
     b->cls_cells.assign(max_views, 0);
     raypc_status st = ctx->alloc((void**)&b->d_table, b->table_bytes, &b->charged);
-    if (st == RAYPC_OK) st = ctx->alloc((void**)&b->d_counter, sizeof(unsigned), &b->charged);
     if (st == RAYPC_OK) st = ctx->alloc((void**)&b->d_pass, sizeof(unsigned) * kMaxVars * max_views, &b->charged);
     if (st == RAYPC_OK) st = ctx->alloc((void**)&b->d_tiles, sizeof(unsigned) * 2 * max_views, &b->charged);
     cudaError_t e = cudaSuccess;
@@ -174,10 +202,8 @@ raypc_status raypc_render_batch(raypc_batch* b, const raypc_view* views, int nvi
     BatchHeader* H = hdr_of(b->h_table[slot]);
     BatchView* T = views_of(b->h_table[slot]);
     int dtype = -1, variant = 0;
-    // a depth output in any view selects the depth instance of the kernel (8x4 tiles)
-    bool depth = false;
-    for (int i = 0; i < nviews; ++i) depth = depth || views[i].opts.depth_dev != nullptr;
-    unsigned long long cls = 0, dist = 0;
+    unsigned long long cls = 0;
+    int dist = 0;
     long long tiles = 0;
     raypc_status st;
     for (int i = 0; i < nviews; ++i) {
@@ -193,12 +219,15 @@ raypc_status raypc_render_batch(raypc_batch* b, const raypc_view* views, int nvi
         if ((st = brush_from_host(V, q.lo, q.hi, q.active_mask, &bv.a.brush))) return st;
         if ((st = pos_from_host(q.pos_lo, q.pos_hi, q.pos_mask, &bv.a.brush))) return st;
         finish_position_brush(bv.a);
-        if (i == 0) variant = depth ? 1 : bv.a.variant;
+        if (i == 0) variant = bv.a.variant;
         bv.a.variant = variant;
+        tiles += (long long)((q.w + block_tile_w(variant) - 1) / block_tile_w(variant)) *
+                 ((q.h + block_tile_h(variant) - 1) / block_tile_h(variant));
+        if (tiles > 0x7fffffffLL) return fail(RAYPC_ERR_INVALID_ARG, "batch has more than 2^31 tiles");
         // per view: brick and sub-brick activity bits, the list of active sub-bricks, and
-        // the sub-bricks' empty-space distance with its scratch (bytes)
+        // the sub-bricks' padded empty-space distance (bytes)
         const size_t nsub = L->nsbricks();
-        const size_t words = L->nwords(), need = words + L->nswords() + nsub + (2 * nsub + 3) / 4;
+        const size_t words = L->nwords(), need = words + L->nswords() + nsub + (padded_bytes(L->n) + 3) / 4;
         if (b->bits_words[i] < need) {
             // growing a slot's masks: no batch may still be reading the old ones
             wait_idle(b);
@@ -213,11 +242,9 @@ raypc_status raypc_render_batch(raypc_batch* b, const raypc_view* views, int nvi
         bv.a.lv.active = b->bits[i];
         bv.a.lv.sactive = b->bits[i] + words;
         bv.slist = b->bits[i] + words + L->nswords();
-        uint8_t* dist_buf = reinterpret_cast<uint8_t*>(b->bits[i] + words + L->nswords() + nsub);
-        bv.a.lv.sdist = bv.a.skip ? dist_buf : nullptr;   // renders with skipping jump by the distance
-        bv.stmp = dist_buf + nsub;
+        bv.a.lv.sdist = reinterpret_cast<uint8_t*>(b->bits[i] + words + L->nswords() + nsub);
         bv.dist_begin = dist;
-        if (bv.a.skip) dist += (nsub + 31) & ~(size_t)31;
+        dist += subbrick_distance_tiles(L->n);
         bv.scount = b->d_tiles + b->max_views + i;
         const size_t cells = (size_t)L->n * L->n * L->n;
         if (b->cls_cells[i] < cells) {
@@ -240,29 +267,33 @@ raypc_status raypc_render_batch(raypc_batch* b, const raypc_view* views, int nvi
         bv.cls_begin = cls;
         bv.cls_sub = (unsigned long long)words * 32;
         cls += (unsigned long long)(words + L->nswords()) * 32;
-        bv.tiles_x = (q.w + block_tile_w(variant) - 1) / block_tile_w(variant);
-        bv.tile_begin = (int)tiles;
-        bv.ntiles = bv.tiles_x * ((q.h + block_tile_h(variant) - 1) / block_tile_h(variant));
-        tiles += (long long)bv.ntiles;
-        bv.tile_done = b->d_tiles + i;
-        bv.done = b->d_done[slot] + i;
-        bv.seq = b->seq + 1;
-        if (tiles > 0x7fffffffLL) return fail(RAYPC_ERR_INVALID_ARG, "batch has more than 2^31 tiles");
         T[i] = bv;
     }
     H->nviews = nviews;
-    H->total_tiles = (int)tiles;
     H->cls_total = cls;
     H->dist_total = dist;
-    if (!b->exec[slot] || b->exec_key[slot] != dtype * 16 + variant + (depth ? 8 : 0))
-        if ((st = capture(b, slot, dtype, variant, depth))) return st;
+    b->launch.resize(nviews);
+    for (int i = 0; i < nviews; ++i) {
+        b->launch[i].a = T[i].a;
+        b->launch[i].t = ViewTiles{b->d_tiles + i, b->d_done[slot] + i, b->seq + 1};
+    }
+    if (!b->exec[slot] || b->exec_dtype[slot] != dtype || b->nodes[slot].size() < (size_t)nviews)
+        if ((st = capture(b, slot, dtype))) return st;
+    for (int i = 0; i < nviews; ++i) {
+        const cudaKernelNodeParams p = render_view_node(b->launch[i], dtype);
+        CK(cudaGraphExecKernelNodeSetParams(b->exec[slot], b->nodes[slot][i], &p), "batch render parameters");
+    }
+    for (; b->enabled[slot] < nviews; ++b->enabled[slot])
+        CK(cudaGraphNodeSetEnabled(b->exec[slot], b->nodes[slot][b->enabled[slot]], 1), "batch render node");
+    for (; b->enabled[slot] > nviews; --b->enabled[slot])
+        CK(cudaGraphNodeSetEnabled(b->exec[slot], b->nodes[slot][b->enabled[slot] - 1], 0), "batch render node");
     CK(cudaGraphLaunch(b->exec[slot], (cudaStream_t)stream), "batch graph launch");
     CK(cudaEventRecord(b->done[slot], (cudaStream_t)stream), "batch completion event");
     b->used[slot] = true;
     b->last_slot = slot;
     b->seq += 1;
     b->cur ^= 1;
-    count_launches(6);
+    count_launches(3 + nviews);
     return RAYPC_OK;
 }
 

@@ -178,12 +178,32 @@ struct LevelArgs {
     const float* bmax;
     const uint32_t* active;    // bitmask, ceil(nb^3/32) words
     const uint32_t* sactive;   // sub-brick bitmask, ceil(nsb^3/32) words
-    const uint8_t* sdist;      // optional: empty-space distance of the sub-bricks under sactive (see
-                               // launch_subbrick_distance); renders with skipping jump by it
+    const uint8_t* sdist;      // optional: padded empty-space distance of the sub-bricks under sactive
+                               // (see launch_subbrick_distance); the march searches it, and renders
+                               // with skipping jump by it
+    int pd;                    // edge of the padded grid, subbrick_pad(n)
+    uint32_t pbias;            // narrow march: added to the packed index (see narrow_bias)
+    uint32_t plast;            // pd^3 - 1
 };
 
 // Cap of the sub-brick empty-space distance (sub-bricks).
 constexpr int kDistCap = 8;
+
+// The padded distance grid of a level of edge n holds, for e = -1 .. (n-1)/4 on
+// every axis, the distance of sub-brick min(max(e, 0), (n-2)/4) at index e + 1:
+// e = floor(u / 4) of an unclamped grid coordinate -1 <= u < n then finds the
+// sub-brick of the clamped cell index min(max(floor(u), 0), n-2).
+__host__ __device__ constexpr int subbrick_pad(int n) { return ((n - 1) >> 2) + 2; }
+constexpr size_t padded_bytes(int n) { return (size_t)subbrick_pad(n) * subbrick_pad(n) * subbrick_pad(n); }
+
+// Sample search of the march: bits of 1.5 * 2^25 + 4 e are kNarrowOne + e, so
+// with b_a those bits on each axis the padded index is (bz pd + by) pd + bx plus
+// this constant (mod 2^32).
+constexpr uint32_t kNarrowOne = 0x4c400000u;
+constexpr uint32_t narrow_bias(int n) {
+    const uint32_t pd = (uint32_t)subbrick_pad(n);
+    return (1u - kNarrowOne) * (pd * pd + pd + 1u);
+}
 
 // Implicit position axes (x, y, z, radius) usable in brushes and as PC axes;
 // PC axis id kPosAxisBase + a names position axis a.
@@ -237,6 +257,9 @@ struct RenderArgs {
     float tf_lo, tf_scale;        // s = (v - tf_lo) * tf_scale
     float bg[4];
     int ert, skip;
+    float jump[3];                // samples to skip at distance >= 2, 4 and kDistCap (whole numbers)
+    int narrow;                   // every sample has -1 <= u < n on each axis (r_out <= 1, a nearby eye)
+                                  // and a pair plane has less than 2^32 bytes
     int variant;                  // 1..kNumVariants (tile shape of the launch)
     uint32_t jit_seed, jit_pass;  // progressive pass (0: the fixed lattice t0 + (k + 1/2) dt)
     float4* accum;                // optional running mean of the passes ([h][w], updated in place)
@@ -260,12 +283,12 @@ struct ViewDone {
     unsigned long long stats[kNStats];
 };
 
-// One view of a batched render: the march arguments (lv.active / lv.sactive /
-// pass_count point at this view's own classification), the
-// level's brick and sub-brick min/max for that classification, and the view's
-// ranges in the flat brick and tile spaces of the batch. A view's flat brick
-// range holds its bricks (padded to a multiple of 32) followed by its
-// sub-bricks.
+// One view of a batched render, as its classification reads it: the march
+// arguments (lv.active / lv.sactive / pass_count point at this view's own
+// classification), the level's brick and sub-brick min/max for that
+// classification, and the view's ranges in the flat brick and distance-tile
+// spaces of the batch. A view's flat brick range holds its bricks (padded to a
+// multiple of 32) followed by its sub-bricks.
 struct BatchView {
     RenderArgs a;
     const float* bmin;
@@ -276,22 +299,25 @@ struct BatchView {
     unsigned long long cls_sub;    // offset of the first sub-brick in the view's range (multiple of 32)
     uint32_t* slist;               // active sub-bricks of the view (any order), for its cell classes
     uint32_t* scount;              // their number (zeroed per launch)
-    int tiles_x;                   // tiles per image row
-    int tile_begin;                // first flat tile index
-    int ntiles;                    // tiles of this view
-    unsigned seq;                  // launch sequence number written on completion
+    int dist_begin;                // first flat tile of the view's empty-space distance (a.lv.sdist)
+};
+
+// Completion of one view of a batch, and the parameters of its render node.
+struct ViewTiles {
     unsigned* tile_done;           // device counter of finished tiles (zeroed per launch)
-    ViewDone* done;                // device alias of the mapped host record (may be null)
-    uint8_t* stmp;                 // nsb^3 bytes of scratch for the view's empty-space distance
-    unsigned long long dist_begin; // first flat sub-brick index of the view's distance range (multiple
-                                   // of 32; the range is empty for views that render without skipping)
+    ViewDone* done;                // device alias of the mapped host record
+    unsigned seq;                  // launch sequence number written on completion
+};
+struct ViewLaunch {
+    RenderArgs a;
+    ViewTiles t;
+    void* arg[2];                  // the node's parameter pointers (set by render_view_node)
 };
 
 struct BatchHeader {
     int nviews;
-    int total_tiles;
     unsigned long long cls_total;  // flat brick range over all views (multiple of 32)
-    unsigned long long dist_total; // flat sub-brick range of the distance passes over all views
+    int dist_total;                // distance tiles over all views
 };
 
 // Render launch variants: a 128-thread block is 2 x 2 warps; each warp marches
@@ -599,15 +625,14 @@ cudaError_t launch_level_bricks(const void* cells, int dtype, int n, int nvars, 
 cudaError_t launch_classify(ClassifyArgs& c, cudaStream_t stream);
 cudaError_t launch_cell_classes(const CellClassArgs& a, int dtype, cudaStream_t stream);
 cudaError_t launch_render(const RenderArgs& a, int dtype, cudaStream_t stream);
-// Batched render: per-view classification (bricks, sub-bricks and the cell
-// classes of the active sub-bricks, into a.cls), then a persistent kernel that
-// pulls (view, tile) work items from *tile_counter (zeroed by the caller).
-// Grids are fixed by the caller (cls_blocks for the grid-stride classification,
-// blocks for the persistent render) so the launch can be captured in a graph;
-// launches are not counted here (the caller counts each replay).
-cudaError_t launch_render_batch(const BatchHeader* hdr, const BatchView* views, unsigned* tile_counter, bool depth,
-                                int dtype, int variant, unsigned cls_blocks, int blocks, cudaStream_t stream);
-int render_batch_blocks_per_sm(int dtype, int variant, bool depth);
+// Batched render: per-view classification (bricks, sub-bricks, the cell classes
+// of the active sub-bricks into a.cls, the empty-space distance into a.lv.sdist),
+// with a grid fixed by the caller so that the launches can be captured in a
+// graph; then one render node per view (v stays alive while the node parameters
+// are used). Launches are not counted here (the caller counts each replay).
+cudaError_t launch_view_classes(const BatchHeader* hdr, const BatchView* views, int dtype, unsigned cls_blocks,
+                                cudaStream_t stream);
+cudaKernelNodeParams render_view_node(ViewLaunch& v, int dtype);
 cudaError_t launch_histogram(const HistArgs& a, int dtype, cudaStream_t stream);
 
 // Image warping (render_kernels.cu).
@@ -642,14 +667,15 @@ struct TfVisArgs {
 };
 cudaError_t launch_tf_visibility(const TfVisArgs& a, cudaStream_t stream);
 
-// Empty-space distance of the nsb^3 sub-bricks under the activity bits sactive:
-// Chebyshev distance in sub-bricks to the nearest active sub-brick, capped at
-// kDistCap, 0 for active ones (volume_kernels.cu). tmp: nsb^3 bytes of scratch.
-cudaError_t launch_subbrick_distance(const uint32_t* sactive, int nsb, uint8_t* dist, uint8_t* tmp,
-                                     cudaStream_t stream);
-// The same for every view of a batch that renders with skipping, from the view's
-// own activity bits into its a.lv.sdist (with its stmp as scratch), after the
-// per-view classification; `blocks` of 256 threads walk the views' ranges.
+// Empty-space distance of the sub-bricks of a level of edge n under the activity
+// bits sactive: Chebyshev distance in sub-bricks to the nearest active one, capped
+// at kDistCap, 0 for active ones (volume_kernels.cu). Writes the padded grid
+// (padded_bytes(n)), or with raw the nsb^3 distances themselves.
+cudaError_t launch_subbrick_distance(const uint32_t* sactive, int n, uint8_t* out, bool raw, cudaStream_t stream);
+// The same for every view of a batch, from the view's own activity bits into its
+// a.lv.sdist, after the per-view classification; `blocks` blocks take the views'
+// tiles (subbrick_distance_tiles(n) per view, from its dist_begin on).
+int subbrick_distance_tiles(int n);
 cudaError_t launch_subbrick_distance_views(const BatchHeader* hdr, const BatchView* views, unsigned blocks,
                                            cudaStream_t stream);
 

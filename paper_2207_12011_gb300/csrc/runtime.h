@@ -60,8 +60,7 @@ struct Level {
     uint16_t* cls = nullptr;      // cell classes under the current brush (n^3), computed on demand
     uint32_t* tf_active = nullptr;   // activity AND TF visibility (renders with tf_skip)
     uint32_t* tf_sactive = nullptr;
-    uint8_t* sdist = nullptr;        // empty-space distance of the sub-bricks (renders with skipping)
-    uint8_t* sdist_tmp = nullptr;
+    uint8_t* sdist = nullptr;        // padded empty-space distance of the sub-bricks (renders)
     const uint32_t* sdist_of = nullptr;   // activity bits the distance was computed from (null: stale)
     bool cls_valid = false;
     bool bricks = false;

@@ -11,8 +11,8 @@
 //      the oldest unlaunched requests (up to the view and pixel caps): their
 //      histogram kernels first, then one batched render launch (one CUDA graph
 //      replay) holding all their coarse passes and then all their full passes,
-//      each group smallest image first. The persistent kernel writes a
-//      completion record per view into mapped host memory, so each pass is
+//      each group smallest image first. Every view's render writes a
+//      completion record into mapped host memory, so each pass is
 //      published as soon as its own tiles are done.
 // Requests that arrive while launches are running are admitted as slots and
 // pool memory free up and join the next launch, so their work overlaps with
@@ -101,7 +101,7 @@ struct Req {
     std::vector<float> edges;
     int status = RAYPC_OK;
     bool admitted = false, coarse_launched = false, full_launched = false;
-    bool coarse_ready = false, done = false;
+    bool coarse_ready = false, full_ready = false, done = false;
     double t_submit = 0, t_admit = 0, t_coarse = 0, t_done = 0;
     char* mem = nullptr;
     size_t mem_bytes = 0;
@@ -275,15 +275,19 @@ raypc_status launch_hist(raypc_server* S, Req* q, int si) {
     return RAYPC_OK;
 }
 
+// The passes of a launch run side by side: a request is finished when its full pass and,
+// with one, its coarse pass are.
 void publish(raypc_server* S, Item& it, double t, unsigned long long marched) {
     Req* q = it.q;
     it.seen = true;
     if (it.pass == kCoarse) {
         q->coarse_ready = true;
         q->t_coarse = t;
-        return;
+    } else {
+        if (it.pass == kFull) q->samples = marched;
+        q->full_ready = true;
     }
-    if (it.pass == kFull) q->samples = marched;
+    if (!q->full_ready || (q->coarse_launched && !q->coarse_ready)) return;
     finish(S, q, RAYPC_OK);
     q->t_done = t;
 }

@@ -690,88 +690,173 @@ __global__ void __launch_bounds__(256) k_tf_visibility(TfVisArgs A) {
 }  // namespace
 
 // Empty-space distance of the 4^3 sub-bricks: the Chebyshev distance, in
-// sub-bricks, to the nearest active one, capped at kDistCap (0: active). The L-inf
-// distance transform is separable: d(p) = min over qz of max(|dz|, min over qy of
-// max(|dy|, min over active qx of |dx|)), each 1D pass a window of +-kDistCap.
-// pass 0: x from the activity bits into a; 1: y from a into b; 2: z from b into a.
-// One sub-brick id < nsb^3 of one pass.
-__device__ __forceinline__ uint8_t subbrick_distance_at(const uint32_t* __restrict__ act, int nsb, int pass,
-                                                      const uint8_t* __restrict__ in, size_t id) {
-    const int x = (int)(id % nsb), y = (int)((id / nsb) % nsb), z = (int)(id / ((size_t)nsb * nsb));
-    int d = kDistCap;
-    if (pass == 0) {
-        for (int o = -kDistCap; o <= kDistCap; ++o) {
-            const int xx = x + o;
-            if (xx < 0 || xx >= nsb) continue;
-            const size_t q = id - x + xx;
-            if ((__ldg(act + (q >> 5)) >> (q & 31)) & 1u) d = min(d, abs(o));
+// sub-bricks, to the nearest active one, capped at kDistCap (0: active). A block
+// takes a tile of kDistTile x kDistTile sub-brick rows (y, z) and up to
+// 32 kDistWords sub-bricks in x, with a halo of kDistCap rows and one word, as
+// bitmasks: one thread per row, a row's words in its registers. It grows the
+// active set by one 3x3x3 dilation per step (x in registers, y and z through
+// shared memory); the step at which a bit first appears is its distance.
+constexpr int kDistTile = 8;
+constexpr int kDistWords = 4;
+constexpr int kDistRows = kDistTile + 2 * kDistCap;          // rows per axis with the halo
+constexpr int kDistThreads = kDistRows * kDistRows;
+
+struct DistanceTiles {
+    int lim, ntx, nt;             // sub-bricks per axis that the tiles cover, tiles in x and in y (= z)
+};
+
+__host__ __device__ inline DistanceTiles distance_tiles(int n, bool raw) {
+    DistanceTiles d;
+    d.lim = raw ? (n + kSub - 1) / kSub : ((n - 2) >> 2) + 1;
+    d.ntx = (d.lim + 32 * kDistWords - 1) / (32 * kDistWords);
+    d.nt = (d.lim + kDistTile - 1) / kDistTile;
+    return d;
+}
+
+// Tile `tile` of a level; all kDistThreads threads of the block call it.
+__device__ __forceinline__ void subbrick_distance_tile(const uint32_t* __restrict__ act, int n, int tile,
+                                                       uint8_t* __restrict__ out, bool raw) {
+    constexpr int W = kDistWords + 2;                        // one halo word on either side
+    __shared__ uint32_t s_row[W][kDistThreads];
+    const int nsb = (n + kSub - 1) / kSub;
+    const uint32_t nbits = (uint32_t)nsb * nsb * nsb;
+    const DistanceTiles T = distance_tiles(n, raw);
+    const int w0 = (tile % T.ntx) * kDistWords, ty = (tile / T.ntx) % T.nt, tz = tile / (T.ntx * T.nt);
+    const int t = threadIdx.x, ry = t % kDistRows, rz = t / kDistRows;
+    const int y = ty * kDistTile + ry - kDistCap, z = tz * kDistTile + rz - kDistCap;
+    const bool row = y >= 0 && y < nsb && z >= 0 && z < nsb;
+    uint32_t a[W], p[3][kDistWords];
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        // bits 32 (w0 + w - 1) .. + 31 of the row, 0 outside it
+        const int x = 32 * (w0 + w - 1);
+        uint32_t v = 0u;
+        if (row && x >= 0 && x < nsb) {
+            const uint32_t id = ((uint32_t)z * nsb + y) * nsb + x;
+            v = __ldg(act + (id >> 5)) >> (id & 31);
+            if ((id & 31) && (id | 31u) + 1u < nbits) v |= __ldg(act + (id >> 5) + 1) << (32 - (id & 31));
+            if (nsb - x < 32) v &= (1u << (nsb - x)) - 1u;
         }
-    } else {
-        const int c = pass == 1 ? y : z;
-        const size_t stride = pass == 1 ? (size_t)nsb : (size_t)nsb * nsb;
-        for (int o = -kDistCap; o <= kDistCap; ++o) {
-            const int cc = c + o;
-            if (cc < 0 || cc >= nsb) continue;
-            d = min(d, max(abs(o), (int)__ldg(in + (size_t)((long long)id + (long long)o * (long long)stride))));
+        a[w] = v;
+    }
+#pragma unroll
+    for (int w = 0; w < kDistWords; ++w) p[0][w] = p[1][w] = p[2][w] = 0u;
+    uint32_t seen[kDistWords];
+#pragma unroll
+    for (int w = 0; w < kDistWords; ++w) seen[w] = a[w + 1];
+    const int up = ry + 1 < kDistRows ? 1 : 0, dn = ry > 0 ? 1 : 0;
+    const int fw = rz + 1 < kDistRows ? kDistRows : 0, bk = rz > 0 ? kDistRows : 0;
+#pragma unroll 1
+    for (int d = 1; d < kDistCap; ++d) {
+        // x: within the row (the outer halo words only need the bits next to the inner ones)
+        uint32_t prev = 0u;
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            const uint32_t cur = a[w], next = w + 1 < W ? a[w + 1] : 0u;
+            a[w] = cur | (cur << 1) | (cur >> 1) | (prev >> 31) | (next << 31);
+            prev = cur;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < W; ++w) s_row[w][t] = a[w];
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < W; ++w) a[w] |= s_row[w][t + up] | s_row[w][t - dn];
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < W; ++w) s_row[w][t] = a[w];
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < W; ++w) a[w] |= s_row[w][t + fw] | s_row[w][t - bk];
+        // first seen at this step: the distance, in three bit planes
+#pragma unroll
+        for (int w = 0; w < kDistWords; ++w) {
+            const uint32_t fresh = a[w + 1] & ~seen[w];
+            seen[w] |= fresh;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) p[k][w] |= ((d >> k) & 1) ? fresh : 0u;
         }
     }
-    return (uint8_t)d;
+    // bytes of the tile's inner rows: planes 0..2 and "never seen" (kDistCap) through shared memory
+    __syncthreads();
+    static_assert(4 * kDistWords * kDistTile * kDistTile <= W * kDistThreads, "planes fit the row buffer");
+    uint32_t* s_plane = &s_row[0][0];                        // [inner row][word][plane]
+    const int iy = ry - kDistCap, iz = rz - kDistCap;
+    if (iy >= 0 && iy < kDistTile && iz >= 0 && iz < kDistTile) {
+        uint32_t* q = s_plane + (iz * kDistTile + iy) * kDistWords * 4;
+#pragma unroll
+        for (int w = 0; w < kDistWords; ++w) {
+            q[4 * w] = p[0][w];
+            q[4 * w + 1] = p[1][w];
+            q[4 * w + 2] = p[2][w];
+            q[4 * w + 3] = ~seen[w];
+        }
+    }
+    __syncthreads();
+    // output entries e of the tile on each axis: its own sub-bricks, and in the padded grid the
+    // borders before the first and after the last one
+    const int pd = raw ? nsb : subbrick_pad(n), pad = raw ? 0 : 1, last = T.lim - 1, end = raw ? nsb - 1 : (n - 1) >> 2;
+    auto range = [&](int first, int len, int& e0, int& e1) {
+        e0 = first == 0 ? -pad : first;
+        e1 = first + len > last ? end : first + len - 1;
+    };
+    int x0, x1, y0, y1, z0, z1;
+    range(32 * w0, 32 * kDistWords, x0, x1);
+    range(ty * kDistTile, kDistTile, y0, y1);
+    range(tz * kDistTile, kDistTile, z0, z1);
+    const int nx = x1 - x0 + 1, ny = y1 - y0 + 1, total = nx * ny * (z1 - z0 + 1);
+    for (int i = t; i < total; i += kDistThreads) {
+        const int ex = x0 + i % nx, ey = y0 + (i / nx) % ny, ez = z0 + i / (nx * ny);
+        const int sx = min(max(ex, 0), last) - 32 * w0;
+        const int sy = min(max(ey, 0), last) - ty * kDistTile, sz = min(max(ez, 0), last) - tz * kDistTile;
+        const uint32_t* q = s_plane + ((sz * kDistTile + sy) * kDistWords + (sx >> 5)) * 4;
+        const int b = sx & 31;
+        const unsigned dist = ((q[0] >> b) & 1u) | (((q[1] >> b) & 1u) << 1) | (((q[2] >> b) & 1u) << 2) |
+                              (((q[3] >> b) & 1u) << 3);
+        out[((size_t)(ez + pad) * pd + ey + pad) * pd + ex + pad] = (uint8_t)dist;
+    }
+    __syncthreads();                                         // s_row is reused by the block's next tile
 }
 
-__global__ void __launch_bounds__(256) k_subbrick_distance(const uint32_t* __restrict__ act, int nsb, int pass,
-                                                           const uint8_t* __restrict__ in, uint8_t* __restrict__ out) {
-    const size_t total = (size_t)nsb * nsb * nsb;
-    const size_t id = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= total) return;
-    out[id] = subbrick_distance_at(act, nsb, pass, in, id);
+static_assert(kDistCap == 8, "three bit planes and the never-seen bit");
+
+__global__ void __launch_bounds__(kDistThreads) k_subbrick_distance(const uint32_t* __restrict__ act, int n,
+                                                                    uint8_t* __restrict__ out, bool raw) {
+    subbrick_distance_tile(act, n, blockIdx.x, out, raw);
 }
 
-// Every view of a batch: the threads walk the views' concatenated distance ranges (a
-// warp's 32 consecutive flat indices always belong to one view); pass 0 writes the
-// view's distance buffer, 1 its scratch, 2 the distance buffer again.
-__global__ void __launch_bounds__(256) k_subbrick_distance_views(const BatchHeader* __restrict__ hdr,
-                                                                 const BatchView* __restrict__ views, int pass) {
-    const unsigned long long total = hdr->dist_total;
-    const int nviews = hdr->nviews;
-    const int lane = threadIdx.x & 31;
-    const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-    for (unsigned long long g = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; g < total; g += stride) {
-        const unsigned long long g0 = g - lane;
-        int lo = 0, hi = nviews - 1;                 // the last view whose range starts at or before g0
+// Every view of a batch: the blocks walk the views' concatenated tiles.
+__global__ void __launch_bounds__(kDistThreads) k_subbrick_distance_views(const BatchHeader* __restrict__ hdr,
+                                                                          const BatchView* __restrict__ views) {
+    const int total = hdr->dist_total, nviews = hdr->nviews;
+    for (int g = blockIdx.x; g < total; g += gridDim.x) {
+        int lo = 0, hi = nviews - 1;                 // the last view whose tiles start at or before g
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
-            if (views[mid].dist_begin <= g0) lo = mid; else hi = mid - 1;
+            if (views[mid].dist_begin <= g) lo = mid; else hi = mid - 1;
         }
         const BatchView& V = views[lo];
-        const int nsb = V.a.lv.nsb;
-        const size_t id = (size_t)(g - V.dist_begin);
-        if (id >= (size_t)nsb * nsb * nsb) continue;   // the padding of the view's range
-        uint8_t* dist = const_cast<uint8_t*>(V.a.lv.sdist);
-        const uint8_t* in = pass == 1 ? dist : V.stmp;
-        uint8_t* out = pass == 1 ? V.stmp : dist;
-        out[id] = subbrick_distance_at(V.a.lv.sactive, nsb, pass, in, id);
+        subbrick_distance_tile(V.a.lv.sactive, V.a.lv.n, g - V.dist_begin, const_cast<uint8_t*>(V.a.lv.sdist), false);
     }
 }
 
-cudaError_t launch_subbrick_distance(const uint32_t* sactive, int nsb, uint8_t* dist, uint8_t* tmp,
-                                     cudaStream_t stream) {
-    const size_t total = (size_t)nsb * nsb * nsb;
-    const unsigned blocks = (unsigned)((total + 255) / 256);
-    k_subbrick_distance<<<blocks, 256, 0, stream>>>(sactive, nsb, 0, nullptr, dist);
-    k_subbrick_distance<<<blocks, 256, 0, stream>>>(sactive, nsb, 1, dist, tmp);
-    k_subbrick_distance<<<blocks, 256, 0, stream>>>(sactive, nsb, 2, tmp, dist);
-    count_launches(3);
+static int distance_tile_count(int n, bool raw) {
+    const DistanceTiles T = distance_tiles(n, raw);
+    return T.ntx * T.nt * T.nt;
+}
+
+int subbrick_distance_tiles(int n) { return distance_tile_count(n, false); }
+
+cudaError_t launch_subbrick_distance(const uint32_t* sactive, int n, uint8_t* out, bool raw, cudaStream_t stream) {
+    k_subbrick_distance<<<distance_tile_count(n, raw), kDistThreads, 0, stream>>>(sactive, n, out, raw);
+    count_launches(1);
     return cudaGetLastError();
 }
 
 cudaError_t launch_subbrick_distance_views(const BatchHeader* hdr, const BatchView* views, unsigned blocks,
                                            cudaStream_t stream) {
-    for (int pass = 0; pass < 3; ++pass) {
-        k_subbrick_distance_views<<<blocks, 256, 0, stream>>>(hdr, views, pass);
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    k_subbrick_distance_views<<<blocks, kDistThreads, 0, stream>>>(hdr, views);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_tf_visibility(const TfVisArgs& a, cudaStream_t stream) {

@@ -649,7 +649,7 @@ def get_tuning(ctx: Context, dtype: int, n: int):
 
 
 class Batch:
-    """A reusable batched render (one persistent launch in a CUDA graph per call)."""
+    """A reusable batched render (one CUDA graph launch per call)."""
 
     def __init__(self, ctx: Context, max_views: int):
         self.ctx = ctx
