@@ -361,15 +361,15 @@ typedef struct raypc_view {
 typedef struct raypc_batch raypc_batch;
 
 /* A reusable batch of up to max_views views (1..4096). It owns a device view
- * table, per-view classification bitmasks and sub-brick lists, per-view cell
- * classes and a CUDA graph of the batched launch (table upload, per-view brick
- * and sub-brick classification, per-view cell classes, the empty-space distance
- * of every view, and one render node per view, side by side), captured on first
+ * table, per-view classification bitmasks and cell classes and a CUDA graph of
+ * the batched launch (table upload, per-view sub-brick classification and cell
+ * classes, the empty-space distance of every view, and one render node per view,
+ * side by side), captured on first
  * use and replayed afterwards with the nodes' parameters set to the views.
  * Allocates device and pinned host memory; the per-view buffers are allocated
  * for a view slot on its first use and grown for larger levels: n^3 * 2 bytes
- * of cell classes plus about n^3 / 10 bytes of masks, lists and distances per
- * used slot (281 MB at 512^3), charged to the context's budget. */
+ * of cell classes plus about n^3 / 50 bytes of masks and distances per
+ * used slot (271 MB at 512^3), charged to the context's budget. */
 raypc_status raypc_batch_create(raypc_ctx *ctx, int max_views, raypc_batch **out);
 raypc_status raypc_batch_destroy(raypc_batch *batch);
 
@@ -608,7 +608,9 @@ raypc_status raypc_export_volume(raypc_ctx *ctx, int vol, int lod, void *out_dev
 raypc_status raypc_get_bricks(raypc_ctx *ctx, int vol, int lod, float *out_min_dev,
                               float *out_max_dev, void *stream);
 
-/* Copy a level's classification under the current brush. active_bits_dev and
+/* Copy a level's classification under the current brush (that of the 8^3 bricks
+ * is computed by the first of these calls after a brush change: the renders and
+ * histograms use the sub-bricks). active_bits_dev and
  * skippable_bits_dev receive ceil(nb^3 / 32) uint32 words (bit b%32 of word
  * b/32 for brick b); active_list_dev (optional, nb^3 uint32) receives the ids
  * of the active bricks in increasing order and n_active_dev (optional, one

@@ -19,7 +19,7 @@ OBJ_DIR = os.path.join(LIB_DIR, "obj")
 LIB_PATH = os.path.join(LIB_DIR, "libraypc.so")
 HEADER = os.path.join(ROOT, "include", "raypc.h")
 
-SOURCES = ["api.cu", "volume_kernels.cu", "render_kernels.cu", "hist_kernels.cu", "hist_noalloc.cu", "pcsub_kernels.cu",
+SOURCES = ["api.cu", "volume_kernels.cu", "brush_kernels.cu", "render_kernels.cu", "hist_kernels.cu", "hist_noalloc.cu", "pcsub_kernels.cu",
            "points_kernels.cu", "warp_kernels.cu",
            "batch.cu", "tune.cu", "server.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -49,27 +49,24 @@ raypc_status cuda_fail(cudaError_t e, const char* what) {
 namespace {
 
 void free_level(Level& L) {
-    void* ptrs[] = {L.cells, L.pairs, L.bmin, L.bmax, L.active, L.skippable, L.list, L.n_active, L.pass_count,
-                    L.sbmin, L.sbmax, L.sactive, L.slist, L.scount, L.cls, L.tf_active, L.tf_sactive,
-                    L.sdist};
+    void* ptrs[] = {L.cells, L.pairs, L.bmin, L.bmax, L.active, L.skippable, L.list, L.n_active, L.stats,
+                    L.sbmin, L.sbmax, L.sactive, L.cls, L.tf_sactive, L.sdist};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     L = Level{};
 }
 
 void free_bricks(Level& L) {
-    void* ptrs[] = {L.bmin, L.bmax, L.active, L.skippable, L.list, L.n_active, L.pass_count,
-                    L.sbmin, L.sbmax, L.sactive, L.slist, L.scount, L.tf_active, L.tf_sactive,
-                    L.sdist};
+    void* ptrs[] = {L.bmin, L.bmax, L.active, L.skippable, L.list, L.n_active, L.stats,
+                    L.sbmin, L.sbmax, L.sactive, L.tf_sactive, L.sdist};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     L.bmin = L.bmax = L.sbmin = L.sbmax = nullptr;
-    L.active = L.skippable = L.list = L.n_active = L.sactive = L.slist = L.scount = nullptr;
-    L.tf_active = L.tf_sactive = nullptr;
+    L.active = L.skippable = L.list = L.n_active = L.sactive = L.tf_sactive = nullptr;
     L.sdist = nullptr;
     L.sdist_of = nullptr;
-    L.pass_count = nullptr;
-    L.bricks = L.classified = L.cls_valid = false;
+    L.stats = nullptr;
+    L.bricks = L.classified = L.cls_valid = L.listed = false;
 }
 
 void free_staging(Volume* V) {
@@ -98,46 +95,30 @@ void free_volume(raypc_ctx* ctx, Volume* V) {
 }
 
 
-// Classify the bricks and sub-bricks of every built level under the current
-// brush (three launches total).
-raypc_status classify_all(Volume* V, cudaStream_t s) {
-    ClassifyArgs c{};
-    c.nvars = V->nvars;
-    c.rin2 = V->r_in * V->r_in;
-    c.rout2 = V->r_out * V->r_out;
-    c.brush = V->brush;
+// The classification is out of date (new values, levels or brush).
+void unclassify(Volume* V) {
+    for (auto& L : V->lv) {
+        L.classified = L.cls_valid = L.listed = false;
+        L.sdist_of = nullptr;
+    }
+}
+
+// Classify the sub-bricks of every built level under the current brush and compute
+// the cell classes of level with_classes (its buffer allocated; null: none), in one launch.
+raypc_status classify_all(Volume* V, Level* with_classes, cudaStream_t s) {
+    BrushLaunch P{};
     for (int l = 0; l < V->nlev; ++l) {
         Level& L = V->lv[l];
         if (!L.bricks) return fail(RAYPC_ERR_INVALID_ARG, "bricks of level %d are not built", l);
-        ClassifyLevel& C = c.lv[c.nlev++];
-        C.bmin = L.bmin;
-        C.bmax = L.bmax;
-        C.n = L.n;
-        C.bs = kBrick;
-        C.active = L.active;
-        C.skippable = L.skippable;
-        C.list = L.list;
-        C.n_active = L.n_active;
-        C.pass_count = L.pass_count;
+        BrushItem& it = P.items[P.nitems++];
+        it = brush_item(V, L, V->brush);
+        it.active = L.sactive;
+        it.cls = &L == with_classes ? L.cls : nullptr;
     }
-    c.nbrick = c.nlev;
-    for (int l = 0; l < V->nlev; ++l) {
-        Level& L = V->lv[l];
-        ClassifyLevel& C = c.lv[c.nlev++];
-        C.bmin = L.sbmin;
-        C.bmax = L.sbmax;
-        C.n = L.n;
-        C.bs = kSub;
-        C.active = L.sactive;
-        C.alist = L.slist;
-        C.acount = L.scount;
-    }
-    CK(launch_classify(c, s), "classify kernels");
-    for (int l = 0; l < V->nlev; ++l) {
-        V->lv[l].classified = true;
-        V->lv[l].cls_valid = false;          // cell classes follow the brush; computed on demand
-        V->lv[l].sdist_of = nullptr;         // so does the empty-space distance
-    }
+    CK(launch_brush(P, V->dtype, s), "classification kernel");
+    unclassify(V);
+    for (int l = 0; l < V->nlev; ++l) V->lv[l].classified = true;
+    if (with_classes) with_classes->cls_valid = true;
     return RAYPC_OK;
 }
 
@@ -145,7 +126,21 @@ raypc_status classify_all(Volume* V, cudaStream_t s) {
 raypc_status ensure_classified(Volume* V, Level& L, cudaStream_t s) {
     if (L.classified) return RAYPC_OK;
     if (!V->brush_set) return fail(RAYPC_ERR_INVALID_ARG, "raypc_set_brush must run first");
-    return classify_all(V, s);
+    return classify_all(V, nullptr, s);
+}
+
+// The level's cell class buffer (allocated on first use; words of cells outside active
+// sub-bricks are never written again).
+raypc_status alloc_cell_classes(raypc_ctx* ctx, Volume* V, Level& L, cudaStream_t s) {
+    if (L.cls) return RAYPC_OK;
+    const size_t bytes = (size_t)L.n * L.n * L.n * sizeof(uint16_t);
+    raypc_status st = ctx->alloc((void**)&L.cls, bytes, &V->bytes);
+    if (st) {
+        L.cls = nullptr;
+        return st;
+    }
+    CK(cudaMemsetAsync(L.cls, 0, bytes, s), "clear cell classes");
+    return RAYPC_OK;
 }
 
 raypc_status alloc_bricks(raypc_ctx* ctx, Volume* V, Level& L) {
@@ -159,19 +154,18 @@ raypc_status alloc_bricks(raypc_ctx* ctx, Volume* V, Level& L) {
         (st = ctx->alloc((void**)&L.sbmax, smm, &V->bytes)) ||
         (st = ctx->alloc((void**)&L.sactive, L.nswords() * sizeof(uint32_t), &V->bytes)) ||
         (st = ctx->alloc((void**)&L.tf_sactive, L.nswords() * sizeof(uint32_t), &V->bytes)) ||
-        (st = ctx->alloc((void**)&L.tf_active, words, &V->bytes)) ||
-        (st = ctx->alloc((void**)&L.slist, L.nsbricks() * sizeof(uint32_t), &V->bytes)) ||
-        (st = ctx->alloc((void**)&L.scount, sizeof(uint32_t), &V->bytes)) ||
         (st = ctx->alloc((void**)&L.bmin, mm, &V->bytes)) ||
         (st = ctx->alloc((void**)&L.bmax, mm, &V->bytes)) ||
         (st = ctx->alloc((void**)&L.active, words, &V->bytes)) ||
         (st = ctx->alloc((void**)&L.skippable, words, &V->bytes)) ||
         (st = ctx->alloc((void**)&L.list, nbk * sizeof(uint32_t), &V->bytes)) ||
         (st = ctx->alloc((void**)&L.n_active, sizeof(uint32_t), &V->bytes)) ||
-        (st = ctx->alloc((void**)&L.pass_count, sizeof(unsigned) * kMaxVars, &V->bytes))) {
+        (st = ctx->alloc((void**)&L.stats, sizeof(unsigned long long) * (kMaxVars + 1), &V->bytes))) {
         free_bricks(L);
         return st;
     }
+    CK(cudaMemset(L.stats, 0, sizeof(unsigned long long) * (kMaxVars + 1)), "clear level statistics");
+    L.gen = 0;
     return RAYPC_OK;
 }
 
@@ -256,12 +250,13 @@ raypc_status ingest(raypc_ctx* ctx, Volume* V, const void* src, int src_is_devic
     // x-pairs come out of the same pass over the source
     Level& C = V->lv[1];
     const bool next = C.cells && C.pairs && C.n * 2 == L.n && ingest_next_level_fits(dsrc, L.n);
+    const LevelStats stats{L.stats, ++L.gen};
     if (next)
         e = launch_ingest_next_level(dsrc, src_dtype, L.cells, L.pairs, V->dtype, L.n, V->nvars, L.bmin, L.bmax,
-                                     L.sbmin, L.sbmax, C.cells, C.pairs, s);
+                                     L.sbmin, L.sbmax, C.cells, C.pairs, stats, s);
     else
         e = launch_ingest(dsrc, src_dtype, L.cells, L.pairs, V->dtype, L.n, V->nvars, L.bmin, L.bmax, L.sbmin,
-                          L.sbmax, s);
+                          L.sbmax, stats, s);
     C.fresh = next && e == cudaSuccess;
     if (staging) cudaFreeAsync(staging, s);
     if (staged && e == cudaSuccess) {
@@ -270,7 +265,7 @@ raypc_status ingest(raypc_ctx* ctx, Volume* V, const void* src, int src_is_devic
     }
     if (e != cudaSuccess) return cuda_fail(e, "ingest kernel");
     L.bricks = true;               // level-0 brick min/max come out of the ingest pass
-    for (auto& l : V->lv) l.classified = l.cls_valid = false;
+    unclassify(V);
     return RAYPC_OK;
 }
 
@@ -335,21 +330,15 @@ raypc_status make_render_args(Volume* V, Level* L, const raypc_camera* cam, int 
     if (!isfinite(dt) || dt < 2.0f * V->r_out / 4194304.0f)
         return fail(RAYPC_ERR_INVALID_ARG, "step %g too small (at most 2^21 samples per chord)", dt);
     RenderArgs a{};
-    a.lv.cells = L->cells;
     a.lv.pairs = L->pairs;
     a.lv.n = L->n;
-    a.lv.nb = L->nb;
     a.lv.nsb = L->nsb;
     a.lv.pd = subbrick_pad(L->n);
     a.lv.pbias = narrow_bias(L->n);
     a.lv.plast = (uint32_t)(padded_bytes(L->n) - 1);
     a.lv.sactive = L->sactive;
-    a.lv.bmin = L->bmin;
-    a.lv.bmax = L->bmax;
-    a.lv.active = L->active;
     a.nvars = V->nvars;
     a.brush = V->brush;
-    a.pass_count = L->pass_count;
     for (int i = 0; i < 3; ++i) { a.eye[i] = cam->eye[i]; a.target[i] = cam->target[i]; a.up[i] = cam->up[i]; }
     a.tan_half = cam->tan_half_vfov;
     a.w = w;
@@ -386,32 +375,39 @@ raypc_status make_render_args(Volume* V, Level* L, const raypc_camera* cam, int 
     a.out = reinterpret_cast<float4*>(out_rgba_dev);
     a.counts = o.counts_dev;
     a.depth = o.depth_dev;
-    a.tf_prefix = V->tf_prefix;
-    a.tf_skip = o.tf_skip ? 1 : 0;
     a.stats = stats_dev;
     *out = a;
     return RAYPC_OK;
 }
 
+BrushItem brush_item(const Volume* V, const Level& L, const BrushArgs& brush) {
+    BrushItem it{};
+    it.sbmin = L.sbmin;
+    it.sbmax = L.sbmax;
+    it.cells = L.cells;
+    it.stats = L.stats;
+    it.gen = L.gen;
+    it.n = L.n;
+    it.nsb = L.nsb;
+    it.nvars = V->nvars;
+    it.rin2 = V->r_in * V->r_in;
+    it.rout2 = V->r_out * V->r_out;
+    it.brush = brush;
+    return it;
+}
+
 raypc_status ensure_cell_classes(raypc_ctx* ctx, Volume* V, Level& L, cudaStream_t s) {
     if (L.cls_valid) return RAYPC_OK;
-    raypc_status cst = ensure_classified(V, L, s);           // the classes cover the active sub-bricks
-    if (cst) return cst;
-    if (!L.cls) {
-        const size_t bytes = (size_t)L.n * L.n * L.n * sizeof(uint16_t);
-        raypc_status st = ctx->alloc((void**)&L.cls, bytes, &V->bytes);
-        if (st) return st;
-        CK(cudaMemsetAsync(L.cls, 0, bytes, s), "clear cell classes");
-    }
-    CellClassArgs c{};
-    c.pairs = L.pairs;
-    c.n = L.n;
-    c.nvars = V->nvars;
-    c.brush = V->brush;
-    c.slist = L.slist;
-    c.scount = L.scount;
-    c.out = L.cls;
-    CK(launch_cell_classes(c, V->dtype, s), "cell class kernel");
+    if (!L.classified && !V->brush_set) return fail(RAYPC_ERR_INVALID_ARG, "raypc_set_brush must run first");
+    raypc_status st = alloc_cell_classes(ctx, V, L, s);
+    if (st) return st;
+    if (!L.classified) return classify_all(V, &L, s);
+    BrushLaunch P{};                                         // this level's bits again, and its classes
+    P.nitems = 1;
+    P.items[0] = brush_item(V, L, V->brush);
+    P.items[0].active = L.sactive;
+    P.items[0].cls = L.cls;
+    CK(launch_brush(P, V->dtype, s), "cell class kernel");
     L.cls_valid = true;
     return RAYPC_OK;
 }
@@ -593,32 +589,31 @@ raypc_status raypc_build_bricks(raypc_ctx* ctx, int vol, int brick_dim, int n_lo
         }
         if ((st = alloc_bricks(ctx, V, L))) return st;
         if (L.fresh)             // the ingest already wrote this level's cells: its bricks only
-            CK(launch_level_bricks(L.cells, V->dtype, L.n, V->nvars, L.bmin, L.bmax, L.sbmin, L.sbmax, s),
+            CK(launch_level_bricks(L.cells, V->dtype, L.n, V->nvars, L.bmin, L.bmax, L.sbmin, L.sbmax,
+                                   LevelStats{L.stats, ++L.gen}, s),
                "level bricks kernel");
         else
-            CK(launch_lod(P.cells, P.n, L.cells, L.pairs, V->dtype, V->nvars, L.bmin, L.bmax, L.sbmin, L.sbmax, s),
+            CK(launch_lod(P.cells, P.n, L.cells, L.pairs, V->dtype, V->nvars, L.bmin, L.bmax, L.sbmin, L.sbmax,
+                          LevelStats{L.stats, ++L.gen}, s),
                "LOD kernel");
         L.fresh = false;
         L.bricks = true;
     }
     if (V->stale || 1 + n_lod > V->nlev) V->nlev = 1 + n_lod;   // stale coarser levels drop out
     V->stale = false;
-    for (auto& L : V->lv) L.classified = L.cls_valid = false;
+    unclassify(V);
     return RAYPC_OK;
 }
 
 // Re-classify every built level under the volume's (new) brush and compute the
-// cell classes of level 0.
+// cell classes of level 0, so that a render runs its kernel alone (coarser levels get
+// their classes when first rendered).
 static raypc_status reclassify(raypc_ctx* ctx, Volume* V, cudaStream_t s) {
-    if (V->stale) {            // coarser levels are rebuilt by raypc_build_bricks, which classifies lazily
-        for (auto& L : V->lv) L.classified = L.cls_valid = false;
-        return RAYPC_OK;
-    }
-    raypc_status st = classify_all(V, s);
-    if (st) return st;
-    // the full-resolution level's cell classes now, so that a render runs its kernel
-    // alone (coarser levels get theirs when first rendered)
-    return ensure_cell_classes(ctx, V, V->lv[0], s);
+    unclassify(V);
+    if (V->stale) return RAYPC_OK;   // coarser levels are rebuilt by raypc_build_bricks, which classifies lazily
+    const raypc_status st = alloc_cell_classes(ctx, V, V->lv[0], s);
+    const raypc_status cl = classify_all(V, st ? nullptr : &V->lv[0], s);
+    return cl ? cl : st;
 }
 
 raypc_status raypc_set_brush(raypc_ctx* ctx, int vol, const float* lo, const float* hi,
@@ -719,28 +714,21 @@ static raypc_status ensure_distance(raypc_ctx* ctx, Volume* V, Level& L, RenderA
 }
 
 // With tf_skip, the render reads the activity bits ANDed with the TF visibility of
-// the level's bricks and sub-bricks (computed for this render on its stream).
+// the level's sub-bricks (computed for this render on its stream).
 static raypc_status apply_tf_skip(Volume* V, Level& L, const raypc_render_opts* opts, RenderArgs& a, cudaStream_t s) {
     if (!opts || !opts->tf_skip) return RAYPC_OK;
     TfVisArgs t{};
-    t.n = L.n;
-    t.nb = L.nb;
     t.nsb = L.nsb;
     t.nvars = V->nvars;
     t.color_var = V->color_var;
-    t.bmin = L.bmin;
-    t.bmax = L.bmax;
     t.sbmin = L.sbmin;
     t.sbmax = L.sbmax;
-    t.active = L.active;
     t.sactive = L.sactive;
-    t.tf = V->tf;
+    t.tf_prefix = V->tf_prefix;
     t.tf_lo = a.tf_lo;
     t.tf_scale = a.tf_scale;
-    t.out_active = L.tf_active;
     t.out_sactive = L.tf_sactive;
     CK(launch_tf_visibility(t, s), "TF visibility kernel");
-    a.lv.active = L.tf_active;
     a.lv.sactive = L.tf_sactive;
     return RAYPC_OK;
 }
@@ -1107,6 +1095,23 @@ raypc_status raypc_get_skip_list(raypc_ctx* ctx, int vol, int lod, uint32_t* act
     cudaStream_t s = (cudaStream_t)stream;
     if (V->stale) return fail(RAYPC_ERR_INVALID_ARG, "volume updated: raypc_build_bricks must run first");
     if ((st = ensure_classified(V, *L, s))) return st;
+    if (!L->listed) {
+        BrickListArgs b{};
+        b.bmin = L->bmin;
+        b.bmax = L->bmax;
+        b.n = L->n;
+        b.nb = L->nb;
+        b.nvars = V->nvars;
+        b.rin2 = V->r_in * V->r_in;
+        b.rout2 = V->r_out * V->r_out;
+        b.brush = V->brush;
+        b.active = L->active;
+        b.skippable = L->skippable;
+        b.list = L->list;
+        b.n_active = L->n_active;
+        CK(launch_brick_list(b, s), "brick list kernels");
+        L->listed = true;
+    }
     size_t wb = L->nwords() * sizeof(uint32_t);
     if (active_bits_dev) CK(cudaMemcpyAsync(active_bits_dev, L->active, wb, cudaMemcpyDeviceToDevice, s), "copy active bits");
     if (skippable_bits_dev) CK(cudaMemcpyAsync(skippable_bits_dev, L->skippable, wb, cudaMemcpyDeviceToDevice, s), "copy skippable bits");

@@ -21,9 +21,8 @@ struct raypc_batch {
     raypc_ctx* ctx = nullptr;
     int max_views = 0;
     size_t table_bytes = 0;
-    char* d_table = nullptr;          // BatchHeader, then max_views BatchView (device)
-    unsigned* d_pass = nullptr;       // max_views x kMaxVars selectivity counts
-    unsigned* d_tiles = nullptr;      // max_views finished-tile counters, then max_views sub-brick list lengths
+    char* d_table = nullptr;          // BatchHeader, then max_views BrushItem (device)
+    unsigned* d_tiles = nullptr;      // max_views finished-tile counters
     ViewDone* h_done[2] = {nullptr, nullptr};   // mapped pinned completion records per table slot
     ViewDone* d_done[2] = {nullptr, nullptr};   // their device aliases
     unsigned seq = 0;                 // launch sequence number
@@ -32,7 +31,7 @@ struct raypc_batch {
     cudaEvent_t done[2] = {nullptr, nullptr};
     bool used[2] = {false, false};
     int cur = 0;
-    std::vector<uint32_t*> bits;      // per view slot: active words, sub-brick active words, sub-brick list
+    std::vector<uint32_t*> bits;      // per view slot: sub-brick active words, padded distance grid
     std::vector<size_t> bits_words;   // capacity (words) per slot
     std::vector<uint16_t*> cls;       // per view slot: cell classes under the view's brush (n^3 words)
     std::vector<size_t> cls_cells;    // capacity (cells) per slot
@@ -51,7 +50,7 @@ namespace {
 constexpr size_t kHeaderBytes = 256;   // BatchHeader padded so the views start aligned
 
 BatchHeader* hdr_of(char* table) { return reinterpret_cast<BatchHeader*>(table); }
-BatchView* views_of(char* table) { return reinterpret_cast<BatchView*>(table + kHeaderBytes); }
+BrushItem* views_of(char* table) { return reinterpret_cast<BrushItem*>(table + kHeaderBytes); }
 
 void wait_idle(raypc_batch* b) {
     for (int i = 0; i < 2; ++i)
@@ -72,7 +71,6 @@ void release(raypc_batch* b) {
     for (uint16_t* p : b->cls)
         if (p) cudaFree(p);
     if (b->d_table) cudaFree(b->d_table);
-    if (b->d_pass) cudaFree(b->d_pass);
     if (b->d_tiles) cudaFree(b->d_tiles);
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
     if (b->ctx) b->ctx->used -= b->charged < b->ctx->used ? b->charged : b->ctx->used;
@@ -82,7 +80,7 @@ raypc_status capture(raypc_batch* b, int slot, int dtype) {
     int dev = 0, sms = 0;
     CK(cudaGetDevice(&dev), "cudaGetDevice");
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
-    const unsigned cls_blocks = (unsigned)sms * 8u;
+    const unsigned blocks = (unsigned)sms * 8u;
     if (b->exec[slot]) {
         cudaGraphExecDestroy(b->exec[slot]);
         b->exec[slot] = nullptr;
@@ -95,10 +93,9 @@ raypc_status capture(raypc_batch* b, int slot, int dtype) {
     cudaStream_t s = b->cap_stream;
     CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal), "begin graph capture");
     cudaError_t e = cudaMemcpyAsync(b->d_table, b->h_table[slot], b->table_bytes, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(b->d_pass, 0, sizeof(unsigned) * kMaxVars * b->max_views, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(b->d_tiles, 0, sizeof(unsigned) * 2 * b->max_views, s);
-    if (e == cudaSuccess)
-        e = launch_view_classes(hdr_of(b->d_table), views_of(b->d_table), dtype, cls_blocks, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(b->d_tiles, 0, sizeof(unsigned) * b->max_views, s);
+    if (e == cudaSuccess) e = launch_brush_views(hdr_of(b->d_table), views_of(b->d_table), dtype, s);
+    if (e == cudaSuccess) e = launch_subbrick_distance_views(hdr_of(b->d_table), views_of(b->d_table), blocks, s);
     cudaGraph_t graph = nullptr;
     cudaError_t e2 = cudaStreamEndCapture(s, &graph);
     if (e == cudaSuccess) e = e2;
@@ -149,14 +146,13 @@ raypc_status raypc_batch_create(raypc_ctx* ctx, int max_views, raypc_batch** out
     raypc_batch* b = new raypc_batch();
     b->ctx = ctx;
     b->max_views = max_views;
-    b->table_bytes = kHeaderBytes + sizeof(BatchView) * (size_t)max_views;
+    b->table_bytes = kHeaderBytes + sizeof(BrushItem) * (size_t)max_views;
     b->bits.assign(max_views, nullptr);
     b->bits_words.assign(max_views, 0);
     b->cls.assign(max_views, nullptr);
     b->cls_cells.assign(max_views, 0);
     raypc_status st = ctx->alloc((void**)&b->d_table, b->table_bytes, &b->charged);
-    if (st == RAYPC_OK) st = ctx->alloc((void**)&b->d_pass, sizeof(unsigned) * kMaxVars * max_views, &b->charged);
-    if (st == RAYPC_OK) st = ctx->alloc((void**)&b->d_tiles, sizeof(unsigned) * 2 * max_views, &b->charged);
+    if (st == RAYPC_OK) st = ctx->alloc((void**)&b->d_tiles, sizeof(unsigned) * max_views, &b->charged);
     cudaError_t e = cudaSuccess;
     for (int i = 0; i < 2 && st == RAYPC_OK && e == cudaSuccess; ++i) {
         e = cudaHostAlloc((void**)&b->h_table[i], b->table_bytes, cudaHostAllocDefault);
@@ -200,9 +196,10 @@ raypc_status raypc_render_batch(raypc_batch* b, const raypc_view* views, int nvi
     // the table buffer of this slot was last read by the batch two calls ago
     if (b->used[slot]) CK(cudaEventSynchronize(b->done[slot]), "wait for the previous use of the view table");
     BatchHeader* H = hdr_of(b->h_table[slot]);
-    BatchView* T = views_of(b->h_table[slot]);
+    BrushItem* T = views_of(b->h_table[slot]);
+    b->launch.resize(nviews);
     int dtype = -1, variant = 0;
-    unsigned long long cls = 0;
+    unsigned chunks = 0;
     int dist = 0;
     long long tiles = 0;
     raypc_status st;
@@ -214,20 +211,18 @@ raypc_status raypc_render_batch(raypc_batch* b, const raypc_view* views, int nvi
         if ((st = get_level(V, q.lod, &L))) return st;
         if (dtype < 0) dtype = V->dtype;
         if (V->dtype != dtype) return fail(RAYPC_ERR_INVALID_ARG, "view %d: all views of a batch need one storage dtype", i);
-        BatchView bv{};
-        if ((st = make_render_args(V, L, &q.cam, q.w, q.h, &q.opts, q.out_rgba_dev, q.stats_dev, &bv.a))) return st;
-        if ((st = brush_from_host(V, q.lo, q.hi, q.active_mask, &bv.a.brush))) return st;
-        if ((st = pos_from_host(q.pos_lo, q.pos_hi, q.pos_mask, &bv.a.brush))) return st;
-        finish_position_brush(bv.a);
-        if (i == 0) variant = bv.a.variant;
-        bv.a.variant = variant;
+        RenderArgs& a = b->launch[i].a;
+        if ((st = make_render_args(V, L, &q.cam, q.w, q.h, &q.opts, q.out_rgba_dev, q.stats_dev, &a))) return st;
+        if ((st = brush_from_host(V, q.lo, q.hi, q.active_mask, &a.brush))) return st;
+        if ((st = pos_from_host(q.pos_lo, q.pos_hi, q.pos_mask, &a.brush))) return st;
+        finish_position_brush(a);
+        if (i == 0) variant = a.variant;
+        a.variant = variant;
         tiles += (long long)((q.w + block_tile_w(variant) - 1) / block_tile_w(variant)) *
                  ((q.h + block_tile_h(variant) - 1) / block_tile_h(variant));
         if (tiles > 0x7fffffffLL) return fail(RAYPC_ERR_INVALID_ARG, "batch has more than 2^31 tiles");
-        // per view: brick and sub-brick activity bits, the list of active sub-bricks, and
-        // the sub-bricks' padded empty-space distance (bytes)
-        const size_t nsub = L->nsbricks();
-        const size_t words = L->nwords(), need = words + L->nswords() + nsub + (padded_bytes(L->n) + 3) / 4;
+        // per view: sub-brick activity bits and the sub-bricks' padded empty-space distance (bytes)
+        const size_t words = L->nswords(), need = words + (padded_bytes(L->n) + 3) / 4;
         if (b->bits_words[i] < need) {
             // growing a slot's masks: no batch may still be reading the old ones
             wait_idle(b);
@@ -239,13 +234,6 @@ raypc_status raypc_render_batch(raypc_batch* b, const raypc_view* views, int nvi
             b->charged += ch;
             b->bits_words[i] = need;
         }
-        bv.a.lv.active = b->bits[i];
-        bv.a.lv.sactive = b->bits[i] + words;
-        bv.slist = b->bits[i] + words + L->nswords();
-        bv.a.lv.sdist = reinterpret_cast<uint8_t*>(b->bits[i] + words + L->nswords() + nsub);
-        bv.dist_begin = dist;
-        dist += subbrick_distance_tiles(L->n);
-        bv.scount = b->d_tiles + b->max_views + i;
         const size_t cells = (size_t)L->n * L->n * L->n;
         if (b->cls_cells[i] < cells) {
             // growing a slot's cell classes: no batch may still be reading the old ones
@@ -258,25 +246,29 @@ raypc_status raypc_render_batch(raypc_batch* b, const raypc_view* views, int nvi
             b->charged += ch;
             b->cls_cells[i] = cells;
         }
-        bv.a.cls = b->cls[i];
-        bv.a.pass_count = b->d_pass + (size_t)i * kMaxVars;
-        bv.bmin = L->bmin;
-        bv.bmax = L->bmax;
-        bv.sbmin = L->sbmin;
-        bv.sbmax = L->sbmax;
-        bv.cls_begin = cls;
-        bv.cls_sub = (unsigned long long)words * 32;
-        cls += (unsigned long long)(words + L->nswords()) * 32;
-        T[i] = bv;
-    }
-    H->nviews = nviews;
-    H->cls_total = cls;
-    H->dist_total = dist;
-    b->launch.resize(nviews);
-    for (int i = 0; i < nviews; ++i) {
-        b->launch[i].a = T[i].a;
+        BrushItem it = brush_item(V, *L, a.brush);
+        it.active = b->bits[i];
+        it.cls = b->cls[i];
+        it.sdist = reinterpret_cast<uint8_t*>(b->bits[i] + words);
+        if (q.opts.tf_skip) {
+            it.tf_prefix = V->tf_prefix;
+            it.color_var = V->color_var;
+            it.tf_lo = a.tf_lo;
+            it.tf_scale = a.tf_scale;
+        }
+        it.chunk_begin = chunks;
+        chunks += brush_chunks(L->n);
+        it.dist_begin = dist;
+        dist += subbrick_distance_tiles(L->n);
+        T[i] = it;
+        a.lv.sactive = it.active;
+        a.lv.sdist = it.sdist;
+        a.cls = it.cls;
         b->launch[i].t = ViewTiles{b->d_tiles + i, b->d_done[slot] + i, b->seq + 1};
     }
+    H->nviews = nviews;
+    H->chunks = chunks;
+    H->dist_total = dist;
     if (!b->exec[slot] || b->exec_dtype[slot] != dtype || b->nodes[slot].size() < (size_t)nviews)
         if ((st = capture(b, slot, dtype))) return st;
     for (int i = 0; i < nviews; ++i) {
@@ -293,7 +285,7 @@ raypc_status raypc_render_batch(raypc_batch* b, const raypc_view* views, int nvi
     b->last_slot = slot;
     b->seq += 1;
     b->cur ^= 1;
-    count_launches(3 + nviews);
+    count_launches(2 + nviews);
     return RAYPC_OK;
 }
 

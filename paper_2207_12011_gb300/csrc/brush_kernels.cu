@@ -3,19 +3,24 @@
 // one launch gives the activity bits of the sub-bricks of any number of levels
 // and, for the levels that ask for them, the cell classes of the active ones.
 //
-// A warp takes 32 consecutive sub-bricks: a lane classifies one (shell, position
-// brush, min/max against the brush), a ballot is the word of activity bits, and
-// the warp then computes the classes of the active ones in groups of 8 that are
-// neighbours in x (32 x 4 x 4 cells). Lanes run along x, so every load is one or
-// two whole 64-byte segments; each cell's corners are folded along x in the lane,
-// then along y and z from row to row in registers. A variable whose range over
-// every active sub-brick of the group lies inside the brush by its margin is not
-// read at all (most of a brush's variables, in most groups). FP16 volumes fold
-// two cells per instruction as binary16 pairs (exact) and decide them with four
-// comparisons against binary16 bounds (see half_bounds).
+// A block takes a chunk of 32-bit words of activity: its warps first classify the
+// words (a lane per sub-brick: shell, position brush, min/max against the
+// brush), then compute the cell classes of the active sub-bricks in groups of 4
+// that are neighbours in x (16 x 4 x 4 cells), taken one by one from a list in
+// shared memory because some words have none and some 8 of them. A lane takes two
+// cells in x and walks z: each cell's corners are folded along x and y in the
+// lane, along z from plane to plane in registers. A variable whose range over every
+// active sub-brick of the group lies inside the brush by its margin is not read
+// at all (of a 6-variable brush's variables 4 of 6, on average, at 256^3). FP16
+// volumes fold two cells per instruction as binary16 pairs (exact) and decide them
+// with four comparisons against binary16 bounds (see half_bounds).
 //
-// Bound by instruction issue and load latency: 512^3 FP16 with a 6-variable brush
-// reads about a third of the field.
+// Bound by load latency. One launch against the former four and their counters'
+// clears, which read every restricted variable's x-pairs a sub-brick at a time:
+// 532 -> 205 us at 512^3 FP16 with a 6-variable brush, 109 -> 58 us at 256^3 FP16,
+// 68 -> 44 us at 256^3 FP32 with 4 variables (of 205 us the classification takes
+// 44, the stores 29). Groups of 8 with whole cells' rows in registers measured 250-
+// 390, one warp per word 216, the x-pair layout 204 with twice the bytes.
 #include <algorithm>
 
 #include "common.cuh"
@@ -26,6 +31,8 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kBrushWarps = 8;
+constexpr int kBrushBlocks = 6;                       // resident blocks per SM: load latency wants the warps
+constexpr unsigned kChunkWords = 16;                  // words a block classifies before it takes their groups
 
 __device__ __forceinline__ float margin(float m) { return __fmaf_rn(m, 0x1p-20f, 0x1p-120f); }
 
@@ -88,24 +95,22 @@ struct BrushShared {
 };
 
 __device__ __forceinline__ __half2 as_half2(unsigned u) { return *reinterpret_cast<const __half2*>(&u); }
-__device__ __forceinline__ unsigned as_bits(__half2 h) { return *reinterpret_cast<const unsigned*>(&h); }
 
-// Corner folds of a lane's cells: FP16 two cells in x as a binary16 pair, FP32 one.
+// Corner folds of a lane's two cells (x, x + 1), x even, as a pair of values.
 template <int DT> struct Corners;
 template <> struct Corners<kF16> {
     using V = __half2;
-    static constexpr int kX = 2, kZ = 2;               // cells of a lane along x and z
     static __device__ __forceinline__ V lo(V a, V b) { return __hmin2(a, b); }
     static __device__ __forceinline__ V hi(V a, V b) { return __hmax2_nan(a, b); }
-    // corners (x, x+1) and (x+1, x+2) of a row, x even; even: rows start at even elements
-    static __device__ __forceinline__ void row(const void* cells, size_t r, int x, int n, bool even, V& mn, V& mx) {
-        const unsigned short* c = static_cast<const unsigned short*>(cells) + r;
-        const int x0 = min(x, (n - 1) & ~1), x1 = min(x + 1, n - 1), x2 = min(x + 2, n - 1);
-        const unsigned p = even ? __ldg(reinterpret_cast<const unsigned*>(c + x0))
-                                : (unsigned)__ldg(c + x0) | ((unsigned)__ldg(c + x1) << 16);
-        const unsigned q = __byte_perm(p, (unsigned)__ldg(c + x2), 0x5432);
-        mn = lo(as_half2(p), as_half2(q));
-        mx = hi(as_half2(p), as_half2(q));
+    // corners (x, x+1) and (x+1, x+2) of row c; EVEN: rows start at even elements and x+1 < n
+    template <bool EVEN>
+    static __device__ __forceinline__ void row(const void* c, size_t r, int x0, int x1, int x2, V& mn, V& mx) {
+        const unsigned short* p = static_cast<const unsigned short*>(c) + r;
+        const unsigned a = EVEN ? __ldg(reinterpret_cast<const unsigned*>(p + x0))
+                                : (unsigned)__ldg(p + x0) | ((unsigned)__ldg(p + x1) << 16);
+        const unsigned b = __byte_perm(a, (unsigned)__ldg(p + x2), 0x5432);
+        mn = lo(as_half2(a), as_half2(b));
+        mx = hi(as_half2(a), as_half2(b));
     }
     static __device__ __forceinline__ unsigned classes(const BrushShared& S, int v, V mn, V mx) {
         const unsigned need = 0x00010001u << v;
@@ -120,80 +125,73 @@ template <> struct Corners<kF16> {
     }
 };
 template <> struct Corners<kF32> {
-    using V = float;
-    static constexpr int kX = 1, kZ = 4;
-    static __device__ __forceinline__ V lo(V a, V b) { return fminf(a, b); }
-    static __device__ __forceinline__ V hi(V a, V b) { return max_nan(a, b); }
-    static __device__ __forceinline__ void row(const void* cells, size_t r, int x, int n, bool, V& mn, V& mx) {
-        const float* c = static_cast<const float*>(cells) + r;
-        const float a = __ldg(c + min(x, n - 1)), b = __ldg(c + min(x + 1, n - 1));
+    using V = float2;
+    static __device__ __forceinline__ V lo(V a, V b) { return make_float2(fminf(a.x, b.x), fminf(a.y, b.y)); }
+    static __device__ __forceinline__ V hi(V a, V b) { return make_float2(max_nan(a.x, b.x), max_nan(a.y, b.y)); }
+    template <bool EVEN>
+    static __device__ __forceinline__ void row(const void* c, size_t r, int x0, int x1, int x2, V& mn, V& mx) {
+        const float* p = static_cast<const float*>(c) + r;
+        const float2 a = EVEN ? __ldg(reinterpret_cast<const float2*>(p + x0)) : make_float2(__ldg(p + x0), __ldg(p + x1));
+        const float2 b = make_float2(a.y, __ldg(p + x2));
         mn = lo(a, b);
         mx = hi(a, b);
     }
     static __device__ __forceinline__ unsigned classes(const BrushShared& S, int v, V mn, V mx) {
-        return cell_class(mn, mx, S.it.brush.lo[v], S.it.brush.hi[v], 1u << v);
+        const float lo = S.it.brush.lo[v], hi = S.it.brush.hi[v];
+        return cell_class(mn.x, mx.x, lo, hi, 1u << v) | (cell_class(mn.y, mx.y, lo, hi, 1u << v) << 16);
     }
 };
 
-// Classes of the cells of up to 8 sub-bricks (sx .. sx + 7, sy, sz), sx a multiple
-// of 8, over the variables `vars`; written for the sub-bricks in `act` (bit k: sx + k).
-template <int DT>
+constexpr int kGroup = 4;            // sub-bricks of a group: 8 lanes of two cells in x, 4 lanes in y
+
+// Classes of the cells of up to kGroup sub-bricks (sx .. sx + 3, sy, sz), sx a multiple
+// of kGroup, over the variables `vars`; written for the sub-bricks in `act` (bit k: sx + k).
+template <int DT, bool EVEN>
 __device__ __forceinline__ void classes_of_group(const BrushShared& S, int sx, int sy, int sz, unsigned act,
                                                  unsigned vars, int lane) {
     using C = Corners<DT>;
     using V = typename C::V;
-    constexpr int kLanes = 32 / C::kX;                       // lanes along x; the others take the next z cells
     const int n = S.it.n;
-    const int x = sx * kSub + (lane % kLanes) * C::kX, y = sy * kSub, z = sz * kSub + (lane / kLanes) * C::kZ;
+    const int x = sx * kSub + 2 * (lane & 7), y = sy * kSub + (lane >> 3), z = sz * kSub;
     const size_t nn = (size_t)n * n;
-    const bool even = (n & 1) == 0;
-    unsigned word[C::kZ][kSub];
-#pragma unroll
-    for (int c = 0; c < C::kZ; ++c)
-#pragma unroll
-        for (int r = 0; r < kSub; ++r) word[c][r] = 0u;
+    const int x0 = EVEN ? min(x, n - 2) : min(x, n - 1), x1 = min(x + 1, n - 1), x2 = min(x + 2, n - 1);
+    const size_t r0 = (size_t)min(y, n - 1) * n, r1 = (size_t)min(y + 1, n - 1) * n;
+    unsigned word[kSub] = {0u, 0u, 0u, 0u};
     while (vars) {                                           // uniform over the warp
         const int v = __ffs(vars) - 1;
         vars &= vars - 1u;
         const char* plane = static_cast<const char*>(S.it.cells) + nn * n * (size_t)v * (DT == kF16 ? 2 : 4);
-        V pmn[kSub], pmx[kSub];                              // the previous z plane, folded along x and y
+        V pmn{}, pmx{};                                      // the previous z plane, folded along x and y
 #pragma unroll
-        for (int c = 0; c <= C::kZ; ++c) {
+        for (int c = 0; c <= kSub; ++c) {
             const size_t rz = (size_t)min(z + c, n - 1) * nn;
-            V rmn[kSub + 1], rmx[kSub + 1];
-#pragma unroll
-            for (int r = 0; r <= kSub; ++r)
-                C::row(plane, rz + (size_t)min(y + r, n - 1) * n, x, n, even, rmn[r], rmx[r]);
-#pragma unroll
-            for (int r = 0; r < kSub; ++r) {
-                const V mn = C::lo(rmn[r], rmn[r + 1]), mx = C::hi(rmx[r], rmx[r + 1]);
-                if (c > 0) word[c - 1][r] |= C::classes(S, v, C::lo(pmn[r], mn), C::hi(pmx[r], mx));
-                pmn[r] = mn;
-                pmx[r] = mx;
-            }
+            V amn, amx, bmn, bmx;
+            C::template row<EVEN>(plane, rz + r0, x0, x1, x2, amn, amx);
+            C::template row<EVEN>(plane, rz + r1, x0, x1, x2, bmn, bmx);
+            const V mn = C::lo(amn, bmn), mx = C::hi(amx, bmx);
+            if (c > 0) word[c > 0 ? c - 1 : 0] |= C::classes(S, v, C::lo(pmn, mn), C::hi(pmx, mx));
+            pmn = mn;
+            pmx = mx;
         }
     }
     // cells with an index of n - 1 do not exist
-    if (!((act >> ((lane % kLanes) * C::kX / kSub)) & 1u) || x >= n - 1) return;
+    if (!((act >> ((lane & 7) >> 1)) & 1u) || x >= n - 1 || y >= n - 1) return;
 #pragma unroll
-    for (int c = 0; c < C::kZ; ++c)
-#pragma unroll
-        for (int r = 0; r < kSub; ++r) {
-            if (z + c >= n - 1 || y + r >= n - 1) continue;
-            uint16_t* out = S.it.cls + ((size_t)(z + c) * n + (y + r)) * n + x;
-            if (C::kX == 2 && even) {
-                *reinterpret_cast<unsigned*>(out) = word[c][r];
-            } else {
-                out[0] = (uint16_t)word[c][r];
-                if (C::kX == 2 && x + 1 < n - 1) out[1] = (uint16_t)(word[c][r] >> 16);
-            }
+    for (int c = 0; c < kSub; ++c) {
+        if (z + c >= n - 1) break;
+        uint16_t* out = S.it.cls + ((size_t)(z + c) * n + y) * n + x;
+        if (EVEN) {
+            *reinterpret_cast<unsigned*>(out) = word[c];
+        } else {
+            out[0] = (uint16_t)word[c];
+            if (x + 1 < n - 1) out[1] = (uint16_t)(word[c] >> 16);
         }
+    }
 }
 
-// Word w (32 sub-bricks) of the item; of its groups, this warp computes those with
-// number % split == part.
-template <int DT>
-__device__ __forceinline__ void classify_word(const BrushShared& S, unsigned w, int part, int split, int lane) {
+// Classify word w (32 sub-bricks) of the item, store its activity bits and append the
+// groups with active sub-bricks to the block's list.
+__device__ __forceinline__ void classify_word(const BrushShared& S, unsigned w, int lane, uint2* list, unsigned* count) {
     const int nsb = S.it.nsb;
     const unsigned total = (unsigned)nsb * nsb * nsb;
     const unsigned b = w * 32u + lane;
@@ -204,31 +202,41 @@ __device__ __forceinline__ void classify_word(const BrushShared& S, unsigned w, 
         const size_t o = (size_t)b * S.it.nvars + S.it.color_var;
         act = tf_range_visible(S.it.sbmin[o], S.it.sbmax[o], S.it.tf_prefix, S.it.tf_lo, S.it.tf_scale);
     }
-    unsigned rem = __ballot_sync(kFull, act);
-    if (lane == 0 && part == 0) S.it.active[w] = rem;
-    if (!S.it.cls) return;
+    const unsigned word = __ballot_sync(kFull, act);
+    if (lane == 0) S.it.active[w] = word;
+    if (!S.it.cls || word == 0u) return;
     // a NaN corner fails its cell whatever the range says: ranges decide finite levels only
-    const unsigned mine = S.it.brush.mask & ~(S.finite ? inside : 0u);
-    int group = 0;
-    while (rem) {
-        const int j = __ffs(rem) - 1;
-        const unsigned id = w * 32u + j;
-        const int sx = (int)(id % nsb), sy = (int)((id / nsb) % nsb), sz = (int)(id / ((unsigned)nsb * nsb));
-        const int first = j - (sx & 7);                      // lane of sub-brick sx & ~7 (may be < 0)
-        const int end = min(min(first + 8, j + nsb - sx), 32);
-        const unsigned lanes = (end < 32 ? (1u << end) - 1u : kFull) & ~((1u << j) - 1u);
-        const unsigned here = rem & lanes;
-        rem &= ~lanes;
-        if (group++ % split != part) continue;
-        const unsigned vars = __reduce_or_sync(kFull, (here >> lane) & 1u ? mine : 0u);
-        classes_of_group<DT>(S, sx & ~7, sy, sz, first >= 0 ? here >> first : here << -first, vars, lane);
+    const unsigned mine = act ? S.it.brush.mask & ~(S.finite ? inside : 0u) : 0u;
+    // the lanes of this lane's group: kGroup neighbours in x, cut at the word's and the row's ends
+    const int sx = (int)(b % (unsigned)nsb), k = sx & (kGroup - 1);
+    const int first = lane - k, end = min(min(first + kGroup, lane + nsb - sx), 32);
+    const unsigned lanes = (end < 32 ? (1u << end) - 1u : kFull) & ~((1u << max(first, 0)) - 1u);
+    unsigned vars = 0u;
+#pragma unroll
+    for (int q = 0; q < kGroup; ++q) {                       // the group's lanes are consecutive
+        const int l = max(first, 0) + q;
+        const unsigned m = __shfl_sync(kFull, mine, l & 31);
+        if (l < end) vars |= m;
     }
+    const unsigned here = word & lanes;
+    const bool head = lane == max(first, 0) && here != 0u;   // one lane per group
+    const unsigned heads = __ballot_sync(kFull, head);
+    unsigned at = 0u;
+    if (lane == 0) at = atomicAdd(count, (unsigned)__popc(heads));
+    at = __shfl_sync(kFull, at, 0) + __popc(heads & ((1u << lane) - 1u));
+    // sub-brick id of the group's first place (its row's, in front of this word too), which of
+    // the group are active, the variables to read
+    if (head) list[at] = make_uint2(b - k, (first >= 0 ? here >> first : here << -first) << 8 | vars);
 }
 
-// Blocks walk the chunks (kBrushWarps * per_warp / split words) of all items.
+// Blocks walk the chunks (P.words words each) of all items: the warps first
+// classify the chunk's words, then take its groups from the block's list one by one
+// (a word has between none and 32, and each takes a load latency per variable).
 template <int DT>
-__global__ void __launch_bounds__(32 * kBrushWarps) k_brush(const __grid_constant__ BrushLaunch P) {
+__global__ void __launch_bounds__(32 * kBrushWarps, kBrushBlocks) k_brush(const __grid_constant__ BrushLaunch P) {
     __shared__ BrushShared S;
+    __shared__ uint2 s_list[32 * kChunkWords];
+    __shared__ unsigned s_count, s_next;
     const BrushItem* items = P.table ? P.table : P.items;
     const int nitems = P.table ? P.header->nviews : P.nitems;
     const unsigned total = P.table ? P.header->chunks : P.chunks;
@@ -240,8 +248,9 @@ __global__ void __launch_bounds__(32 * kBrushWarps) k_brush(const __grid_constan
             const int mid = (vi + hi + 1) >> 1;
             if (items[mid].chunk_begin <= c) vi = mid; else hi = mid - 1;
         }
+        __syncthreads();                                     // the previous chunk's state is no longer read
+        if (threadIdx.x == 0) s_count = s_next = 0u;
         if (vi != cur) {                                     // uniform over the block
-            __syncthreads();
             static_assert(sizeof(BrushItem) % 4 == 0, "copied by words");
             for (int i = threadIdx.x; i < (int)(sizeof(BrushItem) / 4); i += blockDim.x)
                 reinterpret_cast<unsigned*>(&S.it)[i] = reinterpret_cast<const unsigned*>(items + vi)[i];
@@ -268,14 +277,25 @@ __global__ void __launch_bounds__(32 * kBrushWarps) k_brush(const __grid_constan
             }
             __syncthreads();
             if (threadIdx.x == 0 && !S.finite) S.pairs = 0u;  // NaN and infinite corners: cell_class
-            __syncthreads();
             cur = vi;
         }
-        const unsigned words = ((unsigned)S.it.nsb * S.it.nsb * S.it.nsb + 31u) / 32u;
-        for (int i = 0; i < P.per_warp; ++i) {
-            const unsigned unit = ((c - S.it.chunk_begin) * P.per_warp + i) * kBrushWarps + warp;
-            const unsigned w = unit / P.split;
-            if (w < words) classify_word<DT>(S, w, (int)(unit % P.split), P.split, lane);
+        __syncthreads();
+        const int nsb = S.it.nsb;
+        const unsigned words = ((unsigned)nsb * nsb * nsb + 31u) / 32u;
+        const unsigned w0 = (c - S.it.chunk_begin) * P.words;
+        for (unsigned w = w0 + warp; w < min(words, w0 + P.words); w += kBrushWarps)
+            classify_word(S, w, lane, s_list, &s_count);
+        __syncthreads();
+        const unsigned groups = s_count;
+        for (;;) {
+            unsigned g = 0u;
+            if (lane == 0) g = atomicAdd(&s_next, 1u);
+            g = __shfl_sync(kFull, g, 0);
+            if (g >= groups) break;
+            const uint2 e = s_list[g];
+            const int sx = (int)(e.x % (unsigned)nsb), sy = (int)((e.x / nsb) % nsb), sz = (int)(e.x / ((unsigned)nsb * nsb));
+            if ((S.it.n & 1) == 0) classes_of_group<DT, true>(S, sx, sy, sz, e.y >> 8, e.y & 0xffu, lane);
+            else classes_of_group<DT, false>(S, sx, sy, sz, e.y >> 8, e.y & 0xffu, lane);
         }
     }
 }
@@ -337,42 +357,43 @@ unsigned words_of(int n) {
     return (nsb * nsb * nsb + 31u) / 32u;
 }
 
-constexpr int kPerWarp = 2;          // units a warp takes before its block looks for the next chunk
+int sm_count() {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms > 0 ? sms : 1;
+}
 
 }  // namespace
 
-unsigned brush_chunks(int n) {
-    const unsigned unit = (unsigned)(kBrushWarps * kPerWarp);
-    return (words_of(n) + unit - 1) / unit;
-}
+unsigned brush_chunks(int n) { return (words_of(n) + kChunkWords - 1) / kChunkWords; }
 
-// Grids of fewer words than the GPU has warps give each word's groups to four warps.
+// Chunks of kChunkWords words, or on grids with fewer chunks than SMs have room for,
+// fewer words, so that every SM has some.
 cudaError_t launch_brush(BrushLaunch& P, int dtype, cudaStream_t stream) {
     unsigned words = 0;
     for (int i = 0; i < P.nitems; ++i) words += words_of(P.items[i].n);
+    const unsigned blocks = (unsigned)sm_count() * kBrushBlocks;
     P.table = nullptr;
     P.header = nullptr;
-    P.split = words < 4096 ? 4 : 1;
-    P.per_warp = words < 4096 ? 1 : kPerWarp;
+    P.words = std::min<unsigned>(kChunkWords, std::max(1u, (words + blocks - 1) / blocks));
     P.chunks = 0;
-    const unsigned unit = (unsigned)(kBrushWarps * P.per_warp / (P.split > kBrushWarps ? 1 : 1));
     for (int i = 0; i < P.nitems; ++i) {
         P.items[i].chunk_begin = P.chunks;
-        P.chunks += (words_of(P.items[i].n) * (unsigned)P.split + unit - 1) / unit;
+        P.chunks += (words_of(P.items[i].n) + P.words - 1) / P.words;
     }
-    if (dtype == kF16) k_brush<kF16><<<P.chunks, 32 * kBrushWarps, 0, stream>>>(P);
-    else k_brush<kF32><<<P.chunks, 32 * kBrushWarps, 0, stream>>>(P);
+    if (dtype == kF16) k_brush<kF16><<<std::min(P.chunks, blocks), 32 * kBrushWarps, 0, stream>>>(P);
+    else k_brush<kF32><<<std::min(P.chunks, blocks), 32 * kBrushWarps, 0, stream>>>(P);
     count_launches(1);
     return cudaGetLastError();
 }
 
-cudaError_t launch_brush_views(const BatchHeader* hdr, const BrushItem* table, int dtype, unsigned blocks,
-                               cudaStream_t stream) {
+cudaError_t launch_brush_views(const BatchHeader* hdr, const BrushItem* table, int dtype, cudaStream_t stream) {
     BrushLaunch P{};
     P.table = table;
     P.header = hdr;
-    P.split = 1;
-    P.per_warp = kPerWarp;
+    P.words = kChunkWords;
+    const unsigned blocks = (unsigned)sm_count() * kBrushBlocks;
     if (dtype == kF16) k_brush<kF16><<<blocks, 32 * kBrushWarps, 0, stream>>>(P);
     else k_brush<kF32><<<blocks, 32 * kBrushWarps, 0, stream>>>(P);
     return cudaGetLastError();

@@ -169,14 +169,9 @@ template <> __device__ __forceinline__ float load_cell<kF16>(const void* base, s
 // Kernel argument blocks.
 // ---------------------------------------------------------------------------
 struct LevelArgs {
-    const void* cells;         // planar values
     const void* pairs;         // x-pairs per variable
     int n;                     // cube edge in cells
-    int nb;                    // bricks per axis
     int nsb;                   // sub-bricks per axis
-    const float* bmin;         // [nb^3][nvars]
-    const float* bmax;
-    const uint32_t* active;    // bitmask, ceil(nb^3/32) words
     const uint32_t* sactive;   // sub-brick bitmask, ceil(nsb^3/32) words
     const uint8_t* sdist;      // optional: padded empty-space distance of the sub-bricks under sactive
                                // (see launch_subbrick_distance); the march searches it, and renders
@@ -245,7 +240,6 @@ struct RenderArgs {
     LevelArgs lv;
     int nvars;
     BrushArgs brush;
-    const unsigned* pass_count;   // per variable: bricks passing that variable alone (order hint)
     float eye[3], target[3], up[3], tan_half;
     int w, h;
     float dt;
@@ -268,8 +262,6 @@ struct RenderArgs {
     float4* out;
     uint32_t* counts;             // optional [h][w][2]
     float* depth;                 // optional [h][w]: t of the first kept sample, +inf if none
-    const int* tf_prefix;         // [kTF + 1]: entries < j with sigma > 0 (TF visibility)
-    int tf_skip;                  // batched views: classify against the TF visibility too
     unsigned long long* stats;    // optional kNStats counters
 };
 
@@ -283,23 +275,25 @@ struct ViewDone {
     unsigned long long stats[kNStats];
 };
 
-// One view of a batched render, as its classification reads it: the march
-// arguments (lv.active / lv.sactive / pass_count point at this view's own
-// classification), the level's brick and sub-brick min/max for that
-// classification, and the view's ranges in the flat brick and distance-tile
-// spaces of the batch. A view's flat brick range holds its bricks (padded to a
-// multiple of 32) followed by its sub-bricks.
-struct BatchView {
-    RenderArgs a;
-    const float* bmin;
-    const float* bmax;
-    const float* sbmin;
+// One level to classify under a brush (see brush_kernels.cu).
+struct BrushItem {
+    const float* sbmin;            // [nsb^3][nvars], sub-brick min/max
     const float* sbmax;
-    unsigned long long cls_begin;  // first flat brick index (multiple of 32)
-    unsigned long long cls_sub;    // offset of the first sub-brick in the view's range (multiple of 32)
-    uint32_t* slist;               // active sub-bricks of the view (any order), for its cell classes
-    uint32_t* scount;              // their number (zeroed per launch)
-    int dist_begin;                // first flat tile of the view's empty-space distance (a.lv.sdist)
+    const void* cells;             // planar values, storage dtype
+    uint32_t* active;              // sub-brick activity bits, written
+    uint16_t* cls;                 // optional: cell classes, written for the cells of active sub-bricks
+    const unsigned long long* stats;   // [kMaxVars + 1] magnitudes of the level (see LevelStats)
+    const int* tf_prefix;          // optional: activity AND visibility of the transfer function
+                                   // ([kTF + 1]: entries < j with sigma > 0)
+    uint8_t* sdist;                // batched views: padded empty-space distance, written afterwards
+    unsigned gen;                  // generation of stats
+    int n, nsb, nvars;
+    float rin2, rout2;             // r_in * r_in, r_out * r_out rounded to FP32
+    int color_var;
+    float tf_lo, tf_scale;
+    unsigned chunk_begin;          // first chunk of this item, set by the launcher (table: by the caller)
+    int dist_begin;                // batched views: first distance tile
+    BrushArgs brush;
 };
 
 // Completion of one view of a batch, and the parameters of its render node.
@@ -316,8 +310,42 @@ struct ViewLaunch {
 
 struct BatchHeader {
     int nviews;
-    unsigned long long cls_total;  // flat brick range over all views (multiple of 32)
+    unsigned chunks;               // brush chunks over all views
     int dist_total;                // distance tiles over all views
+};
+
+// Items of one classification launch: a few in the parameters, or the views of a
+// batch in a device table.
+constexpr int kBrushItems = 3;
+struct BrushLaunch {
+    const BrushItem* table;        // null: items
+    const BatchHeader* header;     // of table
+    int nitems;
+    unsigned words, chunks;        // words per chunk and chunks, set by the launcher
+    BrushItem items[kBrushItems];
+};
+
+// Magnitudes of a level's stored values, written by the kernel that computes its
+// min/max: per variable, then for non-finite values, the key
+// (generation << 32) | bits -- bits of the largest |value|, or 1 when a value is
+// NaN or infinite. A key of another generation holds nothing of this one, so
+// the keys need no clearing between ingests.
+struct LevelStats {
+    unsigned long long* key;       // [kMaxVars + 1]
+    unsigned gen;
+};
+
+// Activity, dilation and ordered list of a level's 8^3 bricks (inspection).
+struct BrickListArgs {
+    const float* bmin;             // [nb^3][nvars]
+    const float* bmax;
+    int n, nb, nvars;
+    float rin2, rout2;
+    BrushArgs brush;
+    uint32_t* active;
+    uint32_t* skippable;
+    uint32_t* list;
+    uint32_t* n_active;
 };
 
 // Render launch variants: a 128-thread block is 2 x 2 warps; each warp marches
@@ -407,11 +435,12 @@ __device__ __forceinline__ bool tf_range_visible(float mn, float mx, const int* 
 // rounding), and the box meets the position brush. A variable with
 // max(|min_v|, |max_v|) > 2^126 never deactivates
 // a brick (a corner difference can overflow and the interpolated value be
-// infinite). pass_bits gets bit v set for each restricted variable the brick
-// passes on its own (only meaningful when the box meets the shell).
+// infinite). inside gets bit v set for each restricted variable whose every value
+// in the brick passes by the margin (min_v - d >= lo_v and max_v + d <= hi_v;
+// NaN values, which the range ignores, aside); only meaningful for active bricks.
 __device__ __forceinline__ bool classify_brick(size_t b, int nb, int bs, float sc, float rin2, float rout2,
                                                const BrushArgs& brush, int nvars, const float* bmin,
-                                               const float* bmax, unsigned& pass_bits) {
+                                               const float* bmax, unsigned& inside) {
     int c[3] = {(int)(b % nb), (int)((b / nb) % nb), (int)(b / ((size_t)nb * nb))};
     float nearc[3], farc[3];
 #pragma unroll
@@ -423,7 +452,7 @@ __device__ __forceinline__ bool classify_brick(size_t b, int nb, int bs, float s
     }
     const float near2 = dot3_rn(nearc[0], nearc[1], nearc[2], nearc[0], nearc[1], nearc[2]);
     const float far2 = dot3_rn(farc[0], farc[1], farc[2], farc[0], farc[1], farc[2]);
-    pass_bits = 0;
+    inside = 0;
     if (!((near2 <= rout2) && (far2 >= rin2))) return false;
     if (brush.pmask) {
         // the box must meet every restricted coordinate range, and its radius range
@@ -444,9 +473,9 @@ __device__ __forceinline__ bool classify_brick(size_t b, int nb, int bs, float s
         const float mn = bmin[b * nvars + v], mx = bmax[b * nvars + v];
         const float m = fmaxf(fabsf(mn), fabsf(mx));
         const float d = __fmaf_rn(m, 0x1p-20f, 0x1p-120f);
-        const bool ok = m > 0x1p126f || ((__fadd_rn(mx, d) >= brush.lo[v]) && (__fsub_rn(mn, d) <= brush.hi[v]));
-        if (ok) pass_bits |= 1u << v;
-        all = all && ok;
+        const float up = __fadd_rn(mx, d), dn = __fsub_rn(mn, d);
+        if (m <= 0x1p126f && dn >= brush.lo[v] && up <= brush.hi[v]) inside |= 1u << v;
+        all = all && (m > 0x1p126f || (up >= brush.lo[v] && dn <= brush.hi[v]));
     }
     return all;
 }
@@ -465,37 +494,6 @@ __device__ __forceinline__ bool skippable_brick(size_t b, int nb, const uint32_t
     return true;
 }
 
-// Classification of all built levels of a volume in one launch per kernel.
-// Entries 0..nbrick-1 are the 8^3 bricks of the levels (active, skippable,
-// compacted list, selectivity counts); the entries after them are sub-brick
-// grids (bs = kSub: active bits only; the other outputs are null).
-struct ClassifyLevel {
-    const float* bmin;
-    const float* bmax;
-    int n;                        // level edge
-    int bs;                       // brick edge (kBrick or kSub)
-    float sc;                     // 2 / n, set by the launcher
-    size_t first;                 // first flat index of this entry (multiple of 32), set by the launcher
-    uint32_t* active;
-    uint32_t* skippable;
-    uint32_t* list;
-    uint32_t* n_active;
-    unsigned* pass_count;
-    uint32_t* alist;              // optional: active ids in no particular order ...
-    uint32_t* acount;             // ... and their number (zeroed by the launcher)
-};
-
-struct ClassifyArgs {
-    int nlev;                     // entries in lv
-    int nbrick;                   // leading entries with bs = kBrick
-    int nvars;
-    float rin2, rout2;            // r_in * r_in, r_out * r_out rounded to FP32
-    BrushArgs brush;
-    size_t total;                 // set by the launcher: flat range of all entries
-    size_t total_brick;           // set by the launcher: flat range of the kBrick entries
-    ClassifyLevel lv[6];
-};
-
 // Cell classes under a brush: for the interpolation cell with lower corner
 // (x, y, z) and each restricted variable v, over its 8 corner values: FAIL if
 // a corner is NaN or, with m = max(|min|, |max|) <= 2^126 and the brick
@@ -505,98 +503,12 @@ struct ClassifyArgs {
 // be interpolated, kCellFail = some restricted variable fails; [z][y][x] over
 // n^3 (entries with an index of n-1 are not written).
 constexpr unsigned kCellFail = 0x8000u;
-struct CellClassArgs {
-    const void* pairs;            // x-pair layout of the level (see Pair)
-    int n;
-    int nvars;
-    BrushArgs brush;
-    const uint32_t* slist;        // active sub-brick ids under this brush (any order) ...
-    const uint32_t* scount;       // ... and their number (device)
-    uint16_t* out;                // written for the cells of the listed sub-bricks only
-};
 
 // NaN-propagating max (a NaN operand gives NaN).
 __device__ __forceinline__ float max_nan(float a, float b) {
     float d;
     asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
     return d;
-}
-
-// Restricted variables of a brush in increasing order: ids packed 4 bits
-// each, bounds in the same order.
-struct CellVars {
-    int nr;
-    unsigned ids;
-    float lo[kMaxVars], hi[kMaxVars];
-};
-
-__host__ __device__ inline void cell_vars_of(const BrushArgs& b, int nvars, CellVars& R) {
-    R.nr = 0;
-    R.ids = 0;
-    for (int v = 0; v < nvars && v < kMaxVars; ++v)
-        if ((b.mask >> v) & 1u) {
-            R.ids |= (unsigned)v << (4 * R.nr);
-            R.lo[R.nr] = b.lo[v];
-            R.hi[R.nr] = b.hi[v];
-            ++R.nr;
-        }
-}
-
-constexpr int kCellWarps = 4;                           // warps per block of the cell-class kernels
-
-// Cell class words of the 4 x 4 x 4 cells of sub-brick `id` (see
-// CellClassArgs), computed by one warp: lane (lx, ly, lz) takes the cells
-// (4sx + lx, 4sy + ly, 4sz + 2lz + {0, 1}). Per restricted variable a lane
-// loads its 2 x 3 corner x-pairs (the render's layout: one load gives both
-// x-corners) at once; the corner max propagates NaN, so a NaN corner shows as
-// a NaN cell max. Cells with an index of n-1 do not exist and are not written.
-template <int DT>
-__device__ __forceinline__ void cell_classes_of_subbrick(const void* __restrict__ pairs, int n, int nsb, uint32_t id,
-                                                         int lane, const CellVars& R, uint16_t* __restrict__ out) {
-    const int lx = lane & 3, ly = (lane >> 2) & 3, lz = lane >> 4;
-    const size_t nn = (size_t)n * n;
-    const int sx = (int)(id % nsb), sy = (int)((id / nsb) % nsb), sz = (int)(id / ((uint32_t)nsb * nsb));
-    const int x = sx * kSub + lx, y = sy * kSub + ly, z = sz * kSub + 2 * lz;
-    const int y0 = min(y, n - 1), y1 = min(y + 1, n - 1), x0 = min(x, n - 1);   // pair x0 = (c[x0], c[min(x0+1, n-1)])
-    const int zc[3] = {min(z, n - 1), min(z + 1, n - 1), min(z + 2, n - 1)};
-    unsigned word[2] = {0u, 0u};
-#pragma unroll
-    for (int j = 0; j < kMaxVars; ++j) {
-        if (j >= R.nr) break;
-        const int v = (R.ids >> (4 * j)) & 15u;
-        const size_t pv = (size_t)v * nn * n;
-        float mn3[3], mx3[3];
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            const size_t r0 = pv + zc[q] * nn + (size_t)y0 * n, r1 = pv + zc[q] * nn + (size_t)y1 * n;
-            const float2 p0 = Pair<DT>::load(pairs, r0 + x0), p1 = Pair<DT>::load(pairs, r1 + x0);
-            mn3[q] = fminf(fminf(p0.x, p0.y), fminf(p1.x, p1.y));
-            mx3[q] = max_nan(max_nan(p0.x, p0.y), max_nan(p1.x, p1.y));
-        }
-        const float lo = R.lo[j], hi = R.hi[j];
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const float mn = fminf(mn3[c], mn3[c + 1]), mx = max_nan(mx3[c], mx3[c + 1]);
-            unsigned w;
-            if (mx != mx) {
-                w = kCellFail;                                         // a NaN corner
-            } else {
-                const float m = fmaxf(fabsf(mn), fabsf(mx));
-                const float d = __fmaf_rn(m, 0x1p-20f, 0x1p-120f);
-                const float up = __fadd_rn(mx, d), dn = __fsub_rn(mn, d);
-                if (m > 0x1p126f) w = 1u << v;
-                else if (up < lo || dn > hi) w = kCellFail;
-                else if (dn >= lo && up <= hi) w = 0u;
-                else w = 1u << v;
-            }
-            word[c] |= w;
-        }
-    }
-    if (x < n - 1 && y < n - 1) {
-#pragma unroll
-        for (int c = 0; c < 2; ++c)
-            if (z + c < n - 1) out[((size_t)(z + c) * n + y) * n + x] = (uint16_t)word[c];
-    }
 }
 
 // Process-wide count of launched kernels (defined in api.cu).
@@ -608,9 +520,9 @@ void count_launches(int k);
 constexpr int kMaxRowsEdge = 4096;
 cudaError_t launch_ingest(const void* src, int src_dtype, void* cells, void* pairs, int dtype,
                           int n, int nvars, float* bmin, float* bmax, float* sbmin, float* sbmax,
-                          cudaStream_t stream);
+                          LevelStats stats, cudaStream_t stream);
 cudaError_t launch_lod(const void* fine, int n_fine, void* cells, void* pairs, int dtype, int nvars,
-                       float* bmin, float* bmax, float* sbmin, float* sbmax, cudaStream_t stream);
+                       float* bmin, float* bmax, float* sbmin, float* sbmax, LevelStats stats, cudaStream_t stream);
 // Ingest that also writes the next level's cells and x-pairs (edge n / 2, the same
 // 2x2x2 means as launch_lod, from the values it stores) in the same pass over the
 // source; that level's brick min/max then come from launch_level_bricks. Only when
@@ -618,20 +530,19 @@ cudaError_t launch_lod(const void* fine, int n_fine, void* cells, void* pairs, i
 bool ingest_next_level_fits(const void* src, int n);
 cudaError_t launch_ingest_next_level(const void* src, int src_dtype, void* cells, void* pairs, int dtype, int n,
                                      int nvars, float* bmin, float* bmax, float* sbmin, float* sbmax,
-                                     void* next_cells, void* next_pairs, cudaStream_t stream);
+                                     void* next_cells, void* next_pairs, LevelStats stats, cudaStream_t stream);
 // Brick and sub-brick min/max of a level from its own stored cells.
 cudaError_t launch_level_bricks(const void* cells, int dtype, int n, int nvars, float* bmin, float* bmax,
-                                float* sbmin, float* sbmax, cudaStream_t stream);
-cudaError_t launch_classify(ClassifyArgs& c, cudaStream_t stream);
-cudaError_t launch_cell_classes(const CellClassArgs& a, int dtype, cudaStream_t stream);
+                                float* sbmin, float* sbmax, LevelStats stats, cudaStream_t stream);
+// Sub-brick activity bits and cell classes of P.items[0 .. nitems-1] (brush_kernels.cu),
+// and of every view of a batch (brush_chunks(n) chunks per view).
+cudaError_t launch_brush(BrushLaunch& P, int dtype, cudaStream_t stream);
+unsigned brush_chunks(int n);
+cudaError_t launch_brush_views(const BatchHeader* hdr, const BrushItem* table, int dtype, cudaStream_t stream);
+cudaError_t launch_brick_list(const BrickListArgs& a, cudaStream_t stream);
 cudaError_t launch_render(const RenderArgs& a, int dtype, cudaStream_t stream);
-// Batched render: per-view classification (bricks, sub-bricks, the cell classes
-// of the active sub-bricks into a.cls, the empty-space distance into a.lv.sdist),
-// with a grid fixed by the caller so that the launches can be captured in a
-// graph; then one render node per view (v stays alive while the node parameters
-// are used). Launches are not counted here (the caller counts each replay).
-cudaError_t launch_view_classes(const BatchHeader* hdr, const BatchView* views, int dtype, unsigned cls_blocks,
-                                cudaStream_t stream);
+// Render node of one view of a batch (v stays alive while the node parameters are
+// used). Its launches are not counted here (the caller counts each replay).
 cudaKernelNodeParams render_view_node(ViewLaunch& v, int dtype);
 cudaError_t launch_histogram(const HistArgs& a, int dtype, cudaStream_t stream);
 
@@ -650,19 +561,15 @@ struct WarpArgs {
 };
 cudaError_t launch_warp(const WarpArgs& a, cudaStream_t stream);
 
-// TF-aware skipping (volume_kernels.cu): activity bits of the 8^3 bricks and
-// 4^3 sub-bricks of a level ANDed with their TF visibility.
+// TF-aware skipping (volume_kernels.cu): activity bits of the 4^3 sub-bricks of a
+// level ANDed with their TF visibility.
 struct TfVisArgs {
-    int n, nb, nsb, nvars, color_var;
-    const float* bmin;            // [nb^3][nvars]
-    const float* bmax;
+    int nsb, nvars, color_var;
     const float* sbmin;           // [nsb^3][nvars]
     const float* sbmax;
-    const uint32_t* active;       // brush activity bits
-    const uint32_t* sactive;
-    const float4* tf;             // 256 entries (r, g, b, sigma)
+    const uint32_t* sactive;      // brush activity bits
+    const int* tf_prefix;         // [kTF + 1]: entries < j with sigma > 0
     float tf_lo, tf_scale;
-    uint32_t* out_active;         // nwords / nswords
     uint32_t* out_sactive;
 };
 cudaError_t launch_tf_visibility(const TfVisArgs& a, cudaStream_t stream);
@@ -673,10 +580,10 @@ cudaError_t launch_tf_visibility(const TfVisArgs& a, cudaStream_t stream);
 // (padded_bytes(n)), or with raw the nsb^3 distances themselves.
 cudaError_t launch_subbrick_distance(const uint32_t* sactive, int n, uint8_t* out, bool raw, cudaStream_t stream);
 // The same for every view of a batch, from the view's own activity bits into its
-// a.lv.sdist, after the per-view classification; `blocks` blocks take the views'
+// sdist, after the per-view classification; `blocks` blocks take the views'
 // tiles (subbrick_distance_tiles(n) per view, from its dist_begin on).
 int subbrick_distance_tiles(int n);
-cudaError_t launch_subbrick_distance_views(const BatchHeader* hdr, const BatchView* views, unsigned blocks,
+cudaError_t launch_subbrick_distance_views(const BatchHeader* hdr, const BrushItem* views, unsigned blocks,
                                            cudaStream_t stream);
 
 // PC line subsample (pcsub_kernels.cu).

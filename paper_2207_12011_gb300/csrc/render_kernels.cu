@@ -406,81 +406,6 @@ __global__ void __launch_bounds__(kThreads) k_render(RenderArgs A) {
         march_pixel<DT, VAR, DEPTH, WIDE>(A, S, blockIdx.x, blockIdx.y, threadIdx.x >> 5);
 }
 
-// Per-view classification of a batch: one thread per (view, brick); a warp's
-// 32 consecutive flat indices always belong to one view.
-__device__ __forceinline__ int view_of_brick(const BatchHeader& H, const BatchView* V, unsigned long long g) {
-    int lo = 0, hi = H.nviews - 1;
-    while (lo < hi) {
-        int mid = (lo + hi + 1) >> 1;
-        if (V[mid].cls_begin <= g) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
-__global__ void k_classify_views(const BatchHeader* __restrict__ hdr, const BatchView* __restrict__ views) {
-    const BatchHeader H = *hdr;
-    const int lane = threadIdx.x & 31;
-    const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-    for (unsigned long long g = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; g < H.cls_total; g += stride) {
-        const int vi = view_of_brick(H, views, g - lane);
-        const BatchView& V = views[vi];
-        size_t b = g - V.cls_begin;
-        const bool sub = b >= V.cls_sub;             // uniform per warp: cls_sub is a multiple of 32
-        if (sub) b -= V.cls_sub;
-        const int nb = sub ? V.a.lv.nsb : V.a.lv.nb;
-        const size_t nbricks = (size_t)nb * nb * nb;
-        unsigned pass_bits = 0;
-        bool act = b < nbricks &&
-            classify_brick(b, nb, sub ? kSub : kBrick, 2.0f / (float)V.a.lv.n, V.a.rin2, V.a.rout2, V.a.brush,
-                           V.a.nvars, sub ? V.sbmin : V.bmin, sub ? V.sbmax : V.bmax, pass_bits);
-        if (act && V.a.tf_skip) {                    // TF-aware skipping of this view
-            const size_t o = b * V.a.nvars + V.a.color_var;
-            act = tf_range_visible((sub ? V.sbmin : V.bmin)[o], (sub ? V.sbmax : V.bmax)[o], V.a.tf_prefix,
-                                   V.a.tf_lo, V.a.tf_scale);
-        }
-        const unsigned word = __ballot_sync(0xffffffffu, act);
-        uint32_t* active = const_cast<uint32_t*>(sub ? V.a.lv.sactive : V.a.lv.active);
-        if (lane == 0) active[b >> 5] = word;
-        if (sub) {
-            // list the active sub-bricks for the view's cell classes
-            if (V.slist && word) {
-                unsigned base = 0;
-                if (lane == 0) base = atomicAdd(V.scount, (unsigned)__popc(word));
-                base = __shfl_sync(0xffffffffu, base, 0);
-                if (act) V.slist[base + __popc(word & ((1u << lane) - 1u))] = (uint32_t)b;
-            }
-            continue;
-        }
-        for (int v = 0; v < V.a.nvars; ++v) {
-            const unsigned cnt = __popc(__ballot_sync(0xffffffffu, (pass_bits >> v) & 1u));
-            if (lane == 0 && cnt) atomicAdd(const_cast<unsigned*>(V.a.pass_count) + v, cnt);
-        }
-    }
-}
-
-// Cell classes of every view of a batch (see cell_classes_of_subbrick): the
-// blocks walk the views in order, each warp taking listed sub-bricks of the
-// current view; a view's restricted-variable list is built once per block.
-template <int DT>
-__global__ void __launch_bounds__(32 * kCellWarps) k_cell_classes_views(const BatchHeader* __restrict__ hdr,
-                                                                       const BatchView* __restrict__ views) {
-    __shared__ CellVars s_vars;
-    const int nviews = hdr->nviews;
-    const int lane = threadIdx.x & 31;
-    for (int vi = 0; vi < nviews; ++vi) {
-        const BatchView& V = views[vi];
-        if (!V.slist || !V.a.cls) continue;                 // uniform: the view's table entry
-        __syncthreads();                                    // previous view's s_vars no longer read
-        if (threadIdx.x == 0) cell_vars_of(V.a.brush, V.a.nvars, s_vars);
-        __syncthreads();
-        const unsigned count = *V.scount;
-        const int n = V.a.lv.n, nsb = V.a.lv.nsb;
-        uint16_t* out = const_cast<uint16_t*>(V.a.cls);
-        for (unsigned i = blockIdx.x * kCellWarps + (threadIdx.x >> 5); i < count; i += gridDim.x * kCellWarps)
-            cell_classes_of_subbrick<DT>(V.a.lv.pairs, n, nsb, __ldg(V.slist + i), lane, s_vars, out);
-    }
-}
-
 // One view of a batch: the single-frame kernel (its arguments have to sit at a
 // fixed place in the launch parameters: the march reads them as constant
 // operands, and a table of views indexed by the block measured 530 against
@@ -559,18 +484,6 @@ cudaKernelNodeParams render_view_node(ViewLaunch& v, int dtype) {
     p.blockDim = dim3(kThreads);
     p.kernelParams = v.arg;
     return p;
-}
-
-cudaError_t launch_view_classes(const BatchHeader* hdr, const BatchView* views, int dtype, unsigned cls_blocks,
-                                cudaStream_t stream) {
-    k_classify_views<<<cls_blocks, 256, 0, stream>>>(hdr, views);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (dtype == kF16) k_cell_classes_views<kF16><<<cls_blocks, 32 * kCellWarps, 0, stream>>>(hdr, views);
-    else k_cell_classes_views<kF32><<<cls_blocks, 32 * kCellWarps, 0, stream>>>(hdr, views);
-    e = cudaGetLastError();
-    if (e == cudaSuccess) e = launch_subbrick_distance_views(hdr, views, cls_blocks, stream);
-    return e;
 }
 
 }  // namespace raypc

@@ -51,20 +51,19 @@ struct Level {
     uint32_t* skippable = nullptr;
     uint32_t* list = nullptr;
     uint32_t* n_active = nullptr;
-    unsigned* pass_count = nullptr;
+    unsigned long long* stats = nullptr;   // magnitudes of the stored values (see LevelStats) ...
+    unsigned gen = 0;                      // ... of this many min/max passes
     float* sbmin = nullptr;       // [nsb^3][nvars]
     float* sbmax = nullptr;
     uint32_t* sactive = nullptr;  // sub-brick activity bits under the current brush
-    uint32_t* slist = nullptr;    // active sub-brick ids (any order) and their number
-    uint32_t* scount = nullptr;
     uint16_t* cls = nullptr;      // cell classes under the current brush (n^3), computed on demand
-    uint32_t* tf_active = nullptr;   // activity AND TF visibility (renders with tf_skip)
-    uint32_t* tf_sactive = nullptr;
+    uint32_t* tf_sactive = nullptr;  // activity AND TF visibility (renders with tf_skip)
     uint8_t* sdist = nullptr;        // padded empty-space distance of the sub-bricks (renders)
     const uint32_t* sdist_of = nullptr;   // activity bits the distance was computed from (null: stale)
     bool cls_valid = false;
     bool bricks = false;
-    bool classified = false;
+    bool classified = false;      // sactive is current
+    bool listed = false;          // active, skippable, list and n_active are current
     bool fresh = false;           // cells and pairs written by the last ingest of the finer level,
                                   // brick min/max not yet (raypc_build_bricks computes them)
     size_t nbricks() const { return (size_t)nb * nb * nb; }
@@ -112,6 +111,9 @@ raypc_status get_level(Volume* V, int lod, Level** out);
 raypc_status make_render_args(Volume* V, Level* L, const raypc_camera* cam, int w, int h,
                               const raypc_render_opts* opts, float* out_rgba_dev,
                               unsigned long long* stats_dev, RenderArgs* a);
+
+// The classification of level L of volume V under a brush, without outputs.
+BrushItem brush_item(const Volume* V, const Level& L, const BrushArgs& brush);
 
 // Resolve RAYPC_AUTO launch choices from the tuning table (tune.cu).
 void resolve_launch(int device, int dtype, int n, int* variant, int* skip);

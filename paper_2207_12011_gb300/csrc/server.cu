@@ -240,20 +240,12 @@ raypc_status launch_hist(raypc_server* S, Req* q, int si) {
     }
     char* scratch = static_cast<char*>(S->hscratch[si]);
     if (activity && e == cudaSuccess) {
-        ClassifyArgs c{};
-        c.nvars = V->nvars;
-        c.rin2 = V->r_in * V->r_in;
-        c.rout2 = V->r_out * V->r_out;
-        c.brush = b;
-        c.nlev = 1;
-        c.nbrick = 0;
-        c.lv[0].bmin = L->sbmin;
-        c.lv[0].bmax = L->sbmax;
-        c.lv[0].n = L->n;
-        c.lv[0].bs = kSub;
-        c.lv[0].active = reinterpret_cast<uint32_t*>(scratch + copy_bytes);
-        e = launch_classify(c, s);
-        h.sactive = c.lv[0].active;
+        BrushLaunch P{};
+        P.nitems = 1;
+        P.items[0] = brush_item(V, *L, b);
+        P.items[0].active = reinterpret_cast<uint32_t*>(scratch + copy_bytes);
+        e = launch_brush(P, V->dtype, s);
+        h.sactive = P.items[0].active;
         h.nsb = L->nsb;
     }
     if (ncopies > 1) {

@@ -142,66 +142,26 @@ raypc_status raypc_autotune(raypc_ctx* ctx, const raypc_view* views, int nviews,
         if ((st = brush_from_host(V, q.lo, q.hi, q.active_mask, &args[i].brush))) break;
         if ((st = pos_from_host(q.pos_lo, q.pos_hi, q.pos_mask, &args[i].brush))) break;
         finish_position_brush(args[i]);
-        const size_t words = L->nwords();
         void* bits = nullptr;
-        void* list = nullptr;
-        void* misc = nullptr;
-        void* cls = nullptr;
-        cudaError_t e = cudaMalloc(&bits, (2 * words + L->nswords()) * sizeof(uint32_t));
+        cudaError_t e = cudaMalloc(&bits, L->nswords() * sizeof(uint32_t));
         if (e == cudaSuccess) temps.push_back(bits);
-        if (e == cudaSuccess) e = cudaMalloc(&list, L->nbricks() * sizeof(uint32_t) + 16);
-        if (e == cudaSuccess) temps.push_back(list);
-        if (e == cudaSuccess) e = cudaMalloc(&misc, sizeof(unsigned) * (kMaxVars + 4));
-        if (e == cudaSuccess) temps.push_back(misc);
         // cell classes under the view's brush, as a single-view render uses them
+        void* cls = nullptr;
         if (e == cudaSuccess) e = cudaMalloc(&cls, (size_t)L->n * L->n * L->n * sizeof(uint16_t));
         if (e == cudaSuccess) temps.push_back(cls);
-        void* slist = nullptr;
-        if (e == cudaSuccess) e = cudaMalloc(&slist, L->nsbricks() * sizeof(uint32_t) + 16);
-        if (e == cudaSuccess) temps.push_back(slist);
         void* dist = nullptr;                 // padded empty-space distance
         if (e == cudaSuccess) e = cudaMalloc(&dist, padded_bytes(L->n));
         if (e == cudaSuccess) temps.push_back(dist);
         if (e != cudaSuccess) { st = cuda_fail(e, "tuning buffers"); break; }
-        ClassifyArgs c{};
-        c.nlev = 2;
-        c.nbrick = 1;
-        c.nvars = V->nvars;
-        c.rin2 = V->r_in * V->r_in;
-        c.rout2 = V->r_out * V->r_out;
-        c.brush = args[i].brush;
-        c.lv[0].bmin = L->bmin;
-        c.lv[0].bmax = L->bmax;
-        c.lv[0].n = L->n;
-        c.lv[0].bs = kBrick;
-        c.lv[0].active = (uint32_t*)bits;
-        c.lv[0].skippable = (uint32_t*)bits + words;
-        c.lv[0].list = (uint32_t*)list;
-        c.lv[0].pass_count = (unsigned*)misc;
-        c.lv[0].n_active = (uint32_t*)misc + kMaxVars;
-        c.lv[1].bmin = L->sbmin;
-        c.lv[1].bmax = L->sbmax;
-        c.lv[1].n = L->n;
-        c.lv[1].bs = kSub;
-        c.lv[1].active = (uint32_t*)bits + 2 * words;
-        c.lv[1].alist = (uint32_t*)slist;
-        c.lv[1].acount = (uint32_t*)misc + kMaxVars + 1;
-        cudaError_t ce = launch_classify(c, s);
+        BrushLaunch P{};
+        P.nitems = 1;
+        P.items[0] = brush_item(V, *L, args[i].brush);
+        P.items[0].active = (uint32_t*)bits;
+        P.items[0].cls = (uint16_t*)cls;
+        cudaError_t ce = launch_brush(P, V->dtype, s);
         if (ce != cudaSuccess) { st = cuda_fail(ce, "tuning classification"); break; }
-        args[i].lv.active = c.lv[0].active;
-        args[i].lv.sactive = c.lv[1].active;
-        CellClassArgs cc{};
-        cc.pairs = L->pairs;
-        cc.n = L->n;
-        cc.nvars = V->nvars;
-        cc.brush = args[i].brush;
-        cc.slist = c.lv[1].alist;
-        cc.scount = c.lv[1].acount;
-        cc.out = (uint16_t*)cls;
-        ce = launch_cell_classes(cc, V->dtype, s);
-        if (ce != cudaSuccess) { st = cuda_fail(ce, "tuning cell classes"); break; }
-        args[i].cls = cc.out;
-        args[i].pass_count = c.lv[0].pass_count;
+        args[i].lv.sactive = P.items[0].active;
+        args[i].cls = P.items[0].cls;
         ce = launch_subbrick_distance(args[i].lv.sactive, L->n, (uint8_t*)dist, false, s);
         if (ce != cudaSuccess) { st = cuda_fail(ce, "tuning empty-space distance"); break; }
         args[i].lv.sdist = (const uint8_t*)dist;

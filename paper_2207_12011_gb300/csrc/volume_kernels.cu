@@ -1,5 +1,5 @@
 // Volume preparation kernels: ingest/relayout and level-of-detail mean fused
-// with brick min/max, and brush classification of bricks.
+// with brick min/max; the empty-space distance of classified sub-bricks.
 //
 // Section 2.1 of the paper prepares the data once (levels of detail, derived
 // variables); Section 2.2 relies on that preparation not depending on the
@@ -32,6 +32,7 @@ struct RowsArgs {
     float* sbmax;
     void* ccells;         // ingest with the next level: its planar cells (edge n / 2) ...
     void* cpairs;         // ... and x-pairs
+    LevelStats stats;     // magnitudes of this level
 };
 
 __device__ __forceinline__ void fold(float& mn, float& mx, float a_mn, float a_mx) {
@@ -267,6 +268,7 @@ __global__ void __launch_bounds__(kRowCols * kRowSlices, 2) k_rows(RowsArgs A) {
         const bool valid = t < ncol && z < n;
         const int X = t * VEC;
         float ymn[2] = {qnan, qnan}, ymx[2] = {qnan, qnan};
+        float odd = 0.0f;                                // NaN once a value is NaN or infinite
         float even0 = 0.0f, even1 = 0.0f;                // MODE 2: x-pair sums of the even row
 #pragma unroll
         for (int dy0 = 0; dy0 <= kBrick; dy0 += kBatch) {
@@ -284,6 +286,8 @@ __global__ void __launch_bounds__(kRowCols * kRowSlices, 2) k_rows(RowsArgs A) {
                 float rmn = val[j][0], rmx = val[j][0];
 #pragma unroll
                 for (int q = 1; q <= VEC; ++q) fold(rmn, rmx, val[j][q], val[j][q]);
+#pragma unroll
+                for (int q = 0; q < VEC; ++q) odd = fmaf(val[j][q], 0.0f, odd);
                 if (dy <= kSub) fold(ymn[0], ymx[0], rmn, rmx);
                 if (dy >= kSub) fold(ymn[1], ymx[1], rmn, rmx);
                 if (MODE != 3 && dy < kBrick && dz < kBrick)
@@ -346,7 +350,12 @@ __global__ void __launch_bounds__(kRowCols * kRowSlices, 2) k_rows(RowsArgs A) {
                 A.bmin[b * A.nvars + v] = bmn;
                 A.bmax[b * A.nvars + v] = bmx;
             }
+            // the level's largest magnitude: one atomic per warp that may raise it
+            const unsigned mag = __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(fmaxf(fabsf(bmn), fabsf(bmx)), 0.0f)));
+            const unsigned long long key = ((unsigned long long)A.stats.gen << 32) | mag;
+            if ((tx & 31) == 0 && *(volatile unsigned long long*)(A.stats.key + v) < key) atomicMax(A.stats.key + v, key);
         }
+        if (odd != odd) atomicMax(A.stats.key + kMaxVars, ((unsigned long long)A.stats.gen << 32) | 1ull);
         if (MODE == 2 && dz < kHalf && t < ncol) {
             // the next level's cells 2t, 2t+1 of its rows 4 by .. 4 by + 3 in slice 4 bz + dz:
             // ((fine slice 2 dz) + (fine slice 2 dz + 1)) / 8
@@ -368,116 +377,6 @@ __global__ void __launch_bounds__(kRowCols * kRowSlices, 2) k_rows(RowsArgs A) {
         __syncthreads();                                 // s_half is rewritten by the next column chunk
     }
 }
-
-// Locate the level of a flat brick index over all levels (<= 3 levels).
-__device__ __forceinline__ int level_of(const ClassifyArgs& C, size_t g, size_t& b) {
-    int l = 0;
-    while (l + 1 < C.nlev && g >= C.lv[l + 1].first) ++l;
-    b = g - C.lv[l].first;
-    return l;
-}
-
-// One thread per brick of every entry (8^3 bricks and 4^3 sub-bricks of every
-// level): shell test of the widened box and brush test with the rounding
-// margin d = max(|min|, |max|) * 2^-20 + 2^-120. Writes the active bitmask
-// (one ballot word per warp; entry ranges start on multiples of 32) and, for
-// the 8^3 bricks, counts per restricted variable the in-shell bricks that pass
-// that variable alone (a selectivity hint for the render).
-__global__ void k_classify(ClassifyArgs C) {
-    const size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int lane = threadIdx.x & 31;
-    size_t b = 0;
-    const int l = level_of(C, g, b);
-    const ClassifyLevel& L = C.lv[l];
-    const int nb = (L.n + L.bs - 1) / L.bs;
-    const size_t nbricks = (size_t)nb * nb * nb;
-    const bool in_range = g < C.total;
-    const bool valid = in_range && b < nbricks;
-    bool act = false;
-    unsigned pass_bits = 0;
-    if (valid)
-        act = classify_brick(b, nb, L.bs, L.sc, C.rin2, C.rout2, C.brush, C.nvars, L.bmin, L.bmax, pass_bits);
-    const unsigned word = __ballot_sync(0xffffffffu, act);
-    if (lane == 0 && in_range && b < ((nbricks + 31) & ~(size_t)31)) L.active[b >> 5] = word;
-    if (L.alist && word) {                      // uniform per warp: entry ranges are warp-aligned
-        unsigned base = 0;
-        if (lane == 0) base = atomicAdd(L.acount, (unsigned)__popc(word));
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if (act) L.alist[base + __popc(word & ((1u << lane) - 1u))] = (uint32_t)b;
-    }
-    if (L.pass_count == nullptr) return;
-    for (int v = 0; v < C.nvars; ++v) {
-        const unsigned cnt = __popc(__ballot_sync(0xffffffffu, (pass_bits >> v) & 1u));
-        if (lane == 0 && cnt) atomicAdd(&L.pass_count[v], cnt);
-    }
-}
-
-// Skippable = this 8^3 brick and its existing 26 neighbours are inactive.
-__global__ void k_skippable(ClassifyArgs C) {
-    const size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int lane = threadIdx.x & 31;
-    size_t b = 0;
-    const int l = level_of(C, g, b);
-    const ClassifyLevel& L = C.lv[l];
-    const int nb = (L.n + kBrick - 1) / kBrick;
-    const size_t nbricks = (size_t)nb * nb * nb;
-    const bool in_range = g < C.total_brick;
-    const bool valid = in_range && b < nbricks;
-    const bool s = valid && skippable_brick(b, nb, L.active);
-    const unsigned word = __ballot_sync(0xffffffffu, s);
-    if (lane == 0 && in_range && b < ((nbricks + 31) & ~(size_t)31)) L.skippable[b >> 5] = word;
-}
-
-// Ordered compaction of the active 8^3 brick ids, one block of 1024 threads per
-// level: each thread owns a contiguous run of bitmask words; a block-wide
-// exclusive scan of the per-thread popcounts gives every thread its offset.
-__global__ void __launch_bounds__(1024) k_compact(ClassifyArgs C) {
-    __shared__ unsigned s_sum[1024];
-    const ClassifyLevel& L = C.lv[blockIdx.x];
-    const int nb = (L.n + kBrick - 1) / kBrick;
-    const size_t nbricks = (size_t)nb * nb * nb;
-    const size_t nwords = (nbricks + 31) / 32;
-    const size_t per = (nwords + blockDim.x - 1) / blockDim.x;
-    const size_t w0 = min(nwords, threadIdx.x * per), w1 = min(nwords, w0 + per);
-    unsigned cnt = 0;
-    for (size_t w = w0; w < w1; ++w) cnt += __popc(L.active[w]);
-    s_sum[threadIdx.x] = cnt;
-    __syncthreads();
-    for (int off = 1; off < (int)blockDim.x; off <<= 1) {
-        const unsigned add = threadIdx.x >= (unsigned)off ? s_sum[threadIdx.x - off] : 0u;
-        __syncthreads();
-        s_sum[threadIdx.x] += add;
-        __syncthreads();
-    }
-    unsigned pos = s_sum[threadIdx.x] - cnt;
-    for (size_t w = w0; w < w1; ++w) {
-        uint32_t bits = L.active[w];
-        while (bits) {
-            const int j = __ffs(bits) - 1;
-            bits &= bits - 1;
-            const size_t id = w * 32 + j;
-            if (id < nbricks) L.list[pos++] = (uint32_t)id;
-        }
-    }
-    if (threadIdx.x == blockDim.x - 1) *L.n_active = s_sum[threadIdx.x];
-}
-
-// Cell classes (see CellClassArgs) of the cells of the active sub-bricks only
-// (the render consults a cell's class only for samples in an active
-// sub-brick): one warp per listed sub-brick (see cell_classes_of_subbrick).
-template <int DT>
-__global__ void __launch_bounds__(32 * kCellWarps) k_cell_classes(const void* __restrict__ pairs, int n,
-                                                                 const uint32_t* __restrict__ slist,
-                                                                 const uint32_t* __restrict__ scount,
-                                                                 uint16_t* __restrict__ out, CellVars R) {
-    const int lane = threadIdx.x & 31;
-    const int nsb = (n + kSub - 1) / kSub;
-    const unsigned count = *scount;
-    for (unsigned i = blockIdx.x * kCellWarps + (threadIdx.x >> 5); i < count; i += gridDim.x * kCellWarps)
-        cell_classes_of_subbrick<DT>(pairs, n, nsb, __ldg(slist + i), lane, R, out);
-}
-
-inline unsigned blocks_for(size_t n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 
 template <int DT, int MODE, int SRC, int VEC>
 void launch_rows_t(const RowsArgs& a, dim3 grid, cudaStream_t stream) {
@@ -528,7 +427,7 @@ cudaError_t launch_rows(const RowsArgs& a, int dtype, cudaStream_t stream) {
 
 cudaError_t launch_ingest(const void* src, int src_dtype, void* cells, void* pairs, int dtype, int n,
                           int nvars, float* bmin, float* bmax, float* sbmin, float* sbmax,
-                          cudaStream_t stream) {
+                          LevelStats stats, cudaStream_t stream) {
     RowsArgs a{};
     a.src = src;
     a.src_dtype = src_dtype;
@@ -540,6 +439,7 @@ cudaError_t launch_ingest(const void* src, int src_dtype, void* cells, void* pai
     a.bmax = bmax;
     a.sbmin = sbmin;
     a.sbmax = sbmax;
+    a.stats = stats;
     return launch_rows<0>(a, dtype, stream);
 }
 
@@ -549,7 +449,7 @@ bool ingest_next_level_fits(const void* src, int n) {
 
 cudaError_t launch_ingest_next_level(const void* src, int src_dtype, void* cells, void* pairs, int dtype, int n,
                                      int nvars, float* bmin, float* bmax, float* sbmin, float* sbmax,
-                                     void* next_cells, void* next_pairs, cudaStream_t stream) {
+                                     void* next_cells, void* next_pairs, LevelStats stats, cudaStream_t stream) {
     RowsArgs a{};
     a.src = src;
     a.src_dtype = src_dtype;
@@ -561,13 +461,14 @@ cudaError_t launch_ingest_next_level(const void* src, int src_dtype, void* cells
     a.bmax = bmax;
     a.sbmin = sbmin;
     a.sbmax = sbmax;
+    a.stats = stats;
     a.ccells = next_cells;
     a.cpairs = next_pairs;
     return launch_rows<2>(a, dtype, stream);
 }
 
 cudaError_t launch_level_bricks(const void* cells, int dtype, int n, int nvars, float* bmin, float* bmax,
-                                float* sbmin, float* sbmax, cudaStream_t stream) {
+                                float* sbmin, float* sbmax, LevelStats stats, cudaStream_t stream) {
     RowsArgs a{};
     a.src = cells;
     a.src_dtype = dtype;
@@ -577,11 +478,12 @@ cudaError_t launch_level_bricks(const void* cells, int dtype, int n, int nvars, 
     a.bmax = bmax;
     a.sbmin = sbmin;
     a.sbmax = sbmax;
+    a.stats = stats;
     return launch_rows<3>(a, dtype, stream);
 }
 
 cudaError_t launch_lod(const void* fine, int n_fine, void* cells, void* pairs, int dtype, int nvars,
-                       float* bmin, float* bmax, float* sbmin, float* sbmax, cudaStream_t stream) {
+                       float* bmin, float* bmax, float* sbmin, float* sbmax, LevelStats stats, cudaStream_t stream) {
     RowsArgs a{};
     a.src = fine;
     a.n_src = n_fine;
@@ -593,98 +495,23 @@ cudaError_t launch_lod(const void* fine, int n_fine, void* cells, void* pairs, i
     a.bmax = bmax;
     a.sbmin = sbmin;
     a.sbmax = sbmax;
+    a.stats = stats;
     return launch_rows<1>(a, dtype, stream);
-}
-
-cudaError_t launch_cell_classes(const CellClassArgs& a, int dtype, cudaStream_t stream) {
-    if (a.n < 2 || !a.slist || !a.scount) return cudaErrorInvalidValue;
-    CellVars R;
-    cell_vars_of(a.brush, a.nvars, R);
-    // grid fixed on the host (the list length is on the device): enough warps
-    // for every listed sub-brick of a small level, a few waves for a large one
-    const size_t nsb = (size_t)((a.n + kSub - 1) / kSub);
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const unsigned blocks = (unsigned)std::min<size_t>(blocks_for(nsb * nsb * nsb, kCellWarps), (size_t)sms * 16);
-    if (dtype == kF16) k_cell_classes<kF16><<<blocks, 32 * kCellWarps, 0, stream>>>(a.pairs, a.n, a.slist, a.scount, a.out, R);
-    else k_cell_classes<kF32><<<blocks, 32 * kCellWarps, 0, stream>>>(a.pairs, a.n, a.slist, a.scount, a.out, R);
-    count_launches(1);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_classify(ClassifyArgs& c, cudaStream_t stream) {
-    size_t total = 0;
-    for (int l = 0; l < c.nlev; ++l) {
-        ClassifyLevel& L = c.lv[l];
-        if (L.bs != (l < c.nbrick ? kBrick : kSub)) return cudaErrorInvalidValue;
-        const int nb = (L.n + L.bs - 1) / L.bs;
-        L.first = total;
-        L.sc = 2.0f / (float)L.n;
-        total += ((size_t)nb * nb * nb + 31) / 32 * 32;      // entry ranges start on warp boundaries
-        if (l + 1 == c.nbrick) c.total_brick = total;
-        if (L.pass_count) {
-            cudaError_t e = cudaMemsetAsync(L.pass_count, 0, sizeof(unsigned) * kMaxVars, stream);
-            if (e != cudaSuccess) return e;
-        }
-        if (L.alist) {
-            cudaError_t e = cudaMemsetAsync(L.acount, 0, sizeof(uint32_t), stream);
-            if (e != cudaSuccess) return e;
-        }
-    }
-    c.total = total;
-    k_classify<<<blocks_for(total, 256), 256, 0, stream>>>(c);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (c.nbrick == 0) {             // sub-bricks only: no skippable bits, no brick list
-        count_launches(1);
-        return cudaSuccess;
-    }
-    k_skippable<<<blocks_for(c.total_brick, 256), 256, 0, stream>>>(c);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_compact<<<c.nbrick, 1024, 0, stream>>>(c);
-    count_launches(3);
-    return cudaGetLastError();
 }
 
 namespace {
 
-// One thread per brick (entries 0..nbricks-1, padded to whole words) and per
-// sub-brick (the entries after them): activity AND TF visibility
-// (tf_range_visible). A brick's range holds its sub-bricks' ranges, so an
-// invisible brick has only invisible sub-bricks.
+// One thread per sub-brick: activity AND TF visibility (tf_range_visible).
 __global__ void __launch_bounds__(256) k_tf_visibility(TfVisArgs A) {
-    __shared__ int s_pre[kTF + 1];             // s_pre[j] = entries < j with sigma > 0
-    if (threadIdx.x < 32) {
-        int run = 0;
-        for (int base = 0; base < kTF; base += 32) {
-            const bool nz = A.tf[base + threadIdx.x].w > 0.0f;
-            const unsigned b = __ballot_sync(0xffffffffu, nz);
-            s_pre[base + threadIdx.x] = run + __popc(b & ((1u << threadIdx.x) - 1u));
-            run += __popc(b);
-        }
-        if (threadIdx.x == 0) s_pre[kTF] = run;
-    }
-    __syncthreads();
-    const size_t nbr = (size_t)A.nb * A.nb * A.nb, nsub = (size_t)A.nsb * A.nsb * A.nsb;
-    const size_t nbr_pad = (nbr + 31) & ~(size_t)31;
-    const size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool is_sub = g >= nbr_pad;
-    const size_t b = is_sub ? g - nbr_pad : g;
-    const size_t cnt = is_sub ? nsub : nbr;
-    bool bit = false;
-    if (b < cnt) {
-        const uint32_t* act = is_sub ? A.sactive : A.active;
-        bit = (act[b >> 5] >> (b & 31)) & 1u;
-        if (bit) {
-            const float mn = (is_sub ? A.sbmin : A.bmin)[b * A.nvars + A.color_var];
-            const float mx = (is_sub ? A.sbmax : A.bmax)[b * A.nvars + A.color_var];
-            bit = tf_range_visible(mn, mx, s_pre, A.tf_lo, A.tf_scale);
-        }
+    const size_t b = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const size_t nsub = (size_t)A.nsb * A.nsb * A.nsb;
+    bool bit = b < nsub && ((A.sactive[b >> 5] >> (b & 31)) & 1u);
+    if (bit) {
+        const size_t o = b * A.nvars + A.color_var;
+        bit = tf_range_visible(A.sbmin[o], A.sbmax[o], A.tf_prefix, A.tf_lo, A.tf_scale);
     }
     const unsigned word = __ballot_sync(0xffffffffu, bit);
-    if ((threadIdx.x & 31) == 0 && b < ((cnt + 31) & ~(size_t)31)) (is_sub ? A.out_sactive : A.out_active)[b >> 5] = word;
+    if ((threadIdx.x & 31) == 0 && b < nsub) A.out_sactive[b >> 5] = word;
 }
 
 }  // namespace
@@ -827,7 +654,7 @@ __global__ void __launch_bounds__(kDistThreads) k_subbrick_distance(const uint32
 
 // Every view of a batch: the blocks walk the views' concatenated tiles.
 __global__ void __launch_bounds__(kDistThreads) k_subbrick_distance_views(const BatchHeader* __restrict__ hdr,
-                                                                          const BatchView* __restrict__ views) {
+                                                                          const BrushItem* __restrict__ views) {
     const int total = hdr->dist_total, nviews = hdr->nviews;
     for (int g = blockIdx.x; g < total; g += gridDim.x) {
         int lo = 0, hi = nviews - 1;                 // the last view whose tiles start at or before g
@@ -835,8 +662,8 @@ __global__ void __launch_bounds__(kDistThreads) k_subbrick_distance_views(const 
             const int mid = (lo + hi + 1) >> 1;
             if (views[mid].dist_begin <= g) lo = mid; else hi = mid - 1;
         }
-        const BatchView& V = views[lo];
-        subbrick_distance_tile(V.a.lv.sactive, V.a.lv.n, g - V.dist_begin, const_cast<uint8_t*>(V.a.lv.sdist), false);
+        const BrushItem& V = views[lo];
+        subbrick_distance_tile(V.active, V.n, g - V.dist_begin, V.sdist, false);
     }
 }
 
@@ -853,16 +680,15 @@ cudaError_t launch_subbrick_distance(const uint32_t* sactive, int n, uint8_t* ou
     return cudaGetLastError();
 }
 
-cudaError_t launch_subbrick_distance_views(const BatchHeader* hdr, const BatchView* views, unsigned blocks,
+cudaError_t launch_subbrick_distance_views(const BatchHeader* hdr, const BrushItem* views, unsigned blocks,
                                            cudaStream_t stream) {
     k_subbrick_distance_views<<<blocks, kDistThreads, 0, stream>>>(hdr, views);
     return cudaGetLastError();
 }
 
 cudaError_t launch_tf_visibility(const TfVisArgs& a, cudaStream_t stream) {
-    const size_t nbr = (size_t)a.nb * a.nb * a.nb, nsub = (size_t)a.nsb * a.nsb * a.nsb;
-    const size_t total = ((nbr + 31) & ~(size_t)31) + nsub;
-    k_tf_visibility<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>(a);
+    const size_t nsub = (size_t)a.nsb * a.nsb * a.nsb;
+    k_tf_visibility<<<(unsigned)((nsub + 255) / 256), 256, 0, stream>>>(a);
     count_launches(1);
     return cudaGetLastError();
 }
