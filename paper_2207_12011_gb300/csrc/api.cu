@@ -257,6 +257,7 @@ raypc_status ingest(raypc_ctx* ctx, Volume* V, const void* src, int src_is_devic
     else
         e = launch_ingest(dsrc, src_dtype, L.cells, L.pairs, V->dtype, L.n, V->nvars, L.bmin, L.bmax, L.sbmin,
                           L.sbmax, stats, s);
+    for (auto& l : V->lv) l.fresh = false;
     C.fresh = next && e == cudaSuccess;
     if (staging) cudaFreeAsync(staging, s);
     if (staged && e == cudaSuccess) {
@@ -588,14 +589,20 @@ raypc_status raypc_build_bricks(raypc_ctx* ctx, int vol, int brick_dim, int n_lo
             if (st) return st;
         }
         if ((st = alloc_bricks(ctx, V, L))) return st;
-        if (L.fresh)             // the ingest already wrote this level's cells: its bricks only
+        if (L.fresh) {           // the ingest or the pass before already wrote this level's cells: its bricks,
+                                 // and the next level's cells in the same pass where that is allocated too
+            Level* C = l < n_lod && V->lv[l + 1].cells && V->lv[l + 1].n * 2 == L.n &&
+                       ingest_next_level_fits(L.cells, L.n) ? &V->lv[l + 1] : nullptr;
             CK(launch_level_bricks(L.cells, V->dtype, L.n, V->nvars, L.bmin, L.bmax, L.sbmin, L.sbmax,
-                                   LevelStats{L.stats, ++L.gen}, s),
+                                   C ? C->cells : nullptr, C ? C->pairs : nullptr, LevelStats{L.stats, ++L.gen}, s),
                "level bricks kernel");
-        else
+            if (C) C->fresh = true;
+        } else {
             CK(launch_lod(P.cells, P.n, L.cells, L.pairs, V->dtype, V->nvars, L.bmin, L.bmax, L.sbmin, L.sbmax,
                           LevelStats{L.stats, ++L.gen}, s),
                "LOD kernel");
+            if (l < RAYPC_MAX_LOD) V->lv[l + 1].fresh = false;
+        }
         L.fresh = false;
         L.bricks = true;
     }

@@ -531,9 +531,12 @@ bool ingest_next_level_fits(const void* src, int n);
 cudaError_t launch_ingest_next_level(const void* src, int src_dtype, void* cells, void* pairs, int dtype, int n,
                                      int nvars, float* bmin, float* bmax, float* sbmin, float* sbmax,
                                      void* next_cells, void* next_pairs, LevelStats stats, cudaStream_t stream);
-// Brick and sub-brick min/max of a level from its own stored cells.
+// Brick and sub-brick min/max of a level from its own stored cells; with next_cells
+// (and next_pairs; only when ingest_next_level_fits(cells, n)) also the next
+// level's cells and x-pairs.
 cudaError_t launch_level_bricks(const void* cells, int dtype, int n, int nvars, float* bmin, float* bmax,
-                                float* sbmin, float* sbmax, LevelStats stats, cudaStream_t stream);
+                                float* sbmin, float* sbmax, void* next_cells, void* next_pairs, LevelStats stats,
+                                cudaStream_t stream);
 // Sub-brick activity bits and cell classes of P.items[0 .. nitems-1] (brush_kernels.cu),
 // and of every view of a batch (brush_chunks(n) chunks per view).
 cudaError_t launch_brush(BrushLaunch& P, int dtype, cudaStream_t stream);

@@ -131,26 +131,15 @@ __device__ __forceinline__ void store_run(void* cells, void* pairs, size_t i, co
     }
 }
 
-// Values of columns X .. X+VEC of row (y, z) of variable v of the level being
-// produced, rounded to the storage dtype DT; column X+VEC is clamped to n-1.
-//   MODE 0 (ingest): the converted source value (source element type SRC).
-//   MODE 1 (LOD):    FP32 mean of the 2x2x2 fine cells, fine indices clamped,
-//                    ((c000 + c100) + (c010 + c110)) + ((c001 + c101) + (c011 + c111)), x 1/8.
-//   MODE 2 (ingest and the next level): as MODE 0; the kernel also forms the next
-//                    level's means from the values it produced (n a multiple of 16).
-//   MODE 3 (bricks only): the level's own stored cells, for its brick min/max.
-// With VEC > 1 the caller guarantees n % VEC == 0 and, for LOD, an even fine edge.
-template <int DT, int MODE, int SRC, int VEC>
+// Values of columns X .. X+VEC of row (y, z) of variable v of a coarser level, rounded to the
+// storage dtype; column X+VEC is clamped to n-1: the FP32 mean of the 2x2x2 fine cells, fine
+// indices clamped, ((c000 + c100) + (c010 + c110)) + ((c001 + c101) + (c011 + c111)), x 1/8.
+// With VEC > 1 the caller guarantees n % VEC == 0 and an even fine edge.
+template <int DT, int VEC>
 __device__ __forceinline__ void produce_run(const RowsArgs& A, int X, int y, int z, int v, float* val) {
     const int n = A.n;
     const bool right = X + VEC < n;
-    if (MODE != 1) {
-        const size_t row = (((size_t)v * n + z) * n + y) * n;
-        load_run<SRC, VEC>(A.src, row + X, val);
-        load_run<SRC, 1>(A.src, row + (right ? X + VEC : X + VEC - 1), val + VEC);
-#pragma unroll
-        for (int q = 0; q <= VEC; ++q) val[q] = to_stored<DT>(val[q]);
-    } else {
+    {
         const int nf = A.n_src;
         const int y0 = 2 * y, y1 = min(y0 + 1, nf - 1), z0 = 2 * z, z1 = min(z0 + 1, nf - 1);
         const size_t plane = (size_t)v * nf * nf * nf;
@@ -192,7 +181,7 @@ __device__ __forceinline__ void produce_run(const RowsArgs& A, int X, int y, int
     }
 }
 
-// One block per (brick row (by, bz), variable), threads (t, dz): thread t owns
+// Level-of-detail pass. One block per (brick row (by, bz), variable), threads (t, dz): thread t owns
 // the VEC columns X = VEC t .. VEC t + VEC-1 (striding over the level when it
 // is wider than the block) of z-slice z = 8bz + dz, dz in 0..8, and also reads
 // column X+VEC, the right element of its last pair. Each thread streams the
@@ -247,14 +236,21 @@ __device__ __forceinline__ void store_pair_second(void* pairs, size_t i, float v
     else reinterpret_cast<__half*>(pairs)[2 * i + 1] = __float2half_rn(v);
 }
 
-template <int DT, int MODE, int SRC, int VEC>
-__global__ void __launch_bounds__(kRowCols * kRowSlices, 2) k_rows(RowsArgs A) {
+// Record the magnitudes of variable v: odd is NaN in a thread that met a NaN or
+// infinite value, mag the largest |value| the thread knows of (NaN: none), in the
+// warps with `all` set (one atomic per warp that may raise the level's).
+__device__ __forceinline__ void level_stats(const LevelStats& L, int v, float odd, float mag, bool all) {
+    if (odd != odd) atomicMax(L.key + kMaxVars, ((unsigned long long)L.gen << 32) | 1ull);
+    if (!all) return;
+    const unsigned bits = __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(mag, 0.0f)));
+    const unsigned long long key = ((unsigned long long)L.gen << 32) | bits;
+    if ((threadIdx.x & 31) == 0 && *(volatile unsigned long long*)(L.key + v) < key) atomicMax(L.key + v, key);
+}
+
+template <int DT, int VEC>
+__global__ void __launch_bounds__(kRowCols * kRowSlices, 2) k_lod(RowsArgs A) {
     constexpr int G = kSub / VEC;                       // lanes per sub-brick column
-    constexpr int kBatch = MODE == 1 ? 1 : 3;          // rows whose loads are issued together
-    constexpr int kHalf = kBrick / 2;
     __shared__ float s_half[kRowSlices][4][kRowCols];  // per slice: min, max of y half 0, then of half 1
-    // MODE 2: per fine slice and coarse row, the sums over the row pair of the x-pair sums
-    __shared__ float s_next[MODE == 2 ? kBrick : 1][kHalf][2][kRowCols];
     const int n = A.n;
     const int nb = (n + kBrick - 1) / kBrick;
     const int nsb = (n + kSub - 1) / kSub;
@@ -263,47 +259,27 @@ __global__ void __launch_bounds__(kRowCols * kRowSlices, 2) k_rows(RowsArgs A) {
     const int dz = threadIdx.y, tx = threadIdx.x;
     const int z = bz * kBrick + dz;
     const float qnan = __int_as_float(0x7fffffff);
+    float odd = 0.0f, mag = 0.0f;                        // NaN once a value is NaN or infinite; largest |value|
     for (int c0 = 0; c0 < ncol; c0 += blockDim.x) {
         const int t = c0 + tx;
         const bool valid = t < ncol && z < n;
         const int X = t * VEC;
         float ymn[2] = {qnan, qnan}, ymx[2] = {qnan, qnan};
-        float odd = 0.0f;                                // NaN once a value is NaN or infinite
-        float even0 = 0.0f, even1 = 0.0f;                // MODE 2: x-pair sums of the even row
 #pragma unroll
-        for (int dy0 = 0; dy0 <= kBrick; dy0 += kBatch) {
-            float val[kBatch][VEC + 1];
+        for (int dy = 0; dy <= kBrick; ++dy) {
+            const int y = by * kBrick + dy;
+            if (!valid || y >= n) continue;
+            float val[VEC + 1];
+            produce_run<DT, VEC>(A, X, y, z, v, val);
+            float rmn = val[0], rmx = val[0];
 #pragma unroll
-            for (int j = 0; j < kBatch; ++j) {
-                const int y = by * kBrick + dy0 + j;
-                if (valid && dy0 + j <= kBrick && y < n) produce_run<DT, MODE, SRC, VEC>(A, X, y, z, v, val[j]);
-            }
+            for (int q = 1; q <= VEC; ++q) fold(rmn, rmx, val[q], val[q]);
 #pragma unroll
-            for (int j = 0; j < kBatch; ++j) {
-                const int dy = dy0 + j;
-                const int y = by * kBrick + dy;
-                if (!valid || dy > kBrick || y >= n) continue;
-                float rmn = val[j][0], rmx = val[j][0];
-#pragma unroll
-                for (int q = 1; q <= VEC; ++q) fold(rmn, rmx, val[j][q], val[j][q]);
-#pragma unroll
-                for (int q = 0; q < VEC; ++q) odd = fmaf(val[j][q], 0.0f, odd);
-                if (dy <= kSub) fold(ymn[0], ymx[0], rmn, rmx);
-                if (dy >= kSub) fold(ymn[1], ymx[1], rmn, rmx);
-                if (MODE != 3 && dy < kBrick && dz < kBrick)
-                    store_run<DT, VEC>(A.cells, A.pairs, (((size_t)v * n + z) * n + y) * n + X, val[j]);
-                if (MODE == 2 && dy < kBrick && dz < kBrick) {
-                    // the next level's mean, in its order: (c000 + c100) + (c010 + c110) per fine slice
-                    const float p0 = __fadd_rn(val[j][0], val[j][1]), p1 = __fadd_rn(val[j][2], val[j][3]);
-                    if ((dy & 1) == 0) {
-                        even0 = p0;
-                        even1 = p1;
-                    } else {
-                        s_next[MODE == 2 ? dz : 0][dy >> 1][0][tx] = __fadd_rn(even0, p0);
-                        s_next[MODE == 2 ? dz : 0][dy >> 1][1][tx] = __fadd_rn(even1, p1);
-                    }
-                }
-            }
+            for (int q = 0; q < VEC; ++q) odd = fmaf(val[q], 0.0f, odd);
+            if (dy <= kSub) fold(ymn[0], ymx[0], rmn, rmx);
+            if (dy >= kSub) fold(ymn[1], ymx[1], rmn, rmx);
+            if (dy < kBrick && dz < kBrick)
+                store_run<DT, VEC>(A.cells, A.pairs, (((size_t)v * n + z) * n + y) * n + X, val);
         }
         s_half[dz][0][tx] = ymn[0];
         s_half[dz][1][tx] = ymx[0];
@@ -350,74 +326,177 @@ __global__ void __launch_bounds__(kRowCols * kRowSlices, 2) k_rows(RowsArgs A) {
                 A.bmin[b * A.nvars + v] = bmn;
                 A.bmax[b * A.nvars + v] = bmx;
             }
-            // the level's largest magnitude: one atomic per warp that may raise it
-            const unsigned mag = __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(fmaxf(fabsf(bmn), fabsf(bmx)), 0.0f)));
-            const unsigned long long key = ((unsigned long long)A.stats.gen << 32) | mag;
-            if ((tx & 31) == 0 && *(volatile unsigned long long*)(A.stats.key + v) < key) atomicMax(A.stats.key + v, key);
-        }
-        if (odd != odd) atomicMax(A.stats.key + kMaxVars, ((unsigned long long)A.stats.gen << 32) | 1ull);
-        if (MODE == 2 && dz < kHalf && t < ncol) {
-            // the next level's cells 2t, 2t+1 of its rows 4 by .. 4 by + 3 in slice 4 bz + dz:
-            // ((fine slice 2 dz) + (fine slice 2 dz + 1)) / 8
-            const int m = n >> 1;
-            const bool row_end = t + 1 >= ncol, chunk_end = tx + 1 >= (int)blockDim.x;
-            const int s0 = MODE == 2 ? 2 * dz : 0, s1 = MODE == 2 ? 2 * dz + 1 : 0;
-#pragma unroll
-            for (int k = 0; k < kHalf; ++k) {
-                const float v0 = to_stored<DT>(__fmul_rn(__fadd_rn(s_next[s0][k][0][tx], s_next[s1][k][0][tx]), 0.125f));
-                const float v1 = to_stored<DT>(__fmul_rn(__fadd_rn(s_next[s0][k][1][tx], s_next[s1][k][1][tx]), 0.125f));
-                float r = v1;                            // the row's last cell pairs with itself
-                if (!row_end && !chunk_end)
-                    r = to_stored<DT>(__fmul_rn(__fadd_rn(s_next[s0][k][0][tx + 1], s_next[s1][k][0][tx + 1]), 0.125f));
-                const size_t i = (((size_t)v * m + (size_t)(bz * kHalf + dz)) * m + (size_t)(by * kHalf + k)) * m + 2 * t;
-                store_next_level<DT>(A.ccells, A.cpairs, i, v0, v1, r, row_end || !chunk_end);
-                if (tx == 0 && t > 0) store_pair_second<DT>(A.cpairs, i - 1, v0);   // the previous chunk's last pair
-            }
+            mag = fmaxf(mag, fmaxf(fabsf(bmn), fabsf(bmx)));
         }
         __syncthreads();                                 // s_half is rewritten by the next column chunk
     }
+    level_stats(A.stats, v, odd, mag, dz == 0);
+}
+
+// Ingest and brick passes, by MODE: 0 ingest (the converted source, element type SRC), 2 ingest
+// and the next level's cells (n a multiple of 16), 3 the min/max of the level's own
+// stored cells, 4 those and the next level's cells (1 is the level-of-detail pass).
+//
+// A block takes 32 VEC columns of one brick row of one
+// variable, a warp one of its four (y half, z half) quadrants, 5 x 5 rows with the
+// apron, a thread a run of VEC columns (4 where every run is aligned, else 1). The
+// five rows of a slice are loaded together; a run's right neighbour comes from the
+// next lane; a sub-brick in x is 4 / VEC neighbouring lanes; the next level's sums
+// stay in registers from the even to the odd fine slice, and the warps meet once, for
+// the brick.
+//
+// Bound by HBM: 5.7 TB/s of algorithmic bytes at 512^3, FP32 into FP16 with the next
+// level (1.51 ms against 1.79 for blocks of 9 slices with two barriers per 64
+// column runs, which left memory idle at the barriers; 2.32 against 2.40 ms for
+// FP32 storage; 250^3 FP32, one column per thread, 307 against 419 us). Fewer registers than
+// the five rows need spill (8 blocks per SM: 327 against 302 us at 256^3 FP32); the
+// half as wide FP16 sources want the warps instead.
+constexpr int kQuadThreads = 128;
+constexpr int quad_blocks(int mode, int src) { return mode >= 3 || src == kF16 ? 10 : 5; }
+
+template <int DT, int MODE, int SRC, int VEC>
+__global__ void __launch_bounds__(kQuadThreads, quad_blocks(MODE, SRC)) k_quads(RowsArgs A) {
+    constexpr int kRows = kSub + 1, G = kSub / VEC;          // rows of a quadrant; lanes of a sub-brick
+    constexpr bool kNext = (MODE == 2 || MODE == 4) && VEC == 4, kStore = MODE == 0 || MODE == 2;
+    __shared__ float s_mn[4][32], s_mx[4][32];
+    const int n = A.n, ncol = (n + VEC - 1) / VEC, nb = (n + kBrick - 1) / kBrick, nsb = (n + kSub - 1) / kSub;
+    const int nxc = (ncol + 31) / 32;
+    const int lane = threadIdx.x & 31, quad = threadIdx.x >> 5, yh = quad & 1, zh = quad >> 1;
+    const int xc = blockIdx.x % nxc, by = (blockIdx.x / nxc) % nb, bz = blockIdx.x / (nxc * nb), v = blockIdx.y;
+    const int t = xc * 32 + lane, X = t * VEC;
+    const int y0 = by * kBrick + yh * kSub, z0 = bz * kBrick + zh * kSub;
+    const bool valid = t < ncol, last = t == ncol - 1;
+    const float qnan = __int_as_float(0x7fffffff);
+    float mn = qnan, mx = qnan;
+    float odd = 0.0f;                                        // NaN once a value is NaN or infinite
+    float even[kNext ? 2 : 1][2];                            // sums of the even slice: [coarse row][cell]
+#pragma unroll
+    for (int dz = 0; dz < kRows; ++dz) {
+        const int z = z0 + dz;
+        float val[kRows][VEC + 1];
+        // the slice's rows (rows beyond the grid repeat the last one: no new value)
+#pragma unroll
+        for (int dy = 0; dy < kRows; ++dy) {
+            const int y = min(y0 + dy, n - 1);
+#pragma unroll
+            for (int q = 0; q <= VEC; ++q) val[dy][q] = 0.0f;
+            if (!valid || z >= n) continue;
+            const size_t row = (((size_t)v * n + z) * n + y) * n;
+            load_run<SRC, VEC>(A.src, row + X, val[dy]);
+            if (lane == 31 && !last) load_run<SRC, 1>(A.src, row + X + VEC, val[dy] + VEC);
+        }
+#pragma unroll
+        for (int dy = 0; dy < kRows; ++dy) {
+#pragma unroll
+            for (int q = 0; q <= VEC; ++q) val[dy][q] = to_stored<DT>(val[dy][q]);
+            const float right = __shfl_down_sync(0xffffffffu, val[dy][0], 1);
+            if (last) val[dy][VEC] = val[dy][VEC - 1];
+            else if (lane < 31) val[dy][VEC] = right;
+            if (!valid || z >= n) continue;
+#pragma unroll
+            for (int q = 0; q <= VEC; ++q) fold(mn, mx, val[dy][q], val[dy][q]);
+#pragma unroll
+            for (int q = 0; q < VEC; ++q) odd = fmaf(val[dy][q], 0.0f, odd);
+            if (kStore && dy < kSub && dz < kSub && y0 + dy < n)
+                store_run<DT, VEC>(A.cells, A.pairs, (((size_t)v * n + z) * n + y0 + dy) * n + X, val[dy]);
+        }
+        if constexpr (kNext) {
+            if (dz == kSub) continue;
+            // the next level's cells 2t, 2t+1 of its rows (y0 + {0, 2}) / 2, in its order:
+            // (c000 + c100) + (c010 + c110) per fine slice, then the two slices, / 8
+            const int m = n >> 1;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                float sum[2];
+#pragma unroll
+                for (int c = 0; c < 2; ++c)
+                    sum[c] = __fadd_rn(__fadd_rn(val[2 * k][2 * c], val[2 * k][2 * c + 1]),
+                                       __fadd_rn(val[2 * k + 1][2 * c], val[2 * k + 1][2 * c + 1]));
+                if ((dz & 1) == 0) {
+                    even[k][0] = sum[0];
+                    even[k][1] = sum[1];
+                    continue;
+                }
+                const float v0 = to_stored<DT>(__fmul_rn(__fadd_rn(even[k][0], sum[0]), 0.125f));
+                const float v1 = to_stored<DT>(__fmul_rn(__fadd_rn(even[k][1], sum[1]), 0.125f));
+                const float r = __shfl_down_sync(0xffffffffu, v0, 1);
+                if (!valid) continue;
+                const size_t i = (((size_t)v * m + (z >> 1)) * m + ((y0 >> 1) + k)) * m + 2 * t;
+                // the pair of cell 2t+1 needs cell 2t+2: the next lane's, the cell itself at the row's
+                // end, or from the next column chunk's first lane, which writes that half
+                store_next_level<DT>(A.ccells, A.cpairs, i, v0, v1, last ? v1 : r, last || lane < 31);
+                if (lane == 0 && t > 0) store_pair_second<DT>(A.cpairs, i - 1, v0);
+            }
+        }
+    }
+    // sub-bricks, then bricks
+#pragma unroll
+    for (int m = 1; m < G; m <<= 1) fold(mn, mx, __shfl_xor_sync(0xffffffffu, mn, m), __shfl_xor_sync(0xffffffffu, mx, m));
+    if (valid && t % G == 0 && y0 < n && z0 < n) {
+        const size_t sb = ((size_t)(z0 >> 2) * nsb + (y0 >> 2)) * nsb + t / G;
+        A.sbmin[sb * A.nvars + v] = mn;
+        A.sbmax[sb * A.nvars + v] = mx;
+    }
+    s_mn[quad][lane] = y0 < n ? mn : qnan;                   // an absent quadrant adds nothing
+    s_mx[quad][lane] = y0 < n ? mx : qnan;
+    __syncthreads();
+    level_stats(A.stats, v, odd, 0.0f, false);
+    if (quad != 0) return;
+#pragma unroll
+    for (int q = 1; q < 4; ++q) fold(mn, mx, s_mn[q][lane], s_mx[q][lane]);
+    fold(mn, mx, __shfl_xor_sync(0xffffffffu, mn, G), __shfl_xor_sync(0xffffffffu, mx, G));
+    if (valid && t % (2 * G) == 0) {
+        const size_t b = ((size_t)bz * nb + by) * nb + t / (2 * G);
+        A.bmin[b * A.nvars + v] = mn;
+        A.bmax[b * A.nvars + v] = mx;
+    }
+    level_stats(A.stats, v, 0.0f, fmaxf(fabsf(mn), fabsf(mx)), true);
 }
 
 template <int DT, int MODE, int SRC, int VEC>
-void launch_rows_t(const RowsArgs& a, dim3 grid, cudaStream_t stream) {
-    const int ncol = (a.n + VEC - 1) / VEC;
+void launch_quads_t(const RowsArgs& a, cudaStream_t stream) {
+    const int nb = (a.n + kBrick - 1) / kBrick, nxc = ((a.n + VEC - 1) / VEC + 31) / 32;
+    k_quads<DT, MODE, SRC, VEC><<<dim3((unsigned)(nb * nb * nxc), (unsigned)a.nvars), kQuadThreads, 0, stream>>>(a);
+}
+
+template <int DT, int MODE, int SRC>
+void launch_quads_t(const RowsArgs& a, bool vec, cudaStream_t stream) {
+    if (vec || MODE == 2 || MODE == 4) launch_quads_t<DT, MODE, SRC, 4>(a, stream);
+    else launch_quads_t<DT, MODE == 2 ? 0 : MODE == 4 ? 3 : MODE, SRC, 1>(a, stream);
+}
+
+template <int DT, int VEC>
+void launch_lod_t(const RowsArgs& a, cudaStream_t stream) {
+    const int nb = (a.n + kBrick - 1) / kBrick, ncol = (a.n + VEC - 1) / VEC;
     // one thread per column run up to kRowCols (narrow levels use narrow blocks), per z-slice
     const dim3 block(min(kRowCols, max(32, (ncol + 31) / 32 * 32)), kRowSlices);
-    k_rows<DT, MODE, SRC, VEC><<<grid, block, 0, stream>>>(a);
+    k_lod<DT, VEC><<<dim3((unsigned)(nb * nb), (unsigned)a.nvars), block, 0, stream>>>(a);
 }
 
 template <int MODE>
 cudaError_t launch_rows(const RowsArgs& a, int dtype, cudaStream_t stream) {
     if (a.n < 2 || a.n > kMaxRowsEdge) return cudaErrorInvalidValue;
-    const int nb = (a.n + kBrick - 1) / kBrick;
-    dim3 grid((unsigned)(nb * nb), (unsigned)a.nvars);
-    // 4-column runs when every run is aligned -- n % 4 == 0, a 16-byte aligned
-    // source (ingest) or an even fine edge (LOD; n % 4 == 0 makes it 8k) -- and
-    // the level is wide enough to fill a warp with runs.
-    bool vec = a.n % 4 == 0 && a.n >= 128;
-    if (MODE == 1) vec = vec && a.n_src == 2 * a.n;
-    else vec = vec && ((uintptr_t)a.src % 16 == 0);
-    if (MODE == 2) {
-        // the fused next level needs 4-column runs and whole bricks of both levels
-        if (!vec || a.n % 16 != 0 || !a.ccells || !a.cpairs) return cudaErrorInvalidValue;
-        const bool s16 = a.src_dtype == kF16;
-        if (dtype == kF16) { if (s16) launch_rows_t<kF16, 2, kF16, 4>(a, grid, stream); else launch_rows_t<kF16, 2, kF32, 4>(a, grid, stream); }
-        else               { if (s16) launch_rows_t<kF32, 2, kF16, 4>(a, grid, stream); else launch_rows_t<kF32, 2, kF32, 4>(a, grid, stream); }
-    } else if (MODE == 3) {
-        if (dtype == kF16) { if (vec) launch_rows_t<kF16, 3, kF16, 4>(a, grid, stream); else launch_rows_t<kF16, 3, kF16, 1>(a, grid, stream); }
-        else               { if (vec) launch_rows_t<kF32, 3, kF32, 4>(a, grid, stream); else launch_rows_t<kF32, 3, kF32, 1>(a, grid, stream); }
-    } else if (MODE == 0) {
-        const bool s16 = a.src_dtype == kF16;
-        if (dtype == kF16) {
-            if (vec) { if (s16) launch_rows_t<kF16, 0, kF16, 4>(a, grid, stream); else launch_rows_t<kF16, 0, kF32, 4>(a, grid, stream); }
-            else     { if (s16) launch_rows_t<kF16, 0, kF16, 1>(a, grid, stream); else launch_rows_t<kF16, 0, kF32, 1>(a, grid, stream); }
-        } else {
-            if (vec) { if (s16) launch_rows_t<kF32, 0, kF16, 4>(a, grid, stream); else launch_rows_t<kF32, 0, kF32, 4>(a, grid, stream); }
-            else     { if (s16) launch_rows_t<kF32, 0, kF16, 1>(a, grid, stream); else launch_rows_t<kF32, 0, kF32, 1>(a, grid, stream); }
-        }
+    if constexpr (MODE == 1) {
+        // 4-column runs when every run is aligned (n % 4 == 0 and an even fine edge make it 8k)
+        // and the level is wide enough to fill a warp with runs
+        const bool vec = a.n % 4 == 0 && a.n_src == 2 * a.n && a.n >= 128;
+        if (dtype == kF16) { if (vec) launch_lod_t<kF16, 4>(a, stream); else launch_lod_t<kF16, 1>(a, stream); }
+        else               { if (vec) launch_lod_t<kF32, 4>(a, stream); else launch_lod_t<kF32, 1>(a, stream); }
     } else {
-        if (dtype == kF16) { if (vec) launch_rows_t<kF16, 1, kF16, 4>(a, grid, stream); else launch_rows_t<kF16, 1, kF16, 1>(a, grid, stream); }
-        else               { if (vec) launch_rows_t<kF32, 1, kF32, 4>(a, grid, stream); else launch_rows_t<kF32, 1, kF32, 1>(a, grid, stream); }
+        // 4-column runs when every run is aligned: n % 4 == 0 and a 16-byte aligned source
+        const bool vec = a.n % 4 == 0 && (uintptr_t)a.src % 16 == 0;
+        // the fused next level needs them and whole bricks of both levels
+        if ((MODE == 2 || MODE == 4) && (!vec || a.n % 16 != 0 || !a.ccells || !a.cpairs)) return cudaErrorInvalidValue;
+        if constexpr (MODE >= 3) {
+            if (dtype == kF16) launch_quads_t<kF16, MODE, kF16>(a, vec, stream);
+            else launch_quads_t<kF32, MODE, kF32>(a, vec, stream);
+        } else if (a.src_dtype == kF16) {
+            if (dtype == kF16) launch_quads_t<kF16, MODE, kF16>(a, vec, stream);
+            else launch_quads_t<kF32, MODE, kF16>(a, vec, stream);
+        } else {
+            if (dtype == kF16) launch_quads_t<kF16, MODE, kF32>(a, vec, stream);
+            else launch_quads_t<kF32, MODE, kF32>(a, vec, stream);
+        }
     }
     count_launches(1);
     return cudaGetLastError();
@@ -468,7 +547,8 @@ cudaError_t launch_ingest_next_level(const void* src, int src_dtype, void* cells
 }
 
 cudaError_t launch_level_bricks(const void* cells, int dtype, int n, int nvars, float* bmin, float* bmax,
-                                float* sbmin, float* sbmax, LevelStats stats, cudaStream_t stream) {
+                                float* sbmin, float* sbmax, void* next_cells, void* next_pairs, LevelStats stats,
+                                cudaStream_t stream) {
     RowsArgs a{};
     a.src = cells;
     a.src_dtype = dtype;
@@ -478,8 +558,10 @@ cudaError_t launch_level_bricks(const void* cells, int dtype, int n, int nvars, 
     a.bmax = bmax;
     a.sbmin = sbmin;
     a.sbmax = sbmax;
+    a.ccells = next_cells;
+    a.cpairs = next_pairs;
     a.stats = stats;
-    return launch_rows<3>(a, dtype, stream);
+    return next_cells ? launch_rows<4>(a, dtype, stream) : launch_rows<3>(a, dtype, stream);
 }
 
 cudaError_t launch_lod(const void* fine, int n_fine, void* cells, void* pairs, int dtype, int nvars,
