@@ -466,6 +466,10 @@ raypc_status raypc_create(raypc_ctx** out, int device, size_t hbm_budget_bytes) 
     raypc_ctx* c = new raypc_ctx();
     c->device = device;
     c->budget = hbm_budget_bytes;
+    {
+        DeviceGuard g(device);
+        if (g.ok) c->open_pool();
+    }
     *out = c;
     g_err.clear();
     return RAYPC_OK;
@@ -478,6 +482,7 @@ raypc_status raypc_destroy(raypc_ctx* ctx) {
         DeviceGuard g(ctx->device);
         for (auto& kv : ctx->vols) free_volume(ctx, kv.second);
         ctx->vols.clear();
+        if (ctx->pool) cudaMemPoolDestroy(ctx->pool);      // released once its last frees have run
     }
     delete ctx;
     return RAYPC_OK;
@@ -855,33 +860,40 @@ raypc_status raypc_pc_histogram(raypc_ctx* ctx, int vol, int lod, const int* axi
     cudaError_t e = cudaSuccess;
     h.edges_host = edges;
     if (ne > (size_t)kHistInlineEdges) {
-        CK(cudaMallocAsync((void**)&dedges, sizeof(float) * ne, s), "edge buffer");
+        CK(ctx->scratch((void**)&dedges, sizeof(float) * ne, s), "edge buffer");
         e = cudaMemcpyAsync(dedges, edges, sizeof(float) * ne, cudaMemcpyHostToDevice, s);
     }
-    // hot bins of large grids: the blocks spread their atomics over zeroed copies in stream-ordered
-    // scratch, summed into the output afterwards (which then needs no clearing); the same
-    // scratch holds the row counter that balances the warps
+    // large grids list the cells' bins in stream-ordered scratch and count them in shared memory;
+    // without room for that (or with more bins than fit there) the blocks spread their atomics over
+    // zeroed copies, summed into the output afterwards (which then needs no clearing), and the
+    // same scratch holds the row counter that balances the warps
     const size_t count = (size_t)(naxes - 1) * bins * bins;
-    const int ncopies = ((uintptr_t)out_counts_dev & 15u) ? 1 : hist_copies(L->n, naxes, bins);
+    h.edges = dedges;
+    h.out = out_counts_dev;
+    h.sactive = use_activity ? L->sactive : nullptr;
+    h.nsb = L->nsb;
+    if (e == cudaSuccess && hist_by_list(h, V->dtype) && ctx->room(hist_list(h).bytes) &&
+        ctx->scratch(&h.list, hist_list(h).bytes, s) != cudaSuccess) {
+        cudaGetLastError();
+        h.list = nullptr;
+    }
+    const int ncopies = h.list || ((uintptr_t)out_counts_dev & 15u) ? 1 : hist_copies(L->n, naxes, bins);
     const size_t copy_bytes = sizeof(uint32_t) * (count * ncopies + 4);
     uint32_t* copies = nullptr;
     if (e == cudaSuccess && ncopies > 1) {
-        e = cudaMallocAsync((void**)&copies, copy_bytes, s);
+        e = ctx->scratch((void**)&copies, copy_bytes, s);
         if (e == cudaSuccess) e = cudaMemsetAsync(copies, 0, copy_bytes, s);
     } else if (e == cudaSuccess) {
         e = cudaMemsetAsync(out_counts_dev, 0, sizeof(uint32_t) * count, s);
     }
     if (e == cudaSuccess) {
-        h.edges = dedges;
-        h.out = out_counts_dev;
         h.copies = copies;
         h.ncopies = copies ? ncopies : 1;
         h.rowctr = copies ? copies + count * ncopies : nullptr;
-        h.sactive = use_activity ? L->sactive : nullptr;
-        h.nsb = L->nsb;
         e = launch_histogram(h, V->dtype, s);
         if (e == cudaSuccess && copies) e = launch_histogram_reduce(copies, ncopies, count, out_counts_dev, s);
     }
+    if (h.list) cudaFreeAsync(h.list, s);
     if (copies) cudaFreeAsync(copies, s);
     if (dedges) cudaFreeAsync(dedges, s);
     if (e != cudaSuccess) return cuda_fail(e, "histogram");
@@ -942,7 +954,7 @@ raypc_status raypc_pc_subsample(raypc_ctx* ctx, int vol, int lod, uint32_t seed,
     cudaStream_t s = (cudaStream_t)stream;
     // select state and per-block counts: a small device buffer owned by this call (freed in stream order)
     void* scratch = nullptr;
-    CK(cudaMallocAsync(&scratch, pc_subsample_scratch_bytes(), s), "subsample scratch");
+    CK(ctx->scratch(&scratch, pc_subsample_scratch_bytes(), s), "subsample scratch");
     cudaError_t e = launch_pc_subsample(a, V->dtype, m, N, scratch, s);
     cudaFreeAsync(scratch, s);
     if (e != cudaSuccess) return cuda_fail(e, "pc subsample");
@@ -1033,7 +1045,7 @@ raypc_status raypc_warp_image(raypc_ctx* ctx, const raypc_camera* from, const ra
     DeviceGuard g(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
     // per-pixel selection keys: a device buffer owned by this call (freed in stream order)
-    CK(cudaMallocAsync((void**)&a.keys, sizeof(unsigned long long) * (size_t)w * h, s), "warp keys");
+    CK(ctx->scratch((void**)&a.keys, sizeof(unsigned long long) * (size_t)w * h, s), "warp keys");
     cudaError_t e = launch_warp(a, s);
     cudaFreeAsync(a.keys, s);
     if (e != cudaSuccess) return cuda_fail(e, "warp kernels");

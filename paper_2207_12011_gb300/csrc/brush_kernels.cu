@@ -50,13 +50,6 @@ __device__ __forceinline__ unsigned cell_class(float mn, float mx, float lo, flo
     return w;
 }
 
-// binary16 neighbours (bits of non-NaN values; the infinities are their own outer neighbours).
-__device__ __forceinline__ unsigned half_next(unsigned h) {
-    if (h == 0x7c00u) return h;
-    if (h == 0x8000u) h = 0u;
-    return h & 0x8000u ? h - 1u : h + 1u;
-}
-__device__ __forceinline__ unsigned half_prev(unsigned h) { return half_next(h ^ 0x8000u) ^ 0x8000u; }
 __device__ __forceinline__ float half_val(unsigned h) { return __half2float(__ushort_as_half((unsigned short)h)); }
 
 // binary16 bounds of a lower bound lo for corner values of at most M: a cell with

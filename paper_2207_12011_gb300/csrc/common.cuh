@@ -393,7 +393,18 @@ struct HistArgs {
                                   // (null: rows by warp stride)
     const uint32_t* sactive;      // optional: 4^3 sub-brick activity under this brush (cells of inactive
     int nsb;                      // sub-bricks are never counted), sub-bricks per axis
+    void* list;                   // optional scratch of hist_list(*this).bytes: the cells' bins are listed and
+                                  // counted in shared memory (no copies and no rowctr then)
 };
+
+// Scratch of a call that lists its cells' bins, and whether it should.
+struct HistList {
+    int planes;                   // z-planes listed at a time
+    unsigned chunks, batch;       // chunks of the list, chunks a warp takes at a time
+    size_t bins_at, bytes;
+};
+HistList hist_list(const HistArgs& h);
+bool hist_by_list(const HistArgs& h, int dtype);
 
 // World box that the samples assigned to brick b of edge bs (lower
 // interpolation index in [bs b, bs b + bs)) can occupy along one axis, widened
@@ -503,6 +514,14 @@ __device__ __forceinline__ bool skippable_brick(size_t b, int nb, const uint32_t
 // be interpolated, kCellFail = some restricted variable fails; [z][y][x] over
 // n^3 (entries with an index of n-1 are not written).
 constexpr unsigned kCellFail = 0x8000u;
+
+// binary16 neighbours (bits of non-NaN values; the infinities are their own outer neighbours).
+__device__ __forceinline__ unsigned half_next(unsigned h) {
+    if (h == 0x7c00u) return h;
+    if (h == 0x8000u) h = 0u;
+    return h & 0x8000u ? h - 1u : h + 1u;
+}
+__device__ __forceinline__ unsigned half_prev(unsigned h) { return half_next(h ^ 0x8000u) ^ 0x8000u; }
 
 // NaN-propagating max (a NaN operand gives NaN).
 __device__ __forceinline__ float max_nan(float a, float b) {

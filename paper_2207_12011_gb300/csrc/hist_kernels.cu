@@ -2,28 +2,34 @@
 // Fig. 2): for every in-shell (and, optionally, in-brush) cell and every pair
 // of adjacent axes (a, a+1), H[a][bin_a][bin_{a+1}] += 1.
 //
-// A scan over HBM plus the binning of the kept cells. A warp walks one x-row
-// of cells at a time so the planar loads are coalesced; rows whose cells all
-// lie outside the shell are skipped without touching memory. The vector kernel
-// streams 16-byte chunks of a row per variable (8 FP16 or 4 FP32 cells per
-// lane) through a cp.async double buffer in shared memory; the scalar kernel
-// (ragged grid edges, unaligned fields) takes one cell per lane. A cell's axis
-// values that are not brushed are loaded only after its brushed values pass.
-// Position axes and the position brush use the cell centre, coordinate
-// RN((2i + 1 - n) / n). With the volume's own brush the cells of inactive 4^3
-// sub-bricks are skipped without loads: every vertex of such a sub-brick fails
-// the brush (its values lie between the sub-brick's min and max) or lies
-// outside the shell (the sub-brick's widened box, which holds the vertex
-// centres, misses the shell). The in-shell test is integer-exact. Bins come
-// from the FP32 edges held in shared memory (comparisons only, so exact).
-// Increments are aggregated over runs of neighbouring cells that share their
-// bins (one atomicAdd per run), and on large grids spread over partial
-// histograms that a reduction sums, so the hot bins of a smooth field do not
-// serialise in L2.
+// A scan over HBM, the binning of the kept cells, and the counting. Rows whose cells
+// all lie outside the shell are skipped without touching memory. The vector kernels
+// (even grid edge, 16-byte aligned fields) stream 16-byte chunks per variable (8 FP16
+// or 4 FP32 cells per lane): through a cp.async double buffer in shared memory and a
+// compact list of the kept cells when something is brushed, straight into
+// registers when every in-shell cell counts. The scalar kernel (odd grid edges,
+// unaligned fields) takes one cell per lane. Position axes and the position
+// brush use the cell centre, coordinate RN((2i + 1 - n) / n). With the
+// volume's own brush the cells of inactive 4^3 sub-bricks are skipped without loads:
+// every vertex of such a sub-brick fails the brush (its values lie between the
+// sub-brick's min and max) or lies outside the shell (the sub-brick's widened
+// box, which holds the vertex centres, misses the shell). The in-shell test is
+// integer-exact. Bins come from the FP32 edges: an affine guess, checked against every
+// edge when the table is staged, and corrected by comparisons where that finds it inexact.
+//
+// What bounds a large call is the counting: five L2 atomics per cell of six axes, of
+// which few can be merged (neighbouring cells of a 256-bin table rarely share a bin
+// pair) and many meet at hot bins. Large grids therefore list the cells' bins in HBM and
+// count them one pair at a time in shared memory (k_hist_count): 512^3 FP16, 6
+// axes, 256 bins, whole shell 1236 -> 525 us; 4 brushed variables 422 -> 313 us;
+// 250^3 264 -> 115 us. Smaller grids, tables that do not fit and calls without scratch
+// add runs of cells with equal bins straight to L2, on large grids spread over
+// partial histograms that a reduction sums.
 #include <math.h>
 #include <stdint.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "host_math.h"
@@ -33,26 +39,48 @@ namespace raypc {
 namespace {
 
 constexpr int kHistThreads = 256;                    // scalar kernel
-constexpr int kHistWarps = kHistThreads / 32;
 constexpr int kHistVecThreads = 512;                 // vector kernel (two resident blocks per SM)
 constexpr int kHistVecWarps = kHistVecThreads / 32;
 constexpr unsigned kFull = 0xffffffffu;
 
-// Number of interior edges e_1..e_{bins-1} that are <= v, for non-decreasing
-// edges, from the staged table whose first and last entries are -inf and +inf
-// (stage_edges): j from an affine guess is the answer iff e[j] <= v < e[j+1]
-// (both loaded at once); otherwise the guess is walked to the answer with
-// comparisons of interior edges only (exact for any edges; equally spaced
-// edges rarely need a step). NaN compares false everywhere and lands in bin 0;
-// +inf fails only the last check of bin bins-1 and walks back to it.
-__device__ __forceinline__ int bin_of(const float* e, int bins, float v, float scale, float off) {
-    float g = fmaf(v, scale, off);                         // any guess is verified below
-    g = fminf(fmaxf(g, 0.0f), (float)(bins - 1));          // a NaN guess becomes 0
-    int j = __float_as_int(__fadd_rd(g, 0x1p23f)) - 0x4b000000;   // floor(g): 0 <= g < 2^23
-    const float lo = e[j], hi = e[j + 1];
-    if ((v >= lo) & (v < hi)) return j;
+// Affine guess of the bin of v, 0 .. bins - 1, non-decreasing in v (a NaN v gives 0): the place of v
+// among the bins as a fraction, saturated to [0, 1], times top = the float below bins, rounded
+// down to an integer in the low mantissa bits of the result.
+__device__ __forceinline__ unsigned bin_guess_raw(float top, float v, float scale, float off) {
+    return __float_as_uint(__fmaf_rd(__saturatef(fmaf(v, scale, off)), top, 0x1p23f));
+}
+__device__ __forceinline__ int bin_guess(float top, float v, float scale, float off) {
+    return (int)(bin_guess_raw(top, v, scale, off) - 0x4b000000u);
+}
+__device__ __forceinline__ float guess_top(int bins) { return __uint_as_float(__float_as_uint((float)bins) - 1u); }
+
+// How the bins of a call's axes are found from the guess (stage_edges picks one).
+enum BinMode : int {
+    kBinWalk = 0,                  // the guess is walked to the bin, comparing edges
+    kBinNear = 1,                  // the guess is at most one bin off for every v
+    kBinExact = 2,                 // the guess is the bin of every binary16 v
+};
+
+// From a guess to the bin. Out of line: rare, and an inlined copy per axis made the kernels too large
+// to come from HBM in time when their first launch finds the caches full of other data.
+__device__ __noinline__ int walk_bin(const float* e, int bins, float v, int j) {
     while (j > 0 && !(v >= e[j])) --j;
     while (j < bins - 1 && v >= e[j + 1]) ++j;
+    return j;
+}
+
+// Number of interior edges e_1..e_{bins-1} that are <= v, for non-decreasing edges:
+// the guess corrected with comparisons of edges only, so exact for any edges. The
+// staged table holds NaN for e_0 and e_bins, on which no count depends. NaN values
+// compare false everywhere and land in bin 0.
+template <int MODE>
+__device__ __forceinline__ int bin_of(const float* e, int bins, float top, float v, float scale, float off) {
+    int j = bin_guess(top, v, scale, off);
+    if constexpr (MODE == kBinNear) {
+        j += (v >= e[j + 1] ? 1 : 0) - (v < e[j] ? 1 : 0);
+    } else if constexpr (MODE == kBinWalk) {
+        j = walk_bin(e, bins, v, j);
+    }
     return j;
 }
 
@@ -72,12 +100,12 @@ __device__ __forceinline__ void add_runs(uint32_t* hist, unsigned key, bool kept
     }
 }
 
-// Largest integer m >= 0 with m * m <= a (0 <= a < 2^31).
+// Largest integer m >= 0 with m * m <= a (0 <= a < 2^31; m + 1 <= 46341, so the squares fit 32 bits).
 __device__ __forceinline__ int isqrt_floor(int a) {
-    int m = (int)sqrtf((float)a);
-    while ((long long)m * m > a) --m;
-    while ((long long)(m + 1) * (m + 1) <= a) ++m;
-    return m;
+    unsigned m = (unsigned)__fsqrt_rn((float)a);           // at most one off
+    if (m * m > (unsigned)a) --m;
+    if ((m + 1u) * (m + 1u) <= (unsigned)a) ++m;
+    return (int)m;
 }
 
 // Kernel view of a histogram call: the brushed variables and the axes as
@@ -103,9 +131,16 @@ struct HistLaunch {
     uint32_t sbr;                  // bit s: slot s is tested against the brush
     float slo[kMaxVars], shi[kMaxVars];
     uint32_t slo_h2[kMaxVars], shi_h2[kMaxVars];   // FP16 fields: the same bounds as binary16 pairs
-    float guess_scale[kMaxVars], guess_off[kMaxVars];   // bin guess fma(v, scale, off)
+    float guess_scale[kMaxVars], guess_off[kMaxVars];   // bin guess: fma(v, scale, off) of the bins
     long long soff[kMaxVars];      // byte offset of each load slot's plane (vector kernel)
+    int item0, items;              // rows (or segments) of this launch: item0 .. items - 1
     int rot;                       // row order: plane z is rotated in y by z * rot (mod n)
+    int batch;                     // segments a warp of the group walk takes at a time (1 .. 32)
+    // list mode: bins of the counted cells instead of counts (see ListSlots)
+    unsigned char* list;
+    unsigned char* list_mask;      // one byte per 8 cells of the list: the ones that count
+    unsigned* list_next;           // zeroed: chunks taken
+    unsigned list_chunks, list_batch;   // chunks that fit, chunks a warp takes at a time
     uint32_t* rowctr;              // zeroed row counter, or null: rows by warp stride
     int s_in, s_out;               // shell test on 2x+1-n etc., clamped to int
     uint32_t* out;                 // nout histograms; block b adds to copy b % nout
@@ -116,15 +151,65 @@ struct HistLaunch {
     float edges_inl[kInlineEdges];
 };
 
-// Copy the edge table into shared memory (all threads; the caller syncs), with
-// each axis's outer edges e_0 and e_bins, which no count depends on, replaced by
-// -inf and +inf so that bin_of checks a guess with two comparisons.
-__device__ __forceinline__ void stage_edges(const HistLaunch& A, float* s_edges) {
-    const int ne = A.naxes * (A.bins + 1);
+// The bin edges of a call in shared memory, and how its bins are found.
+struct BinTable {
+    float off[kMaxVars];           // guess offsets
+    int ok[kMaxVars];              // bit c < kOffsets: the guess with offset c is exact; bit kOffsets: near
+};
+constexpr int kOffsets = 4;
+__device__ __forceinline__ float offset_of(float off, int c, float bin) {
+    return off + bin * (c == 0 ? 0.0f : c == 1 ? 0x1p-15f : c == 2 ? -0x1p-15f : 0x1p-14f);
+}
+
+// Copy the edges of axes a0 .. a0 + naxes - 1 into shared memory (all threads), with
+// each axis's outer edges e_0 and e_bins replaced by NaN (see bin_of), and choose the
+// mode; syncs. The guess and the bin are both non-decreasing in v, so the guess is
+// at most one off everywhere if at every interior edge e_k it is k - 1 or more and
+// just below it k or less, and it is the bin of every binary16 value if it is k or
+// more at the smallest one >= e_k and k - 1 or less at the one before. A guess
+// that misses that by its rounding at some edge is tried with its offset moved by
+// a few 2^-15 of a bin.
+template <int DT>
+__device__ __forceinline__ int stage_edges(const HistLaunch& A, int a0, int naxes, float* s_edges, BinTable& T) {
+    const int bins = A.bins, ne = naxes * (bins + 1);
+    const float top = guess_top(bins), bin = 1.0f / (float)bins;
+    const int all = DT == kF16 ? (2 << kOffsets) - 1 : 1 << kOffsets;
+    if (threadIdx.x < kMaxVars) T.ok[threadIdx.x] = all;
+    __syncthreads();
     for (int i = threadIdx.x; i < ne; i += blockDim.x) {
-        const int k = i % (A.bins + 1);
-        s_edges[i] = k == 0 ? -INFINITY : k == A.bins ? INFINITY : A.edges ? __ldg(A.edges + i) : A.edges_inl[i];
+        const int a = i / (bins + 1), k = i - a * (bins + 1), src = a0 * (bins + 1) + i;
+        float e = __int_as_float(0x7fffffff);
+        if (k != 0 && k != bins) {
+            e = A.edges ? __ldg(A.edges + src) : A.edges_inl[src];
+            const float scale = A.guess_scale[a0 + a], off = A.guess_off[a0 + a];
+            int ok = bin_guess(top, e, scale, off) >= k - 1 &&
+                     bin_guess(top, nextafterf(e, -INFINITY), scale, off) <= k ? 1 << kOffsets : 0;
+            if (DT == kF16) {
+                const unsigned up = __half_as_ushort(__float2half_ru(e)), dn = half_prev(up);
+                const float vu = __half2float(__ushort_as_half((unsigned short)up));
+                const float vd = __half2float(__ushort_as_half((unsigned short)dn));
+#pragma unroll 1
+                for (int c = 0; c < kOffsets; ++c)
+                    if (bin_guess(top, vu, scale, offset_of(off, c, bin)) >= k && bin_guess(top, vd, scale, offset_of(off, c, bin)) < k)
+                        ok |= 1 << c;
+            }
+            if (ok != all) atomicAnd(&T.ok[a], ok);
+        }
+        s_edges[i] = e;
     }
+    __syncthreads();
+    bool near = true, exact = DT == kF16;
+    for (int a = 0; a < naxes; ++a) {
+        const int av = A.avar[a0 + a];
+        near = near && (T.ok[a] >> kOffsets);
+        exact = exact && av < kPosAxisBase && (T.ok[a] & ((1 << kOffsets) - 1));
+    }
+    if (threadIdx.x < naxes) {
+        const int c = exact ? __ffs(T.ok[threadIdx.x]) - 1 : 0;
+        T.off[threadIdx.x] = offset_of(A.guess_off[a0 + threadIdx.x], c, bin);
+    }
+    __syncthreads();
+    return exact ? kBinExact : near ? kBinNear : kBinWalk;
 }
 
 // Row geometry shared by both kernels: the x range of the r-th row (y, z) inside the
@@ -147,7 +232,8 @@ struct RowSpan {
 __device__ __forceinline__ bool row_span(const HistLaunch& A, int r, RowSpan& R) {
     const int n = A.n;
     R.z = r / n;
-    R.y = r - R.z * n + (R.z * A.rot) % n;                  // z * rot < 2^24 for n <= 4096
+    R.y = r - R.z * n;
+    if (A.rot) R.y += (R.z * A.rot) % n;                    // z * rot < 2^24 for n <= 4096
     if (R.y >= n) R.y -= n;
     const int dy = 2 * R.y + 1 - n, dz = 2 * R.z + 1 - n;
     R.syz = dy * dy + dz * dz;                              // < 2^31 for n <= 4096
@@ -185,8 +271,8 @@ __device__ __forceinline__ unsigned first_batch(const HistLaunch& A, int gwarp) 
 
 __device__ __forceinline__ int take_row(const HistLaunch& A, int r, int rows, int nwarps, int lane, unsigned& rq) {
     if (!A.rowctr) return r + nwarps;
-    if (r >= 0 && (r + 1) % kRowBatch != 0) return r + 1;
-    const int t = (int)__shfl_sync(kFull, rq, 0) * kRowBatch;
+    if (r >= A.item0 && (r - A.item0 + 1) % kRowBatch != 0) return r + 1;
+    const int t = A.item0 + (int)__shfl_sync(kFull, rq, 0) * kRowBatch;
     if (t < rows && lane == 0) rq = (unsigned)nwarps + atomicAdd(A.rowctr, 1u);
     return t;
 }
@@ -221,8 +307,9 @@ __device__ __forceinline__ bool cell_geometry_passes(const HistLaunch& A, const 
 template <int DT>
 __global__ void __launch_bounds__(kHistThreads) k_hist_scalar(const __grid_constant__ HistLaunch A) {
     extern __shared__ float s_edges[];
-    stage_edges(A, s_edges);
-    __syncthreads();
+    __shared__ BinTable T;
+    const int mode = stage_edges<DT>(A, 0, A.naxes, s_edges, T);
+    const float top = guess_top(A.bins);
 
     const int lane = threadIdx.x & 31;
     const int n = A.n;
@@ -280,7 +367,9 @@ __global__ void __launch_bounds__(kHistThreads) k_hist_scalar(const __grid_const
                     if (keep[j]) {
                         const float v = av >= kPosAxisBase ? pos_axis(cx, R.cy, R.cz, cr2, av - kPosAxisBase)
                                                            : load_cell<DT>(A.cells, av * plane + R.base + x);
-                        b = (unsigned)bin_of(s_edges + a * (bins + 1), bins, v, A.guess_scale[a], A.guess_off[a]);
+                        const float* e = s_edges + a * (bins + 1);
+                        b = (unsigned)(mode != kBinWalk ? bin_of<kBinNear>(e, bins, top, v, A.guess_scale[a], T.off[a])
+                                                        : bin_of<kBinWalk>(e, bins, top, v, A.guess_scale[a], T.off[a]));
                     }
                     if (a > 0) add_runs(out + (size_t)(a - 1) * bins * bins, prev * (unsigned)bins + b, keep[j], km, lane);
                     prev = b;
@@ -328,21 +417,22 @@ __device__ __forceinline__ unsigned span_bits(int lo, int hi) {
     return l > h ? 0u : (2u << h) - (1u << l);
 }
 
-// Geometric keep bits of this lane's chunk (x0 .. x0 + VEC - 1; x0 and n multiples
-// of VEC): in the shell (the row's ranges), in an active sub-brick when the
-// activity is given, inside the position brush. A chunk with a cell in the shell
-// lies inside the row, so its sub-brick ids are valid.
+// Geometric keep bits of this lane's chunk (cells x0 .. x0 + VEC - 1, x0 any): in the
+// shell (the row's ranges), in an active sub-brick when the activity is given, inside
+// the position brush.
 template <int VEC>
 __device__ __forceinline__ unsigned chunk_geometry(const HistLaunch& A, const RowSpan& R, int x0) {
     unsigned kb = span_bits<VEC>(R.xa - x0, R.xb - x0) & ~span_bits<VEC>(R.ca - x0, R.cb - x0);
     if (kb && A.sactive) {
-        // the chunk's VEC / 4 sub-bricks sit in one activity word unless the first is bit 31
-        const uint32_t sid = R.srow + (uint32_t)(x0 >> 2);
+        // the activity of the sub-bricks that the chunk's cells lie in, from the first kept cell's on
+        const int xs = x0 + __ffs(kb) - 1, s0 = xs >> 2;
+        const uint32_t sid = R.srow + (uint32_t)s0;
         unsigned act = __ldg(A.sactive + (sid >> 5)) >> (sid & 31);
-        if (VEC > 4 && (sid & 31) > 32 - VEC / 4) act |= __ldg(A.sactive + (sid >> 5) + 1) << (32 - (sid & 31));
+        const int more = min((x0 + 31 - __clz(kb)) >> 2, A.nsb - 1) - s0;   // to the last kept cell's
+        if ((int)(sid & 31) + more > 31) act |= __ldg(A.sactive + (sid >> 5) + 1) << (32 - (sid & 31));
 #pragma unroll
-        for (int q = 0; q < VEC / 4; ++q)
-            if (!((act >> q) & 1u)) kb &= ~(0xfu << (4 * q));
+        for (int q = 0; q < VEC / 4 + 1; ++q)
+            if (!((act >> q) & 1u)) kb &= ~span_bits<VEC>(4 * (s0 + q) - x0, 4 * (s0 + q) + 3 - x0);
     }
     if (kb && A.pmask) {
         BrushArgs pb;
@@ -365,16 +455,19 @@ __device__ __forceinline__ unsigned chunk_geometry(const HistLaunch& A, const Ro
 template <int VEC>
 __device__ __forceinline__ void next_chunk_row(const HistLaunch& A, int nwarps, int lane, ChunkRow& C) {
     constexpr int CH = 32 * VEC;
-    const int rows = A.n * A.n;
+    const int rows = A.items;
     int r = C.r, xw = C.xw + CH;
-    bool have_row = r >= 0;
+    bool have_row = r >= A.item0;
     for (;;) {
         if (!have_row || xw > C.R.xb) {
             r = take_row(A, r, rows, nwarps, lane, C.rq);
             if (r >= rows) { C.r = -1; C.kb = 0u; return; }
             if (!row_span(A, r, C.R)) { have_row = false; continue; }
             have_row = true;
-            xw = C.R.xa & ~(VEC - 1);
+            // chunks start on 16-byte boundaries of the plane: before x = 0 of the row when the edge is
+            // no multiple of VEC (the cells in front are another row's)
+            const int lead = (int)(C.R.base & (VEC - 1));
+            xw = ((C.R.xa + lead) & ~(VEC - 1)) - lead;
         }
         const unsigned kb = chunk_geometry<VEC>(A, C.R, xw + lane * VEC);
         if (__ballot_sync(kFull, kb != 0u) != 0u) {
@@ -387,28 +480,177 @@ __device__ __forceinline__ void next_chunk_row(const HistLaunch& A, int nwarps, 
     }
 }
 
-// One binning round of the vector kernel: lane l holds a cell iff kept (the kept lanes
-// are a prefix, km their mask) with its axis values val[a]. Bins come from the FP32 edges in
-// shared memory; a lane whose bin tuple differs from its left neighbour's starts a run and
-// adds the run's length to each adjacent-axis pair (one atomic per pair and run).
-__device__ __forceinline__ void bin_round(const HistLaunch& A, const float* s_edges, uint32_t* out,
-                                          const float (&val)[kMaxVars], bool kept, unsigned km, int lane) {
-    const int naxes = A.naxes, bins = A.bins;
-    unsigned bn[kMaxVars];
-    unsigned packed[3] = {0u, 0u, 0u};                      // three bins per word, 10 bits each
-#pragma unroll
-    for (int a = 0; a < kMaxVars; ++a) {
-        bn[a] = 0u;
-        if (a >= naxes || !kept) continue;
-        bn[a] = (unsigned)bin_of(s_edges + a * (bins + 1), bins, val[a], A.guess_scale[a], A.guess_off[a]);
-        packed[a / 3] |= bn[a] << (10 * (a % 3));
+// How a warp of the vector kernel walks the cells: chunk rows of whole x-rows, or
+// groups of active sub-bricks. Both hold the current chunk's geometric keep bits kb,
+// this lane's element offset off (its VEC consecutive cells) and, for position
+// axes, the centre of listed cell c (lane c / VEC, cell c % VEC).
+template <int VEC>
+struct RowWalk {
+    ChunkRow C;
+    int nwarps;
+    unsigned kb;
+    size_t off;
+    __device__ __forceinline__ void start(const HistLaunch& A, int gwarp, int nw) {
+        nwarps = nw;
+        C.r = A.item0 + gwarp - nw;
+        C.xw = 0;
+        C.rq = first_batch(A, gwarp);
     }
+    __device__ __forceinline__ bool more() const { return C.r >= 0; }
+    __device__ __forceinline__ void next(const HistLaunch& A, int lane) {
+        next_chunk_row<VEC>(A, nwarps, lane, C);
+        kb = C.kb;
+        off = C.R.base + C.xw + lane * VEC;
+    }
+    __device__ __forceinline__ void centre(const HistLaunch& A, int c, float& cx, float& cy, float& cz) const {
+        cx = cell_centre_rn(C.xw + c, A.n);
+        cy = C.R.cy;
+        cz = C.R.cz;
+    }
+};
+
+// For listed calls: groups of 2 VEC / 4 sub-bricks that are neighbours in x, with an active one among
+// them: 2 VEC x 4 x 4 cells, lane 2 r + h the h-th half of row r (y = r % 4, z =
+// r / 4), taken from segments of 8 sub-bricks of a sub-brick row. Under a brush the
+// active sub-bricks are few and short in x: a chunk row of 32 VEC cells of one
+// x-row has a third of its lanes at work, a group two thirds, and no row needs its
+// sphere's chord (256^3 FP16, 3 brushed variables: 42 -> 25 M warp instructions). The
+// segments come in batches, their bits loaded at once (512^3: 352 -> 214 us).
+template <int VEC>
+struct GroupWalk {
+    static constexpr int kSubs = VEC / 2;              // sub-bricks of a group
+    int nwarps, base;                                  // first segment of the batch (-1: no more)
+    unsigned rq, segs, mine, bits, kb;                 // segments left in the batch, lane j's: the bits of segment j
+    int sx, sy, sz;                                    // first sub-brick of the segment's bits, and its row
+    int gx;                                            // first sub-brick of the current group
+    size_t off;
+    __device__ __forceinline__ void start(const HistLaunch& A, int gwarp, int nw) {
+        nwarps = nw;
+        base = 0;
+        rq = (unsigned)gwarp;
+        segs = bits = 0u;
+    }
+    __device__ __forceinline__ bool more() const { return base >= 0; }
+    // The activity bits of the warp's next batch of segments, one segment per lane: the batch's
+    // number was taken from the row counter a batch ahead, and
+    // empty segments cost a bit each instead of a load's latency.
+    __device__ __forceinline__ bool next_batch(const HistLaunch& A, int lane) {
+        const unsigned b = __shfl_sync(kFull, rq, 0);
+        const long long first = A.item0 + (long long)b * A.batch;
+        if (first >= A.items) {
+            base = -1;
+            return false;
+        }
+        base = (int)first;
+        if (lane == 0) rq = (unsigned)nwarps + atomicAdd(A.rowctr, 1u);
+        mine = 0u;
+        const int seg = base + lane, per_row = (A.nsb + 7) >> 3;
+        if (lane < A.batch && seg < A.items) {
+            const int row = seg / per_row, x = (seg - row * per_row) << 3;
+            const uint32_t id = (uint32_t)row * A.nsb + x;
+            const int here = min(8, A.nsb - x);        // sub-bricks of the segment
+            mine = __ldg(A.sactive + (id >> 5)) >> (id & 31);
+            if ((int)(id & 31) + here > 32) mine |= __ldg(A.sactive + (id >> 5) + 1) << (32 - (id & 31));
+            mine &= (1u << here) - 1u;
+        }
+        segs = __ballot_sync(kFull, mine != 0u);
+        return true;
+    }
+    __device__ __forceinline__ void next(const HistLaunch& A, int lane) {
+        const int n = A.n, nsb = A.nsb, per_row = (nsb + 7) >> 3;
+        kb = 0u;
+        for (;;) {
+            if (bits == 0u) {                          // uniform over the warp
+                while (segs == 0u)
+                    if (!next_batch(A, lane)) return;
+                const int j = __ffs(segs) - 1;
+                segs &= segs - 1u;
+                bits = __shfl_sync(kFull, mine, j);
+                const int row = (base + j) / per_row;
+                sx = (base + j - row * per_row) << 3;
+                sz = row / nsb;
+                sy = row - sz * nsb;
+            }
+            const int g = (__ffs(bits) - 1) & ~(kSubs - 1);
+            const unsigned act = (bits >> g) & ((1u << kSubs) - 1u);
+            bits &= ~(((1u << kSubs) - 1u) << g);
+            gx = sx + g;
+            const int half = lane & 1, row = lane >> 1;
+            const int x = gx * 4 + half * VEC, y = sy * 4 + (row & 3), z = sz * 4 + (row >> 2);
+            if (x < n) {                               // n is a multiple of VEC and of 4
+#pragma unroll
+                for (int q = 0; q < VEC / 4; ++q)
+                    if ((act >> (half * (VEC / 4) + q)) & 1u) kb |= 0xfu << (4 * q);
+            }
+            const int dy = 2 * y + 1 - n, dz = 2 * z + 1 - n, syz = dy * dy + dz * dz;
+            if (kb) {
+                // |2x + 1 - n| over the run: all of it in the shell, or cell by cell
+                const int d0 = 2 * x + 1 - n, d1 = d0 + 2 * (VEC - 1);
+                const int far = max(abs(d0), abs(d1)), near = d0 > 0 ? d0 : (d1 < 0 ? -d1 : 0);
+                if (!(near * near + syz >= A.s_in && far * far + syz <= A.s_out)) {
+#pragma unroll
+                    for (int q = 0; q < VEC; ++q) {
+                        const int d = d0 + 2 * q, sh = d * d + syz;
+                        if (!(sh >= A.s_in && sh <= A.s_out)) kb &= ~(1u << q);
+                    }
+                }
+            }
+            if (kb && A.pmask) {
+                BrushArgs pb;
+#pragma unroll
+                for (int a = 0; a < kNumPos; ++a) { pb.plo[a] = A.plo[a]; pb.phi[a] = A.phi[a]; }
+                pb.pmask = A.pmask;
+                const float cy = cell_centre_rn(y, n), cz = cell_centre_rn(z, n);
+#pragma unroll
+                for (int q = 0; q < VEC; ++q) {
+                    const float cx = cell_centre_rn(x + q, n);
+                    if (((kb >> q) & 1u) && !pos_pass(cx, cy, cz, dot3_rn(cx, cy, cz, cx, cy, cz), pb)) kb &= ~(1u << q);
+                }
+            }
+            if (__ballot_sync(kFull, kb != 0u) != 0u) {
+                off = ((size_t)z * n + y) * n + x;
+                return;
+            }
+        }
+    }
+    __device__ __forceinline__ void centre(const HistLaunch& A, int c, float& cx, float& cy, float& cz) const {
+        const int l = c / VEC, row = l >> 1;
+        cx = cell_centre_rn(gx * 4 + (l & 1) * VEC + c % VEC, A.n);
+        cy = cell_centre_rn(sy * 4 + (row & 3), A.n);
+        cz = cell_centre_rn(sz * 4 + (row >> 2), A.n);
+    }
+};
+
+// One binning round of the vector kernel: lane l holds a cell iff kept (the kept lanes
+// are a prefix) with its axis values val[a]; bn[a] receives their bins. NAX: the number of
+// axes, 0: A.naxes.
+template <int NAX, int MODE>
+__device__ __forceinline__ void bins_of(const HistLaunch& A, const float* s_edges, const BinTable& T,
+                                        const float (&val)[kMaxVars], unsigned (&bn)[kMaxVars]) {
+    const float top = guess_top(A.bins);
+#pragma unroll
+    for (int a = 0; a < (NAX ? NAX : kMaxVars); ++a) {
+        bn[a] = 0u;
+        if (!NAX && a >= A.naxes) continue;
+        bn[a] = (unsigned)bin_of<MODE>(s_edges + a * (A.bins + 1), A.bins, top, val[a], A.guess_scale[a], T.off[a]);
+    }
+}
+
+// Direct counts: a lane whose bin tuple differs from its left neighbour's starts a run
+// and adds the run's length to each adjacent-axis pair (one L2 atomic per pair and
+// run; km: mask of the kept lanes).
+__device__ __forceinline__ void add_tuples(const HistLaunch& A, uint32_t* out, const unsigned (&bn)[kMaxVars], bool kept,
+                                           unsigned km, int lane) {
+    const int naxes = A.naxes, bins = A.bins;
     bool same = lane > 0;
 #pragma unroll
     for (int w = 0; w < 3; ++w) {
         if (3 * w >= naxes) break;
-        const unsigned left = __shfl_up_sync(kFull, packed[w], 1);   // every lane takes part
-        same = same && left == packed[w];
+        unsigned packed = 0u;                               // three bins, 10 bits each
+#pragma unroll
+        for (int a = 3 * w; a < 3 * w + 3 && a < kMaxVars; ++a) packed |= bn[a] << (10 * (a % 3));
+        const unsigned left = __shfl_up_sync(kFull, packed, 1);   // by every lane: outside the condition
+        same = same && left == packed;
     }
     const bool head = kept && !same;
     const unsigned hm = __ballot_sync(kFull, head);
@@ -416,142 +658,212 @@ __device__ __forceinline__ void bin_round(const HistLaunch& A, const float* s_ed
         const unsigned after = lane == 31 ? 0u : (kFull << (lane + 1));
         const unsigned stop = (hm | ~km) & after;            // next run start or the last kept lane
         const unsigned len = (unsigned)((stop ? __ffs(stop) - 1 : 32) - lane);
+        const unsigned bb = (unsigned)(bins * bins);
 #pragma unroll
         for (int a = 1; a < kMaxVars; ++a) {
             if (a >= naxes) break;
-            atomicAdd(out + (size_t)(a - 1) * bins * bins + bn[a - 1] * (unsigned)bins + bn[a], len);
+            atomicAdd(out + ((a - 1) * bb + bn[a - 1] * (unsigned)bins + bn[a]), len);
         }
     }
 }
 
+// A warp's place in the list of binned cells. The list is made of chunks of 32 units of
+// 8 cells, each axis's bins contiguous within a chunk (bytes up to 256 bins, else 16
+// bits), with one mask byte per unit. A warp takes list_batch chunks at a time from a
+// counter, the first ones when it has a cell to list.
+constexpr int kListCells = 256;
+constexpr unsigned kListBatch = 4;                           // most chunks taken at a time
+struct ListSlots {
+    unsigned chunk, left;                                    // current chunk, chunks of its batch after it
+    unsigned fill;                                           // used cells (k_hist_bins: used units) of the chunk
+    unsigned after;                                          // the next batch (lane 0), taken with the last
+    bool early;                                              // chunk of its batch, when batches have several
+    __device__ __forceinline__ void start(unsigned full) {
+        chunk = ~0u;
+        left = after = 0u;
+        fill = full;
+        early = false;
+    }
+    __device__ __forceinline__ void advance(const HistLaunch& A, int lane) {
+        if (left) {
+            --left;
+            ++chunk;
+        } else {
+            if (!early && lane == 0) after = atomicAdd(A.list_next, A.list_batch);
+            chunk = __shfl_sync(kFull, after, 0);
+            left = A.list_batch - 1u;
+            early = false;
+            if (left) return;
+        }
+        if (left == 0u && A.list_batch > 1u) {
+            early = true;
+            if (lane == 0) after = atomicAdd(A.list_next, A.list_batch);
+        }
+    }
+    __device__ __forceinline__ void mask(const HistLaunch& A, unsigned c, unsigned unit, unsigned bits) const {
+        if (c < A.list_chunks) A.list_mask[(size_t)c * 32 + unit] = (unsigned char)bits;
+    }
+    // masks of the chunk's units: the first fill cells
+    __device__ __forceinline__ void close(const HistLaunch& A, int lane) {
+        mask(A, chunk, lane, (1u << min(8, max(0, (int)fill - 8 * lane))) - 1u);
+    }
+    // the rest of the chunk from unit u on, the rest of its batch and the batch taken early are empty
+    __device__ __forceinline__ void finish(const HistLaunch& A, unsigned u, int lane) {
+        if (lane >= (int)u) mask(A, chunk, lane, 0u);
+        for (unsigned i = 1; i <= left; ++i) mask(A, chunk + i, lane, 0u);
+        const unsigned next = __shfl_sync(kFull, after, 0);
+        for (unsigned i = 0; early && i < A.list_batch; ++i) mask(A, next + i, lane, 0u);
+    }
+    // a round of up to 32 cells, take of them kept (a prefix of the lanes)
+    template <int NAX>
+    __device__ __forceinline__ void put(const HistLaunch& A, const unsigned (&bn)[kMaxVars], bool kept, int take, int lane) {
+        const int naxes = NAX ? NAX : A.naxes;
+        if (fill + 32 > kListCells) {
+            close(A, lane);
+            advance(A, lane);
+            fill = 0u;
+        }
+        if (kept && chunk < A.list_chunks) {                 // the list is sized for every in-shell cell
+            const size_t at = (size_t)chunk * (size_t)(naxes * kListCells) + fill + lane;
+#pragma unroll
+            for (int a = 0; a < (NAX ? NAX : kMaxVars); ++a) {
+                if (!NAX && a >= naxes) break;
+                if (A.bins <= 256) A.list[at + a * kListCells] = (unsigned char)bn[a];
+                else reinterpret_cast<unsigned short*>(A.list)[at + a * kListCells] = (unsigned short)bn[a];
+            }
+        }
+        fill += (unsigned)take;
+    }
+};
+
 // Vector kernel (grid edge a multiple of the chunk, 16-byte aligned planes, at most
-// kMaxVars load slots). A warp walks x-rows in chunk rows of 32 lanes x 16 bytes
-// (8 FP16 or 4 FP32 cells per lane). While it tests and bins one chunk row it has
-// the next one's slots copied into its other shared buffer with cp.async (only
-// chunks with a cell that passes the shell, sub-brick and position tests), so
-// HBM latency hides behind the binning and no registers wait on loads. All
-// brushed slots are tested (FP16: two cells at a time against exact binary16
-// bounds); the surviving cells go into a compact list in x order (warp prefix
-// sum) from which the warp bins 32 cells per round, reading the axis values
-// from the buffer. Neighbouring lanes then hold neighbouring cells, whose bin
-// tuples mostly agree on a smooth field: a lane whose tuple differs from its
-// left neighbour's starts a run and adds the run's length to each
-// adjacent-axis pair (one atomic per pair and run). Persistent grid, rows from
-// the row counter or by warp stride; the edge table is staged once per resident
-// block.
-template <int DT>
+// kMaxVars load slots). While a warp tests and bins one chunk of its walk (32 lanes x
+// 16 bytes, 8 FP16 or 4 FP32 cells per lane) it has the next one's slots copied
+// into its other shared buffer with cp.async (only chunks with a cell that passes
+// the shell, sub-brick and position tests), so HBM latency hides behind the
+// binning and no registers wait on loads. All brushed slots are tested (FP16: two
+// cells at a time against exact binary16 bounds); the surviving cells go into a
+// compact list (warp prefix sum) from which the warp bins 32 cells per round,
+// reading the axis values from the buffer. LIST: the bins go into a list that
+// k_hist_count turns into counts; else straight into L2 atomics. Persistent grid;
+// rows or segments from the row counter or by warp stride; the edge table is staged
+// once per resident block. NAX: 0 with a position axis or a position brush, else the
+// number of axes, or -1 for any (fixed loops have no checks and immediate offsets: 89 -> 82
+// us at 250^3 FP16 by groups).
+template <int DT, typename Walk, int NAX, bool LIST>
 __global__ void __launch_bounds__(kHistVecThreads, 2) k_hist(const __grid_constant__ HistLaunch A) {
     constexpr int VEC = DT == kF16 ? 8 : 4;
+    constexpr int kMost = NAX > 0 ? NAX : kMaxVars;
+    constexpr bool kCarry = DT == kF16 && NAX != 0;            // FP16: a remainder waits for the next chunk
     extern __shared__ __align__(16) unsigned char s_raw[];
+    __shared__ BinTable T;
     float* s_edges = reinterpret_cast<float*>(s_raw);
     const int ne16 = (A.naxes * (A.bins + 1) + 3) & ~3;
-    const int nslot = A.nslot, naxes = A.naxes;
-    const int buf_bytes = nslot * 512;                          // one chunk row of every slot
+    const int nslot = A.nslot, naxes = NAX > 0 ? NAX : A.naxes;
+    const int buf_bytes = nslot * 512;                          // one chunk of every slot
     unsigned char* s_warp = s_raw + sizeof(float) * ne16 + (size_t)(threadIdx.x >> 5) * (2 * buf_bytes + 256);
     unsigned char* s_list = s_warp + 2 * buf_bytes;
-    stage_edges(A, s_edges);
-    __syncthreads();
+    const int mode = stage_edges<DT>(A, 0, naxes, s_edges, T);
 
     const int lane = threadIdx.x & 31;
-    const int n = A.n;
-    const int nwarps = (int)((gridDim.x * blockDim.x) >> 5);
-    const int bins = A.bins;
     const uint32_t sbr = A.sbr;
-    uint32_t* const out = A.out + (size_t)(blockIdx.x % (unsigned)A.nout) * (naxes - 1) * bins * bins;
+    uint32_t* const out = LIST ? nullptr : A.out + (size_t)(blockIdx.x % (unsigned)A.nout) * (naxes - 1) * A.bins * A.bins;
 
-    // copies of chunk row C into buffer b (lanes whose chunk has no passing cell copy nothing)
-    auto prefetch = [&](const ChunkRow& C, int b) {
-        if (C.r >= 0 && C.kb) {
-            const int x0 = C.xw + lane * VEC;
+    // copies of chunk W into buffer b (lanes whose cells all fail copy nothing)
+    auto prefetch = [&](const Walk& W, int b) {
+        if (W.more() && W.kb) {
             unsigned char* dst = s_warp + b * buf_bytes + lane * 16;
-            const char* src = static_cast<const char*>(A.cells) + (C.R.base + x0) * (16 / VEC);
+            const char* src = static_cast<const char*>(A.cells) + W.off * (16 / VEC);
 #pragma unroll
             for (int s = 0; s < kMaxVars; ++s)
-                if (s < nslot && A.svar[s] >= 0) cp_async16(dst + s * 512, src + A.soff[s]);
+                if (s < NAX || (s < nslot && (NAX < 0 || A.svar[s] >= 0))) cp_async16(dst + s * 512, src + A.soff[s]);
         }
         cp_async_commit();
     };
 
-    const bool carry = DT == kF16 && !A.use_pos;
+    ListSlots slots;
+    slots.start(kListCells);
     int q = 0;                                                  // carried cells, in lanes 0..q-1
-    unsigned cpk[kMaxVars / 2] = {0u, 0u, 0u, 0u};              // a carried cell's values, binary16 pairs
+    unsigned cpk[(kMost + 1) / 2] = {};                         // a carried cell's values, binary16 pairs
 
-    ChunkRow cur;
-    cur.r = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) - nwarps;
-    cur.xw = 0;
-    cur.rq = first_batch(A, (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5));
-    next_chunk_row<VEC>(A, nwarps, lane, cur);
-    prefetch(cur, 0);
+    Walk cur;
+    cur.start(A, (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), (int)((gridDim.x * blockDim.x) >> 5));
+    cur.kb = 0u;                                                // an empty chunk before the first
+    bool have = true;
     int b = 0;
-    while (cur.r >= 0) {
-        ChunkRow nxt = cur;
-        next_chunk_row<VEC>(A, nwarps, lane, nxt);
-        prefetch(nxt, b ^ 1);
-        cp_async_wait_prev();                                   // this chunk row's copies have landed
-        __syncwarp();
+    for (;;) {                                                  // no chunk left: only the last carried cells are
+        if (!have && q == 0) break;
+        Walk nxt = cur;
         const unsigned char* buf = s_warp + b * buf_bytes;
-        unsigned kb = cur.kb;
-        // brushed slots
-        if constexpr (DT == kF16) {
-            unsigned acc[4] = {kFull, kFull, kFull, kFull};
+        int total = 0;
+        if (have) {
+            nxt.next(A, lane);
+            prefetch(nxt, b ^ 1);
+            cp_async_wait_prev();                               // this chunk's copies have landed
+            __syncwarp();
+            unsigned kb = cur.kb;
+            // brushed slots
+            if constexpr (DT == kF16) {
+                unsigned acc[4] = {kFull, kFull, kFull, kFull};
 #pragma unroll
-            for (int s = 0; s < kMaxVars; ++s) {
-                if (s < nslot && ((sbr >> s) & 1u)) {
-                    const uint4 v = *reinterpret_cast<const uint4*>(buf + s * 512 + lane * 16);
-                    const __half2 lo2 = u32_as_half2(A.slo_h2[s]), hi2 = u32_as_half2(A.shi_h2[s]);
-                    const unsigned w[4] = {v.x, v.y, v.z, v.w};
+                for (int s = 0; s < kMaxVars; ++s) {
+                    if ((sbr >> s) & 1u) {
+                        const uint4 v = *reinterpret_cast<const uint4*>(buf + s * 512 + lane * 16);
+                        const __half2 lo2 = u32_as_half2(A.slo_h2[s]), hi2 = u32_as_half2(A.shi_h2[s]);
+                        const unsigned w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        acc[q] &= __hge2_mask(u32_as_half2(w[q]), lo2) & __hle2_mask(u32_as_half2(w[q]), hi2);
+                        for (int i = 0; i < 4; ++i)
+                            acc[i] &= __hge2_mask(u32_as_half2(w[i]), lo2) & __hle2_mask(u32_as_half2(w[i]), hi2);
+                    }
                 }
-            }
-            unsigned pass = 0u;
+                unsigned pass = 0u;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) pass |= ((acc[q] & 1u) | ((acc[q] >> 15) & 2u)) << (2 * q);
-            kb &= pass;
-        } else {
+                for (int i = 0; i < 4; ++i) pass |= ((acc[i] & 1u) | ((acc[i] >> 15) & 2u)) << (2 * i);
+                kb &= pass;
+            } else {
 #pragma unroll
-            for (int s = 0; s < kMaxVars; ++s) {
-                if (s < nslot && ((sbr >> s) & 1u)) {
-                    const uint4 v = *reinterpret_cast<const uint4*>(buf + s * 512 + lane * 16);
-                    const float lo = A.slo[s], hi = A.shi[s];
+                for (int s = 0; s < kMaxVars; ++s) {
+                    if ((sbr >> s) & 1u) {
+                        const uint4 v = *reinterpret_cast<const uint4*>(buf + s * 512 + lane * 16);
+                        const float lo = A.slo[s], hi = A.shi[s];
 #pragma unroll
-                    for (int j = 0; j < VEC; ++j) {
-                        const float x = chunk_elem<DT>(v, j);
-                        if (!(x >= lo && x <= hi)) kb &= ~(1u << j);
+                        for (int j = 0; j < VEC; ++j) {
+                            const float x = chunk_elem<DT>(v, j);
+                            if (!(x >= lo && x <= hi)) kb &= ~(1u << j);
+                        }
                     }
                 }
             }
-        }
-        // compact list of the surviving cells (chunk-row offsets) in x order: the exclusive
-        // prefix of the per-lane counts from an inclusive shuffle scan
-        const unsigned cnt = (unsigned)__popc(kb);
-        unsigned inc = cnt;
+            // compact list of the surviving cells (lane * VEC + j) in order: the exclusive
+            // prefix of the per-lane counts from an inclusive shuffle scan
+            const unsigned cnt = (unsigned)__popc(kb);
+            unsigned inc = cnt;
 #pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const unsigned t = __shfl_up_sync(kFull, inc, d);
-            if (lane >= d) inc += t;
-        }
-        int pos = (int)(inc - cnt);
-        const int total = (int)__shfl_sync(kFull, inc, 31);
+            for (int d = 1; d < 32; d <<= 1) {
+                const unsigned t = __shfl_up_sync(kFull, inc, d);
+                if (lane >= d) inc += t;
+            }
+            int pos = (int)(inc - cnt);
+            total = (int)__shfl_sync(kFull, inc, 31);
 #pragma unroll
-        for (int j = 0; j < VEC; ++j)
-            if ((kb >> j) & 1u) s_list[pos++] = (unsigned char)(lane * VEC + j);
-        __syncwarp();
+            for (int j = 0; j < VEC; ++j)
+                if ((kb >> j) & 1u) s_list[pos++] = (unsigned char)(lane * VEC + j);
+            __syncwarp();
+        }
         // bin the surviving cells 32 per round. FP16 without position axes carries a remainder
-        // of fewer than 32 cells to the next chunk row (their values in the lanes' registers),
-        // so that sparse chunk rows still fill whole rounds
+        // of fewer than 32 cells to the next chunk (their values in the lanes' registers),
+        // so that sparse chunks still fill whole rounds
         int consumed = 0;
 #pragma unroll 1
         for (;;) {
             const int avail = q + total - consumed;
             if (avail == 0) break;
-            if (carry && avail < 32) {
+            if (kCarry && have && avail < 32) {
                 if (lane >= q && lane < avail) {
                     const int c = s_list[consumed + lane - q];
 #pragma unroll
-                    for (int a = 0; a < kMaxVars; ++a) {
-                        if (a >= naxes) break;
+                    for (int a = 0; a < kMost; ++a) {
+                        if (NAX < 0 && a >= naxes) break;
                         const unsigned hb = reinterpret_cast<const unsigned short*>(buf + a * 512)[c];
                         cpk[a >> 1] = (cpk[a >> 1] & (0xffff0000u >> (16 * (a & 1)))) | (hb << (16 * (a & 1)));
                     }
@@ -565,48 +877,320 @@ __global__ void __launch_bounds__(kHistVecThreads, 2) k_hist(const __grid_consta
             float val[kMaxVars];
 #pragma unroll
             for (int a = 0; a < kMaxVars; ++a) val[a] = 0.0f;
-            if (kept && lane < q) {                             // a carried cell
+            if (kCarry && kept && lane < q) {                   // a carried cell
 #pragma unroll
-                for (int a = 0; a < kMaxVars; ++a)
-                    if (a < naxes)
-                        val[a] = __half2float(__ushort_as_half((unsigned short)(cpk[a >> 1] >> (16 * (a & 1)))));
+                for (int a = 0; a < kMost; ++a)
+                    val[a] = __half2float(__ushort_as_half((unsigned short)(cpk[a >> 1] >> (16 * (a & 1)))));
             } else if (kept) {
-                const int c = s_list[consumed + lane - q];       // cell cur.xw + c
-                float cx = 0.0f, cr2 = 0.0f;
-                if (A.use_pos) {
-                    cx = cell_centre_rn(cur.xw + c, n);
-                    cr2 = dot3_rn(cx, cur.R.cy, cur.R.cz, cx, cur.R.cy, cur.R.cz);
+                const int c = s_list[consumed + lane - q];
+                float cx = 0.0f, cy = 0.0f, cz = 0.0f, cr2 = 0.0f;
+                if (!NAX && A.use_pos) {
+                    cur.centre(A, c, cx, cy, cz);
+                    cr2 = dot3_rn(cx, cy, cz, cx, cy, cz);
                 }
 #pragma unroll
-                for (int a = 0; a < kMaxVars; ++a) {
-                    if (a >= naxes) break;
-                    const int av = A.avar[a];
-                    if (av >= kPosAxisBase)
-                        val[a] = pos_axis(cx, cur.R.cy, cur.R.cz, cr2, av - kPosAxisBase);
+                for (int a = 0; a < kMost; ++a) {
+                    if (NAX <= 0 && a >= naxes) break;
+                    if (!NAX && A.avar[a] >= kPosAxisBase)
+                        val[a] = pos_axis(cx, cy, cz, cr2, A.avar[a] - kPosAxisBase);
                     else if (DT == kF16)
                         val[a] = __half2float(__ushort_as_half(reinterpret_cast<const unsigned short*>(buf + a * 512)[c]));
                     else
                         val[a] = reinterpret_cast<const float*>(buf + a * 512)[c];
                 }
             }
-            bin_round(A, s_edges, out, val, kept, km, lane);
+            unsigned bn[kMaxVars] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+            if (DT == kF16 && NAX && mode == kBinExact) bins_of<(NAX > 0 ? NAX : 0), kBinExact>(A, s_edges, T, val, bn);
+            else if (mode != kBinWalk) bins_of<(NAX > 0 ? NAX : 0), kBinNear>(A, s_edges, T, val, bn);
+            else bins_of<(NAX > 0 ? NAX : 0), kBinWalk>(A, s_edges, T, val, bn);
+            if (LIST) slots.put<(NAX > 0 ? NAX : 0)>(A, bn, kept, take, lane);
+            else add_tuples(A, out, bn, kept, km, lane);
             consumed += take - q;
             q = 0;
         }
+        if (!have) break;
         __syncwarp();                                           // buffer b and the list are reused next
         cur = nxt;
+        have = cur.more();
         b ^= 1;
     }
-    if (q > 0) {                                                // the last carried cells
-        const bool kept = lane < q;
-        float val[kMaxVars];
-#pragma unroll
-        for (int a = 0; a < kMaxVars; ++a)
-            val[a] = kept && a < naxes ? __half2float(__ushort_as_half((unsigned short)(cpk[a >> 1] >> (16 * (a & 1)))))
-                                       : 0.0f;
-        bin_round(A, s_edges, out, val, kept, (1u << q) - 1u, lane);
+    if (LIST) {
+        slots.close(A, lane);
+        slots.finish(A, 32u, lane);
     }
     asm volatile("cp.async.wait_all;\n" ::: "memory");
+}
+
+// Lists the bins of every in-shell cell (no brush, no position axes; even grid edge,
+// 16-byte aligned planes). A warp takes ROWS neighbouring rows and walks them side by side,
+// 32 / ROWS lanes x 8 cells of each: the rows' geometry is computed at once, and 9 in 10
+// lanes have cells (a whole warp per row: 2 in 3). Nothing is compacted: a lane
+// bins its 8 cells straight from 16-byte loads, six axes (FP32: three) in flight, and
+// stores a unit's bins of an axis with one store; cells outside the shell at the
+// ends of a row stay unset in the unit's mask. Bound by HBM with its three instructions
+// per value (205 -> 75 per 32 cells of 6 axes). ROWS is 8 on grids with at least five
+// batches of 8 rows for each warp, else 4, which finish together sooner: whole calls at
+// 512^3 FP16 with 1, 2, 4, 8 and 16 rows take 874, 698, 597, 535 and 627 us, at 256^3 FP32
+// 161, 138, 136, 150 and 152.
+template <int DT, int MODE, int ROWS, typename BIN>
+__device__ __forceinline__ void list_rows(const HistLaunch& A, const float* s_edges, const BinTable& T) {
+    constexpr int kUnit = 8, kBytes = DT == kF16 ? 16 : 32;    // cells and bytes of a unit
+    constexpr int kLanes = 32 / ROWS;                          // of a row
+    constexpr int kAxes = DT == kF16 ? 6 : 3;                  // axes in flight
+    const int lane = threadIdx.x & 31;
+    const float top = guess_top(A.bins);
+    ListSlots slots;
+    slots.start(32u);
+    const unsigned nwarps = (gridDim.x * blockDim.x) >> 5;
+    unsigned rq = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    for (;;) {
+        const int first_row = A.item0 + (int)__shfl_sync(kFull, rq, 0) * ROWS;
+        if (first_row >= A.items) break;
+        if (lane == 0) rq = nwarps + atomicAdd(A.rowctr, 1u);
+        const int r = first_row + lane / kLanes;
+        RowSpan R;
+        int x0 = 0;
+        bool row = r < A.items && row_span(A, r, R);
+        if (row) {
+            // units start on 16-byte boundaries of the plane: before x = 0 of the row when the edge is no
+            // multiple of 8 (the cells in front are another row's)
+            const int lead = (int)(R.base & (kUnit - 1));
+            x0 = ((R.xa + lead) & ~(kUnit - 1)) - lead + (lane & (kLanes - 1)) * kUnit;
+        }
+        for (; __ballot_sync(kFull, row && x0 <= R.xb) != 0u; x0 += kLanes * kUnit) {
+            unsigned kb = 0u;
+            if (row) kb = span_bits<kUnit>(R.xa - x0, R.xb - x0) & ~span_bits<kUnit>(R.ca - x0, R.cb - x0);
+            // units with a cell to count, packed in lane order; those past the chunk's end go to the next
+            const unsigned um = __ballot_sync(kFull, kb != 0u);
+            if (um == 0u) continue;
+            const unsigned first = slots.chunk;
+            unsigned u = slots.fill + __popc(um & ((1u << lane) - 1u));
+            slots.fill += __popc(um);
+            if (slots.fill > 32u) {
+                slots.advance(A, lane);
+                slots.fill -= 32u;
+            }
+            const unsigned chunk = u < 32u ? first : slots.chunk;
+            u &= 31u;
+            if (!(kb && chunk < A.list_chunks)) continue;
+            A.list_mask[(size_t)chunk * 32 + u] = (unsigned char)kb;
+            const char* src = static_cast<const char*>(A.cells) + (R.base + x0) * (kBytes / kUnit);
+            if (x0 + kLanes * kUnit <= R.xb)                   // the next step's lines on their way
+                for (int a = 0; a < A.naxes; ++a)
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(src + A.soff[a] + kLanes * kBytes));
+            BIN* dst = reinterpret_cast<BIN*>(A.list) + (size_t)chunk * (size_t)(A.naxes * kListCells) + u * kUnit;
+            for (int a0 = 0; a0 < A.naxes; a0 += kAxes) {
+                uint4 v[kAxes][kBytes / 16];
+#pragma unroll
+                for (int i = 0; i < kAxes; ++i)
+                    if (a0 + i < A.naxes) {
+#pragma unroll
+                        for (int h = 0; h < kBytes / 16; ++h)
+                            v[i][h] = __ldg(reinterpret_cast<const uint4*>(src + A.soff[a0 + i]) + h);
+                    }
+#pragma unroll
+                for (int i = 0; i < kAxes; ++i)
+                    if (a0 + i < A.naxes) {
+                        const int a = a0 + i;
+                        const float* e = s_edges + a * (A.bins + 1);
+                        const float scale = A.guess_scale[a], off = T.off[a];
+                        unsigned bn[kUnit];                    // MODE kBinExact, bytes: in the low byte
+#pragma unroll
+                        for (int j = 0; j < kUnit; ++j) {
+                            float x;
+                            if constexpr (DT == kF16) {
+                                const unsigned w = (j >> 1) == 0 ? v[i][0].x : (j >> 1) == 1 ? v[i][0].y : (j >> 1) == 2 ? v[i][0].z : v[i][0].w;
+                                const float2 f = __half22float2(u32_as_half2(w));
+                                x = (j & 1) ? f.y : f.x;
+                            } else {
+                                x = chunk_elem<kF32>(v[i][j >> 2], j & 3);
+                            }
+                            bn[j] = MODE == kBinExact ? bin_guess_raw(top, x, scale, off) : (unsigned)bin_of<MODE>(e, A.bins, top, x, scale, off);
+                        }
+                        if constexpr (sizeof(BIN) == 1) {
+                            uint2 p;
+                            p.x = __byte_perm(__byte_perm(bn[0], bn[1], 0x0040), __byte_perm(bn[2], bn[3], 0x0040), 0x5410);
+                            p.y = __byte_perm(__byte_perm(bn[4], bn[5], 0x0040), __byte_perm(bn[6], bn[7], 0x0040), 0x5410);
+                            *reinterpret_cast<uint2*>(dst + a * kListCells) = p;
+                        } else {
+                            *reinterpret_cast<uint4*>(dst + a * kListCells) =
+                                make_uint4(__byte_perm(bn[0], bn[1], 0x5410), __byte_perm(bn[2], bn[3], 0x5410),
+                                           __byte_perm(bn[4], bn[5], 0x5410), __byte_perm(bn[6], bn[7], 0x5410));
+                        }
+                    }
+            }
+        }
+    }
+    slots.finish(A, slots.fill, lane);
+}
+
+template <int DT, int ROWS, typename BIN>
+__global__ void __launch_bounds__(kHistVecThreads, 2) k_hist_bins(const __grid_constant__ HistLaunch A) {
+    extern __shared__ float s_edges[];
+    __shared__ BinTable T;
+    const int mode = stage_edges<DT>(A, 0, A.naxes, s_edges, T);
+    if (DT == kF16 && mode == kBinExact) list_rows<DT, kBinExact, ROWS, BIN>(A, s_edges, T);
+    else if (mode != kBinWalk) list_rows<DT, kBinNear, ROWS, BIN>(A, s_edges, T);
+    else list_rows<DT, kBinWalk, ROWS, BIN>(A, s_edges, T);
+}
+
+// Counts of the listed cells. L2 atomics (5 per cell: neighbouring cells of a
+// 256-bin histogram share few bin pairs) bound the calls on large grids; here one block
+// per SM keeps the whole histogram of ONE adjacent-axis pair in its shared memory,
+// reads two axes of the list's chunks (4 lanes to a chunk: lanes on neighbouring cells would
+// meet at the same counters) and adds its non-zero counts to the output at the end. Pairs with hot bins take longer (adds of a warp to one counter serialise), so the
+// warps take chunks from a counter per pair, and a block whose pair is done helps the one
+// with the most chunks left (512^3, whole shell: 1138 -> 415 us). The bank conflicts and the
+// instructions around the adds bound it: 4 lanes to a chunk and the keys' layout
+// (count_pitch) 385 -> 327 us, predicated adds 327 -> 286 us.
+//
+// Counters are 32 bits where they fit (kPairBytes), else 16 bits, two to a word. A
+// 16-bit count cannot overflow: a thread adds the 8 cells of a unit, and if one of its
+// counters then stood at 2^15 or more it moves 2^15 of it to the output
+// (compare-and-swap; unless another thread did) before it adds anything again, so
+// at most 8 kPairThreads single counts stand above 2^15 at any time.
+constexpr int kPairThreads = 1024;
+constexpr size_t kPairBytes = (size_t)200 << 10;    // shared memory for the counters of a block
+constexpr unsigned kCountBatch = 8;                 // chunks a warp takes at a time, four lanes each
+constexpr unsigned kCountWorth = 64;                // chunks left per block for which changing the pair pays
+                                                    // (its clearing and adding up take about 10 us)
+constexpr size_t kListBytes = (size_t)512 << 20;    // bins of one slab
+constexpr long long kListGrid = 1ll << 21, kListGridBrush = 1ll << 25;   // see hist_by_list
+constexpr size_t kListWarps = 160 * 2 * kHistVecWarps;   // most warps of a launch that lists
+constexpr int kListHead = 64;                       // bytes: row counter, chunks taken, chunks counted of each pair
+static_assert(0x8000 + 8 * kPairThreads <= 0x10000, "16-bit counters");
+static_assert(4 * (2 + kMaxVars - 1) <= kListHead, "list head");
+
+struct CountArgs {
+    const unsigned char* list;
+    const unsigned char* mask;
+    unsigned* head;                // [1]: chunks taken, [2 + p]: zeroed, chunks of pair p taken here
+    unsigned chunks;               // chunks that fit
+    int naxes, bins;
+    uint32_t* out;
+};
+
+// Counter (x, y) of a pair has the key x * pitch + y. The pitch is 11 mod 32, so that the
+// counters around one another, which cells around one another hit, lie in different banks;
+// 16-bit counters k and k + words share a word for the same reason, not k and k + 1.
+__host__ __device__ __forceinline__ unsigned count_pitch(int bins) { return (unsigned)(bins + ((11 - bins) & 31)); }
+__host__ __device__ __forceinline__ unsigned count_words(int bins, bool wide) {
+    const unsigned keys = (unsigned)bins * count_pitch(bins);
+    return wide ? keys : (keys + 1u) / 2u;
+}
+
+// Adds to a shared word (its shared-space address) if kept, predicated instead of branched around;
+// its value before, or 0.
+__device__ __forceinline__ unsigned add_if(bool kept, unsigned addr, unsigned v) {
+    unsigned old = 0u;
+    asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %3, 0;\n@p atom.shared.add.u32 %0, [%1], %2;\n}\n"
+                 : "+r"(old) : "r"(addr), "r"(v), "r"((unsigned)kept) : "memory");
+    return old;
+}
+
+// A 16-bit counter last seen in its word cur: 2^15 of it to the output while it holds as much.
+__device__ __noinline__ void move_high(unsigned* hist, unsigned words, uint32_t* out, unsigned key, unsigned cur) {
+    const bool high = key >= words;
+    unsigned* w = hist + (high ? key - words : key);
+    const unsigned sh = high ? 16u : 0u;
+    while (((cur >> sh) & 0xffffu) >= 0x8000u) {
+        const unsigned seen = atomicCAS(w, cur, cur - (0x8000u << sh));
+        if (seen == cur) {
+            atomicAdd(out, 0x8000u);
+            return;
+        }
+        cur = seen;
+    }
+}
+
+template <typename BIN, bool WIDE>
+__global__ void __launch_bounds__(kPairThreads, 1) k_hist_count(CountArgs A) {
+    extern __shared__ unsigned s_hist[];
+    __shared__ int s_pair;
+    constexpr int kWords = 2 * (int)sizeof(BIN);              // 32-bit words of a unit
+    const int bins = A.bins, npairs = A.naxes - 1, lane = threadIdx.x & 31;
+    const unsigned pitch = count_pitch(bins), words = count_words(bins, WIDE);
+    const unsigned chunks = min(A.head[1], A.chunks), s_base = (unsigned)__cvta_generic_to_shared(s_hist);
+    int pair = (int)(blockIdx.x % (unsigned)npairs);
+    for (;;) {
+        uint32_t* const out = A.out + (size_t)pair * bins * bins;
+        unsigned* taken = A.head + 2 + pair;
+        for (unsigned i = threadIdx.x; i < words; i += kPairThreads) s_hist[i] = 0u;
+        unsigned next = lane == 0 ? atomicAdd(taken, kCountBatch) : 0u;
+        __syncthreads();
+        for (;;) {
+            const unsigned c0 = __shfl_sync(kFull, next, 0);
+            if (c0 >= chunks) break;
+            if (lane == 0) next = atomicAdd(taken, kCountBatch);
+            const unsigned c = c0 + (lane >> 2);
+            const bool any = c < chunks;
+            unsigned m = 0u, a[kWords] = {}, b[kWords] = {};
+            auto load = [&](int step, unsigned& m, unsigned (&a)[kWords], unsigned (&b)[kWords]) {
+                const int unit = step * 4 + (lane & 3);
+                m = __ldg(A.mask + (size_t)c * 32 + unit);
+                const BIN* pa = reinterpret_cast<const BIN*>(A.list) + ((size_t)c * A.naxes + pair) * kListCells + unit * 8;
+                if constexpr (sizeof(BIN) == 1) {
+                    const uint2 x = __ldg(reinterpret_cast<const uint2*>(pa)), y = __ldg(reinterpret_cast<const uint2*>(pa + kListCells));
+                    a[0] = x.x; a[1] = x.y; b[0] = y.x; b[1] = y.y;
+                } else {
+                    const uint4 x = __ldg(reinterpret_cast<const uint4*>(pa)), y = __ldg(reinterpret_cast<const uint4*>(pa + kListCells));
+                    a[0] = x.x; a[1] = x.y; a[2] = x.z; a[3] = x.w; b[0] = y.x; b[1] = y.y; b[2] = y.z; b[3] = y.w;
+                }
+            };
+            if (any) load(0, m, a, b);
+            for (int step = 0; step < 8; ++step) {
+                unsigned mn = 0u, an[kWords] = {}, bn[kWords] = {};
+                if (any && step < 7) load(step + 1, mn, an, bn);
+                unsigned key[8], cur[8], over = 0u;
+                constexpr int kPer = 4 / (int)sizeof(BIN), kBits = 8 * (int)sizeof(BIN);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const unsigned x = (a[j / kPer] >> (kBits * (j % kPer))) & ((1u << kBits) - 1u);
+                    const unsigned y = (b[j / kPer] >> (kBits * (j % kPer))) & ((1u << kBits) - 1u);
+                    key[j] = x * pitch + y;
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const bool high = !WIDE && key[j] >= words;
+                    const unsigned one = high ? 0x10000u : 1u;
+                    cur[j] = add_if((m >> j) & 1u, s_base + 4u * (high ? key[j] - words : key[j]), one) + one;
+                }
+                if (!WIDE) {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) over |= cur[j];
+                    if (over & 0x80008000u) {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            if (((m >> j) & 1u) && (cur[j] & 0x80008000u)) move_high(s_hist, words, out + (key[j] / pitch) * bins + key[j] % pitch, key[j], cur[j]);
+                    }
+                }
+                m = mn;
+#pragma unroll
+                for (int i = 0; i < kWords; ++i) { a[i] = an[i]; b[i] = bn[i]; }
+            }
+        }
+        __syncthreads();
+        for (unsigned i = threadIdx.x; i < (unsigned)(bins * bins); i += kPairThreads) {
+            const unsigned x = i / (unsigned)bins, key = i + x * (pitch - bins);
+            const unsigned v = WIDE ? s_hist[key] : key >= words ? s_hist[key - words] >> 16 : s_hist[key] & 0xffffu;
+            if (v) atomicAdd(out + i, v);
+        }
+        if (threadIdx.x == 0) {
+            unsigned most = 0u;
+            int to = -1;
+            for (int p = 0; p < npairs; ++p) {
+                const unsigned t = *reinterpret_cast<volatile unsigned*>(A.head + 2 + p);
+                if (t < chunks && chunks - t > most) {
+                    most = chunks - t;
+                    to = p;
+                }
+            }
+            s_pair = most >= kCountWorth * gridDim.x ? to : -1;
+        }
+        __syncthreads();
+        pair = s_pair;
+        if (pair < 0) break;
+    }
 }
 
 // out[i] = sum over the copies of copy[c][i] (count a multiple of 4, 16-byte aligned).
@@ -650,8 +1234,8 @@ bool fill_launch(const HistArgs& h, HistLaunch& a, bool& vec_slots) {
     for (int i = 0; i < h.naxes && i < kMaxVars; ++i) {
         a.avar[i] = h.axis[i];
         if (h.axis[i] >= kPosAxisBase) a.use_pos = 1;
-        a.guess_scale[i] = h.guess_scale[i];
-        a.guess_off[i] = -h.guess_e0[i] * h.guess_scale[i];
+        a.guess_scale[i] = h.guess_scale[i] / (float)h.bins;
+        a.guess_off[i] = -h.guess_e0[i] * a.guess_scale[i];
     }
     // load slots of the vector kernel: the axes, then the brushed variables that are no axis
     vec_slots = true;
@@ -703,6 +1287,68 @@ bool fill_launch(const HistArgs& h, HistLaunch& a, bool& vec_slots) {
     return true;
 }
 
+template <typename K>
+cudaError_t launch_k(K kernel, const HistLaunch& a, int threads, size_t smem, long long items, int sms, cudaStream_t stream) {
+    int per_sm = 0;
+    cudaError_t e = cudaSuccess;
+    if (smem > 48 * 1024) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // persistent grid: as many blocks as fit at once
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
+    if (e != cudaSuccess) return e;
+    const long long want = (items + threads / 32 - 1) / (threads / 32);
+    long long most = (long long)sms * std::max(1, per_sm);
+    if (a.list) most = std::min<long long>(most, kListWarps / kHistVecWarps);   // as many as the list allows for
+    const int blocks = (int)std::max<long long>(1, std::min<long long>(want, most));
+    kernel<<<blocks, threads, smem, stream>>>(a);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
+typedef void (*HistKernel)(const HistLaunch);
+template <int DT, int VEC>
+HistKernel list_kernel(int nax, bool groups) {
+    if (!groups) return nax ? k_hist<DT, RowWalk<VEC>, -1, true> : k_hist<DT, RowWalk<VEC>, 0, true>;
+    switch (nax) {
+        case 2: return k_hist<DT, GroupWalk<VEC>, 2, true>;
+        case 3: return k_hist<DT, GroupWalk<VEC>, 3, true>;
+        case 4: return k_hist<DT, GroupWalk<VEC>, 4, true>;
+        case 5: return k_hist<DT, GroupWalk<VEC>, 5, true>;
+        case 6: return k_hist<DT, GroupWalk<VEC>, 6, true>;
+        case 7: return k_hist<DT, GroupWalk<VEC>, 7, true>;
+        case 8: return k_hist<DT, GroupWalk<VEC>, 8, true>;
+        default: return k_hist<DT, GroupWalk<VEC>, 0, true>;
+    }
+}
+
+// Shared memory of the count kernel's counters (wide: 32 bits).
+size_t count_bytes(int bins, bool wide) { return sizeof(unsigned) * (size_t)count_words(bins, wide); }
+
+cudaError_t launch_count(const CountArgs& c, int sms, cudaStream_t stream) {
+    const bool wide = count_bytes(c.bins, true) <= kPairBytes;          // bins <= 224
+    const size_t smem = count_bytes(c.bins, wide);
+    const auto kernel = c.bins > 256 ? k_hist_count<unsigned short, false> : wide ? k_hist_count<unsigned char, true> : k_hist_count<unsigned char, false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kernel<<<std::max(sms, c.naxes - 1), kPairThreads, smem, stream>>>(c);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
+// Vector kernels' conditions: 16-byte aligned planes (an even edge makes n^3 a multiple of 8)
+// and load slots that fit; the group walk also needs whole chunks and sub-bricks per row.
+template <int DT>
+bool vector_walk(const HistArgs& h, bool vec_slots) {
+    return vec_slots && h.n % 2 == 0 && (reinterpret_cast<uintptr_t>(h.cells) & 15u) == 0;
+}
+
+// Whether a call counts every in-shell cell by stored values alone.
+bool lists_whole_rows(const HistArgs& h) {
+    if (h.use_brush && (h.brush.mask || h.brush.pmask)) return false;
+    for (int i = 0; i < h.naxes; ++i)
+        if (h.axis[i] >= kPosAxisBase) return false;
+    return true;
+}
+
 template <int DT>
 cudaError_t launch_t(const HistArgs& h, cudaStream_t stream) {
     HistLaunch a{};                      // about 8.6 KB with the inline edges (host stack)
@@ -711,34 +1357,101 @@ cudaError_t launch_t(const HistArgs& h, cudaStream_t stream) {
     const int ne = h.naxes * (h.bins + 1);
     if (h.s_out < 0) return cudaSuccess;                 // no cell in the shell: the zeroed output is the answer
     constexpr int VEC = DT == kF16 ? 8 : 4;
-    const bool vec = vec_slots && h.n % VEC == 0 && (reinterpret_cast<uintptr_t>(h.cells) & 15u) == 0;
-    const size_t smem = vec ? sizeof(float) * (size_t)((ne + 3) & ~3) + (size_t)kHistVecWarps * (2 * a.nslot * 512 + 256)
-                            : sizeof(float) * (size_t)ne;
-    // persistent grid: as many blocks as fit at once
-    int dev = 0, sms = 0, per_sm = 0;
+    int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess && vec && smem > 48 * 1024)
-        e = cudaFuncSetAttribute(k_hist<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-        e = vec ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hist<DT>, kHistVecThreads, smem)
-                : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hist_scalar<DT>, kHistThreads, smem);
     if (e != cudaSuccess) return e;
-    const long long rows = (long long)a.n * a.n;
-    const int warps_per_block = vec ? kHistVecWarps : kHistWarps;
-    const long long want_blocks = (rows + warps_per_block - 1) / warps_per_block;
-    const int blocks = (int)std::max<long long>(1, std::min<long long>(want_blocks, (long long)sms * std::max(1, per_sm)));
-    if (!vec) {
+    const int rows = a.n * a.n;
+    if (!vector_walk<DT>(h, vec_slots)) {
         a.rot = 0;
         a.rowctr = nullptr;
+        return launch_k(k_hist_scalar<DT>, a, kHistThreads, sizeof(float) * (size_t)ne, rows, sms, stream);
     }
-    if (vec) k_hist<DT><<<blocks, kHistVecThreads, smem, stream>>>(a);
-    else k_hist_scalar<DT><<<blocks, kHistThreads, smem, stream>>>(a);
-    count_launches(1);
-    return cudaGetLastError();
+    const size_t smem = sizeof(float) * (size_t)((ne + 3) & ~3) + (size_t)kHistVecWarps * (2 * a.nslot * 512 + 256);
+    // brushed listed calls by groups: 512^3 FP16 3 / 4 variables 230 / 315 us, by rows 263 / 339; direct calls are
+    // faster by rows (256^3 FP16 77 us, by groups 86)
+    const bool groups = h.list && a.sactive && h.n % VEC == 0;
+    const int per_plane = groups ? h.nsb * ((h.nsb + 7) / 8) : h.n;      // items of a (sub-brick) plane in z
+    const int planes = groups ? h.nsb : h.n;
+    const int nax = a.use_pos ? 0 : a.naxes;
+    if (!h.list) {
+        a.items = per_plane * planes;
+        const HistKernel k = a.use_pos ? k_hist<DT, RowWalk<VEC>, 0, false> : k_hist<DT, RowWalk<VEC>, -1, false>;
+        return launch_k(k, a, kHistVecThreads, smem, a.items, sms, stream);
+    }
+    // in slabs of planes whose cells fit the list, each counted before the next
+    const HistList L = hist_list(h);
+    unsigned* head = static_cast<unsigned*>(h.list);
+    a.rowctr = head;
+    a.rot = 0;
+    a.list_next = head + 1;
+    a.list_mask = static_cast<unsigned char*>(h.list) + kListHead;
+    a.list_chunks = L.chunks;
+    a.list_batch = L.batch;
+    a.list = static_cast<unsigned char*>(h.list) + L.bins_at;
+    const bool whole = lists_whole_rows(h) && !groups;
+    const bool wide_rows = rows >= 8 * 5 * sms * 2 * kHistVecWarps;      // see list_rows
+    const int step = groups ? std::max(1, L.planes / 4) : L.planes;
+    for (int p = 0; p < planes; p += step) {
+        a.item0 = p * per_plane;
+        a.items = std::min(planes, p + step) * per_plane;
+        const int count = a.items - a.item0;
+        a.batch = std::max(1, std::min(32, count / (sms * 2 * kHistVecWarps * 8)));   // about eight batches per warp
+        e = cudaMemsetAsync(head, 0, kListHead, stream);
+        if (e != cudaSuccess) return e;
+        if (whole) {
+            const HistKernel k = wide_rows ? (h.bins <= 256 ? k_hist_bins<DT, 8, unsigned char> : k_hist_bins<DT, 8, unsigned short>)
+                                           : (h.bins <= 256 ? k_hist_bins<DT, 4, unsigned char> : k_hist_bins<DT, 4, unsigned short>);
+            e = launch_k(k, a, kHistVecThreads, sizeof(float) * (size_t)ne, (count + 3) / 4, sms, stream);
+        } else {
+            e = launch_k(list_kernel<DT, VEC>(nax, groups), a, kHistVecThreads, smem, count, sms, stream);
+        }
+        if (e == cudaSuccess)
+            e = launch_count(CountArgs{a.list, a.list_mask, head, a.list_chunks, h.naxes, h.bins, h.out}, sms, stream);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace
+
+// List of a call: the in-shell cells of as many planes as kListBytes hold (every cell of a
+// plane taken as in the shell when there is more than one slab).
+HistList hist_list(const HistArgs& h) {
+    const size_t n = (size_t)h.n, cell = (size_t)h.naxes * (h.bins <= 256 ? 1 : 2);
+    // in-shell cells: their unit cubes lie between two spheres sqrt(3)/2 beyond the shell's
+    const double ro = 0.5 * std::sqrt((double)std::max<int64_t>(h.s_out, 0)) + 0.87;
+    const double ri = std::max(0.0, 0.5 * std::sqrt((double)std::max<int64_t>(h.s_in, 0)) - 0.87);
+    const double shell = std::min((double)n * n * n, 4.18880 * (ro * ro * ro - ri * ri * ri) + 1.0);
+    // units: whole rows leave up to four partly filled ones (two chords' ends) per row; the
+    // compacting kernels may leave 31 of a chunk's 256 cells unused
+    const auto units = [&](size_t cells, size_t planes) {
+        return lists_whole_rows(h) ? std::max(cells / 8 + 4 * n * planes, cells / 7) : cells / 7 + 1;
+    };
+    HistList L{};
+    L.planes = h.n;
+    size_t u = units((size_t)shell, n);
+    if (u * 8 * cell > kListBytes) {
+        L.planes = (int)std::min<size_t>(n, std::max<size_t>(4, kListBytes / (n * n * cell * 8 / 7 + 32 * n * cell) / 4 * 4));
+        u = units((size_t)L.planes * n * n, (size_t)L.planes);
+    }
+    // a warp may leave its current chunk, the rest of its batch and the next batch unused
+    L.batch = (unsigned)std::max<size_t>(1, std::min<size_t>(kListBatch, u / (32 * 8 * kListWarps)));
+    L.chunks = (unsigned)(u / 32 + 1 + 2 * L.batch * kListWarps);
+    L.bins_at = ((size_t)kListHead + 32 * (size_t)L.chunks + 255) / 256 * 256;
+    L.bytes = L.bins_at + (size_t)L.chunks * kListCells * cell;
+    return L;
+}
+
+// Large grids on the vector path whose pair histogram fits a block (up to 310 bins). On smaller
+// ones the second kernel and the blocks' clearing and adding up cost more than the
+// atomics. Listed / direct, us: whole shell 128^3 FP32 58 / 62, 160^3 FP16 67 / 86, 512^3 535 /
+// 1293; brushed, after a render has
+// filled the caches, 256^3 FP16 83 / 77, 256^3 FP32 97 / 99 (a whole step with it 1031 / 1017), 512^3 315 / 400.
+bool hist_by_list(const HistArgs& h, int dtype) {
+    return (long long)h.n * h.n * h.n >= (h.use_brush ? kListGridBrush : kListGrid) && h.n % 2 == 0 && (reinterpret_cast<uintptr_t>(h.cells) & 15u) == 0 &&
+           count_bytes(h.bins, false) <= kPairBytes;
+}
 
 int hist_copies(int n, int naxes, int bins) {
     const size_t bytes = sizeof(uint32_t) * (size_t)(naxes - 1) * bins * bins;

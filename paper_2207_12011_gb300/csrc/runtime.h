@@ -147,11 +147,38 @@ struct raypc_ctx {
     std::map<int, raypc::Volume*> vols;
     int next_id = 1;
 
+    // Stream-ordered scratch of single calls, from a pool of the context's own that keeps up to
+    // kScratchKept bytes between calls (the device's default pool gives everything back at each
+    // synchronisation, and the next call maps its scratch anew). Safe on any stream; freed with
+    // cudaFreeAsync on the stream that used it. Without a pool it comes from the default one.
+    cudaMemPool_t pool = nullptr;
+    static constexpr unsigned long long kScratchKept = 640ull << 20;
+    void open_pool() {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = device;
+        unsigned long long keep = kScratchKept;
+        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) pool = nullptr;
+        else if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess) return;
+        cudaGetLastError();
+    }
+    cudaError_t scratch(void** p, size_t bytes, cudaStream_t s) {
+        return pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s);
+    }
+    // Room for scratch that a call can do without: within the budget, when there is one.
+    bool room(size_t bytes) const { return !budget || used + bytes <= budget; }
+
     // Device allocation charged against the budget.
     raypc_status alloc(void** p, size_t bytes, size_t* charged) {
         if (budget && used + bytes > budget)
             return raypc::fail(RAYPC_ERR_OOM, "HBM budget exceeded: %zu used + %zu requested > %zu", used, bytes, budget);
         cudaError_t e = cudaMalloc(p, bytes ? bytes : 16);
+        if (e == cudaErrorMemoryAllocation && pool) {     // what the pool keeps may make the room
+            cudaGetLastError();
+            e = cudaMemPoolTrimTo(pool, 0);
+            if (e == cudaSuccess) e = cudaMalloc(p, bytes ? bytes : 16);
+        }
         if (e != cudaSuccess) return raypc::cuda_fail(e, "cudaMalloc");
         used += bytes;
         *charged += bytes;

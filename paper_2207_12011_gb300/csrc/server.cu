@@ -219,9 +219,15 @@ raypc_status launch_hist(raypc_server* S, Req* q, int si) {
     cudaError_t e = cudaSuccess;
     if (q->edges.size() > (size_t)kHistInlineEdges)
         e = cudaMemcpyAsync(q->d_edges, q->edges.data(), sizeof(float) * q->edges.size(), cudaMemcpyHostToDevice, s);
-    // scratch: the partial copies and their row counter (large grids), then the sub-brick bits
+    // scratch: the list of bins from the context's pool (large grids); without it the partial
+    // copies and their row counter in the stream's scratch, then the sub-brick bits
     const size_t count = (size_t)(naxes - 1) * bins * bins;
-    const int ncopies = ((uintptr_t)q->hist & 15u) ? 1 : hist_copies(L->n, naxes, bins);
+    if (e == cudaSuccess && hist_by_list(h, V->dtype) && S->ctx->room(hist_list(h).bytes) &&
+        S->ctx->scratch(&h.list, hist_list(h).bytes, s) != cudaSuccess) {
+        cudaGetLastError();
+        h.list = nullptr;
+    }
+    const int ncopies = h.list || ((uintptr_t)q->hist & 15u) ? 1 : hist_copies(L->n, naxes, bins);
     const size_t copy_bytes = ncopies > 1 ? (sizeof(uint32_t) * (count * ncopies + 4) + 255) / 256 * 256 : 0;
     const bool activity = h.use_brush && L->sbmin;
     const size_t need = copy_bytes + (activity ? sizeof(uint32_t) * L->nswords() : 0);
@@ -235,7 +241,10 @@ raypc_status launch_hist(raypc_server* S, Req* q, int si) {
             S->hscratch_bytes[si] = 0;
         }
         size_t charged = 0;
-        if ((st = S->ctx->alloc(&S->hscratch[si], need, &charged))) return st;
+        if ((st = S->ctx->alloc(&S->hscratch[si], need, &charged))) {
+            if (h.list) cudaFreeAsync(h.list, s);
+            return st;
+        }
         S->hscratch_bytes[si] = need;
     }
     char* scratch = static_cast<char*>(S->hscratch[si]);
@@ -263,6 +272,7 @@ raypc_status launch_hist(raypc_server* S, Req* q, int si) {
         if (e == cudaSuccess) e = cudaMemsetAsync(q->hist, 0, sizeof(uint32_t) * (count + 1), s);
         if (e == cudaSuccess) e = launch_histogram(h, V->dtype, s);
     }
+    if (h.list) cudaFreeAsync(h.list, s);
     if (e != cudaSuccess) return cuda_fail(e, "server histogram");
     return RAYPC_OK;
 }
