@@ -55,12 +55,16 @@ inline unsigned long long count_in_shell(int n, int64_t s_in, int64_t s_out) {
         const int64_t xa = std::max<int64_t>(0, (n - m) / 2), xb = std::min<int64_t>(n - 1, (n - 1 + m) / 2);
         return xb >= xa ? xb - xa + 1 : 0;
     };
+    // rows of one eighth of the (y, z) plane stand for their mirror images (256^3: 65536 -> 8256 rows,
+    // a third of the host's time for a subsample of 100 000 lines)
     unsigned long long total = 0;
-    for (int z = 0; z < n; ++z)
-        for (int y = 0; y < n; ++y) {
+    for (int z = n / 2; z < n; ++z)
+        for (int y = n / 2; y <= z; ++y) {
             const int64_t dy = 2 * y + 1 - n, dz = 2 * z + 1 - n, syz = dy * dy + dz * dz;
             const int64_t row = upto(s_out - syz) - upto(s_in - 1 - syz);   // <= 0 when s_in > s_out
-            total += row > 0 ? (unsigned long long)row : 0ull;
+            if (row <= 0) continue;
+            const int images = (dy ? 2 : 1) * (dz ? 2 : 1) * (y < z ? 2 : 1);
+            total += (unsigned long long)row * (unsigned long long)images;
         }
     return total;
 }

@@ -17,7 +17,15 @@
 // return at once. An ordered compaction follows: warps own contiguous row
 // segments, count their selected cells, one block scans the counts, and each
 // warp writes its cells' indices in cell order from its segment's offset; one
-// thread per line then gathers the line's axis values and brush flag.
+// thread per line then gathers the line's axis values and brush flag. The block that
+// finishes a round last picks its digit, and the one that counts last scans.
+//
+// The four passes over the cells are bound by instructions (a key is some 40 of them), and were by
+// the rows' 64-bit divisions and square-root corrections and by a thousand blocks' tables
+// of digits added to L2: 256^3, 100 000 lines 223 -> 197 us of kernels in 11 launches
+// instead of 18, the call with its filter 337 -> 222 us.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace raypc {
@@ -28,30 +36,33 @@ constexpr int kDigitBits = 12;
 constexpr int kDigits = 1 << kDigitBits;
 constexpr int kRounds = 6;             // 6 x 12 >= 64 bits
 constexpr int kSubThreads = 256;
+constexpr int kSubBlocks = 304;        // two per SM
+constexpr int kSubWide = 1024;         // rounds and counts: fewer blocks with a table of digits each
 
 struct SubState {
     unsigned long long prefix;         // resolved top bits of the m-th smallest key
     unsigned long long need;           // cells still to take among keys sharing the prefix
     int nbits;                         // resolved bits, 0..64
     int done;                          // selection final: top nbits bits <= prefix (nbits 0: all)
+    unsigned ticket;                   // blocks of the running kernel that have finished
     unsigned long long hist[kDigits];
     unsigned seg_cnt[kSubMaxSegments];   // selected cells per compaction segment
     unsigned seg_off[kSubMaxSegments];   // their exclusive prefix sums
 };
 
-// Largest integer m >= 0 with m * m <= a (0 <= a < 2^31).
+// Largest integer m >= 0 with m * m <= a (0 <= a < 2^31; m + 1 <= 46341, so the squares fit 32 bits).
 __device__ __forceinline__ int isqrt_floor_dev(int a) {
-    int m = (int)sqrtf((float)a);
-    while ((long long)m * m > a) --m;
-    while ((long long)(m + 1) * (m + 1) <= a) ++m;
-    return m;
+    unsigned m = (unsigned)__fsqrt_rn((float)a);           // at most one off
+    if (m * m > (unsigned)a) --m;
+    if ((m + 1u) * (m + 1u) <= (unsigned)a) ++m;
+    return (int)m;
 }
 
-// x range [xa, xb] of row (y, z) whose cells can lie inside the outer sphere;
-// false if none can. syz = dy^2 + dz^2 of the row.
-__device__ __forceinline__ bool row_range(const SubsampleArgs& A, long long r, int& xa, int& xb, int& syz) {
+// x range [xa, xb] of row r = z * n + y (32 bits: n < 46340) whose cells can lie inside the outer
+// sphere; false if none can. syz = dy^2 + dz^2 of the row.
+__device__ __forceinline__ bool row_range(const SubsampleArgs& A, int r, int& xa, int& xb, int& syz) {
     const int n = A.n;
-    const int y = (int)(r % n), z = (int)(r / n);
+    const int z = r / n, y = r - z * n;
     const int dy = 2 * y + 1 - n, dz = 2 * z + 1 - n;
     syz = dy * dy + dz * dz;
     if (syz > A.s_out) return false;
@@ -59,6 +70,21 @@ __device__ __forceinline__ bool row_range(const SubsampleArgs& A, long long r, i
     xa = max(0, (n - m) / 2);
     xb = min(n - 1, (n - 1 + m) / 2);
     return xa <= xb;
+}
+
+// Whether this block is the last of the launch to get here, with the other blocks' writes visible to
+// it (all threads call it; the ticket is left at zero for the next kernel).
+__device__ __forceinline__ bool last_block(SubState* S) {
+    __shared__ bool s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s_last = atomicAdd(&S->ticket, 1u) == gridDim.x - 1u;
+        if (s_last) S->ticket = 0u;
+    }
+    __syncthreads();
+    if (s_last) __threadfence();
+    return s_last;
 }
 
 __device__ __forceinline__ bool in_shell(const SubsampleArgs& A, int x, int syz) {
@@ -78,54 +104,23 @@ __global__ void k_sub_init(SubState* S, unsigned long long m, int all) {
         S->need = m;
         S->nbits = 0;
         S->done = all;
+        S->ticket = 0u;
     }
 }
 
-// One round: histogram of the next digit of the keys that share the prefix.
-__global__ void __launch_bounds__(kSubThreads) k_sub_hist(SubsampleArgs A, SubState* S) {
-    __shared__ unsigned h[kDigits];
-    if (S->done) return;
-    const int nbits = S->nbits;
-    const unsigned long long prefix = S->prefix;
-    const int width = min(kDigitBits, 64 - nbits);
-    const int shift = 64 - nbits - width;
-    const unsigned dmask = (1u << width) - 1u;
-    for (int i = threadIdx.x; i < kDigits; i += blockDim.x) h[i] = 0u;
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    const long long rows = (long long)A.n * A.n;
-    const long long gwarp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long r = gwarp; r < rows; r += nwarps) {
-        int xa, xb, syz;
-        if (!row_range(A, r, xa, xb, syz)) continue;
-        for (int x = xa + lane; x <= xb; x += 32) {
-            if (!in_shell(A, x, syz)) continue;
-            const unsigned long long key = splitmix64_at(A.key, (unsigned long long)r * A.n + x);
-            if (nbits != 0 && (key >> (64 - nbits)) != prefix) continue;
-            atomicAdd(&h[(unsigned)(key >> shift) & dmask], 1u);
-        }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < kDigits; i += blockDim.x)
-        if (h[i]) atomicAdd(&S->hist[i], (unsigned long long)h[i]);
-}
-
-// One block of 1024 threads: the digit whose bucket holds the next needed key.
-__global__ void __launch_bounds__(1024) k_sub_pick(SubState* S) {
-    __shared__ unsigned long long s_sum[1024];
-    if (S->done) return;
-    constexpr int kPer = kDigits / 1024;
+// The digit whose bucket holds the next needed key (one block; width: bits of the digit).
+__device__ __forceinline__ void pick_digit(SubState* S, int width) {
+    __shared__ unsigned long long s_sum[kSubWide];
+    constexpr int kPer = kDigits / kSubWide;
     const int t = threadIdx.x;
     // the state is read before the first barrier: the owner thread rewrites it after the last one
-    const int width = min(kDigitBits, 64 - S->nbits);
     const unsigned long long need = S->need;
     unsigned long long loc[kPer], tot = 0ull;
 #pragma unroll
-    for (int i = 0; i < kPer; ++i) { loc[i] = S->hist[t * kPer + i]; tot += loc[i]; }
+    for (int i = 0; i < kPer; ++i) { loc[i] = __ldcg(&S->hist[t * kPer + i]); tot += loc[i]; }
     s_sum[t] = tot;
     __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
+    for (int off = 1; off < kSubWide; off <<= 1) {
         const unsigned long long add = t >= off ? s_sum[t - off] : 0ull;
         __syncthreads();
         s_sum[t] += add;
@@ -147,54 +142,80 @@ __global__ void __launch_bounds__(1024) k_sub_pick(SubState* S) {
             before += loc[i];
         }
     }
-    __syncthreads();
 #pragma unroll
     for (int i = 0; i < kPer; ++i) S->hist[t * kPer + i] = 0ull;
 }
 
+// One round: histogram of the next digit of the keys that share the prefix, and the digit.
+__global__ void __launch_bounds__(kSubWide) k_sub_round(SubsampleArgs A, SubState* S) {
+    __shared__ unsigned h[kDigits];
+    if (S->done) return;                                       // set by an earlier launch: the same in all blocks
+    const int nbits = S->nbits;
+    const unsigned long long prefix = S->prefix;
+    const int width = min(kDigitBits, 64 - nbits);
+    const int shift = 64 - nbits - width;
+    const unsigned dmask = (1u << width) - 1u;
+    for (int i = threadIdx.x; i < kDigits; i += kSubWide) h[i] = 0u;
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const int rows = A.n * A.n;
+    const int nwarps = (int)((gridDim.x * blockDim.x) >> 5);
+    for (int r = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); r < rows; r += nwarps) {
+        int xa, xb, syz;
+        if (!row_range(A, r, xa, xb, syz)) continue;
+        for (int x = xa + lane; x <= xb; x += 32) {
+            if (!in_shell(A, x, syz)) continue;
+            const unsigned long long key = splitmix64_at(A.key, (unsigned long long)r * A.n + x);
+            if (nbits != 0 && (key >> (64 - nbits)) != prefix) continue;
+            atomicAdd(&h[(unsigned)(key >> shift) & dmask], 1u);
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kDigits; i += kSubWide)
+        if (h[i]) atomicAdd(&S->hist[i], (unsigned long long)h[i]);
+    if (last_block(S)) pick_digit(S, width);
+}
+
 // Rows [r0, r1) of compaction segment g (one warp per segment, segments in row order).
-__device__ __forceinline__ void segment_rows(const SubsampleArgs& A, long long g, int nseg, long long& r0, long long& r1) {
-    const long long rows = (long long)A.n * A.n;
-    const long long per = (rows + nseg - 1) / nseg;
-    r0 = min(rows, g * per);
+__device__ __forceinline__ void segment_rows(const SubsampleArgs& A, int g, int nseg, int& r0, int& r1) {
+    const int rows = A.n * A.n;
+    const int per = (rows + nseg - 1) / nseg;
+    r0 = min(rows, g * per);                                   // g * per < rows + nseg * 2
     r1 = min(rows, r0 + per);
 }
 
-__global__ void __launch_bounds__(kSubThreads) k_sub_count(SubsampleArgs A, SubState* S, int nseg) {
-    const long long g = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (g >= nseg) return;                                     // whole warps
-    const int lane = threadIdx.x & 31;
-    const int nbits = S->nbits;
-    const unsigned long long prefix = S->prefix;
-    long long r0, r1;
-    segment_rows(A, g, nseg, r0, r1);
-    unsigned cnt = 0;
-    for (long long r = r0; r < r1; ++r) {
-        int xa, xb, syz;
-        if (!row_range(A, r, xa, xb, syz)) continue;
-        for (int x = xa + lane; x <= xb; x += 32)
-            if (in_shell(A, x, syz) && selected(splitmix64_at(A.key, (unsigned long long)r * A.n + x), nbits, prefix))
-                ++cnt;
+// Selected cells of each segment, and their exclusive prefix sums (m < 2^31).
+__global__ void __launch_bounds__(kSubWide) k_sub_count(SubsampleArgs A, SubState* S, int nseg) {
+    __shared__ unsigned s_sum[kSubWide];
+    const int g = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (g < nseg) {                                            // whole warps
+        const int nbits = S->nbits;
+        const unsigned long long prefix = S->prefix;
+        int r0, r1;
+        segment_rows(A, g, nseg, r0, r1);
+        unsigned cnt = 0;
+        for (int r = r0; r < r1; ++r) {
+            int xa, xb, syz;
+            if (!row_range(A, r, xa, xb, syz)) continue;
+            for (int x = xa + lane; x <= xb; x += 32)
+                if (in_shell(A, x, syz) && selected(splitmix64_at(A.key, (unsigned long long)r * A.n + x), nbits, prefix))
+                    ++cnt;
+        }
+        cnt = __reduce_add_sync(0xffffffffu, cnt);
+        if (lane == 0) S->seg_cnt[g] = cnt;
     }
-    cnt = __reduce_add_sync(0xffffffffu, cnt);
-    if (lane == 0) S->seg_cnt[g] = cnt;
-}
-
-// One block of 1024 threads: exclusive scan of the segment counts (m < 2^31).
-__global__ void __launch_bounds__(1024) k_sub_scan(SubState* S, int nseg) {
-    __shared__ unsigned s_sum[1024];
-    constexpr int kPer = kSubMaxSegments / 1024;
+    if (!last_block(S)) return;
+    constexpr int kPer = kSubMaxSegments / kSubWide;
     const int t = threadIdx.x;
     unsigned loc[kPer], tot = 0u;
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {
-        const int g = t * kPer + i;
-        loc[i] = g < nseg ? S->seg_cnt[g] : 0u;
+        loc[i] = t * kPer + i < nseg ? __ldcg(&S->seg_cnt[t * kPer + i]) : 0u;
         tot += loc[i];
     }
     s_sum[t] = tot;
     __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
+    for (int off = 1; off < kSubWide; off <<= 1) {
         const unsigned add = t >= off ? s_sum[t - off] : 0u;
         __syncthreads();
         s_sum[t] += add;
@@ -203,23 +224,22 @@ __global__ void __launch_bounds__(1024) k_sub_scan(SubState* S, int nseg) {
     unsigned run = s_sum[t] - tot;
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {
-        const int g = t * kPer + i;
-        if (g < nseg) S->seg_off[g] = run;
+        if (t * kPer + i < nseg) S->seg_off[t * kPer + i] = run;
         run += loc[i];
     }
 }
 
 __global__ void __launch_bounds__(kSubThreads) k_sub_write(SubsampleArgs A, SubState* S, int nseg) {
-    const long long g = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int g = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (g >= nseg) return;                                     // whole warps
     const int lane = threadIdx.x & 31;
     const int nbits = S->nbits;
     const unsigned long long prefix = S->prefix;
     unsigned long long base = S->seg_off[g];
-    long long r0, r1;
+    int r0, r1;
     segment_rows(A, g, nseg, r0, r1);
     const int n = A.n;
-    for (long long r = r0; r < r1; ++r) {
+    for (int r = r0; r < r1; ++r) {
         int xa, xb, syz;
         if (!row_range(A, r, xa, xb, syz)) continue;        // uniform over the warp
         for (int x0 = xa; x0 <= xb; x0 += 32) {
@@ -273,24 +293,18 @@ cudaError_t launch_pc_subsample(const SubsampleArgs& a, int dtype, unsigned long
     SubState* S = reinterpret_cast<SubState*>(scratch);
     if (m == 0) return cudaSuccess;
     k_sub_init<<<1, 1024, 0, stream>>>(S, m, m >= N ? 1 : 0);
-    const long long rows = (long long)a.n * a.n;
-    const long long want = (rows + (kSubThreads / 32) - 1) / (kSubThreads / 32);
-    const int hist_blocks = (int)(want < 1024 ? want : 1024);
-    for (int round = 0; round < kRounds; ++round) {
-        k_sub_hist<<<hist_blocks, kSubThreads, 0, stream>>>(a, S);
-        k_sub_pick<<<1, 1024, 0, stream>>>(S);
-    }
-    const int nseg = (int)(rows < kSubMaxSegments ? rows : kSubMaxSegments);
-    const int seg_blocks = (nseg + kSubThreads / 32 - 1) / (kSubThreads / 32);
-    k_sub_count<<<seg_blocks, kSubThreads, 0, stream>>>(a, S, nseg);
-    k_sub_scan<<<1, 1024, 0, stream>>>(S, nseg);
-    k_sub_write<<<seg_blocks, kSubThreads, 0, stream>>>(a, S, nseg);
+    const int rows = a.n * a.n;
+    const int round_blocks = std::min((rows + kSubWide / 32 - 1) / (kSubWide / 32), kSubBlocks);
+    for (int round = 0; round < kRounds; ++round) k_sub_round<<<round_blocks, kSubWide, 0, stream>>>(a, S);
+    const int nseg = std::min(rows, kSubMaxSegments);
+    k_sub_count<<<(nseg + kSubWide / 32 - 1) / (kSubWide / 32), kSubWide, 0, stream>>>(a, S, nseg);
+    k_sub_write<<<(nseg + kSubThreads / 32 - 1) / (kSubThreads / 32), kSubThreads, 0, stream>>>(a, S, nseg);
     const int gblocks = (int)((m + kSubThreads - 1) / kSubThreads);
     if (dtype == kF16)
         k_sub_gather<kF16><<<gblocks, kSubThreads, 0, stream>>>(a);
     else
         k_sub_gather<kF32><<<gblocks, kSubThreads, 0, stream>>>(a);
-    count_launches(5 + 2 * kRounds);
+    count_launches(4 + kRounds);
     return cudaGetLastError();
 }
 
