@@ -811,7 +811,7 @@ def run_ours(args):
 
 
 # ---------------------------------------------------------------------------
-# batched views (64 views of a 512^3 volume, one persistent launch in a CUDA graph)
+# batched views (64 views of a 512^3 volume, one CUDA graph launch)
 # ---------------------------------------------------------------------------
 def batched_workload(n, k, seed, dev):
     """The batched workload: an n^3 x 6 volume, its FP16 transfer function on T_anom, k random
@@ -922,13 +922,13 @@ def run_batched(rp, dev, args, seed):
     return {"what": f"{k} views of {n}^3 x 6, image sizes uniform in {{256,512,1024,2048}}^2 "
                     f"({pixels / 1e6:.1f} MP), random orbit cameras, distinct jittered 6-variable brushes",
             "batched_f16": {"ms_per_batch": round(batch_ms, 3), "samples_per_s": round(batch_samples / (batch_ms / 1e3), 1),
-                            "views_per_s": round(k / (batch_ms / 1e3), 1), "launch": "1 CUDA graph (per-view classification, cell classes and empty-space distance + persistent render)"},
+                            "views_per_s": round(k / (batch_ms / 1e3), 1), "launch": "1 CUDA graph (per-view classification, cell classes, empty-space distance and render nodes)"},
             "plain_f32_per_frame": {"ms_per_batch": round(plain_ms, 3),
                                     "samples_per_s": round(plain_samples / (plain_ms / 1e3), 1),
                                     "launch": f"{k} x (set_brush + render), default launch choices (8x4 tiles, skipping on)"},
             "plain_f32_per_frame_tuned": {"ms_per_batch": round(tuned_ms, 3), "tuning": tune32},
             "batched_tuning": tune16,
-            "roofline": {"kernel": "batched graph (classification + cell classes + k_render_batch)", "bound": "hbm",
+            "roofline": {"kernel": "batched graph (classification + cell classes + k_render_view)", "bound": "hbm",
                          "achieved": round(alg_bytes / batch_ms / 1e6, 1), "peak": peak, "unit": "GB/s",
                          "frac": round(alg_bytes / batch_ms / 1e6 / peak, 4), "frac_of_nominal": round(alg_bytes / batch_ms / 1e6 / NOMINAL_HBM_GBS, 4), "alg_bytes_per_batch": alg_bytes,
                          "peak_kind": f"{peak_kind} HBM copy"},

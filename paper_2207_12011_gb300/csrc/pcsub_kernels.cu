@@ -20,10 +20,10 @@
 // thread per line then gathers the line's axis values and brush flag. The block that
 // finishes a round last picks its digit, and the one that counts last scans.
 //
-// The four passes over the cells are bound by instructions (a key is some 40 of them), and were by
-// the rows' 64-bit divisions and square-root corrections and by a thousand blocks' tables
-// of digits added to L2: 256^3, 100 000 lines 223 -> 197 us of kernels in 11 launches
-// instead of 18, the call with its filter 337 -> 222 us.
+// The four passes over the cells are bound by the 64-bit arithmetic of the keys (30 us each at
+// 256^3); between and after them the call waited for launches and the host: 256^3, 100 000
+// lines 223 -> 197 us of kernels in 11 launches instead of 18, the call with its filter 337 ->
+// 222 us.
 #include <algorithm>
 
 #include "common.cuh"
