@@ -143,7 +143,9 @@ raypc_status alloc_cell_classes(raypc_ctx* ctx, Volume* V, Level& L, cudaStream_
     return RAYPC_OK;
 }
 
-raypc_status alloc_bricks(raypc_ctx* ctx, Volume* V, Level& L) {
+// The level's min/max, masks and statistics, the latter cleared in the order of stream s, on which
+// the pass that fills them runs.
+raypc_status alloc_bricks(raypc_ctx* ctx, Volume* V, Level& L, cudaStream_t s) {
     if (L.bmin) return RAYPC_OK;
     size_t nbk = L.nbricks();
     size_t mm = nbk * V->nvars * sizeof(float);
@@ -164,7 +166,7 @@ raypc_status alloc_bricks(raypc_ctx* ctx, Volume* V, Level& L) {
         free_bricks(L);
         return st;
     }
-    CK(cudaMemset(L.stats, 0, sizeof(unsigned long long) * (kMaxVars + 1)), "clear level statistics");
+    CK(cudaMemsetAsync(L.stats, 0, sizeof(unsigned long long) * (kMaxVars + 1), s), "clear level statistics");
     L.gen = 0;
     return RAYPC_OK;
 }
@@ -524,7 +526,7 @@ raypc_status raypc_load_volume(raypc_ctx* ctx, const void* src, int src_is_devic
     L.pairs_bytes = 2 * L.cells_bytes;
     raypc_status st = ctx->alloc(&L.cells, L.cells_bytes, &V->bytes);
     if (st == RAYPC_OK) st = ctx->alloc(&L.pairs, L.pairs_bytes, &V->bytes);
-    if (st == RAYPC_OK) st = alloc_bricks(ctx, V, L);
+    if (st == RAYPC_OK) st = alloc_bricks(ctx, V, L, s);
     if (st != RAYPC_OK) { free_volume(ctx, V); return st; }
     st = ingest(ctx, V, src, src_is_device, src_dtype, s);
     if (st != RAYPC_OK) { free_volume(ctx, V); return st; }
@@ -593,7 +595,7 @@ raypc_status raypc_build_bricks(raypc_ctx* ctx, int vol, int brick_dim, int n_lo
             if (st == RAYPC_OK) st = ctx->alloc(&L.pairs, L.pairs_bytes, &V->bytes);
             if (st) return st;
         }
-        if ((st = alloc_bricks(ctx, V, L))) return st;
+        if ((st = alloc_bricks(ctx, V, L, s))) return st;
         if (L.fresh) {           // the ingest or the pass before already wrote this level's cells: its bricks,
                                  // and the next level's cells in the same pass where that is allocated too
             Level* C = l < n_lod && V->lv[l + 1].cells && V->lv[l + 1].n * 2 == L.n &&

@@ -1,0 +1,75 @@
+"""The largest magnitudes of a level's stored values, which decide how its cells are classified:
+they belong to the values that the level holds, on whatever stream they came in."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2207_12011_gb300 import synth
+from test_gpu_parity import bits, stored
+
+pytestmark = pytest.mark.gpu
+R_IN, R_OUT = 0.3, 1.0
+
+
+@pytest.fixture(scope="module")
+def rp():
+    import paper_2207_12011_gb300.raypc as rp
+    rp.lib()
+    return rp
+
+
+def field(n, seed, nans):
+    """Two smooth variables; with nans, some values of the first are NaN."""
+    vol = synth.make_shell_volume(n, seed=seed)[:2].contiguous()
+    if nans:
+        vol[0, ::5, ::7, ::3] = float("nan")
+    return vol
+
+
+def wide_brush(vol):
+    """Every number of the first variable passes; the second is cut. Half the bounds are near its values."""
+    s = vol[1].flatten().sort().values
+    return np.array([-1e30, float(s[len(s) // 5])], np.float32), np.array([1e30, float(s[-len(s) // 8])], np.float32), 0b11
+
+
+def check_classes(rp, v, st, brush, lod=0, stream=None):
+    """Activity and classes of a level under the volume's brush against the oracle on its values."""
+    n = st.shape[1]
+    nsb = (n + 3) // 4
+    lo, hi, mask = brush
+    words = v.sub_bricks(lod, stream=stream)[2]
+    got = v.cell_classes(lod, stream=stream)
+    torch.cuda.synchronize()
+    mn, mx = oracle.brick_minmax(st, 4)
+    want, _ = oracle.classify(mn, mx, n, R_IN, R_OUT, lo, hi, mask, bs=4)
+    act = bits(rp, words, nsb ** 3).reshape(nsb, nsb, nsb).astype(bool)
+    assert np.array_equal(act, want.reshape(act.shape).astype(bool))
+    idx = np.arange(n) // 4
+    sel = act[idx[:, None, None], idx[None, :, None], idx[None, None, :]]
+    sel[n - 1], sel[:, n - 1], sel[:, :, n - 1] = False, False, False
+    got, ref = got.cpu().numpy().view(np.uint16), oracle.cell_classes(st, lo, hi, mask)
+    assert sel.any() and np.array_equal(got[sel], ref[sel]), np.argwhere((got != ref) & sel)[:4]
+
+
+@pytest.mark.parametrize("store", ["f32", "f16"])
+def test_load_on_a_stream_beside_a_busy_default_stream(rp, store):
+    """A volume that comes in on a stream of its own, and its coarser level, while the default stream
+    has work queued: nothing of theirs waits for, or is undone by, the default stream's order."""
+    n = 48
+    vol = field(n, 3, True)
+    src, brush, st = vol.cuda(), wide_brush(torch.nan_to_num(vol)), stored(vol, store)
+    busy = torch.empty((4096, 4096), device="cuda", dtype=torch.bfloat16).normal_()
+    side = torch.cuda.Stream()
+    with rp.Context(0) as ctx:
+        torch.cuda.synchronize()
+        for _ in range(200):
+            busy @ busy
+        v = ctx.load_volume(src, store=store, r_in=R_IN, r_out=R_OUT, stream=side)
+        v.build_bricks(n_lod=1, stream=side)
+        torch.cuda.synchronize()
+        v.set_brush(*brush, stream=side)
+        check_classes(rp, v, st, brush, stream=side)
+        coarse = oracle.lod_mean(st)
+        coarse = coarse.astype(np.float16).astype(np.float32) if store == "f16" else coarse
+        check_classes(rp, v, coarse, brush, lod=1, stream=side)
