@@ -143,9 +143,7 @@ raypc_status alloc_cell_classes(raypc_ctx* ctx, Volume* V, Level& L, cudaStream_
     return RAYPC_OK;
 }
 
-// The level's min/max, masks and statistics, the latter cleared in the order of stream s, on which
-// the pass that fills them runs.
-raypc_status alloc_bricks(raypc_ctx* ctx, Volume* V, Level& L, cudaStream_t s) {
+raypc_status alloc_bricks(raypc_ctx* ctx, Volume* V, Level& L) {
     if (L.bmin) return RAYPC_OK;
     size_t nbk = L.nbricks();
     size_t mm = nbk * V->nvars * sizeof(float);
@@ -162,12 +160,10 @@ raypc_status alloc_bricks(raypc_ctx* ctx, Volume* V, Level& L, cudaStream_t s) {
         (st = ctx->alloc((void**)&L.skippable, words, &V->bytes)) ||
         (st = ctx->alloc((void**)&L.list, nbk * sizeof(uint32_t), &V->bytes)) ||
         (st = ctx->alloc((void**)&L.n_active, sizeof(uint32_t), &V->bytes)) ||
-        (st = ctx->alloc((void**)&L.stats, sizeof(unsigned long long) * (kMaxVars + 1), &V->bytes))) {
+        (st = ctx->alloc((void**)&L.stats, kLevelStatsBytes, &V->bytes))) {
         free_bricks(L);
         return st;
     }
-    CK(cudaMemsetAsync(L.stats, 0, sizeof(unsigned long long) * (kMaxVars + 1), s), "clear level statistics");
-    L.gen = 0;
     return RAYPC_OK;
 }
 
@@ -252,13 +248,12 @@ raypc_status ingest(raypc_ctx* ctx, Volume* V, const void* src, int src_is_devic
     // x-pairs come out of the same pass over the source
     Level& C = V->lv[1];
     const bool next = C.cells && C.pairs && C.n * 2 == L.n && ingest_next_level_fits(dsrc, L.n);
-    const LevelStats stats{L.stats, ++L.gen};
     if (next)
         e = launch_ingest_next_level(dsrc, src_dtype, L.cells, L.pairs, V->dtype, L.n, V->nvars, L.bmin, L.bmax,
-                                     L.sbmin, L.sbmax, C.cells, C.pairs, stats, s);
+                                     L.sbmin, L.sbmax, C.cells, C.pairs, L.stats, s);
     else
         e = launch_ingest(dsrc, src_dtype, L.cells, L.pairs, V->dtype, L.n, V->nvars, L.bmin, L.bmax, L.sbmin,
-                          L.sbmax, stats, s);
+                          L.sbmax, L.stats, s);
     for (auto& l : V->lv) l.fresh = false;
     C.fresh = next && e == cudaSuccess;
     if (staging) cudaFreeAsync(staging, s);
@@ -389,7 +384,6 @@ BrushItem brush_item(const Volume* V, const Level& L, const BrushArgs& brush) {
     it.sbmax = L.sbmax;
     it.cells = L.cells;
     it.stats = L.stats;
-    it.gen = L.gen;
     it.n = L.n;
     it.nsb = L.nsb;
     it.nvars = V->nvars;
@@ -526,7 +520,7 @@ raypc_status raypc_load_volume(raypc_ctx* ctx, const void* src, int src_is_devic
     L.pairs_bytes = 2 * L.cells_bytes;
     raypc_status st = ctx->alloc(&L.cells, L.cells_bytes, &V->bytes);
     if (st == RAYPC_OK) st = ctx->alloc(&L.pairs, L.pairs_bytes, &V->bytes);
-    if (st == RAYPC_OK) st = alloc_bricks(ctx, V, L, s);
+    if (st == RAYPC_OK) st = alloc_bricks(ctx, V, L);
     if (st != RAYPC_OK) { free_volume(ctx, V); return st; }
     st = ingest(ctx, V, src, src_is_device, src_dtype, s);
     if (st != RAYPC_OK) { free_volume(ctx, V); return st; }
@@ -595,18 +589,18 @@ raypc_status raypc_build_bricks(raypc_ctx* ctx, int vol, int brick_dim, int n_lo
             if (st == RAYPC_OK) st = ctx->alloc(&L.pairs, L.pairs_bytes, &V->bytes);
             if (st) return st;
         }
-        if ((st = alloc_bricks(ctx, V, L, s))) return st;
+        if ((st = alloc_bricks(ctx, V, L))) return st;
         if (L.fresh) {           // the ingest or the pass before already wrote this level's cells: its bricks,
                                  // and the next level's cells in the same pass where that is allocated too
             Level* C = l < n_lod && V->lv[l + 1].cells && V->lv[l + 1].n * 2 == L.n &&
                        ingest_next_level_fits(L.cells, L.n) ? &V->lv[l + 1] : nullptr;
             CK(launch_level_bricks(L.cells, V->dtype, L.n, V->nvars, L.bmin, L.bmax, L.sbmin, L.sbmax,
-                                   C ? C->cells : nullptr, C ? C->pairs : nullptr, LevelStats{L.stats, ++L.gen}, s),
+                                   C ? C->cells : nullptr, C ? C->pairs : nullptr, L.stats, s),
                "level bricks kernel");
             if (C) C->fresh = true;
         } else {
             CK(launch_lod(P.cells, P.n, L.cells, L.pairs, V->dtype, V->nvars, L.bmin, L.bmax, L.sbmin, L.sbmax,
-                          LevelStats{L.stats, ++L.gen}, s),
+                          L.stats, s),
                "LOD kernel");
             if (l < RAYPC_MAX_LOD) V->lv[l + 1].fresh = false;
         }

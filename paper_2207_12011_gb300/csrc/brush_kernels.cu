@@ -250,9 +250,7 @@ __global__ void __launch_bounds__(32 * kBrushWarps, kBrushBlocks) k_brush(const 
             if (threadIdx.x == 0) S.pairs = 0u;
             __syncthreads();
             if (threadIdx.x <= kMaxVars) {
-                // magnitudes of the level: keys of another generation hold nothing of this one
-                const unsigned long long key = S.it.stats[threadIdx.x];
-                const unsigned bits = (unsigned)(key >> 32) == S.it.gen ? (unsigned)key : 0u;
+                const unsigned bits = S.it.stats[threadIdx.x];        // magnitudes of the level
                 const int v = threadIdx.x;
                 if (v == kMaxVars) {
                     S.finite = bits == 0u;

@@ -282,11 +282,10 @@ struct BrushItem {
     const void* cells;             // planar values, storage dtype
     uint32_t* active;              // sub-brick activity bits, written
     uint16_t* cls;                 // optional: cell classes, written for the cells of active sub-bricks
-    const unsigned long long* stats;   // [kMaxVars + 1] magnitudes of the level (see LevelStats)
+    const unsigned* stats;         // [kMaxVars + 1] magnitudes of the level (see kLevelStatsBytes)
     const int* tf_prefix;          // optional: activity AND visibility of the transfer function
                                    // ([kTF + 1]: entries < j with sigma > 0)
     uint8_t* sdist;                // batched views: padded empty-space distance, written afterwards
-    unsigned gen;                  // generation of stats
     int n, nsb, nvars;
     float rin2, rout2;             // r_in * r_in, r_out * r_out rounded to FP32
     int color_var;
@@ -326,14 +325,10 @@ struct BrushLaunch {
 };
 
 // Magnitudes of a level's stored values, written by the kernel that computes its
-// min/max: per variable, then for non-finite values, the key
-// (generation << 32) | bits -- bits of the largest |value|, or 1 when a value is
-// NaN or infinite. A key of another generation holds nothing of this one, so
-// the keys need no clearing between ingests.
-struct LevelStats {
-    unsigned long long* key;       // [kMaxVars + 1]
-    unsigned gen;
-};
+// min/max: per variable the bits of the largest |value|, then 1 when a value is NaN
+// or infinite. Cleared in stream order in front of each such pass (36 bytes), so that
+// they belong to the values they are read with also when passes replay from graphs.
+constexpr size_t kLevelStatsBytes = sizeof(unsigned) * (kMaxVars + 1);
 
 // Activity, dilation and ordered list of a level's 8^3 bricks (inspection).
 struct BrickListArgs {
@@ -539,9 +534,9 @@ void count_launches(int k);
 constexpr int kMaxRowsEdge = 4096;
 cudaError_t launch_ingest(const void* src, int src_dtype, void* cells, void* pairs, int dtype,
                           int n, int nvars, float* bmin, float* bmax, float* sbmin, float* sbmax,
-                          LevelStats stats, cudaStream_t stream);
+                          unsigned* stats, cudaStream_t stream);
 cudaError_t launch_lod(const void* fine, int n_fine, void* cells, void* pairs, int dtype, int nvars,
-                       float* bmin, float* bmax, float* sbmin, float* sbmax, LevelStats stats, cudaStream_t stream);
+                       float* bmin, float* bmax, float* sbmin, float* sbmax, unsigned* stats, cudaStream_t stream);
 // Ingest that also writes the next level's cells and x-pairs (edge n / 2, the same
 // 2x2x2 means as launch_lod, from the values it stores) in the same pass over the
 // source; that level's brick min/max then come from launch_level_bricks. Only when
@@ -549,12 +544,12 @@ cudaError_t launch_lod(const void* fine, int n_fine, void* cells, void* pairs, i
 bool ingest_next_level_fits(const void* src, int n);
 cudaError_t launch_ingest_next_level(const void* src, int src_dtype, void* cells, void* pairs, int dtype, int n,
                                      int nvars, float* bmin, float* bmax, float* sbmin, float* sbmax,
-                                     void* next_cells, void* next_pairs, LevelStats stats, cudaStream_t stream);
+                                     void* next_cells, void* next_pairs, unsigned* stats, cudaStream_t stream);
 // Brick and sub-brick min/max of a level from its own stored cells; with next_cells
 // (and next_pairs; only when ingest_next_level_fits(cells, n)) also the next
 // level's cells and x-pairs.
 cudaError_t launch_level_bricks(const void* cells, int dtype, int n, int nvars, float* bmin, float* bmax,
-                                float* sbmin, float* sbmax, void* next_cells, void* next_pairs, LevelStats stats,
+                                float* sbmin, float* sbmax, void* next_cells, void* next_pairs, unsigned* stats,
                                 cudaStream_t stream);
 // Sub-brick activity bits and cell classes of P.items[0 .. nitems-1] (brush_kernels.cu),
 // and of every view of a batch (brush_chunks(n) chunks per view).

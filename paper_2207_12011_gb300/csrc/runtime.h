@@ -51,8 +51,7 @@ struct Level {
     uint32_t* skippable = nullptr;
     uint32_t* list = nullptr;
     uint32_t* n_active = nullptr;
-    unsigned long long* stats = nullptr;   // magnitudes of the stored values (see LevelStats) ...
-    unsigned gen = 0;                      // ... of this many min/max passes
+    unsigned* stats = nullptr;    // magnitudes of the stored values (see kLevelStatsBytes)
     float* sbmin = nullptr;       // [nsb^3][nvars]
     float* sbmax = nullptr;
     uint32_t* sactive = nullptr;  // sub-brick activity bits under the current brush

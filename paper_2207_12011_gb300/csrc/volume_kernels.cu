@@ -32,7 +32,7 @@ struct RowsArgs {
     float* sbmax;
     void* ccells;         // ingest with the next level: its planar cells (edge n / 2) ...
     void* cpairs;         // ... and x-pairs
-    LevelStats stats;     // magnitudes of this level
+    unsigned* stats;      // magnitudes of this level
 };
 
 __device__ __forceinline__ void fold(float& mn, float& mx, float a_mn, float a_mx) {
@@ -239,12 +239,11 @@ __device__ __forceinline__ void store_pair_second(void* pairs, size_t i, float v
 // Record the magnitudes of variable v: odd is NaN in a thread that met a NaN or
 // infinite value, mag the largest |value| the thread knows of (NaN: none), in the
 // warps with `all` set (one atomic per warp that may raise the level's).
-__device__ __forceinline__ void level_stats(const LevelStats& L, int v, float odd, float mag, bool all) {
-    if (odd != odd) atomicMax(L.key + kMaxVars, ((unsigned long long)L.gen << 32) | 1ull);
+__device__ __forceinline__ void level_stats(unsigned* stats, int v, float odd, float mag, bool all) {
+    if (odd != odd) atomicMax(stats + kMaxVars, 1u);
     if (!all) return;
     const unsigned bits = __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(mag, 0.0f)));
-    const unsigned long long key = ((unsigned long long)L.gen << 32) | bits;
-    if ((threadIdx.x & 31) == 0 && *(volatile unsigned long long*)(L.key + v) < key) atomicMax(L.key + v, key);
+    if ((threadIdx.x & 31) == 0 && *(volatile unsigned*)(stats + v) < bits) atomicMax(stats + v, bits);
 }
 
 template <int DT, int VEC>
@@ -476,6 +475,8 @@ void launch_lod_t(const RowsArgs& a, cudaStream_t stream) {
 template <int MODE>
 cudaError_t launch_rows(const RowsArgs& a, int dtype, cudaStream_t stream) {
     if (a.n < 2 || a.n > kMaxRowsEdge) return cudaErrorInvalidValue;
+    const cudaError_t e = cudaMemsetAsync(a.stats, 0, kLevelStatsBytes, stream);
+    if (e != cudaSuccess) return e;
     if constexpr (MODE == 1) {
         // 4-column runs when every run is aligned (n % 4 == 0 and an even fine edge make it 8k)
         // and the level is wide enough to fill a warp with runs
@@ -506,7 +507,7 @@ cudaError_t launch_rows(const RowsArgs& a, int dtype, cudaStream_t stream) {
 
 cudaError_t launch_ingest(const void* src, int src_dtype, void* cells, void* pairs, int dtype, int n,
                           int nvars, float* bmin, float* bmax, float* sbmin, float* sbmax,
-                          LevelStats stats, cudaStream_t stream) {
+                          unsigned* stats, cudaStream_t stream) {
     RowsArgs a{};
     a.src = src;
     a.src_dtype = src_dtype;
@@ -528,7 +529,7 @@ bool ingest_next_level_fits(const void* src, int n) {
 
 cudaError_t launch_ingest_next_level(const void* src, int src_dtype, void* cells, void* pairs, int dtype, int n,
                                      int nvars, float* bmin, float* bmax, float* sbmin, float* sbmax,
-                                     void* next_cells, void* next_pairs, LevelStats stats, cudaStream_t stream) {
+                                     void* next_cells, void* next_pairs, unsigned* stats, cudaStream_t stream) {
     RowsArgs a{};
     a.src = src;
     a.src_dtype = src_dtype;
@@ -547,7 +548,7 @@ cudaError_t launch_ingest_next_level(const void* src, int src_dtype, void* cells
 }
 
 cudaError_t launch_level_bricks(const void* cells, int dtype, int n, int nvars, float* bmin, float* bmax,
-                                float* sbmin, float* sbmax, void* next_cells, void* next_pairs, LevelStats stats,
+                                float* sbmin, float* sbmax, void* next_cells, void* next_pairs, unsigned* stats,
                                 cudaStream_t stream) {
     RowsArgs a{};
     a.src = cells;
@@ -565,7 +566,7 @@ cudaError_t launch_level_bricks(const void* cells, int dtype, int n, int nvars, 
 }
 
 cudaError_t launch_lod(const void* fine, int n_fine, void* cells, void* pairs, int dtype, int nvars,
-                       float* bmin, float* bmax, float* sbmin, float* sbmax, LevelStats stats, cudaStream_t stream) {
+                       float* bmin, float* bmax, float* sbmin, float* sbmax, unsigned* stats, cudaStream_t stream) {
     RowsArgs a{};
     a.src = fine;
     a.n_src = n_fine;

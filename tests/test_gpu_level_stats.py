@@ -73,3 +73,42 @@ def test_load_on_a_stream_beside_a_busy_default_stream(rp, store):
         coarse = oracle.lod_mean(st)
         coarse = coarse.astype(np.float16).astype(np.float32) if store == "f16" else coarse
         check_classes(rp, v, coarse, brush, lod=1, stream=side)
+
+
+@pytest.mark.parametrize("store", ["f32", "f16"])
+@pytest.mark.parametrize("n", [48, 128])                     # level 1 by its own pass, and from the ingest
+def test_recorded_time_steps_in_turn(rp, store, n):
+    """Two time steps with NaN and a finite one, whose update, levels and brush edit are recorded in
+    graphs: replayed in turn, and after a direct update, each leaves the classes of its own values."""
+    steps = [field(n, 3, True), field(n, 5, True).flip(1) * 7, field(n, 5, False)]
+    brush = wide_brush(steps[2])
+    srcs, sts = [s.cuda() for s in steps], [stored(s, store) for s in steps]
+    side = torch.cuda.Stream()
+    with rp.Context(0) as ctx:
+        v = ctx.load_volume(srcs[1], store=store, r_in=R_IN, r_out=R_OUT)
+
+        def step(i):
+            s = torch.cuda.current_stream()
+            v.update(srcs[i], stream=s)
+            v.build_bricks(n_lod=1, stream=s)
+            v.set_brush(*brush, stream=s)
+            return v.cell_classes(stream=s)
+
+        v.build_bricks(n_lod=1)
+        step(0)                                              # the buffers exist from here on
+        torch.cuda.synchronize()
+        graphs, outs = [], []
+        for i in range(3):
+            graphs.append(torch.cuda.CUDAGraph())
+            with torch.cuda.graph(graphs[i], stream=side):
+                outs.append(step(i))
+        for i in (0, 1, 0, 2, 1, None, 0, 2):
+            if i is None:
+                step(1)
+            else:
+                graphs[i].replay()
+            torch.cuda.synchronize()
+            if i is not None:
+                check_classes(rp, v, sts[i], brush)
+                assert torch.equal(outs[i], v.cell_classes())
+        del graphs
