@@ -238,12 +238,14 @@ __device__ __forceinline__ void store_pair_second(void* pairs, size_t i, float v
 
 // Record the magnitudes of variable v: odd is NaN in a thread that met a NaN or
 // infinite value, mag the largest |value| the thread knows of (NaN: none), in the
-// warps with `all` set (one atomic per warp that may raise the level's).
+// warps with `all` set. One atomic per warp that may raise the level's: an atomic per
+// thread that met a NaN took 512^3 FP16 with NaN outside the shell from 1.79 to 9.42 ms.
 __device__ __forceinline__ void level_stats(unsigned* stats, int v, float odd, float mag, bool all) {
-    if (odd != odd) atomicMax(stats + kMaxVars, 1u);
-    if (!all) return;
-    const unsigned bits = __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(mag, 0.0f)));
-    if ((threadIdx.x & 31) == 0 && *(volatile unsigned*)(stats + v) < bits) atomicMax(stats + v, bits);
+    auto raise = [&](int k, unsigned bits) {
+        if ((threadIdx.x & 31) == 0 && *(volatile unsigned*)(stats + k) < bits) atomicMax(stats + k, bits);
+    };
+    if (__any_sync(0xffffffffu, odd != odd)) raise(kMaxVars, 1u);
+    if (all) raise(v, __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(mag, 0.0f))));
 }
 
 template <int DT, int VEC>

@@ -112,3 +112,28 @@ def test_recorded_time_steps_in_turn(rp, store, n):
                 check_classes(rp, v, sts[i], brush)
                 assert torch.equal(outs[i], v.cell_classes())
         del graphs
+
+
+def test_update_with_nan_takes_the_time_of_one_without(rp):
+    """Masked data has NaN in half of its cells: their ingest moves the same bytes as any other and has
+    to take about its time (one atomic per thread that met a NaN took five times as long)."""
+    n = 256
+    vol = synth.make_shell_volume(n, device="cuda").half()
+    masked = vol.clone()
+    masked[:, ::2] = float("nan")
+    with rp.Context(0) as ctx:
+        v = ctx.load_volume(vol, store="f16")
+
+        def ms(src):
+            best = []
+            for _ in range(8):
+                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                a.record()
+                v.update(src)
+                b.record()
+                torch.cuda.synchronize()
+                best.append(a.elapsed_time(b))
+            return min(best)
+
+        ms(vol)
+        assert ms(masked) < 2.0 * ms(vol)
