@@ -326,8 +326,9 @@ struct BrushLaunch {
 
 // Magnitudes of a level's stored values, written by the kernel that computes its
 // min/max: per variable the bits of the largest |value|, then 1 when a value is NaN
-// or infinite. Cleared in stream order in front of each such pass (36 bytes), so that
-// they belong to the values they are read with also when passes replay from graphs.
+// or infinite. Every ingest clears those of all levels in stream order before its pass
+// (one clear of 108 bytes: a coarser level's values change only after an ingest), so
+// that they belong to the values they are read with also when passes replay from graphs.
 constexpr size_t kLevelStatsBytes = sizeof(unsigned) * (kMaxVars + 1);
 
 // Activity, dilation and ordered list of a level's 8^3 bricks (inspection).

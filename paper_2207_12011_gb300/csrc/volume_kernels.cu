@@ -477,8 +477,6 @@ void launch_lod_t(const RowsArgs& a, cudaStream_t stream) {
 template <int MODE>
 cudaError_t launch_rows(const RowsArgs& a, int dtype, cudaStream_t stream) {
     if (a.n < 2 || a.n > kMaxRowsEdge) return cudaErrorInvalidValue;
-    const cudaError_t e = cudaMemsetAsync(a.stats, 0, kLevelStatsBytes, stream);
-    if (e != cudaSuccess) return e;
     if constexpr (MODE == 1) {
         // 4-column runs when every run is aligned (n % 4 == 0 and an even fine edge make it 8k)
         // and the level is wide enough to fill a warp with runs
