@@ -50,7 +50,7 @@ namespace {
 
 void free_level(Level& L) {
     void* ptrs[] = {L.cells, L.pairs, L.bmin, L.bmax, L.active, L.skippable, L.list, L.n_active,
-                    L.sbmin, L.sbmax, L.sactive, L.cls, L.tf_sactive, L.sdist};
+                    L.sbmin, L.sbmax, L.stats.odd, L.sactive, L.cls, L.tf_sactive, L.sdist};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     L = Level{};
@@ -58,13 +58,14 @@ void free_level(Level& L) {
 
 void free_bricks(Level& L) {
     void* ptrs[] = {L.bmin, L.bmax, L.active, L.skippable, L.list, L.n_active,
-                    L.sbmin, L.sbmax, L.sactive, L.tf_sactive, L.sdist};
+                    L.sbmin, L.sbmax, L.stats.odd, L.sactive, L.tf_sactive, L.sdist};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     L.bmin = L.bmax = L.sbmin = L.sbmax = nullptr;
     L.active = L.skippable = L.list = L.n_active = L.sactive = L.tf_sactive = nullptr;
     L.sdist = nullptr;
     L.sdist_of = nullptr;
+    L.stats.odd = nullptr;
     L.bricks = L.classified = L.cls_valid = L.listed = false;
 }
 
@@ -87,7 +88,7 @@ void free_staging(Volume* V) {
 void free_volume(raypc_ctx* ctx, Volume* V) {
     free_staging(V);
     for (auto& L : V->lv) free_level(L);
-    if (V->stats) cudaFree(V->stats);
+    if (V->mags) cudaFree(V->mags);
     if (V->tf) cudaFree(V->tf);
     if (V->tf_prefix) cudaFree(V->tf_prefix);
     ctx->used -= V->bytes < ctx->used ? V->bytes : ctx->used;
@@ -152,6 +153,7 @@ raypc_status alloc_bricks(raypc_ctx* ctx, Volume* V, Level& L) {
     raypc_status st;
     if ((st = ctx->alloc((void**)&L.sbmin, smm, &V->bytes)) ||
         (st = ctx->alloc((void**)&L.sbmax, smm, &V->bytes)) ||
+        (st = ctx->alloc((void**)&L.stats.odd, L.nsbricks() * V->nvars, &V->bytes)) ||
         (st = ctx->alloc((void**)&L.sactive, L.nswords() * sizeof(uint32_t), &V->bytes)) ||
         (st = ctx->alloc((void**)&L.tf_sactive, L.nswords() * sizeof(uint32_t), &V->bytes)) ||
         (st = ctx->alloc((void**)&L.bmin, mm, &V->bytes)) ||
@@ -247,7 +249,7 @@ raypc_status ingest(raypc_ctx* ctx, Volume* V, const void* src, int src_is_devic
     // x-pairs come out of the same pass over the source
     Level& C = V->lv[1];
     const bool next = C.cells && C.pairs && C.n * 2 == L.n && ingest_next_level_fits(dsrc, L.n);
-    e = cudaMemsetAsync(V->stats, 0, kLevelStatsBytes * (1 + RAYPC_MAX_LOD), s);
+    e = cudaMemsetAsync(V->mags, 0, kLevelStatsBytes * (1 + RAYPC_MAX_LOD), s);
     if (e == cudaSuccess && next)
         e = launch_ingest_next_level(dsrc, src_dtype, L.cells, L.pairs, V->dtype, L.n, V->nvars, L.bmin, L.bmax,
                                      L.sbmin, L.sbmax, C.cells, C.pairs, L.stats, s);
@@ -521,9 +523,9 @@ raypc_status raypc_load_volume(raypc_ctx* ctx, const void* src, int src_is_devic
     raypc_status st = ctx->alloc(&L.cells, L.cells_bytes, &V->bytes);
     if (st == RAYPC_OK) st = ctx->alloc(&L.pairs, L.pairs_bytes, &V->bytes);
     if (st == RAYPC_OK) st = alloc_bricks(ctx, V, L);
-    if (st == RAYPC_OK) st = ctx->alloc((void**)&V->stats, kLevelStatsBytes * (1 + RAYPC_MAX_LOD), &V->bytes);
+    if (st == RAYPC_OK) st = ctx->alloc((void**)&V->mags, kLevelStatsBytes * (1 + RAYPC_MAX_LOD), &V->bytes);
     if (st != RAYPC_OK) { free_volume(ctx, V); return st; }
-    for (int l = 0; l <= RAYPC_MAX_LOD; ++l) V->lv[l].stats = V->stats + l * (kMaxVars + 1);
+    for (int l = 0; l <= RAYPC_MAX_LOD; ++l) V->lv[l].stats.mag = V->mags + l * (kMaxVars + 1);
     st = ingest(ctx, V, src, src_is_device, src_dtype, s);
     if (st != RAYPC_OK) { free_volume(ctx, V); return st; }
     if (!src_is_device) {

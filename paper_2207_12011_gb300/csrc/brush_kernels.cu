@@ -13,7 +13,10 @@
 // active sub-brick of the group lies inside the brush by its margin is not read
 // at all (of a 6-variable brush's variables 4 of 6, on average, at 256^3). FP16
 // volumes fold two cells per instruction as binary16 pairs (exact) and decide them
-// with four comparisons against binary16 bounds (see half_bounds).
+// with four comparisons against binary16 bounds (see half_bounds). Both hold for
+// sub-bricks without NaN or infinite values, which the ingest marks; others read every
+// variable that has some and are decided value by value (512^3 FP16 with NaN outside the
+// shell: 242 us; 568 where one NaN took both from the whole level, 545 before either).
 //
 // Bound by load latency. One launch against the former four and their counters'
 // clears, which read every restricted variable's x-pairs a sub-brick at a time:
@@ -105,9 +108,10 @@ template <> struct Corners<kF16> {
         mn = lo(as_half2(a), as_half2(b));
         mx = hi(as_half2(a), as_half2(b));
     }
+    template <bool ODD>
     static __device__ __forceinline__ unsigned classes(const BrushShared& S, int v, V mn, V mx) {
         const unsigned need = 0x00010001u << v;
-        if ((S.pairs >> v) & 1u) {
+        if (!ODD && ((S.pairs >> v) & 1u)) {
             const unsigned fail = __hle2_mask(mx, as_half2(S.fail_lo[v])) | __hge2_mask(mn, as_half2(S.fail_hi[v]));
             const unsigned in = __hge2_mask(mn, as_half2(S.in_lo[v])) & __hle2_mask(mx, as_half2(S.in_hi[v]));
             return (fail & 0x80008000u) | (~(fail | in) & need);
@@ -129,17 +133,20 @@ template <> struct Corners<kF32> {
         mn = lo(a, b);
         mx = hi(a, b);
     }
+    template <bool>
     static __device__ __forceinline__ unsigned classes(const BrushShared& S, int v, V mn, V mx) {
         const float lo = S.it.brush.lo[v], hi = S.it.brush.hi[v];
         return cell_class(mn.x, mx.x, lo, hi, 1u << v) | (cell_class(mn.y, mx.y, lo, hi, 1u << v) << 16);
     }
 };
 
+constexpr unsigned kOdd = 1u << 16;  // in a list entry: NaN or infinite values
 constexpr int kGroup = 4;            // sub-bricks of a group: 8 lanes of two cells in x, 4 lanes in y
 
 // Classes of the cells of up to kGroup sub-bricks (sx .. sx + 3, sy, sz), sx a multiple
-// of kGroup, over the variables `vars`; written for the sub-bricks in `act` (bit k: sx + k).
-template <int DT, bool EVEN>
+// of kGroup, over the variables `vars`; written for the sub-bricks in `act` (bit k: sx + k). ODD: one
+// of them may hold NaN or infinite values, which the binary16 bounds do not decide.
+template <int DT, bool EVEN, bool ODD>
 __device__ __forceinline__ void classes_of_group(const BrushShared& S, int sx, int sy, int sz, unsigned act,
                                                  unsigned vars, int lane) {
     using C = Corners<DT>;
@@ -162,7 +169,7 @@ __device__ __forceinline__ void classes_of_group(const BrushShared& S, int sx, i
             C::template row<EVEN>(plane, rz + r0, x0, x1, x2, amn, amx);
             C::template row<EVEN>(plane, rz + r1, x0, x1, x2, bmn, bmx);
             const V mn = C::lo(amn, bmn), mx = C::hi(amx, bmx);
-            if (c > 0) word[c > 0 ? c - 1 : 0] |= C::classes(S, v, C::lo(pmn, mn), C::hi(pmx, mx));
+            if (c > 0) word[c > 0 ? c - 1 : 0] |= C::template classes<ODD>(S, v, C::lo(pmn, mn), C::hi(pmx, mx));
             pmn = mn;
             pmx = mx;
         }
@@ -198,8 +205,16 @@ __device__ __forceinline__ void classify_word(const BrushShared& S, unsigned w, 
     const unsigned word = __ballot_sync(kFull, act);
     if (lane == 0) S.it.active[w] = word;
     if (!S.it.cls || word == 0u) return;
-    // a NaN corner fails its cell whatever the range says: ranges decide finite levels only
-    const unsigned mine = act ? S.it.brush.mask & ~(S.finite ? inside : 0u) : 0u;
+    // a NaN corner fails its cell whatever the range says: ranges do not decide variables that may
+    // have one. Such a variable sets kOdd beside the variables to read.
+    unsigned mine = act ? S.it.brush.mask & ~inside : 0u;
+    if (act && !S.finite) {
+        for (unsigned m = S.it.brush.mask; m; m &= m - 1u) {
+            const int v = __ffs(m) - 1;
+            const uint8_t* odd = S.it.stats.odd + (size_t)v * total + b;
+            if (odd[0] || (b % (unsigned)nsb + 1u < (unsigned)nsb && odd[1])) mine |= (1u << v) | kOdd;
+        }
+    }
     // the lanes of this lane's group: kGroup neighbours in x, cut at the word's and the row's ends
     const int sx = (int)(b % (unsigned)nsb), k = sx & (kGroup - 1);
     const int first = lane - k, end = min(min(first + kGroup, lane + nsb - sx), 32);
@@ -250,7 +265,7 @@ __global__ void __launch_bounds__(32 * kBrushWarps, kBrushBlocks) k_brush(const 
             if (threadIdx.x == 0) S.pairs = 0u;
             __syncthreads();
             if (threadIdx.x <= kMaxVars) {
-                const unsigned bits = S.it.stats[threadIdx.x];        // magnitudes of the level
+                const unsigned bits = S.it.stats.mag[threadIdx.x];   // magnitude of the variable
                 const int v = threadIdx.x;
                 if (v == kMaxVars) {
                     S.finite = bits == 0u;
@@ -267,7 +282,6 @@ __global__ void __launch_bounds__(32 * kBrushWarps, kBrushBlocks) k_brush(const 
                 }
             }
             __syncthreads();
-            if (threadIdx.x == 0 && !S.finite) S.pairs = 0u;  // NaN and infinite corners: cell_class
             cur = vi;
         }
         __syncthreads();
@@ -285,8 +299,11 @@ __global__ void __launch_bounds__(32 * kBrushWarps, kBrushBlocks) k_brush(const 
             if (g >= groups) break;
             const uint2 e = s_list[g];
             const int sx = (int)(e.x % (unsigned)nsb), sy = (int)((e.x / nsb) % nsb), sz = (int)(e.x / ((unsigned)nsb * nsb));
-            if ((S.it.n & 1) == 0) classes_of_group<DT, true>(S, sx, sy, sz, e.y >> 8, e.y & 0xffu, lane);
-            else classes_of_group<DT, false>(S, sx, sy, sz, e.y >> 8, e.y & 0xffu, lane);
+            const bool odd = DT == kF16 && (e.y & kOdd), even = (S.it.n & 1) == 0;
+            if (even && !odd) classes_of_group<DT, true, false>(S, sx, sy, sz, e.y >> 8, e.y & 0xffu, lane);
+            else if (even) classes_of_group<DT, true, DT == kF16>(S, sx, sy, sz, e.y >> 8, e.y & 0xffu, lane);
+            else if (!odd) classes_of_group<DT, false, false>(S, sx, sy, sz, e.y >> 8, e.y & 0xffu, lane);
+            else classes_of_group<DT, false, DT == kF16>(S, sx, sy, sz, e.y >> 8, e.y & 0xffu, lane);
         }
     }
 }

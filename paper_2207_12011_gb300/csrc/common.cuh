@@ -275,6 +275,19 @@ struct ViewDone {
     unsigned long long stats[kNStats];
 };
 
+// What else the kernel that computes a level's min/max says of its stored values.
+// mag: per variable the bits of the largest |value|, then 1 when a value is NaN or
+// infinite. odd, [nvars][nsb^3]: 1 for every sub-brick that holds such a value (perhaps
+// for its neighbours in a brick too), but for its vertices at x = 4s + 4, which are the
+// next sub-brick's. Every ingest clears mag of all levels in stream order before its pass
+// (one clear of 108 bytes: a coarser level's values change only after an ingest), so
+// that they belong to the values they are read with also when passes replay from graphs.
+struct LevelStats {
+    unsigned* mag;                 // [kMaxVars + 1]
+    uint8_t* odd;
+};
+constexpr size_t kLevelStatsBytes = sizeof(unsigned) * (kMaxVars + 1);
+
 // One level to classify under a brush (see brush_kernels.cu).
 struct BrushItem {
     const float* sbmin;            // [nsb^3][nvars], sub-brick min/max
@@ -282,7 +295,7 @@ struct BrushItem {
     const void* cells;             // planar values, storage dtype
     uint32_t* active;              // sub-brick activity bits, written
     uint16_t* cls;                 // optional: cell classes, written for the cells of active sub-bricks
-    const unsigned* stats;         // [kMaxVars + 1] magnitudes of the level (see kLevelStatsBytes)
+    LevelStats stats;              // of the level
     const int* tf_prefix;          // optional: activity AND visibility of the transfer function
                                    // ([kTF + 1]: entries < j with sigma > 0)
     uint8_t* sdist;                // batched views: padded empty-space distance, written afterwards
@@ -323,13 +336,6 @@ struct BrushLaunch {
     unsigned words, chunks;        // words per chunk and chunks, set by the launcher
     BrushItem items[kBrushItems];
 };
-
-// Magnitudes of a level's stored values, written by the kernel that computes its
-// min/max: per variable the bits of the largest |value|, then 1 when a value is NaN
-// or infinite. Every ingest clears those of all levels in stream order before its pass
-// (one clear of 108 bytes: a coarser level's values change only after an ingest), so
-// that they belong to the values they are read with also when passes replay from graphs.
-constexpr size_t kLevelStatsBytes = sizeof(unsigned) * (kMaxVars + 1);
 
 // Activity, dilation and ordered list of a level's 8^3 bricks (inspection).
 struct BrickListArgs {
@@ -535,9 +541,9 @@ void count_launches(int k);
 constexpr int kMaxRowsEdge = 4096;
 cudaError_t launch_ingest(const void* src, int src_dtype, void* cells, void* pairs, int dtype,
                           int n, int nvars, float* bmin, float* bmax, float* sbmin, float* sbmax,
-                          unsigned* stats, cudaStream_t stream);
+                          LevelStats stats, cudaStream_t stream);
 cudaError_t launch_lod(const void* fine, int n_fine, void* cells, void* pairs, int dtype, int nvars,
-                       float* bmin, float* bmax, float* sbmin, float* sbmax, unsigned* stats, cudaStream_t stream);
+                       float* bmin, float* bmax, float* sbmin, float* sbmax, LevelStats stats, cudaStream_t stream);
 // Ingest that also writes the next level's cells and x-pairs (edge n / 2, the same
 // 2x2x2 means as launch_lod, from the values it stores) in the same pass over the
 // source; that level's brick min/max then come from launch_level_bricks. Only when
@@ -545,12 +551,12 @@ cudaError_t launch_lod(const void* fine, int n_fine, void* cells, void* pairs, i
 bool ingest_next_level_fits(const void* src, int n);
 cudaError_t launch_ingest_next_level(const void* src, int src_dtype, void* cells, void* pairs, int dtype, int n,
                                      int nvars, float* bmin, float* bmax, float* sbmin, float* sbmax,
-                                     void* next_cells, void* next_pairs, unsigned* stats, cudaStream_t stream);
+                                     void* next_cells, void* next_pairs, LevelStats stats, cudaStream_t stream);
 // Brick and sub-brick min/max of a level from its own stored cells; with next_cells
 // (and next_pairs; only when ingest_next_level_fits(cells, n)) also the next
 // level's cells and x-pairs.
 cudaError_t launch_level_bricks(const void* cells, int dtype, int n, int nvars, float* bmin, float* bmax,
-                                float* sbmin, float* sbmax, void* next_cells, void* next_pairs, unsigned* stats,
+                                float* sbmin, float* sbmax, void* next_cells, void* next_pairs, LevelStats stats,
                                 cudaStream_t stream);
 // Sub-brick activity bits and cell classes of P.items[0 .. nitems-1] (brush_kernels.cu),
 // and of every view of a batch (brush_chunks(n) chunks per view).

@@ -51,7 +51,7 @@ struct Level {
     uint32_t* skippable = nullptr;
     uint32_t* list = nullptr;
     uint32_t* n_active = nullptr;
-    unsigned* stats = nullptr;    // magnitudes of the stored values (see kLevelStatsBytes; the volume's)
+    LevelStats stats{};           // of the stored values; mag is the volume's
     float* sbmin = nullptr;       // [nsb^3][nvars]
     float* sbmax = nullptr;
     uint32_t* sactive = nullptr;  // sub-brick activity bits under the current brush
@@ -82,7 +82,7 @@ struct Volume {
     float r_in = 0.f, r_out = 1.f;
     int nlev = 0;             // built levels (1 + coarser)
     Level lv[1 + RAYPC_MAX_LOD];
-    unsigned* stats = nullptr;    // the levels' statistics, one after another
+    unsigned* mags = nullptr;     // the levels' magnitudes, one after another
     bool brush_set = false;
     BrushArgs brush{};
     float4* tf = nullptr;

@@ -32,7 +32,7 @@ struct RowsArgs {
     float* sbmax;
     void* ccells;         // ingest with the next level: its planar cells (edge n / 2) ...
     void* cpairs;         // ... and x-pairs
-    unsigned* stats;      // magnitudes of this level
+    LevelStats stats;
 };
 
 __device__ __forceinline__ void fold(float& mn, float& mx, float a_mn, float a_mx) {
@@ -252,6 +252,7 @@ template <int DT, int VEC>
 __global__ void __launch_bounds__(kRowCols * kRowSlices, 2) k_lod(RowsArgs A) {
     constexpr int G = kSub / VEC;                       // lanes per sub-brick column
     __shared__ float s_half[kRowSlices][4][kRowCols];  // per slice: min, max of y half 0, then of half 1
+    __shared__ float s_odd[kRowSlices][kRowCols];
     const int n = A.n;
     const int nb = (n + kBrick - 1) / kBrick;
     const int nsb = (n + kSub - 1) / kSub;
@@ -260,12 +261,12 @@ __global__ void __launch_bounds__(kRowCols * kRowSlices, 2) k_lod(RowsArgs A) {
     const int dz = threadIdx.y, tx = threadIdx.x;
     const int z = bz * kBrick + dz;
     const float qnan = __int_as_float(0x7fffffff);
-    float odd = 0.0f, mag = 0.0f;                        // NaN once a value is NaN or infinite; largest |value|
+    float all_odd = 0.0f, mag = 0.0f;                    // NaN once a value is NaN or infinite; largest |value|
     for (int c0 = 0; c0 < ncol; c0 += blockDim.x) {
         const int t = c0 + tx;
         const bool valid = t < ncol && z < n;
         const int X = t * VEC;
-        float ymn[2] = {qnan, qnan}, ymx[2] = {qnan, qnan};
+        float ymn[2] = {qnan, qnan}, ymx[2] = {qnan, qnan}, odd = 0.0f;
 #pragma unroll
         for (int dy = 0; dy <= kBrick; ++dy) {
             const int y = by * kBrick + dy;
@@ -286,6 +287,8 @@ __global__ void __launch_bounds__(kRowCols * kRowSlices, 2) k_lod(RowsArgs A) {
         s_half[dz][1][tx] = ymx[0];
         s_half[dz][2][tx] = ymn[1];
         s_half[dz][3][tx] = ymx[1];
+        s_odd[dz][tx] = odd;
+        all_odd += odd;
         __syncthreads();
         if (dz == 0) {
             // (y half, z half) h = j + 2i: slices 0..4 make z half 0, slices 4..8 z half 1
@@ -303,6 +306,12 @@ __global__ void __launch_bounds__(kRowCols * kRowSlices, 2) k_lod(RowsArgs A) {
 #pragma unroll
                 for (int h = 0; h < 4; ++h)
                     fold(mn[h], mx[h], __shfl_xor_sync(0xffffffffu, mn[h], m), __shfl_xor_sync(0xffffffffu, mx[h], m));
+            // a NaN or infinite value in any of the column's rows marks its four sub-bricks
+            float any = 0.0f;
+#pragma unroll
+            for (int sl = 0; sl < kRowSlices; ++sl) any += s_odd[sl][tx];
+#pragma unroll
+            for (int m = 1; m < G; m <<= 1) any += __shfl_xor_sync(0xffffffffu, any, m);
             const bool tcol = t < ncol;
             const int sx = t / G;
             if (tcol && t % G == 0) {
@@ -310,9 +319,10 @@ __global__ void __launch_bounds__(kRowCols * kRowSlices, 2) k_lod(RowsArgs A) {
                 for (int h = 0; h < 4; ++h) {
                     const int sy = 2 * by + (h & 1), sz = 2 * bz + (h >> 1);
                     if (sy < nsb && sz < nsb && sx < nsb) {
-                        const size_t sb = ((size_t)sz * nsb + sy) * nsb + sx;
+                        const size_t sb = ((size_t)sz * nsb + sy) * nsb + sx, nsub = (size_t)nsb * nsb * nsb;
                         A.sbmin[sb * A.nvars + v] = mn[h];
                         A.sbmax[sb * A.nvars + v] = mx[h];
+                        A.stats.odd[v * nsub + sb] = any != any;
                     }
                 }
             }
@@ -331,7 +341,7 @@ __global__ void __launch_bounds__(kRowCols * kRowSlices, 2) k_lod(RowsArgs A) {
         }
         __syncthreads();                                 // s_half is rewritten by the next column chunk
     }
-    level_stats(A.stats, v, odd, mag, dz == 0);
+    level_stats(A.stats.mag, v, all_odd, mag, dz == 0);
 }
 
 // Ingest and brick passes, by MODE: 0 ingest (the converted source, element type SRC), 2 ingest
@@ -433,15 +443,17 @@ __global__ void __launch_bounds__(kQuadThreads, quad_blocks(MODE, SRC)) k_quads(
     // sub-bricks, then bricks
 #pragma unroll
     for (int m = 1; m < G; m <<= 1) fold(mn, mx, __shfl_xor_sync(0xffffffffu, mn, m), __shfl_xor_sync(0xffffffffu, mx, m));
+    const unsigned om = __ballot_sync(0xffffffffu, odd != odd) >> (lane & ~(G - 1));
     if (valid && t % G == 0 && y0 < n && z0 < n) {
         const size_t sb = ((size_t)(z0 >> 2) * nsb + (y0 >> 2)) * nsb + t / G;
         A.sbmin[sb * A.nvars + v] = mn;
         A.sbmax[sb * A.nvars + v] = mx;
+        A.stats.odd[(size_t)v * nsb * nsb * nsb + sb] = (om & ((1u << G) - 1u)) != 0u;
     }
     s_mn[quad][lane] = y0 < n ? mn : qnan;                   // an absent quadrant adds nothing
     s_mx[quad][lane] = y0 < n ? mx : qnan;
     __syncthreads();
-    level_stats(A.stats, v, odd, 0.0f, false);
+    level_stats(A.stats.mag, v, odd, 0.0f, false);
     if (quad != 0) return;
 #pragma unroll
     for (int q = 1; q < 4; ++q) fold(mn, mx, s_mn[q][lane], s_mx[q][lane]);
@@ -451,7 +463,7 @@ __global__ void __launch_bounds__(kQuadThreads, quad_blocks(MODE, SRC)) k_quads(
         A.bmin[b * A.nvars + v] = mn;
         A.bmax[b * A.nvars + v] = mx;
     }
-    level_stats(A.stats, v, 0.0f, fmaxf(fabsf(mn), fabsf(mx)), true);
+    level_stats(A.stats.mag, v, 0.0f, fmaxf(fabsf(mn), fabsf(mx)), true);
 }
 
 template <int DT, int MODE, int SRC, int VEC>
@@ -507,7 +519,7 @@ cudaError_t launch_rows(const RowsArgs& a, int dtype, cudaStream_t stream) {
 
 cudaError_t launch_ingest(const void* src, int src_dtype, void* cells, void* pairs, int dtype, int n,
                           int nvars, float* bmin, float* bmax, float* sbmin, float* sbmax,
-                          unsigned* stats, cudaStream_t stream) {
+                          LevelStats stats, cudaStream_t stream) {
     RowsArgs a{};
     a.src = src;
     a.src_dtype = src_dtype;
@@ -529,7 +541,7 @@ bool ingest_next_level_fits(const void* src, int n) {
 
 cudaError_t launch_ingest_next_level(const void* src, int src_dtype, void* cells, void* pairs, int dtype, int n,
                                      int nvars, float* bmin, float* bmax, float* sbmin, float* sbmax,
-                                     void* next_cells, void* next_pairs, unsigned* stats, cudaStream_t stream) {
+                                     void* next_cells, void* next_pairs, LevelStats stats, cudaStream_t stream) {
     RowsArgs a{};
     a.src = src;
     a.src_dtype = src_dtype;
@@ -548,7 +560,7 @@ cudaError_t launch_ingest_next_level(const void* src, int src_dtype, void* cells
 }
 
 cudaError_t launch_level_bricks(const void* cells, int dtype, int n, int nvars, float* bmin, float* bmax,
-                                float* sbmin, float* sbmax, void* next_cells, void* next_pairs, unsigned* stats,
+                                float* sbmin, float* sbmax, void* next_cells, void* next_pairs, LevelStats stats,
                                 cudaStream_t stream) {
     RowsArgs a{};
     a.src = cells;
@@ -566,7 +578,7 @@ cudaError_t launch_level_bricks(const void* cells, int dtype, int n, int nvars, 
 }
 
 cudaError_t launch_lod(const void* fine, int n_fine, void* cells, void* pairs, int dtype, int nvars,
-                       float* bmin, float* bmax, float* sbmin, float* sbmax, unsigned* stats, cudaStream_t stream) {
+                       float* bmin, float* bmax, float* sbmin, float* sbmax, LevelStats stats, cudaStream_t stream) {
     RowsArgs a{};
     a.src = fine;
     a.n_src = n_fine;
