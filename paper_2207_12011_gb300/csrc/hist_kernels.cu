@@ -1045,20 +1045,28 @@ __global__ void __launch_bounds__(kHistVecThreads, 2) k_hist_bins(const __grid_c
 // (count_pitch) 385 -> 327 us, predicated adds 327 -> 286 us.
 //
 // Counters are 32 bits where they fit (kPairBytes), else 16 bits, two to a word. A
-// 16-bit count cannot overflow: a thread adds the 8 cells of a unit, and if one of its
-// counters then stood at 2^15 or more it moves 2^15 of it to the output
-// (compare-and-swap; unless another thread did) before it adds anything again, so
-// at most 8 kPairThreads single counts stand above 2^15 at any time.
+// 16-bit count cannot overflow: the thread whose add makes it 2^15 moves 2^15 of it to
+// the output, and should that take long, so does every thread that finds it at kFull16 or
+// more, before it adds anything again (a thread adds the 8 cells of a unit at a time), so
+// at most 8 kPairThreads single counts stand above kFull16 at any time. A move clears the
+// counter's top bit: whoever finds it set owns the 2^15, and nobody tries twice. Adds of
+// a warp to one 16-bit counter serialise (the hardware merges adds of 1 to 32-bit ones),
+// so a warp with kSameUnits or more units of a single bin pair each adds those units
+// whole. A constant field at 512^3 FP16, 256 bins: 2138 us with every thread above
+// 2^15 in a compare-and-swap loop, 1347 with the moves as they are, 520 with whole units
+// (32-bit counters: 559); a smooth one 558, now 561.
 constexpr int kPairThreads = 1024;
 constexpr size_t kPairBytes = (size_t)200 << 10;    // shared memory for the counters of a block
 constexpr unsigned kCountBatch = 8;                 // chunks a warp takes at a time, four lanes each
+constexpr int kSameUnits = 8;                       // units of one bin pair in a warp from which they are added whole
 constexpr unsigned kCountWorth = 64;                // chunks left per block for which changing the pair pays
                                                     // (its clearing and adding up take about 10 us)
 constexpr size_t kListBytes = (size_t)512 << 20;    // bins of one slab
 constexpr long long kListGrid = 1ll << 21, kListGridBrush = 1ll << 25;   // see hist_by_list
 constexpr size_t kListWarps = 160 * 2 * kHistVecWarps;   // most warps of a launch that lists
 constexpr int kListHead = 64;                       // bytes: row counter, chunks taken, chunks counted of each pair
-static_assert(0x8000 + 8 * kPairThreads <= 0x10000, "16-bit counters");
+constexpr unsigned kFull16 = 0xc000;                // see k_hist_count
+static_assert(kFull16 + 8 * kPairThreads <= 0x10000, "16-bit counters");
 static_assert(4 * (2 + kMaxVars - 1) <= kListHead, "list head");
 
 struct CountArgs {
@@ -1088,19 +1096,11 @@ __device__ __forceinline__ unsigned add_if(bool kept, unsigned addr, unsigned v)
     return old;
 }
 
-// A 16-bit counter last seen in its word cur: 2^15 of it to the output while it holds as much.
-__device__ __noinline__ void move_high(unsigned* hist, unsigned words, uint32_t* out, unsigned key, unsigned cur) {
-    const bool high = key >= words;
-    unsigned* w = hist + (high ? key - words : key);
-    const unsigned sh = high ? 16u : 0u;
-    while (((cur >> sh) & 0xffffu) >= 0x8000u) {
-        const unsigned seen = atomicCAS(w, cur, cur - (0x8000u << sh));
-        if (seen == cur) {
-            atomicAdd(out, 0x8000u);
-            return;
-        }
-        cur = seen;
-    }
+// A 16-bit counter (top: its highest bit) that an add has taken from `was` to `at`: 2^15 of
+// it to the output, if it is this thread's to move and still there.
+__device__ __noinline__ void move_high(unsigned* word, unsigned top, unsigned was, unsigned at, uint32_t* out) {
+    if (at >= 0x8000u && (was < 0x8000u || at >= kFull16))
+        if (atomicAnd(word, ~top) & top) atomicAdd(out, 0x8000u);
 }
 
 template <typename BIN, bool WIDE>
@@ -1141,8 +1141,26 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_hist_count(CountArgs A) {
             for (int step = 0; step < 8; ++step) {
                 unsigned mn = 0u, an[kWords] = {}, bn[kWords] = {};
                 if (any && step < 7) load(step + 1, mn, an, bn);
-                unsigned key[8], cur[8], over = 0u;
                 constexpr int kPer = 4 / (int)sizeof(BIN), kBits = 8 * (int)sizeof(BIN);
+                if constexpr (!WIDE) {
+                    // a unit of one bin pair: one add (see above)
+                    constexpr unsigned kEach = sizeof(BIN) == 1 ? 0x01010101u : 0x00010001u;
+                    unsigned differ = 0u;
+#pragma unroll
+                    for (int i = 1; i < kWords; ++i) differ |= (a[0] ^ a[i]) | (b[0] ^ b[i]);
+                    if (__popc(__ballot_sync(kFull, differ == 0u && m != 0u)) >= kSameUnits) {
+                        const unsigned x = a[0] & ((1u << kBits) - 1u), y = b[0] & ((1u << kBits) - 1u);
+                        if (differ == 0u && m && a[0] == x * kEach && b[0] == y * kEach) {
+                            const unsigned k = x * pitch + y, sh = k >= words ? 16u : 0u, count = __popc(m);
+                            unsigned* word = s_hist + (sh ? k - words : k);
+                            const unsigned at = ((atomicAdd(word, count << sh) >> sh) & 0xffffu) + count;
+                            if (at >= 0x8000u) move_high(word, 0x8000u << sh, at - count, at, out + x * bins + y);
+                            m = 0u;
+                        }
+                    }
+                }
+                unsigned key[8], cur[8], over = 0u;
+                if (WIDE || __any_sync(kFull, m != 0u)) {
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const unsigned x = (a[j / kPer] >> (kBits * (j % kPer))) & ((1u << kBits) - 1u);
@@ -1161,8 +1179,14 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_hist_count(CountArgs A) {
                     if (over & 0x80008000u) {
 #pragma unroll
                         for (int j = 0; j < 8; ++j)
-                            if (((m >> j) & 1u) && (cur[j] & 0x80008000u)) move_high(s_hist, words, out + (key[j] / pitch) * bins + key[j] % pitch, key[j], cur[j]);
+                            if (((m >> j) & 1u) && (cur[j] & 0x80008000u)) {
+                                const bool high = key[j] >= words;
+                                const unsigned at = high ? cur[j] >> 16 : cur[j] & 0xffffu;
+                                move_high(s_hist + (high ? key[j] - words : key[j]), high ? 0x80000000u : 0x8000u, at - 1u, at,
+                                          out + (key[j] / pitch) * bins + key[j] % pitch);
+                            }
                     }
+                }
                 }
                 m = mn;
 #pragma unroll
