@@ -872,7 +872,7 @@ raypc_status raypc_pc_histogram(raypc_ctx* ctx, int vol, int lod, const int* axi
     h.out = out_counts_dev;
     h.sactive = use_activity ? L->sactive : nullptr;
     h.nsb = L->nsb;
-    if (e == cudaSuccess && hist_by_list(h, V->dtype) && ctx->room(hist_list(h).bytes) &&
+    if (e == cudaSuccess && hist_by_list(h) && ctx->room(hist_list(h).bytes) &&
         ctx->scratch(&h.list, hist_list(h).bytes, s) != cudaSuccess) {
         cudaGetLastError();
         h.list = nullptr;

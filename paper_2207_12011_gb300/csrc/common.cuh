@@ -406,7 +406,7 @@ struct HistList {
     size_t bins_at, bytes;
 };
 HistList hist_list(const HistArgs& h);
-bool hist_by_list(const HistArgs& h, int dtype);
+bool hist_by_list(const HistArgs& h);
 
 // World box that the samples assigned to brick b of edge bs (lower
 // interpolation index in [bs b, bs b + bs)) can occupy along one axis, widened

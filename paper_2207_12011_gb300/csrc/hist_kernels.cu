@@ -1247,10 +1247,9 @@ __global__ void __launch_bounds__(256) k_hist_reduce(const uint4* __restrict__ c
 }
 
 // Kernel view of h. False when the edge table is neither small enough for the
-// launch parameters nor on the device; vec_slots reports whether the load
-// slots fit the vector kernel.
+// launch parameters nor on the device.
 template <int DT>
-bool fill_launch(const HistArgs& h, HistLaunch& a, bool& vec_slots) {
+bool fill_launch(const HistArgs& h, HistLaunch& a) {
     a.cells = h.cells;
     a.n = h.n;
     a.bins = h.bins;
@@ -1274,8 +1273,8 @@ bool fill_launch(const HistArgs& h, HistLaunch& a, bool& vec_slots) {
         a.guess_scale[i] = h.guess_scale[i] / (float)h.bins;
         a.guess_off[i] = -h.guess_e0[i] * a.guess_scale[i];
     }
-    // load slots of the vector kernel: the axes, then the brushed variables that are no axis
-    vec_slots = true;
+    // load slots of the vector kernel: the axes, then the brushed variables that are no axis (those
+    // that fit: see load_slots)
     a.nslot = h.naxes;
     for (int i = 0; i < h.naxes && i < kMaxVars; ++i) {
         a.svar[i] = h.axis[i] >= kPosAxisBase ? -1 : h.axis[i];
@@ -1287,7 +1286,7 @@ bool fill_launch(const HistArgs& h, HistLaunch& a, bool& vec_slots) {
         for (int i = 0; i < h.naxes; ++i)
             if (a.svar[i] == a.bvar[k]) { s = i; break; }
         if (s < 0) {
-            if (a.nslot >= kMaxVars) { vec_slots = false; break; }
+            if (a.nslot >= kMaxVars) break;
             s = a.nslot++;
             a.svar[s] = a.bvar[k];
         }
@@ -1377,11 +1376,21 @@ cudaError_t launch_count(const CountArgs& c, int sms, cudaStream_t stream) {
     return cudaGetLastError();
 }
 
+// Load slots that the vector kernels would take: the axes, and the brushed variables that are no axis.
+int load_slots(const HistArgs& h) {
+    int slots = h.naxes;
+    for (int v = 0; h.use_brush && v < h.nvars && v < kMaxVars; ++v) {
+        bool axis = !((h.brush.mask >> v) & 1u);
+        for (int i = 0; i < h.naxes; ++i) axis = axis || h.axis[i] == v;
+        if (!axis) ++slots;
+    }
+    return slots;
+}
+
 // Vector kernels' conditions: 16-byte aligned planes (an even edge makes n^3 a multiple of 8)
 // and load slots that fit; the group walk also needs whole chunks and sub-bricks per row.
-template <int DT>
-bool vector_walk(const HistArgs& h, bool vec_slots) {
-    return vec_slots && h.n % 2 == 0 && (reinterpret_cast<uintptr_t>(h.cells) & 15u) == 0;
+bool vector_walk(const HistArgs& h) {
+    return h.n % 2 == 0 && (reinterpret_cast<uintptr_t>(h.cells) & 15u) == 0 && load_slots(h) <= kMaxVars;
 }
 
 // Whether a call counts every in-shell cell by stored values alone.
@@ -1395,8 +1404,7 @@ bool lists_whole_rows(const HistArgs& h) {
 template <int DT>
 cudaError_t launch_t(const HistArgs& h, cudaStream_t stream) {
     HistLaunch a{};                      // about 8.6 KB with the inline edges (host stack)
-    bool vec_slots = true;
-    if (!fill_launch<DT>(h, a, vec_slots)) return cudaErrorInvalidValue;
+    if (!fill_launch<DT>(h, a)) return cudaErrorInvalidValue;
     const int ne = h.naxes * (h.bins + 1);
     if (h.s_out < 0) return cudaSuccess;                 // no cell in the shell: the zeroed output is the answer
     constexpr int VEC = DT == kF16 ? 8 : 4;
@@ -1405,7 +1413,7 @@ cudaError_t launch_t(const HistArgs& h, cudaStream_t stream) {
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const int rows = a.n * a.n;
-    if (!vector_walk<DT>(h, vec_slots)) {
+    if (!vector_walk(h)) {
         a.rot = 0;
         a.rowctr = nullptr;
         return launch_k(k_hist_scalar<DT>, a, kHistThreads, sizeof(float) * (size_t)ne, rows, sms, stream);
@@ -1491,8 +1499,8 @@ HistList hist_list(const HistArgs& h) {
 // atomics. Listed / direct, us: whole shell 128^3 FP32 58 / 62, 160^3 FP16 67 / 86, 512^3 535 /
 // 1293; brushed, after a render has
 // filled the caches, 256^3 FP16 83 / 77, 256^3 FP32 97 / 99 (a whole step with it 1031 / 1017), 512^3 315 / 400.
-bool hist_by_list(const HistArgs& h, int dtype) {
-    return (long long)h.n * h.n * h.n >= (h.use_brush ? kListGridBrush : kListGrid) && h.n % 2 == 0 && (reinterpret_cast<uintptr_t>(h.cells) & 15u) == 0 &&
+bool hist_by_list(const HistArgs& h) {
+    return (long long)h.n * h.n * h.n >= (h.use_brush ? kListGridBrush : kListGrid) && vector_walk(h) &&
            count_bytes(h.bins, false) <= kPairBytes;
 }
 

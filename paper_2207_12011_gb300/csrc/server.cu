@@ -222,7 +222,7 @@ raypc_status launch_hist(raypc_server* S, Req* q, int si) {
     // scratch: the list of bins from the context's pool (large grids); without it the partial
     // copies and their row counter in the stream's scratch, then the sub-brick bits
     const size_t count = (size_t)(naxes - 1) * bins * bins;
-    if (e == cudaSuccess && hist_by_list(h, V->dtype) && S->ctx->room(hist_list(h).bytes) &&
+    if (e == cudaSuccess && hist_by_list(h) && S->ctx->room(hist_list(h).bytes) &&
         S->ctx->scratch(&h.list, hist_list(h).bytes, s) != cudaSuccess) {
         cudaGetLastError();
         h.list = nullptr;

@@ -60,3 +60,27 @@ def test_even_edges_take_no_longer_than_odd_ones(rp):
 
     ms(250)
     assert ms(250) < 1.5 * ms(251)
+
+
+def test_more_slots_than_the_chunked_kernel_has(rp):
+    """A large brushed call with more axes and brushed variables than fit the chunked kernel's load slots
+    takes no list: its counts spread over copies, which a second kernel sums."""
+    n, bins = 324, 64
+    vol = synth.make_shell_volume(n, device="cuda").half()
+    order = (0, rp.AXIS_POS(rp.POS_R), 2, rp.AXIS_POS(rp.POS_X), rp.AXIS_POS(rp.POS_Y), rp.AXIS_POS(rp.POS_Z))
+    edges = np.array(synth.make_edges(vol.float(), (0, 0, 2, 0, 0, 0), bins), dtype=np.float32)
+    edges[1] = np.linspace(0.5, 1, bins + 1)
+    edges[3:] = np.linspace(-1, 1, bins + 1)
+    brush = synth.make_brush(vol.float(), "c3")
+    mask = brush.active_mask | 0b111010                      # four brushed variables beside the two axes
+    with rp.Context(0) as ctx:
+        v = ctx.load_volume(vol, store="f16", r_in=R_IN, r_out=R_OUT)
+        v.build_bricks()
+        v.set_brush(brush.lo, brush.hi, mask)
+        v.pc_histogram(order, edges)
+        before = rp.kernel_launches()
+        got = v.pc_histogram(order, edges).cpu().numpy().astype(np.uint32)
+        assert rp.kernel_launches() - before == 2
+        st = vol.float().cpu().numpy()
+        want = oracle.histogram(st, R_IN, R_OUT, brush.lo, brush.hi, mask, order, edges, use_brush=True)[0]
+        assert np.array_equal(got, want)
