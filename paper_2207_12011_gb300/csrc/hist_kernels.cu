@@ -748,8 +748,7 @@ struct ListSlots {
     }
 };
 
-// Vector kernel (grid edge a multiple of the chunk, 16-byte aligned planes, at most
-// kMaxVars load slots). While a warp tests and bins one chunk of its walk (32 lanes x
+// Vector kernel (even grid edge, 16-byte aligned planes, at most kMaxVars load slots). While a warp tests and bins one chunk of its walk (32 lanes x
 // 16 bytes, 8 FP16 or 4 FP32 cells per lane) it has the next one's slots copied
 // into its other shared buffer with cp.async (only chunks with a cell that passes
 // the shell, sub-brick and position tests), so HBM latency hides behind the
@@ -1094,11 +1093,15 @@ struct CountArgs {
 // Counter (x, y) of a pair has the key x * pitch + y. The pitch is 11 mod 32, so that the
 // counters around one another, which cells around one another hit, lie in different banks;
 // 16-bit counters k and k + words share a word for the same reason, not k and k + 1.
-__host__ __device__ __forceinline__ unsigned count_pitch(int bins) { return (unsigned)(bins + ((11 - bins) & 31)); }
-__host__ __device__ __forceinline__ unsigned count_words(int bins, bool wide) {
+__host__ __device__ constexpr unsigned count_pitch(int bins) { return (unsigned)(bins + ((11 - bins) & 31)); }
+__host__ __device__ constexpr unsigned count_words(int bins, bool wide) {
     const unsigned keys = (unsigned)bins * count_pitch(bins);
     return wide ? keys : (keys + 1u) / 2u;
 }
+// Most bins of 32-bit counters, and of 16-bit ones (of lists).
+constexpr int kWideBins = 217, kListBins = 309;
+static_assert(4 * count_words(kWideBins, true) <= kPairBytes && 4 * count_words(kWideBins + 1, true) > kPairBytes &&
+              4 * count_words(kListBins, false) <= kPairBytes && 4 * count_words(kListBins + 1, false) > kPairBytes, "counters");
 
 // Adds to a shared word (its shared-space address) if kept, predicated instead of branched around;
 // its value before, or 0.
@@ -1366,7 +1369,7 @@ HistKernel list_kernel(int nax, bool groups) {
 size_t count_bytes(int bins, bool wide) { return sizeof(unsigned) * (size_t)count_words(bins, wide); }
 
 cudaError_t launch_count(const CountArgs& c, int sms, cudaStream_t stream) {
-    const bool wide = count_bytes(c.bins, true) <= kPairBytes;          // bins <= 224
+    const bool wide = c.bins <= kWideBins;
     const size_t smem = count_bytes(c.bins, wide);
     const auto kernel = c.bins > 256 ? k_hist_count<unsigned short, false> : wide ? k_hist_count<unsigned char, true> : k_hist_count<unsigned char, false>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1494,14 +1497,13 @@ HistList hist_list(const HistArgs& h) {
     return L;
 }
 
-// Large grids on the vector path whose pair histogram fits a block (up to 310 bins). On smaller
+// Large grids on the vector path whose pair histogram fits a block (up to kListBins bins). On smaller
 // ones the second kernel and the blocks' clearing and adding up cost more than the
 // atomics. Listed / direct, us: whole shell 128^3 FP32 58 / 62, 160^3 FP16 67 / 86, 512^3 535 /
 // 1293; brushed, after a render has
 // filled the caches, 256^3 FP16 83 / 77, 256^3 FP32 97 / 99 (a whole step with it 1031 / 1017), 512^3 315 / 400.
 bool hist_by_list(const HistArgs& h) {
-    return (long long)h.n * h.n * h.n >= (h.use_brush ? kListGridBrush : kListGrid) && vector_walk(h) &&
-           count_bytes(h.bins, false) <= kPairBytes;
+    return (long long)h.n * h.n * h.n >= (h.use_brush ? kListGridBrush : kListGrid) && vector_walk(h) && h.bins <= kListBins;
 }
 
 int hist_copies(int n, int naxes, int bins) {
