@@ -1332,11 +1332,16 @@ bool fill_launch(const HistArgs& h, HistLaunch& a) {
     return true;
 }
 
+// The limit of a kernel's dynamic shared memory is the process's, not the call's: it is always set to
+// the most that any call takes, because one set to a call's own size could be lowered by another
+// thread's call between here and the launch.
+constexpr size_t kMostShared = sizeof(float) * ((kMaxVars * (1024 + 1) + 3) & ~3) + (size_t)kHistVecWarps * (2 * kMaxVars * 512 + 256);
+
 template <typename K>
 cudaError_t launch_k(K kernel, const HistLaunch& a, int threads, size_t smem, long long items, int sms, cudaStream_t stream) {
     int per_sm = 0;
     cudaError_t e = cudaSuccess;
-    if (smem > 48 * 1024) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem > 48 * 1024) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMostShared);
     // persistent grid: as many blocks as fit at once
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
     if (e != cudaSuccess) return e;
@@ -1372,7 +1377,7 @@ cudaError_t launch_count(const CountArgs& c, int sms, cudaStream_t stream) {
     const bool wide = c.bins <= kWideBins;
     const size_t smem = count_bytes(c.bins, wide);
     const auto kernel = c.bins > 256 ? k_hist_count<unsigned short, false> : wide ? k_hist_count<unsigned char, true> : k_hist_count<unsigned char, false>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairBytes);
     if (e != cudaSuccess) return e;
     kernel<<<std::max(sms, c.naxes - 1), kPairThreads, smem, stream>>>(c);
     count_launches(1);
