@@ -160,7 +160,11 @@ raypc_status raypc_create(raypc_ctx **out, int device, size_t hbm_budget_bytes);
 /* Free every volume and the context. NULL is accepted. */
 raypc_status raypc_destroy(raypc_ctx *ctx);
 
-/* Bytes of device memory the context currently holds. */
+/* Bytes of device memory the context currently holds: volumes, levels, bricks and
+ * batches, and the scratch of single calls that it keeps for the next ones (up to
+ * 640 MB after a histogram of a large grid, see raypc_pc_histogram; given back
+ * when a context of the library on this device needs the memory, and by
+ * raypc_destroy). */
 raypc_status raypc_memory_used(raypc_ctx *ctx, size_t *out_bytes);
 
 /* ---------------------------------------------------------------------- */
@@ -517,7 +521,11 @@ raypc_status raypc_get_tuning(raypc_ctx *ctx, int dtype, int n, raypc_tuning *ou
  * position brush. Its bin on axis a is
  * the number of interior edges e_1..e_{bins-1} of row a that are <= its value.
  * out_counts_dev ([naxes-1][bins][bins] uint32, caller-owned) is zeroed and
- * filled: H[p][bin_p][bin_{p+1}] counts cells. Counts are exact integers. */
+ * filled: H[p][bin_p][bin_{p+1}] counts cells. Counts are exact integers.
+ * Grids from 128^3 (brushed: about 324^3) of even edge with up to 309 bins take
+ * scratch for a list of the cells' bins, at most about 575 MB, from memory that
+ * the context keeps between calls; where that does not fit the budget or the
+ * device, or for other calls, they take at most 32 MB. */
 raypc_status raypc_pc_histogram(raypc_ctx *ctx, int vol, int lod, const int *axis_order,
                                 int naxes, int bins, const float *edges, int use_brush,
                                 uint32_t *out_counts_dev, void *stream);

@@ -9,10 +9,13 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <atomic>
 #include <map>
 #include <mutex>
 #include <string>
+#include <utility>
+#include <vector>
 
 #include "host_math.h"
 #include "runtime.h"
@@ -239,7 +242,7 @@ raypc_status ingest(raypc_ctx* ctx, Volume* V, const void* src, int src_is_devic
     }
     if (!src_is_device && !staged) {
         size_t src_bytes = nvox * V->nvars * elem_size(src_dtype);
-        e = cudaMallocAsync(&staging, src_bytes, s);
+        e = allocate(ctx->device, [&] { return cudaMallocAsync(&staging, src_bytes, s); });
         if (e != cudaSuccess) return cuda_fail(e, "staging allocation");
         e = cudaMemcpyAsync(staging, src, src_bytes, cudaMemcpyHostToDevice, s);
         if (e != cudaSuccess) { cudaFreeAsync(staging, s); return cuda_fail(e, "host to device copy"); }
@@ -276,6 +279,36 @@ void raypc::count_launches(int k) { g_launches.fetch_add((unsigned long long)k, 
 namespace raypc {
 
 void set_last_error(const char* msg) { g_err = msg; }
+
+namespace {
+std::mutex g_pools_mu;
+std::vector<std::pair<int, cudaMemPool_t>> g_pools;
+}  // namespace
+
+void pool_opened(int device, cudaMemPool_t pool) {
+    std::lock_guard<std::mutex> lk(g_pools_mu);
+    g_pools.emplace_back(device, pool);
+}
+
+void pool_closed(cudaMemPool_t pool) {
+    std::lock_guard<std::mutex> lk(g_pools_mu);
+    g_pools.erase(std::remove_if(g_pools.begin(), g_pools.end(), [&](const auto& p) { return p.second == pool; }), g_pools.end());
+}
+
+bool trim_pools(int device, bool wait) {
+    std::lock_guard<std::mutex> lk(g_pools_mu);
+    unsigned long long held = 0;
+    for (const auto& p : g_pools) {
+        unsigned long long v = 0;
+        if (p.first == device && cudaMemPoolGetAttribute(p.second, cudaMemPoolAttrReservedMemCurrent, &v) == cudaSuccess) held += v;
+    }
+    if (!held) return false;
+    if (wait) cudaDeviceSynchronize();
+    for (const auto& p : g_pools)
+        if (p.first == device) cudaMemPoolTrimTo(p.second, 0);
+    cudaGetLastError();
+    return true;
+}
 
 raypc_status get_volume(raypc_ctx* ctx, int vol, Volume** out) {
     auto it = ctx->vols.find(vol);
@@ -480,7 +513,10 @@ raypc_status raypc_destroy(raypc_ctx* ctx) {
         DeviceGuard g(ctx->device);
         for (auto& kv : ctx->vols) free_volume(ctx, kv.second);
         ctx->vols.clear();
-        if (ctx->pool) cudaMemPoolDestroy(ctx->pool);      // released once its last frees have run
+        if (ctx->pool) {
+            pool_closed(ctx->pool);
+            cudaMemPoolDestroy(ctx->pool);                 // released once its last frees have run
+        }
     }
     delete ctx;
     return RAYPC_OK;
@@ -489,7 +525,7 @@ raypc_status raypc_destroy(raypc_ctx* ctx) {
 raypc_status raypc_memory_used(raypc_ctx* ctx, size_t* out_bytes) {
     if (!ctx || !out_bytes) return fail(RAYPC_ERR_INVALID_ARG, "NULL argument");
     std::lock_guard<std::mutex> lk(ctx->mu);
-    *out_bytes = ctx->used;
+    *out_bytes = ctx->used + ctx->pool_held();
     return RAYPC_OK;
 }
 
@@ -872,11 +908,7 @@ raypc_status raypc_pc_histogram(raypc_ctx* ctx, int vol, int lod, const int* axi
     h.out = out_counts_dev;
     h.sactive = use_activity ? L->sactive : nullptr;
     h.nsb = L->nsb;
-    if (e == cudaSuccess && hist_by_list(h) && ctx->room(hist_list(h).bytes) &&
-        ctx->scratch(&h.list, hist_list(h).bytes, s) != cudaSuccess) {
-        cudaGetLastError();
-        h.list = nullptr;
-    }
+    if (e == cudaSuccess && hist_by_list(h)) h.list = ctx->spare_scratch(hist_list(h).bytes, s);
     const int ncopies = h.list || ((uintptr_t)out_counts_dev & 15u) ? 1 : hist_copies(L->n, naxes, bins);
     const size_t copy_bytes = sizeof(uint32_t) * (count * ncopies + 4);
     uint32_t* copies = nullptr;

@@ -6,6 +6,7 @@
 #include <stdarg.h>
 #include <stdio.h>
 
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <string>
@@ -106,6 +107,25 @@ inline size_t elem_size(int dtype) { return dtype == RAYPC_F16 ? 2 : 4; }
 raypc_status get_volume(raypc_ctx* ctx, int vol, Volume** out);
 raypc_status get_level(Volume* V, int lod, Level** out);
 
+// The contexts' scratch pools. trim_pools gives back what those of a device keep (with wait,
+// after the work in flight); false when they keep nothing.
+void pool_opened(int device, cudaMemPool_t pool);
+void pool_closed(cudaMemPool_t pool);
+bool trim_pools(int device, bool wait);
+
+// An allocation (f() -> cudaError_t) that the idle memory of the device's scratch pools must not
+// make fail: tried again without it.
+template <typename F>
+cudaError_t allocate(int device, F f) {
+    cudaError_t e = f();
+    for (int wait = 0; e == cudaErrorMemoryAllocation && wait < 2; ++wait) {
+        cudaGetLastError();
+        if (!trim_pools(device, wait != 0)) break;
+        e = f();
+    }
+    return e;
+}
+
 // Fill the march arguments of one render of level L of volume V (brush and
 // classification taken from V / L; callers may override them).
 raypc_status make_render_args(Volume* V, Level* L, const raypc_camera* cam, int w, int h,
@@ -151,6 +171,9 @@ struct raypc_ctx {
     // kScratchKept bytes between calls (the device's default pool gives everything back at each
     // synchronisation, and the next call maps its scratch anew). Safe on any stream; freed with
     // cudaFreeAsync on the stream that used it. Without a pool it comes from the default one.
+    // What the pool holds counts as memory used, and is given back when any context of the device
+    // needs it. At 512^3 FP16 a listed whole-shell histogram takes 1.20 ms when it maps its 540 MB
+    // and 0.53 ms when the pool holds them.
     cudaMemPool_t pool = nullptr;
     static constexpr unsigned long long kScratchKept = 640ull << 20;
     void open_pool() {
@@ -159,26 +182,44 @@ struct raypc_ctx {
         props.location.type = cudaMemLocationTypeDevice;
         props.location.id = device;
         unsigned long long keep = kScratchKept;
-        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) pool = nullptr;
-        else if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess) return;
-        cudaGetLastError();
+        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+            pool = nullptr;
+            cudaGetLastError();
+            return;
+        }
+        raypc::pool_opened(device, pool);
+        if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) cudaGetLastError();
     }
+    size_t pool_bytes(cudaMemPoolAttr what) const {
+        unsigned long long v = 0;
+        if (pool && cudaMemPoolGetAttribute(pool, what, &v) != cudaSuccess) cudaGetLastError();
+        return (size_t)v;
+    }
+    size_t pool_held() const { return pool_bytes(cudaMemPoolAttrReservedMemCurrent); }
     cudaError_t scratch(void** p, size_t bytes, cudaStream_t s) {
-        return pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s);
+        return raypc::allocate(device, [&] { return pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s); });
     }
-    // Room for scratch that a call can do without: within the budget, when there is one.
-    bool room(size_t bytes) const { return !budget || used + bytes <= budget; }
+    // Scratch that a call can do without (null: none), within the budget when there is one.
+    void* spare_scratch(size_t bytes, cudaStream_t s) {
+        void* p = nullptr;
+        if (budget && used + std::max(pool_held(), pool_bytes(cudaMemPoolAttrUsedMemCurrent) + bytes) > budget) return nullptr;
+        if ((pool ? cudaMallocFromPoolAsync(&p, bytes, pool, s) : cudaMallocAsync(&p, bytes, s)) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        if (budget && used + pool_held() > budget) {        // other streams' scratch is not free yet
+            cudaFreeAsync(p, s);
+            return nullptr;
+        }
+        return p;
+    }
 
     // Device allocation charged against the budget.
     raypc_status alloc(void** p, size_t bytes, size_t* charged) {
         if (budget && used + bytes > budget)
             return raypc::fail(RAYPC_ERR_OOM, "HBM budget exceeded: %zu used + %zu requested > %zu", used, bytes, budget);
-        cudaError_t e = cudaMalloc(p, bytes ? bytes : 16);
-        if (e == cudaErrorMemoryAllocation && pool) {     // what the pool keeps may make the room
-            cudaGetLastError();
-            e = cudaMemPoolTrimTo(pool, 0);
-            if (e == cudaSuccess) e = cudaMalloc(p, bytes ? bytes : 16);
-        }
+        if (budget && used + pool_held() + bytes > budget) cudaMemPoolTrimTo(pool, 0);   // idle scratch makes way
+        const cudaError_t e = raypc::allocate(device, [&] { return cudaMalloc(p, bytes ? bytes : 16); });
         if (e != cudaSuccess) return raypc::cuda_fail(e, "cudaMalloc");
         used += bytes;
         *charged += bytes;

@@ -222,11 +222,7 @@ raypc_status launch_hist(raypc_server* S, Req* q, int si) {
     // scratch: the list of bins from the context's pool (large grids); without it the partial
     // copies and their row counter in the stream's scratch, then the sub-brick bits
     const size_t count = (size_t)(naxes - 1) * bins * bins;
-    if (e == cudaSuccess && hist_by_list(h) && S->ctx->room(hist_list(h).bytes) &&
-        S->ctx->scratch(&h.list, hist_list(h).bytes, s) != cudaSuccess) {
-        cudaGetLastError();
-        h.list = nullptr;
-    }
+    if (e == cudaSuccess && hist_by_list(h)) h.list = S->ctx->spare_scratch(hist_list(h).bytes, s);
     const int ncopies = h.list || ((uintptr_t)q->hist & 15u) ? 1 : hist_copies(L->n, naxes, bins);
     const size_t copy_bytes = ncopies > 1 ? (sizeof(uint32_t) * (count * ncopies + 4) + 255) / 256 * 256 : 0;
     const bool activity = h.use_brush && L->sbmin;

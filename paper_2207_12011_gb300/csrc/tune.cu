@@ -143,14 +143,14 @@ raypc_status raypc_autotune(raypc_ctx* ctx, const raypc_view* views, int nviews,
         if ((st = pos_from_host(q.pos_lo, q.pos_hi, q.pos_mask, &args[i].brush))) break;
         finish_position_brush(args[i]);
         void* bits = nullptr;
-        cudaError_t e = cudaMalloc(&bits, L->nswords() * sizeof(uint32_t));
+        cudaError_t e = allocate(ctx->device, [&] { return cudaMalloc(&bits, L->nswords() * sizeof(uint32_t)); });
         if (e == cudaSuccess) temps.push_back(bits);
         // cell classes under the view's brush, as a single-view render uses them
         void* cls = nullptr;
-        if (e == cudaSuccess) e = cudaMalloc(&cls, (size_t)L->n * L->n * L->n * sizeof(uint16_t));
+        if (e == cudaSuccess) e = allocate(ctx->device, [&] { return cudaMalloc(&cls, (size_t)L->n * L->n * L->n * sizeof(uint16_t)); });
         if (e == cudaSuccess) temps.push_back(cls);
         void* dist = nullptr;                 // padded empty-space distance
-        if (e == cudaSuccess) e = cudaMalloc(&dist, padded_bytes(L->n));
+        if (e == cudaSuccess) e = allocate(ctx->device, [&] { return cudaMalloc(&dist, padded_bytes(L->n)); });
         if (e == cudaSuccess) temps.push_back(dist);
         if (e != cudaSuccess) { st = cuda_fail(e, "tuning buffers"); break; }
         BrushLaunch P{};
