@@ -617,8 +617,8 @@ raypc_status raypc_get_bricks(raypc_ctx *ctx, int vol, int lod, float *out_min_d
                               float *out_max_dev, void *stream);
 
 /* Copy a level's classification under the current brush (that of the 8^3 bricks
- * is computed by the first of these calls after a brush change: the renders and
- * histograms use the sub-bricks). active_bits_dev and
+ * is computed by each of these calls, for the brush at the time of the call: the
+ * renders and histograms use the sub-bricks). active_bits_dev and
  * skippable_bits_dev receive ceil(nb^3 / 32) uint32 words (bit b%32 of word
  * b/32 for brick b); active_list_dev (optional, nb^3 uint32) receives the ids
  * of the active bricks in increasing order and n_active_dev (optional, one

@@ -69,7 +69,7 @@ void free_bricks(Level& L) {
     L.sdist = nullptr;
     L.sdist_of = nullptr;
     L.stats.odd = nullptr;
-    L.bricks = L.classified = L.cls_valid = L.listed = false;
+    L.bricks = L.classified = L.cls_valid = false;
 }
 
 void free_staging(Volume* V) {
@@ -102,7 +102,7 @@ void free_volume(raypc_ctx* ctx, Volume* V) {
 // The classification is out of date (new values, levels or brush).
 void unclassify(Volume* V) {
     for (auto& L : V->lv) {
-        L.classified = L.cls_valid = L.listed = false;
+        L.classified = L.cls_valid = false;
         L.sdist_of = nullptr;
     }
 }
@@ -1146,23 +1146,22 @@ raypc_status raypc_get_skip_list(raypc_ctx* ctx, int vol, int lod, uint32_t* act
     cudaStream_t s = (cudaStream_t)stream;
     if (V->stale) return fail(RAYPC_ERR_INVALID_ARG, "volume updated: raypc_build_bricks must run first");
     if ((st = ensure_classified(V, *L, s))) return st;
-    if (!L->listed) {
-        BrickListArgs b{};
-        b.bmin = L->bmin;
-        b.bmax = L->bmax;
-        b.n = L->n;
-        b.nb = L->nb;
-        b.nvars = V->nvars;
-        b.rin2 = V->r_in * V->r_in;
-        b.rout2 = V->r_out * V->r_out;
-        b.brush = V->brush;
-        b.active = L->active;
-        b.skippable = L->skippable;
-        b.list = L->list;
-        b.n_active = L->n_active;
-        CK(launch_brick_list(b, s), "brick list kernels");
-        L->listed = true;
-    }
+    // by every call, in its own stream's order: a list kept from one call could be read before the
+    // stream that computes it gets there
+    BrickListArgs b{};
+    b.bmin = L->bmin;
+    b.bmax = L->bmax;
+    b.n = L->n;
+    b.nb = L->nb;
+    b.nvars = V->nvars;
+    b.rin2 = V->r_in * V->r_in;
+    b.rout2 = V->r_out * V->r_out;
+    b.brush = V->brush;
+    b.active = L->active;
+    b.skippable = L->skippable;
+    b.list = L->list;
+    b.n_active = L->n_active;
+    CK(launch_brick_list(b, s), "brick list kernels");
     size_t wb = L->nwords() * sizeof(uint32_t);
     if (active_bits_dev) CK(cudaMemcpyAsync(active_bits_dev, L->active, wb, cudaMemcpyDeviceToDevice, s), "copy active bits");
     if (skippable_bits_dev) CK(cudaMemcpyAsync(skippable_bits_dev, L->skippable, wb, cudaMemcpyDeviceToDevice, s), "copy skippable bits");

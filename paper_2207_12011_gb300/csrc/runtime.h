@@ -63,7 +63,6 @@ struct Level {
     bool cls_valid = false;
     bool bricks = false;
     bool classified = false;      // sactive is current
-    bool listed = false;          // active, skippable, list and n_active are current
     bool fresh = false;           // cells and pairs written by the last ingest of the finer level,
                                   // brick min/max not yet (raypc_build_bricks computes them)
     size_t nbricks() const { return (size_t)nb * nb * nb; }
