@@ -53,7 +53,7 @@ namespace {
 
 void free_level(Level& L) {
     void* ptrs[] = {L.cells, L.pairs, L.bmin, L.bmax, L.active, L.skippable, L.list, L.n_active,
-                    L.sbmin, L.sbmax, L.stats.odd, L.sactive, L.cls, L.tf_sactive, L.sdist};
+                    L.sbmin, L.sbmax, L.stats.odd, L.sactive, L.cls, L.tf_sactive, L.sdist, L.tf_sdist};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     L = Level{};
@@ -61,12 +61,12 @@ void free_level(Level& L) {
 
 void free_bricks(Level& L) {
     void* ptrs[] = {L.bmin, L.bmax, L.active, L.skippable, L.list, L.n_active,
-                    L.sbmin, L.sbmax, L.stats.odd, L.sactive, L.tf_sactive, L.sdist};
+                    L.sbmin, L.sbmax, L.stats.odd, L.sactive, L.tf_sactive, L.sdist, L.tf_sdist};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     L.bmin = L.bmax = L.sbmin = L.sbmax = nullptr;
     L.active = L.skippable = L.list = L.n_active = L.sactive = L.tf_sactive = nullptr;
-    L.sdist = nullptr;
+    L.sdist = L.tf_sdist = nullptr;
     L.sdist_of = nullptr;
     L.stats.odd = nullptr;
     L.bricks = L.classified = L.cls_valid = false;
@@ -741,23 +741,24 @@ raypc_status raypc_set_tf(raypc_ctx* ctx, int vol, const float* rgbs, int color_
 }
 
 // Empty-space distance of the sub-bricks under the activity bits the render reads (the
-// brush's, or the TF-visible ones with tf_skip): the grid the march searches. A render
-// without skipping only needs the activity, and reads the bits where the grid cannot be had.
-static raypc_status ensure_distance(raypc_ctx* ctx, Volume* V, Level& L, RenderArgs& a, bool recompute,
-                                    cudaStream_t s) {
-    if (!L.sdist) {
-        raypc_status st = ctx->alloc((void**)&L.sdist, padded_bytes(L.n), &V->bytes);
-        if (st) {
-            L.sdist = nullptr;
-            return a.skip ? st : RAYPC_OK;
-        }
-        L.sdist_of = nullptr;
+// brush's, or the TF-visible ones with tf_skip, in a grid of their own): the grid the march
+// searches. It is kept until the brush or the values change, but for tf_skip and for renders
+// without skipping: these only need the activity (they read the bits where the grid cannot be
+// had), so what they see is that of their own stream's order, also when a graph replays them.
+static raypc_status ensure_distance(raypc_ctx* ctx, Volume* V, Level& L, RenderArgs& a, bool tf, cudaStream_t s) {
+    uint8_t** grid = tf ? &L.tf_sdist : &L.sdist;
+    if (!*grid) {
+        const raypc_status st = ctx->alloc((void**)grid, padded_bytes(L.n), &V->bytes);
+        if (st) *grid = nullptr;
+        else if (!tf) L.sdist_of = nullptr;
+        if (st && tf && L.sdist) grid = &L.sdist;            // no room for two: the other one is stale then
+        else if (st) return a.skip ? st : RAYPC_OK;
     }
-    if (recompute || L.sdist_of != a.lv.sactive) {
-        CK(launch_subbrick_distance(a.lv.sactive, L.n, L.sdist, false, s), "empty-space distance");
-        L.sdist_of = a.lv.sactive;
+    if (tf || !a.skip || L.sdist_of != a.lv.sactive) {
+        CK(launch_subbrick_distance(a.lv.sactive, L.n, *grid, false, s), "empty-space distance");
+        if (grid == &L.sdist && (tf || a.skip)) L.sdist_of = tf ? nullptr : a.lv.sactive;
     }
-    a.lv.sdist = L.sdist;
+    a.lv.sdist = *grid;
     return RAYPC_OK;
 }
 

@@ -59,7 +59,8 @@ struct Level {
     uint16_t* cls = nullptr;      // cell classes under the current brush (n^3), computed on demand
     uint32_t* tf_sactive = nullptr;  // activity AND TF visibility (renders with tf_skip)
     uint8_t* sdist = nullptr;        // padded empty-space distance of the sub-bricks (renders)
-    const uint32_t* sdist_of = nullptr;   // activity bits the distance was computed from (null: stale)
+    uint8_t* tf_sdist = nullptr;     // the same under tf_sactive
+    const uint32_t* sdist_of = nullptr;   // activity bits that sdist was computed from (null: stale)
     bool cls_valid = false;
     bool bricks = false;
     bool classified = false;      // sactive is current
