@@ -333,6 +333,7 @@ void finish_position_brush(RenderArgs& a) {
         a.keep_hi2 = fminf(a.keep_hi2, H);
     }
     a.keep_lo2 = fminf(a.keep_lo2, 0x1p100f);          // finite (the core-jump bound scales it)
+    a.open = a.brush.mask == 0u && a.brush.pmask == 0u;
 }
 
 raypc_status make_render_args(Volume* V, Level* L, const raypc_camera* cam, int w, int h,
@@ -744,8 +745,10 @@ raypc_status raypc_set_tf(raypc_ctx* ctx, int vol, const float* rgbs, int color_
 // brush's, or the TF-visible ones with tf_skip, in a grid of their own): the grid the march
 // searches. It is kept until the brush or the values change, but for tf_skip and for renders
 // without skipping: these only need the activity (they read the bits where the grid cannot be
-// had), so what they see is that of their own stream's order, also when a graph replays them.
+// had, and nothing when nothing is restricted), so what they see is that of their own stream's
+// order, also when a graph replays them.
 static raypc_status ensure_distance(raypc_ctx* ctx, Volume* V, Level& L, RenderArgs& a, bool tf, cudaStream_t s) {
+    if (a.open && !a.skip) return RAYPC_OK;
     uint8_t** grid = tf ? &L.tf_sdist : &L.sdist;
     if (!*grid) {
         const raypc_status st = ctx->alloc((void**)grid, padded_bytes(L.n), &V->bytes);
@@ -779,6 +782,7 @@ static raypc_status apply_tf_skip(Volume* V, Level& L, const raypc_render_opts* 
     t.out_sactive = L.tf_sactive;
     CK(launch_tf_visibility(t, s), "TF visibility kernel");
     a.lv.sactive = L.tf_sactive;
+    a.open = 0;
     return RAYPC_OK;
 }
 

@@ -251,6 +251,7 @@ raypc_status raypc_render_batch(raypc_batch* b, const raypc_view* views, int nvi
         it.cls = b->cls[i];
         it.sdist = reinterpret_cast<uint8_t*>(b->bits[i] + words);
         if (q.opts.tf_skip) {
+            a.open = 0;
             it.tf_prefix = V->tf_prefix;
             it.color_var = V->color_var;
             it.tf_lo = a.tf_lo;

@@ -252,6 +252,7 @@ struct RenderArgs {
     float bg[4];
     int ert, skip;
     float jump[3];                // samples to skip at distance >= 2, 4 and kDistCap (whole numbers)
+    int open;                     // nothing is restricted: every sample of the shell is in an active sub-brick
     int narrow;                   // every sample has -1 <= u < n on each axis (r_out <= 1, a nearby eye)
                                   // and a pair plane has less than 2^32 bytes
     int variant;                  // 1..kNumVariants (tile shape of the launch)
