@@ -67,7 +67,9 @@ typedef int raypc_status;
 #define RAYPC_STAT_MARCHED 0      /* lattice samples from entry to termination  */
 #define RAYPC_STAT_EVALUATED 1    /* samples whose field values were fetched    */
 #define RAYPC_STAT_KEPT 2         /* samples in shell and in brush (composited) */
-#define RAYPC_STAT_SKIPPED 3      /* lattice samples jumped by brick skipping   */
+#define RAYPC_STAT_SKIPPED 3      /* lattice samples jumped over together by empty-space
+                                   * skipping; the up to 8 samples that are looked up
+                                   * before a jump do not count                  */
 #define RAYPC_STAT_RAYS 4         /* rays that hit the outer sphere             */
 #define RAYPC_STAT_ERT 5          /* rays ended by early ray termination        */
 #define RAYPC_NSTATS 8
@@ -281,8 +283,8 @@ raypc_status raypc_set_tf(raypc_ctx *ctx, int vol, const float *rgbs, int color_
  * The integer decisions use correctly rounded FP32 operations in one fixed
  * order, so they do not depend on skipping, tiling or launch shape. Samples
  * in inactive 4^3 sub-bricks are rejected before any interpolation; with
- * skipping on, a ray jumps over the rest of an inactive sub-brick (or of an
- * inactive 8^3 brick), and the jump never changes the image. Requires set_brush
+ * skipping on, rays that are far from any active sub-brick jump over the samples
+ * in between together, and the jump never changes the image. Requires set_brush
  * and set_tf.
  * stats_dev: optional RAYPC_NSTATS uint64 device counters the kernel adds to.
  * opts may be NULL only if the defaults with ert = 1 are wanted. */

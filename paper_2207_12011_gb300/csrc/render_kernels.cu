@@ -47,16 +47,6 @@ __device__ __forceinline__ bool bit_of(const uint32_t* bits, uint32_t id) {
     return (__ldg(bits + (id >> 5)) >> (id & 31)) & 1u;
 }
 
-// x-pair at byte address p.
-template <int DT> __device__ __forceinline__ float2 load_pair(const char* p);
-template <> __device__ __forceinline__ float2 load_pair<kF32>(const char* p) {
-    return __ldg(reinterpret_cast<const float2*>(p));
-}
-template <> __device__ __forceinline__ float2 load_pair<kF16>(const char* p) {
-    const unsigned w = __ldg(reinterpret_cast<const unsigned*>(p));
-    return __half22float2(*reinterpret_cast<const __half2*>(&w));
-}
-
 // Byte offsets inside one variable's x-pair plane: 32 bits when the plane is
 // smaller than 4 GB (WIDE = false), else 64.
 template <bool WIDE> struct Offset { using type = uint32_t; };
@@ -66,10 +56,10 @@ template <> struct Offset<true> { using type = size_t; };
 // (x0, x0+1) at (y0,z0), (y1,z0), (y0,z1), (y1,z1).
 template <int DT, typename OFF>
 __device__ __forceinline__ float interp_var(const char* plane, OFF base, OFF sy, OFF sz, float fx, float fy, float fz) {
-    const float2 a = load_pair<DT>(plane + base);
-    const float2 b = load_pair<DT>(plane + (OFF)(base + sy));
-    const float2 c = load_pair<DT>(plane + (OFF)(base + sz));
-    const float2 d = load_pair<DT>(plane + (OFF)(base + sz + sy));
+    const float2 a = Pair<DT>::load(plane + base, 0);
+    const float2 b = Pair<DT>::load(plane + (OFF)(base + sy), 0);
+    const float2 c = Pair<DT>::load(plane + (OFF)(base + sz), 0);
+    const float2 d = Pair<DT>::load(plane + (OFF)(base + sz + sy), 0);
     return trilerp_rn(a.x, a.y, b.x, b.y, c.x, c.y, d.x, d.y, fx, fy, fz);
 }
 
@@ -412,7 +402,7 @@ __global__ void __launch_bounds__(kThreads) k_render(RenderArgs A) {
     __shared__ ViewShared S;
     load_view_shared(A, S);
     __syncthreads();
-        march_pixel<DT, VAR, DEPTH, WIDE>(A, S, blockIdx.x, blockIdx.y, threadIdx.x >> 5);
+    march_pixel<DT, VAR, DEPTH, WIDE>(A, S, blockIdx.x, blockIdx.y, threadIdx.x >> 5);
 }
 
 // One view of a batch: the single-frame kernel (its arguments have to sit at a

@@ -474,8 +474,9 @@ void launch_quads_t(const RowsArgs& a, cudaStream_t stream) {
 
 template <int DT, int MODE, int SRC>
 void launch_quads_t(const RowsArgs& a, bool vec, cudaStream_t stream) {
-    if (vec || MODE == 2 || MODE == 4) launch_quads_t<DT, MODE, SRC, 4>(a, stream);
-    else launch_quads_t<DT, MODE == 2 ? 0 : MODE == 4 ? 3 : MODE, SRC, 1>(a, stream);
+    if constexpr (MODE == 2 || MODE == 4) launch_quads_t<DT, MODE, SRC, 4>(a, stream);
+    else if (vec) launch_quads_t<DT, MODE, SRC, 4>(a, stream);
+    else launch_quads_t<DT, MODE, SRC, 1>(a, stream);
 }
 
 template <int DT, int VEC>
