@@ -53,7 +53,7 @@ namespace {
 
 void free_level(Level& L) {
     void* ptrs[] = {L.cells, L.pairs, L.bmin, L.bmax, L.active, L.skippable, L.list, L.n_active,
-                    L.sbmin, L.sbmax, L.stats.odd, L.sactive, L.cls, L.tf_sactive, L.sdist, L.tf_sdist};
+                    L.sbmin, L.sbmax, L.sactive, L.cls, L.tf_sactive, L.sdist, L.tf_sdist};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     L = Level{};
@@ -61,7 +61,7 @@ void free_level(Level& L) {
 
 void free_bricks(Level& L) {
     void* ptrs[] = {L.bmin, L.bmax, L.active, L.skippable, L.list, L.n_active,
-                    L.sbmin, L.sbmax, L.stats.odd, L.sactive, L.tf_sactive, L.sdist, L.tf_sdist};
+                    L.sbmin, L.sbmax, L.sactive, L.tf_sactive, L.sdist, L.tf_sdist};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     L.bmin = L.bmax = L.sbmin = L.sbmax = nullptr;
@@ -156,8 +156,7 @@ raypc_status alloc_bricks(raypc_ctx* ctx, Volume* V, Level& L) {
     raypc_status st;
     if ((st = ctx->alloc((void**)&L.sbmin, smm, &V->bytes)) ||
         (st = ctx->alloc((void**)&L.sbmax, smm, &V->bytes)) ||
-        (st = ctx->alloc((void**)&L.stats.odd, L.nsbricks() * V->nvars, &V->bytes)) ||
-        (st = ctx->alloc((void**)&L.sactive, L.nswords() * sizeof(uint32_t), &V->bytes)) ||
+        (st = ctx->alloc((void**)&L.sactive, L.nswords() * sizeof(uint32_t) + L.nsbricks() * V->nvars, &V->bytes)) ||
         (st = ctx->alloc((void**)&L.tf_sactive, L.nswords() * sizeof(uint32_t), &V->bytes)) ||
         (st = ctx->alloc((void**)&L.bmin, mm, &V->bytes)) ||
         (st = ctx->alloc((void**)&L.bmax, mm, &V->bytes)) ||
@@ -168,6 +167,7 @@ raypc_status alloc_bricks(raypc_ctx* ctx, Volume* V, Level& L) {
         free_bricks(L);
         return st;
     }
+    L.stats.odd = reinterpret_cast<uint8_t*>(L.sactive + L.nswords());   // behind the words of the same allocation
     return RAYPC_OK;
 }
 
