@@ -744,11 +744,13 @@ raypc_status raypc_set_tf(raypc_ctx* ctx, int vol, const float* rgbs, int color_
 // Empty-space distance of the sub-bricks under the activity bits the render reads (the
 // brush's, or the TF-visible ones with tf_skip, in a grid of their own): the grid the march
 // searches. It is kept until the brush or the values change, but for tf_skip and for renders
-// without skipping: these only need the activity (they read the bits where the grid cannot be
-// had, and nothing when nothing is restricted), so what they see is that of their own stream's
-// order, also when a graph replays them.
-static raypc_status ensure_distance(raypc_ctx* ctx, Volume* V, Level& L, RenderArgs& a, bool tf, cudaStream_t s) {
+// asked to go without skipping: these only need the activity (they read the bits where the grid
+// cannot be had, and nothing when nothing is restricted), so what they see is that of their own
+// stream's order, also when a graph replays them.
+static raypc_status ensure_distance(raypc_ctx* ctx, Volume* V, Level& L, RenderArgs& a, const raypc_render_opts* opts,
+                                    cudaStream_t s) {
     if (a.open && !a.skip) return RAYPC_OK;
+    const bool tf = opts && opts->tf_skip, off = opts && opts->skip == RAYPC_SKIP_OFF;
     uint8_t** grid = tf ? &L.tf_sdist : &L.sdist;
     if (!*grid) {
         const raypc_status st = ctx->alloc((void**)grid, padded_bytes(L.n), &V->bytes);
@@ -757,9 +759,9 @@ static raypc_status ensure_distance(raypc_ctx* ctx, Volume* V, Level& L, RenderA
         if (st && tf && L.sdist) grid = &L.sdist;            // no room for two: the other one is stale then
         else if (st) return a.skip ? st : RAYPC_OK;
     }
-    if (tf || !a.skip || L.sdist_of != a.lv.sactive) {
+    if (tf || off || L.sdist_of != a.lv.sactive) {
         CK(launch_subbrick_distance(a.lv.sactive, L.n, *grid, false, s), "empty-space distance");
-        if (grid == &L.sdist && (tf || a.skip)) L.sdist_of = tf ? nullptr : a.lv.sactive;
+        if (grid == &L.sdist && (tf || !off)) L.sdist_of = tf ? nullptr : a.lv.sactive;
     }
     a.lv.sdist = *grid;
     return RAYPC_OK;
@@ -803,7 +805,7 @@ raypc_status raypc_render(raypc_ctx* ctx, int vol, int lod, const raypc_camera* 
     if ((st = ensure_cell_classes(ctx, V, *L, (cudaStream_t)stream))) return st;
     a.cls = L->cls;
     if ((st = apply_tf_skip(V, *L, opts, a, (cudaStream_t)stream))) return st;
-    if ((st = ensure_distance(ctx, V, *L, a, opts && opts->tf_skip, (cudaStream_t)stream))) return st;
+    if ((st = ensure_distance(ctx, V, *L, a, opts, (cudaStream_t)stream))) return st;
     CK(launch_render(a, V->dtype, (cudaStream_t)stream), "render kernel");
     return RAYPC_OK;
 }
@@ -833,7 +835,7 @@ raypc_status raypc_render_progressive(raypc_ctx* ctx, int vol, int lod, const ra
     a.accum = reinterpret_cast<float4*>(accum_rgba_dev);
     a.accum_w = 1.0f / (float)((double)pass + 1.0);
     if ((st = apply_tf_skip(V, *L, opts, a, (cudaStream_t)stream))) return st;
-    if ((st = ensure_distance(ctx, V, *L, a, opts && opts->tf_skip, (cudaStream_t)stream))) return st;
+    if ((st = ensure_distance(ctx, V, *L, a, opts, (cudaStream_t)stream))) return st;
     CK(launch_render(a, V->dtype, (cudaStream_t)stream), "render kernel");
     return RAYPC_OK;
 }
