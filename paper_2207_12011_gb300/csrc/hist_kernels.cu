@@ -21,9 +21,9 @@
 // which few can be merged (neighbouring cells of a 256-bin table rarely share a bin
 // pair) and many meet at hot bins. Large grids therefore list the cells' bins in HBM and
 // count them one pair at a time in shared memory (k_hist_count): 512^3 FP16, 6
-// axes, 256 bins, whole shell 1236 -> 525 us; 4 brushed variables 422 -> 313 us;
+// axes, 256 bins, whole shell 1401 -> 557 us; 4 brushed variables 422 -> 313 us;
 // 250^3 264 -> 115 us. Smaller grids, tables that do not fit and calls without scratch
-// add runs of cells with equal bins straight to L2, on large grids spread over
+// add runs of equal bins straight to L2 (see by_pair), on large grids spread over
 // partial histograms that a reduction sums.
 #include <math.h>
 #include <stdint.h>
@@ -1504,8 +1504,7 @@ HistList hist_list(const HistArgs& h) {
 
 // Large grids on the vector path whose pair histogram fits a block (up to kListBins bins). On smaller
 // ones the second kernel and the blocks' clearing and adding up cost more than the
-// atomics. Listed / direct, us: whole shell 128^3 FP32 58 / 62, 160^3 FP16 67 / 86, 512^3 535 /
-// 1293; brushed, after a render has
+// atomics. Listed / direct, us: whole shell 128^3 FP32 59 / 62, 256^3 FP32 141 / 189; brushed, after a render has
 // filled the caches, 256^3 FP16 83 / 77, 256^3 FP32 97 / 99 (a whole step with it 1031 / 1017), 512^3 315 / 400.
 bool hist_by_list(const HistArgs& h) {
     return (long long)h.n * h.n * h.n >= (h.use_brush ? kListGridBrush : kListGrid) && vector_walk(h) && h.bins <= kListBins;
