@@ -62,12 +62,6 @@ template <> __device__ __forceinline__ void load_run<kF32, 4>(const void* base, 
     const float4 a = __ldg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(base) + i));
     out[0] = a.x; out[1] = a.y; out[2] = a.z; out[3] = a.w;
 }
-template <> __device__ __forceinline__ void load_run<kF16, 4>(const void* base, size_t i, float* out) {
-    const uint2 w = __ldg(reinterpret_cast<const uint2*>(reinterpret_cast<const __half*>(base) + i));
-    const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&w.x));
-    const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&w.y));
-    out[0] = a.x; out[1] = a.y; out[2] = b.x; out[3] = b.y;
-}
 template <> __device__ __forceinline__ void load_run<kF32, 8>(const void* base, size_t i, float* out) {
     load_run<kF32, 4>(base, i, out);
     load_run<kF32, 4>(base, i + 4, out + 4);
@@ -82,6 +76,37 @@ template <> __device__ __forceinline__ void load_run<kF16, 8>(const void* base, 
         out[2 * q + 1] = f.y;
     }
 }
+
+// The same in two steps, so that no conversion waits between the loads of several runs.
+template <int T, int VEC> struct RawRun;
+template <> struct RawRun<kF32, 1> {
+    float v;
+    __device__ __forceinline__ void load(const void* base, size_t i) { v = __ldg(reinterpret_cast<const float*>(base) + i); }
+    __device__ __forceinline__ void get(float* out) const { out[0] = v; }
+};
+template <> struct RawRun<kF32, 4> {
+    float4 v;
+    __device__ __forceinline__ void load(const void* base, size_t i) {
+        v = __ldg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(base) + i));
+    }
+    __device__ __forceinline__ void get(float* out) const { out[0] = v.x; out[1] = v.y; out[2] = v.z; out[3] = v.w; }
+};
+template <> struct RawRun<kF16, 1> {
+    unsigned short v;
+    __device__ __forceinline__ void load(const void* base, size_t i) { v = __ldg(reinterpret_cast<const unsigned short*>(base) + i); }
+    __device__ __forceinline__ void get(float* out) const { out[0] = __half2float(__ushort_as_half(v)); }
+};
+template <> struct RawRun<kF16, 4> {
+    uint2 v;
+    __device__ __forceinline__ void load(const void* base, size_t i) {
+        v = __ldg(reinterpret_cast<const uint2*>(reinterpret_cast<const __half*>(base) + i));
+    }
+    __device__ __forceinline__ void get(float* out) const {
+        const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&v.x));
+        const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&v.y));
+        out[0] = a.x; out[1] = a.y; out[2] = b.x; out[3] = b.y;
+    }
+};
 
 // Store VEC stored values (already rounded to DT) of one row run: the cells
 // and their x-pairs (c[x], c[x+1]); val[VEC] is the value right of the run.
@@ -360,13 +385,15 @@ __global__ void __launch_bounds__(kRowCols * kRowSlices, 2) k_lod(RowsArgs A) {
 // level (1.51 ms against 1.79 for blocks of 9 slices with two barriers per 64
 // column runs, which left memory idle at the barriers; 2.32 against 2.40 ms for
 // FP32 storage; 250^3 FP32, one column per thread, 307 against 419 us). Fewer registers than
-// the five rows need spill (8 blocks per SM: 327 against 302 us at 256^3 FP32); the
-// half as wide FP16 sources want the warps instead.
+// the five rows need spill (8 blocks per SM: 327 against 302 us at 256^3 FP32; FP16 into FP16
+// still gains from 8). The loads are raw: with the conversion of an FP16 source behind
+// each, the next one waited for it (with the next level, 256^3 FP32 from FP16 325 -> 277 us,
+// 512^3 FP16 from FP16 1729 -> 1307; 251^3 FP32 from FP16 435 -> 306).
 constexpr int kQuadThreads = 128;
-constexpr int quad_blocks(int mode, int src) { return mode >= 3 || src == kF16 ? 10 : 5; }
+constexpr int quad_blocks(int mode, int dt, int src) { return mode >= 3 ? 10 : dt == kF16 && src == kF16 ? 8 : 5; }
 
 template <int DT, int MODE, int SRC, int VEC>
-__global__ void __launch_bounds__(kQuadThreads, quad_blocks(MODE, SRC)) k_quads(RowsArgs A) {
+__global__ void __launch_bounds__(kQuadThreads, quad_blocks(MODE, DT, SRC)) k_quads(RowsArgs A) {
     constexpr int kRows = kSub + 1, G = kSub / VEC;          // rows of a quadrant; lanes of a sub-brick
     constexpr bool kNext = (MODE == 2 || MODE == 4) && VEC == 4, kStore = MODE == 0 || MODE == 2;
     __shared__ float s_mn[4][32], s_mx[4][32];
@@ -385,19 +412,23 @@ __global__ void __launch_bounds__(kQuadThreads, quad_blocks(MODE, SRC)) k_quads(
     for (int dz = 0; dz < kRows; ++dz) {
         const int z = z0 + dz;
         float val[kRows][VEC + 1];
+        RawRun<SRC, VEC> raw[kRows];
+        RawRun<SRC, 1> edge[kRows];
         // the slice's rows (rows beyond the grid repeat the last one: no new value)
 #pragma unroll
         for (int dy = 0; dy < kRows; ++dy) {
             const int y = min(y0 + dy, n - 1);
-#pragma unroll
-            for (int q = 0; q <= VEC; ++q) val[dy][q] = 0.0f;
+            raw[dy] = {};
+            edge[dy] = {};
             if (!valid || z >= n) continue;
             const size_t row = (((size_t)v * n + z) * n + y) * n;
-            load_run<SRC, VEC>(A.src, row + X, val[dy]);
-            if (lane == 31 && !last) load_run<SRC, 1>(A.src, row + X + VEC, val[dy] + VEC);
+            raw[dy].load(A.src, row + X);
+            if (lane == 31 && !last) edge[dy].load(A.src, row + X + VEC);
         }
 #pragma unroll
         for (int dy = 0; dy < kRows; ++dy) {
+            raw[dy].get(val[dy]);
+            edge[dy].get(val[dy] + VEC);
 #pragma unroll
             for (int q = 0; q <= VEC; ++q) val[dy][q] = to_stored<DT>(val[dy][q]);
             const float right = __shfl_down_sync(0xffffffffu, val[dy][0], 1);
