@@ -309,7 +309,9 @@ template <int DT>
 __global__ void __launch_bounds__(kHistThreads) k_hist_scalar(const __grid_constant__ HistLaunch A) {
     extern __shared__ float s_edges[];
     __shared__ BinTable T;
-    const int mode = stage_edges<DT>(A, 0, A.naxes, s_edges, T);
+    // (without the check against binary16 values, which the near form here does not need: the table's
+    // staging is a third of a small call, 65^3 FP16 24.5 -> 19.0 us)
+    const int mode = stage_edges<kF32>(A, 0, A.naxes, s_edges, T);
     const float top = guess_top(A.bins);
 
     const int lane = threadIdx.x & 31;
