@@ -1066,9 +1066,9 @@ __global__ void __launch_bounds__(kHistVecThreads, 2) k_hist_bins(const __grid_c
 // counter's top bit: whoever finds it set owns the 2^15, and nobody tries twice. Adds of
 // a warp to one 16-bit counter serialise (the hardware merges adds of 1 to 32-bit ones),
 // so a warp with kSameUnits or more units of a single bin pair each adds those units
-// whole. A constant field at 512^3 FP16, 256 bins: 2138 us with every thread above
-// 2^15 in a compare-and-swap loop, 1347 with the moves as they are, 520 with whole units
-// (32-bit counters: 559); a smooth one 558, now 561.
+// whole (until a step of its batch has fewer: the check would cost smooth fields 1-2 %). A constant field at 512^3 FP16, 256 bins: 2138 us with every thread above
+// 2^15 in a compare-and-swap loop, 1347 with the moves as they are, 506 with whole units
+// (32-bit counters: 559); a smooth one 559, now 545.
 constexpr int kPairThreads = 1024;
 constexpr size_t kPairBytes = (size_t)200 << 10;    // shared memory for the counters of a block
 constexpr unsigned kCountBatch = 8;                 // chunks a warp takes at a time, four lanes each
@@ -1156,17 +1156,19 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_hist_count(CountArgs A) {
                 }
             };
             if (any) load(0, m, a, b);
+            [[maybe_unused]] bool same = true;                   // the batch's steps so far had units of one bin pair
             for (int step = 0; step < 8; ++step) {
                 unsigned mn = 0u, an[kWords] = {}, bn[kWords] = {};
                 if (any && step < 7) load(step + 1, mn, an, bn);
                 constexpr int kPer = 4 / (int)sizeof(BIN), kBits = 8 * (int)sizeof(BIN);
-                if constexpr (!WIDE) {
+                if (!WIDE && same) {
                     // a unit of one bin pair: one add (see above)
                     constexpr unsigned kEach = sizeof(BIN) == 1 ? 0x01010101u : 0x00010001u;
                     unsigned differ = 0u;
 #pragma unroll
                     for (int i = 1; i < kWords; ++i) differ |= (a[0] ^ a[i]) | (b[0] ^ b[i]);
-                    if (__popc(__ballot_sync(kFull, differ == 0u && m != 0u)) >= kSameUnits) {
+                    same = __popc(__ballot_sync(kFull, differ == 0u && m != 0u)) >= kSameUnits;
+                    if (same) {
                         const unsigned x = a[0] & ((1u << kBits) - 1u), y = b[0] & ((1u << kBits) - 1u);
                         if (differ == 0u && m && a[0] == x * kEach && b[0] == y * kEach) {
                             const unsigned k = x * pitch + y, sh = k >= words ? 16u : 0u, count = __popc(m);
