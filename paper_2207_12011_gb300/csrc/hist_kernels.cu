@@ -21,7 +21,7 @@
 // which few can be merged (neighbouring cells of a 256-bin table rarely share a bin
 // pair) and many meet at hot bins. Large grids therefore list the cells' bins in HBM and
 // count them one pair at a time in shared memory (k_hist_count): 512^3 FP16, 6
-// axes, 256 bins, whole shell 1401 -> 557 us; 4 brushed variables 422 -> 313 us;
+// axes, 256 bins, whole shell 1438 -> 537 us; 4 brushed variables 422 -> 313 us;
 // 250^3 264 -> 115 us. Smaller grids, tables that do not fit and calls without scratch
 // add runs of equal bins straight to L2 (see by_pair), on large grids spread over
 // partial histograms that a reduction sums.
