@@ -28,7 +28,7 @@ def field(n, seed, nans):
 
 
 def wide_brush(vol):
-    """Every number of the first variable passes; the second is cut. Half the bounds are near its values."""
+    """Every number of the first variable passes; the second is cut at two of its values."""
     s = vol[1].flatten().sort().values
     return np.array([-1e30, float(s[len(s) // 5])], np.float32), np.array([1e30, float(s[-len(s) // 8])], np.float32), 0b11
 
